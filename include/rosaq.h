@@ -150,8 +150,9 @@ int rosaq_calib_cov(rosaq_ctx *ctx, const void *X, int x_dtype, int64_t n_tokens
  *       subnormal (bits 0x0001) and an infinite one by the largest finite value (0x7bff),
  *   z = clamp(-rint(lo/s), 0, 2^bits-1), stored as +0 when lo >= 0,
  *   code = clamp(rint(w/s) + z, 0, 2^bits-1), all IEEE fp32, ties to even.
- * Allocates the result (*out, release with rosaq_weight_free) and a temporary fp32
- * W' of d_in*d_out floats that is freed before returning.  Synchronizes `stream`.
+ * Allocates the result (*out, release with rosaq_weight_free) from the context's memory pool, which keeps up to 64 MB
+ * of freed operands for reuse and is released with the context.  A rotation with a column permutation may grow the
+ * context workspace (by at most 16 MB, or one 128-column strip of W' in fp32).  Synchronizes `stream`.
  * d_in % 128 == 0 required; d_out >= 1 (padded internally to a multiple of 128).
  */
 int rosaq_quantize(rosaq_ctx *ctx, const void *W, int d_in, int d_out, const rosaq_rot *rot,
@@ -163,8 +164,7 @@ int rosaq_quantize(rosaq_ctx *ctx, const void *W, int d_in, int d_out, const ros
  *   in_scale  DEVICE fp32 [d_in], the diagonal of D; NULL = rosaq_quantize.  The paper gives no rule for D:
  *             it is an input, like R; the caller feeds rosaq_linear the activations x D^-1 (R).
  * W'' = R^T (D W): each product d[i] * W[i][n] is rounded once to fp32, then the chain of rosaq_quantize runs
- * on those values (rot == NULL: W'' = D W).  With rot and in_scale both given a second temporary of
- * d_in*d_out floats is allocated and freed.  Everything else as rosaq_quantize.
+ * on those values (rot == NULL: W'' = D W).  Everything else as rosaq_quantize.
  */
 int rosaq_quantize_scaled(rosaq_ctx *ctx, const void *W, int d_in, int d_out, const rosaq_rot *rot,
                           const float *in_scale, int bits, int group, int k_salient, rosaq_weight **out,

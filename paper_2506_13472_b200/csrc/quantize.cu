@@ -6,248 +6,211 @@
 // intrinsics (__fmaf_rn, __fdiv_rn, ...) so that the compiler can neither contract nor
 // reorder it: the codes must be reproducible bit for bit by a sequential IEEE fp32
 // implementation.
+#include <algorithm>
+
 #include "rosaq_internal.cuh"
 
 namespace rosaq {
 
 // =====================================================================================
-// out[i][n] (+)= sum_k A[k][i] * B[k][n]   -- one fused multiply-add per term, k ascending,
-// a single fp32 accumulator per output started at +0 (the canonical chain of W' = R^T W;
-// also used, with A = B = X, for the Gram matrix of fp32 calibration activations).
-// 128 x 128 output tile per CTA, 256 threads, 8 x 8 outputs per thread, K stepped by 16
-// through shared memory.  Zero padding outside [I) x [N) x [K) is harmless: fma(0, 0, acc)
-// returns acc.
+// The fp32 chain.  out[i][n] = sum_k A[k][i] * B[k][n] as one fused multiply-add per term, k ascending, a single
+// fp32 accumulator per output started at +0: the canonical order of W' = R^T W (and, with A = B = X, the Gram
+// matrix of fp32 calibration activations).  A CTA of 128 threads computes a 128 x 128 tile, 8 x 16 outputs per
+// thread, K stepped by 8 through two shared-memory buffers.  Zero padding is harmless: fma(0, 0, acc) = acc.
+//
+// Bound: the fp32 pipe (one multiply-add per lane and cycle, 128 lanes per SM) -- as long as the operands keep up.
+// A 16-byte shared-memory load occupies the SM's load path for four cycles whatever it broadcasts, so an 8 x 8 thread
+// tile (four loads per 64 multiply-adds) is bound by its loads; an 8 x 16 one (six per 128) is not.  Scalar
+// multiply-adds then lose a quarter of their issue cycles to register-port stalls (3.27 ms in the example below);
+// fma.rn.f32x2, two independent IEEE multiply-adds on register pairs, does not and leaves issue slots free.
+// Measured at 4096 -> 4096 INT4, dense R, the rotation and the quantization: 3.41 ms (41 TFLOP/s; 8 x 8 scalar per
+// thread, one buffer, W' through global memory) before, 2.59 ms (53 TFLOP/s) after.
 // =====================================================================================
+constexpr int kBM = 128, kBN = 128, kBK = 8;
+constexpr int kFmaThreads = 128;
+constexpr int kFmaBufFloats = kBK * (kBM + kBN);
+constexpr int kTilePitch = 132;                                  // floats; the finished tile reuses the buffers
+constexpr int kFmaSmemBytes = 128 * kTilePitch * 4;
+
+// this thread's outputs: rows ty * 4 + {0..3} and 64 + ty * 4 + {0..3}; columns tx * 4 + {0..3} of each 32-column
+// quarter.  A warp covers 4 x 8 of the 16 x 8 (ty, tx).
+struct FmaThread {
+  int ty, tx;
+  __device__ FmaThread() {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ty = warp * 4 + (lane >> 3);
+    tx = lane & 7;
+  }
+  __device__ int row(int ia) const { return ia < 4 ? ty * 4 + ia : 64 + ty * 4 + ia - 4; }
+};
+
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ float4 unpack4(unsigned long long a, unsigned long long b) {
+  float4 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(a));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.z), "=f"(v.w) : "l"(b));
+  return v;
+}
+// two independent IEEE fp32 multiply-adds
+__device__ __forceinline__ void fma2(unsigned long long &c, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+
+// Four values of one operand row as they come from memory.  They are converted when they are stored to shared memory,
+// one K step after the load was issued: converted in place they would stall the warp for the whole latency.
 template <typename T>
-__device__ __forceinline__ float to_f32(T v);
+struct Raw4;
 template <>
-__device__ __forceinline__ float to_f32<float>(float v) { return v; }
+struct Raw4<float> {
+  float4 v;
+  __device__ __forceinline__ void zero() { v = make_float4(0.f, 0.f, 0.f, 0.f); }
+  __device__ __forceinline__ void load4(const float *p) { v = *reinterpret_cast<const float4 *>(p); }
+  __device__ __forceinline__ void set(int e, float x) { reinterpret_cast<float *>(&v)[e] = x; }
+  __device__ __forceinline__ float4 expand() const { return v; }
+};
 template <>
-__device__ __forceinline__ float to_f32<__half>(__half v) { return __half2float(v); }
+struct Raw4<__half> {
+  __half2 v[2];
+  __device__ __forceinline__ void zero() { v[0] = v[1] = __float2half2_rn(0.f); }
+  __device__ __forceinline__ void load4(const __half *p) { *reinterpret_cast<uint2 *>(v) = *reinterpret_cast<const uint2 *>(p); }
+  __device__ __forceinline__ void set(int e, __half x) {
+    if (e & 1) v[e >> 1].y = x;
+    else v[e >> 1].x = x;
+  }
+  __device__ __forceinline__ float4 expand() const {
+    const float2 a = __half22float2(v[0]), b = __half22float2(v[1]);
+    return make_float4(a.x, a.y, b.x, b.y);
+  }
+};
 
-constexpr int kBM = 128, kBN = 128, kBK = 16;
-
-template <typename TA, typename TB, bool kAccumulate>
-__global__ void __launch_bounds__(256)
-gemm_tn_fma_kernel(const TA *__restrict__ A, long long lda, long long strideA,
-                   const TB *__restrict__ B, long long ldb, long long strideB,
-                   float *__restrict__ out, long long ldo, long long strideO,
-                   int I, int N, long long K) {
-  __shared__ __align__(16) float As[kBK][kBM];
-  __shared__ __align__(16) float Bs[kBK][kBN];
-  A += blockIdx.z * strideA;
-  B += blockIdx.z * strideB;
-  out += blockIdx.z * strideO;
-  const int i0 = blockIdx.y * kBM, n0 = blockIdx.x * kBN;
-  const int tid = threadIdx.x;
-  const int ty = tid >> 4, tx = tid & 15;
-  // loader mapping: 16 rows x 128 columns, 8 consecutive columns per thread
-  const int lr = tid >> 4, lc = (tid & 15) * 8;
-
-  float acc[8][8];
+// The K loop.  fetch_a(k, c, raw) / fetch_b(k, c, raw) deliver A[k][c .. c + 3] / B[k][c .. c + 3] (tile columns; 0 outside
+// the operand, also for k >= K); with kScaled row k of B is multiplied by fetch_s(k), one rounding per product.
+// acc[ia][2 q + e] is row(ia), columns 32 q + tx * 4 + 2 e, + 1.
+template <typename TA, typename TB, bool kScaled, typename FA, typename FB, typename FS>
+__device__ __forceinline__ void fma_tile(float *smem, int K, const FmaThread &ft, FA fetch_a, FB fetch_b, FS fetch_s, unsigned long long acc[8][8]) {
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
+  for (int ia = 0; ia < 8; ++ia)
 #pragma unroll
-    for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
-
-  float ra[8], rb[8];
-  auto fetch = [&](long long k0) {
-    long long k = k0 + lr;
+    for (int ib = 0; ib < 8; ++ib) acc[ia][ib] = 0ull;
+  const int lr = threadIdx.x >> 5, lc = (threadIdx.x & 31) * 4;      // loader: rows lr and lr + 4 of the K step, four columns
+  Raw4<TA> ra[2];
+  Raw4<TB> rb[2];
+  float rs[2];
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      int i = i0 + lc + e, n = n0 + lc + e;
-      ra[e] = (k < K && i < I) ? to_f32<TA>(A[k * lda + i]) : 0.0f;
-      rb[e] = (k < K && n < N) ? to_f32<TB>(B[k * ldb + n]) : 0.0f;
+    for (int h = 0; h < 2; ++h) {
+      fetch_a(k0 + lr + 4 * h, lc, ra[h]);
+      fetch_b(k0 + lr + 4 * h, lc, rb[h]);
+      if (kScaled) rs[h] = fetch_s(k0 + lr + 4 * h);
+    }
+  };
+  auto put = [&](float *buf) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      *reinterpret_cast<float4 *>(buf + (lr + 4 * h) * kBM + lc) = ra[h].expand();
+      float4 b = rb[h].expand();
+      if (kScaled) b = make_float4(__fmul_rn(rs[h], b.x), __fmul_rn(rs[h], b.y), __fmul_rn(rs[h], b.z), __fmul_rn(rs[h], b.w));
+      *reinterpret_cast<float4 *>(buf + kBK * kBM + (lr + 4 * h) * kBN + lc) = b;
     }
   };
   fetch(0);
-  for (long long k0 = 0; k0 < K; k0 += kBK) {
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      As[lr][lc + e] = ra[e];
-      Bs[lr][lc + e] = rb[e];
-    }
-    __syncthreads();
-    if (k0 + kBK < K) fetch(k0 + kBK);
+  put(smem);
+  __syncthreads();
+  int cur = 0;
+  for (int k0 = 0; k0 < K; k0 += kBK) {
+    const bool more = k0 + kBK < K;
+    if (more) fetch(k0 + kBK);
+    const float *as = smem + cur * kFmaBufFloats + ft.ty * 4, *bs = smem + cur * kFmaBufFloats + kBK * kBM + ft.tx * 4;
 #pragma unroll
     for (int kk = 0; kk < kBK; ++kk) {
-      float a[8], b[8];
-      *reinterpret_cast<float4 *>(&a[0]) = *reinterpret_cast<const float4 *>(&As[kk][ty * 4]);
-      *reinterpret_cast<float4 *>(&a[4]) = *reinterpret_cast<const float4 *>(&As[kk][64 + ty * 4]);
-      *reinterpret_cast<float4 *>(&b[0]) = *reinterpret_cast<const float4 *>(&Bs[kk][tx * 4]);
-      *reinterpret_cast<float4 *>(&b[4]) = *reinterpret_cast<const float4 *>(&Bs[kk][64 + tx * 4]);
+      __align__(16) float a[8];
+      ulonglong2 b[4];
 #pragma unroll
-      for (int ia = 0; ia < 8; ++ia)
+      for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(a + 4 * h) = *reinterpret_cast<const float4 *>(as + kk * kBM + 64 * h);
 #pragma unroll
-        for (int ib = 0; ib < 8; ++ib) acc[ia][ib] = __fmaf_rn(a[ia], b[ib], acc[ia][ib]);
+      for (int q = 0; q < 4; ++q) b[q] = *reinterpret_cast<const ulonglong2 *>(bs + kk * kBN + 32 * q);
+#pragma unroll
+      for (int ia = 0; ia < 8; ++ia) {
+        const unsigned long long aa = pack2(a[ia], a[ia]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          fma2(acc[ia][2 * q], aa, b[q].x);
+          fma2(acc[ia][2 * q + 1], aa, b[q].y);
+        }
+      }
     }
+    if (more) put(smem + (cur ^ 1) * kFmaBufFloats);
+    __syncthreads();
+    cur ^= 1;
   }
+}
+
+__device__ __forceinline__ void store_tile_smem(float *tile, const FmaThread &ft, const unsigned long long acc[8][8]) {
 #pragma unroll
-  for (int ia = 0; ia < 8; ++ia) {
-    int i = i0 + (ia < 4 ? ty * 4 + ia : 64 + ty * 4 + ia - 4);
-    if (i >= I) continue;
+  for (int ia = 0; ia < 8; ++ia)
 #pragma unroll
-    for (int ib = 0; ib < 8; ++ib) {
-      int n = n0 + (ib < 4 ? tx * 4 + ib : 64 + tx * 4 + ib - 4);
-      if (n >= N) continue;
-      float *o = out + (long long)i * ldo + n;
-      *o = kAccumulate ? __fadd_rn(*o, acc[ia][ib]) : acc[ia][ib];
-    }
-  }
-}
-
-// Block-diagonal (head-wise, Eq. 6) and/or permuted rotation: output row j takes column
-// perm[j] of blockdiag(Rb); the chain runs over the dh rows of that column's block only.
-// One CTA per output row, threads along the output columns.
-template <typename TQ, typename TW>
-__global__ void __launch_bounds__(256)
-rotate_weights_blockdiag_kernel(const TQ *__restrict__ Rb, int d_in, int dh, const int32_t *__restrict__ perm,
-                                const TW *__restrict__ W, int d_out, float *__restrict__ Wp) {
-  extern __shared__ float rcol[];  // [dh]
-  const int j = blockIdx.x;
-  const int p = perm ? perm[j] : j;
-  const int h = p / dh, c = p % dh;
-  const TQ *R = Rb + (long long)h * dh * dh;
-  for (int k = threadIdx.x; k < dh; k += blockDim.x) rcol[k] = to_f32<TQ>(R[(long long)k * dh + c]);
-  __syncthreads();
-  const TW *Wb = W + (long long)h * dh * d_out;
-  for (int n = blockIdx.y * blockDim.x + threadIdx.x; n < d_out; n += gridDim.y * blockDim.x) {
-    float acc = 0.0f;
-    for (int k = 0; k < dh; ++k) acc = __fmaf_rn(rcol[k], to_f32<TW>(Wb[(long long)k * d_out + n]), acc);
-    Wp[(long long)j * d_out + n] = acc;
-  }
-}
-
-__global__ void cast_weights_kernel(const __half *__restrict__ W, long long n, float *__restrict__ Wp) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long stride = (long long)gridDim.x * blockDim.x;
-  for (; i < n; i += stride) Wp[i] = __half2float(W[i]);
-}
-
-// D W of the scaled (AWQ-style) variant: out[i][n] = d[i] * W[i][n], one fp32 rounding per product
-__global__ void scale_rows_kernel(const __half *__restrict__ W, const float *__restrict__ d, int d_out, long long n,
-                                  float *__restrict__ out) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long stride = (long long)gridDim.x * blockDim.x;
-  for (; i < n; i += stride) out[i] = __fmul_rn(d[i / d_out], __half2float(W[i]));
-}
-
-template <typename TW>
-static int rotate_weights_typed(const void *q, int q_is_f32, int d_in, int n_blocks, const int32_t *perm, const TW *W,
-                                int d_out, float *Wp, cudaStream_t s) {
-  if (n_blocks == 1 && perm == nullptr && q_is_f32) {
-    dim3 grid((d_out + kBN - 1) / kBN, (d_in + kBM - 1) / kBM, 1);
-    gemm_tn_fma_kernel<float, TW, false><<<grid, 256, 0, s>>>(
-        static_cast<const float *>(q), d_in, 0, W, d_out, 0, Wp, d_out, 0, d_in, d_out, d_in);
-  } else {
-    int dh = d_in / n_blocks;
-    size_t smem = sizeof(float) * dh;
-    if (smem > 48 * 1024) {
-      cudaError_t e;
-      if (q_is_f32)
-        e = cudaFuncSetAttribute(rotate_weights_blockdiag_kernel<float, TW>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      else
-        e = cudaFuncSetAttribute(rotate_weights_blockdiag_kernel<__half, TW>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
-    }
-    dim3 grid(d_in, min((d_out + 255) / 256, 8));
-    if (q_is_f32)
-      rotate_weights_blockdiag_kernel<float, TW><<<grid, 256, smem, s>>>(static_cast<const float *>(q), d_in, dh,
-                                                                           perm, W, d_out, Wp);
-    else
-      rotate_weights_blockdiag_kernel<__half, TW><<<grid, 256, smem, s>>>(static_cast<const __half *>(q), d_in, dh,
-                                                                            perm, W, d_out, Wp);
-  }
-  return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
-}
-
-int launch_rotate_weights(const void *q, int q_is_f32, int d_in, int n_blocks, const int32_t *perm,
-                          const __half *W, int d_out, float *Wp, cudaStream_t s) {
-  return rotate_weights_typed<__half>(q, q_is_f32, d_in, n_blocks, perm, W, d_out, Wp, s);
-}
-
-// the same chain on a weight that is already fp32 (the scaled weight D W)
-int launch_rotate_weights_w32(const void *q, int q_is_f32, int d_in, int n_blocks, const int32_t *perm,
-                              const float *W32, int d_out, float *Wp, cudaStream_t s) {
-  return rotate_weights_typed<float>(q, q_is_f32, d_in, n_blocks, perm, W32, d_out, Wp, s);
-}
-
-int launch_scale_rows(const __half *W, const float *in_scale, int d_in, int d_out, float *out, cudaStream_t s) {
-  long long n = (long long)d_in * d_out;
-  long long want = (n + 255) / 256;
-  int blocks = (int)(want < 148 * 16 ? want : 148 * 16);
-  scale_rows_kernel<<<blocks, 256, 0, s>>>(W, in_scale, d_out, n, out);
-  return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
-}
-
-int launch_cast_weights(const __half *W, int d_in, int d_out, float *Wp, cudaStream_t s) {
-  long long n = (long long)d_in * d_out;
-  long long want = (n + 255) / 256;
-  int blocks = (int)(want < 148 * 16 ? want : 148 * 16);
-  cast_weights_kernel<<<blocks, 256, 0, s>>>(W, n, Wp);
-  return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
-}
-
-// Gram matrix on CUDA cores (fp32 products, fp32 accumulate): exact-product path for fp32
-// calibration activations and the fallback for shapes the tensor-core kernel does not take.
-int launch_cov_fma(const void *X, int x_dtype, long long n_tokens, int d, long long ldx, int n_blocks, float *C,
-                   cudaStream_t s) {
-  int dh = d / n_blocks;
-  dim3 grid((dh + kBN - 1) / kBN, (dh + kBM - 1) / kBM, n_blocks);
-  if (x_dtype == ROSAQ_F32) {
-    const float *x = static_cast<const float *>(X);
-    gemm_tn_fma_kernel<float, float, true><<<grid, 256, 0, s>>>(x, ldx, dh, x, ldx, dh, C, dh, (long long)dh * dh,
-                                                                 dh, dh, n_tokens);
-  } else {
-    const __half *x = static_cast<const __half *>(X);
-    gemm_tn_fma_kernel<__half, __half, true><<<grid, 256, 0, s>>>(x, ldx, dh, x, ldx, dh, C, dh,
-                                                                   (long long)dh * dh, dh, dh, n_tokens);
-  }
-  return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
+    for (int q = 0; q < 4; ++q)
+      *reinterpret_cast<float4 *>(tile + ft.row(ia) * kTilePitch + 32 * q + ft.tx * 4) =
+          unpack4(acc[ia][2 * q], acc[ia][2 * q + 1]);
 }
 
 // =====================================================================================
-// Eq. 3 / Section 3.3: salient rows -> fp16; other groups -> asymmetric min/max RTN codes,
-// written straight into the tiled layout.  One thread per (group, output column).
+// Eq. 3 / Section 3.3: one 128 x 128 tile of W' in shared memory = one group of 128 output columns.  Salient rows ->
+// fp16; other groups -> asymmetric min/max RTN codes, written straight into the tiled layout.  kParts
+// threads per column (a CTA of 128 * kParts threads), each with its share of the rows; the parts' extremes are joined in
+// row order through `ends`, so a tie between zeros of either sign falls as in one scan.
 // =====================================================================================
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   return (uint32_t)__half_as_ushort(__float2half_rn(lo)) | ((uint32_t)__half_as_ushort(__float2half_rn(hi)) << 16);
 }
 
-template <int kBits>
-__global__ void __launch_bounds__(kTileN)
-quant_pack_kernel(const float *__restrict__ Wp, TiledOperand t) {
-  const int nt = blockIdx.x, g = blockIdx.y, nl = threadIdx.x;
-  const int n = nt * kTileN + nl;
-  const bool live = n < t.d_out;
-  uint8_t *tile = t.blob + tile_offset(t, nt, g);
-  const float *col = Wp + (long long)g * kGroup * t.d_out + n;
+template <int kBits, int kParts>
+__device__ __forceinline__ void quant_tile(const float *tile, float2 *ends, const TiledOperand &t, int nt, int g) {
+  constexpr int kRows = kGroup / kParts;
+  static_assert(kRows % 32 == 0, "a part holds whole INT3 sets");
+  const int nl = threadIdx.x & 127, part = threadIdx.x >> 7, k0 = part * kRows;
+  const bool live = nt * kTileN + nl < t.d_out;
+  uint8_t *out = t.blob + tile_offset(t, nt, g);
+  const float *col = tile + k0 * kTilePitch + nl;
   if (g < t.g_fp16) {
-    for (int k8 = 0; k8 < kGroup; k8 += 8) {
+    for (int k8 = 0; k8 < kRows; k8 += 8) {
       float v[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = live ? col[(long long)(k8 + e) * t.d_out] : 0.0f;
-      *reinterpret_cast<uint4 *>(tile + fp16_tile_byte(k8, nl)) =
+      for (int e = 0; e < 8; ++e) v[e] = live ? col[(k8 + e) * kTilePitch] : 0.0f;
+      *reinterpret_cast<uint4 *>(out + fp16_tile_byte(k0 + k8, nl)) =
           make_uint4(pack_half2(v[0], v[1]), pack_half2(v[2], v[3]), pack_half2(v[4], v[5]), pack_half2(v[6], v[7]));
     }
     return;
   }
-  constexpr int kWords = kBits == 4 ? 16 : 12;
+  float lo = col[0], hi = col[0];
+#pragma unroll 16
+  for (int k = 1; k < kRows; ++k) {
+    const float w = col[k * kTilePitch];
+    lo = w < lo ? w : lo;
+    hi = w > hi ? w : hi;
+  }
+  if (kParts > 1) {
+    ends[threadIdx.x] = make_float2(lo, hi);
+    __syncthreads();
+    lo = ends[nl].x, hi = ends[nl].y;
+#pragma unroll
+    for (int q = 1; q < kParts; ++q) {
+      const float2 e = ends[q * 128 + nl];
+      lo = e.x < lo ? e.x : lo;
+      hi = e.y > hi ? e.y : hi;
+    }
+  }
+  constexpr int kWords = (kBits == 4 ? 16 : 12) / kParts;
   uint32_t words[kWords];
 #pragma unroll
   for (int w = 0; w < kWords; ++w) words[w] = 0;
   __half sh = __ushort_as_half(0), zh = __ushort_as_half(0);
   if (live) {
     const float qmax = (float)((1 << kBits) - 1);
-    float lo = col[0], hi = col[0];
-    for (int k = 1; k < kGroup; ++k) {
-      float w = col[(long long)k * t.d_out];
-      lo = w < lo ? w : lo;
-      hi = w > hi ? w : hi;
-    }
     float range = __fsub_rn(hi, lo);
     if (range < 1e-5f) range = 1e-5f;
     unsigned short sb = __half_as_ushort(__float2half_rn(__fdiv_rn(range, qmax)));
@@ -259,23 +222,260 @@ quant_pack_kernel(const float *__restrict__ Wp, TiledOperand t) {
     if (z <= 0.0f) z = 0.0f;
     if (z > qmax) z = qmax;
     zh = __float2half_rn(z);
-#pragma unroll 8
-    for (int k = 0; k < kGroup; ++k) {
-      float q = __fadd_rn(rintf(__fdiv_rn(col[(long long)k * t.d_out], sf)), z);
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+      float q = __fadd_rn(rintf(__fdiv_rn(col[k * kTilePitch], sf)), z);
       if (q < 0.0f) q = 0.0f;
       if (q > qmax) q = qmax;
       put_code<kBits>(words, k, (uint32_t)q);
     }
   }
-  store_quant_tile_column<kBits>(tile, nl, words, sh, zh);
+  if (kParts == 1) {
+    store_quant_tile_column<kBits>(out, nl, words, sh, zh);
+    return;
+  }
+  if (kBits == 4) {
+#pragma unroll
+    for (int j = 0; j < kWords / 4; ++j)
+      *reinterpret_cast<uint4 *>(out + ((part * kWords / 4 + j) * kTileN + nl) * 16) =
+          make_uint4(words[4 * j], words[4 * j + 1], words[4 * j + 2], words[4 * j + 3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) *reinterpret_cast<uint32_t *>(out + int3_word_byte(part * kWords + j, nl)) = words[j];
+  }
+  if (part == 0)
+    *reinterpret_cast<uint32_t *>(out + quant_code_bytes(kBits) + nl * 4) =
+        (uint32_t)__half_as_ushort(sh) | ((uint32_t)__half_as_ushort(zh) << 16);
 }
 
-int launch_quant_pack(const float *Wp, const TiledOperand &t, cudaStream_t s) {
-  dim3 grid(t.n_tiles, groups_per_tile(t));
+struct RotateArgs {
+  const void *q;            // [n_blocks][dh][dh]
+  const int32_t *perm;      // output row j takes column perm[j] of blockdiag(q), or NULL
+  const int32_t *inv;       // its inverse (kSpill only), or NULL
+  const __half *W;          // [d_in][d_out]
+  const float *in_scale;    // [d_in]: the chain runs on the fp32 products in_scale[i] * W[i][n]; or NULL
+  float *spill;             // kSpill: W' columns [n_base, n_base + spill_cols), row-major
+  int d_in, d_out, dh, n_base, spill_cols;
+};
+
+// W' = R^T W for one 128 x 128 tile, then either quantized and packed from shared memory (kSpill = false: the tile is
+// a whole group, so W' never reaches global memory), or, when the rows of a group come from different head blocks (a
+// block-diagonal R with a column order), stored to a slab of W' that quant_tile_kernel reads.
+template <typename TQ, int kBits, bool kSpill, bool kScaled>
+__global__ void __launch_bounds__(kFmaThreads, 2)
+rotate_tile_kernel(const RotateArgs a, const TiledOperand t) {
+  extern __shared__ __align__(16) float smem[];
+  const FmaThread ft;
+  const int nt = blockIdx.x, n0 = a.n_base + nt * kBN;
+  // rows of the tile: output channels of group blockIdx.y, or (kSpill) source columns of one head block
+  const int per_block = (a.dh + kBM - 1) / kBM;
+  const int h = kSpill ? (int)blockIdx.y / per_block : (a.perm ? 0 : (int)blockIdx.y * kBM / a.dh);
+  const int c0 = kSpill ? ((int)blockIdx.y % per_block) * kBM : (int)blockIdx.y * kBM - h * a.dh;   // first column inside the block
+  const TQ *R = static_cast<const TQ *>(a.q) + (long long)h * a.dh * a.dh;
+  const __half *W = a.W + (long long)h * a.dh * a.d_out;
+  const int32_t *perm = kSpill ? nullptr : a.perm;
+  int pc[4];                                                         // the four columns of R this thread loads
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int i = (threadIdx.x & 31) * 4 + e + c0;
+    pc[e] = i >= a.dh ? -1 : (perm ? perm[i] : i);
+  }
+  const bool a_vec = perm == nullptr && a.dh % 8 == 0, b_vec = a.d_out % 8 == 0;
+  auto fetch_a = [&](int k, int, Raw4<TQ> &raw) {
+    if (k < a.dh && a_vec && pc[3] >= 0) {
+      raw.load4(R + (long long)k * a.dh + pc[0]);
+      return;
+    }
+    raw.zero();
+    if (k < a.dh)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (pc[e] >= 0) raw.set(e, R[(long long)k * a.dh + pc[e]]);
+  };
+  auto fetch_b = [&](int k, int c, Raw4<__half> &raw) {
+    const int n = n0 + c;
+    if (k < a.dh && b_vec && n + 3 < a.d_out) {
+      raw.load4(W + (long long)k * a.d_out + n);
+      return;
+    }
+    raw.zero();
+    if (k < a.dh)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (n + e < a.d_out) raw.set(e, W[(long long)k * a.d_out + n + e]);
+  };
+  const float *ds = kScaled ? a.in_scale + (long long)h * a.dh : nullptr;
+  unsigned long long acc[8][8];
+  fma_tile<TQ, __half, kScaled>(smem, a.dh, ft, fetch_a, fetch_b, [&](int k) { return k < a.dh ? ds[k] : 0.f; }, acc);
+  if (!kSpill) {
+    store_tile_smem(smem, ft, acc);                                  // (the K loop ends with a barrier)
+    __syncthreads();
+    quant_tile<kBits, 1>(smem, nullptr, t, nt, blockIdx.y);
+  } else {
+#pragma unroll
+    for (int ia = 0; ia < 8; ++ia) {
+      const int c = c0 + ft.row(ia);
+      if (c >= a.dh) continue;
+      const int p = h * a.dh + c, j = a.inv ? a.inv[p] : p;
+      float *dst = a.spill + (long long)j * a.spill_cols + nt * kBN + ft.tx * 4;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<float4 *>(dst + 32 * q) = unpack4(acc[ia][2 * q], acc[ia][2 * q + 1]);
+    }
+  }
+}
+
+// Quantizes and packs tiles whose W' is already there: a slab of fp32 W' (spill), or no rotation at all, W or D W
+// (one fp32 rounding per product).  Bound: HBM (2 bytes per weight in, half a byte out).
+constexpr int kQuantParts = 4, kQuantThreads = 128 * kQuantParts;
+constexpr int kQuantSmemBytes = kFmaSmemBytes + kQuantThreads * (int)sizeof(float2);
+
+template <int kBits>
+__global__ void __launch_bounds__(kQuantThreads, 3)
+quant_tile_kernel(const float *__restrict__ spill, const __half *__restrict__ W, const float *__restrict__ in_scale, int nt0,
+                  int spill_cols, const TiledOperand t) {
+  extern __shared__ __align__(16) float tile[];
+  const int nt = nt0 + blockIdx.x, g = blockIdx.y;
+  const int lr = threadIdx.x >> 4, lc = (threadIdx.x & 15) * 8;      // 32 rows per step, eight columns per thread
+  const int n = nt * kTileN + lc;
+#pragma unroll
+  for (int r0 = 0; r0 < kGroup; r0 += kQuantThreads / 16) {
+    const long long i = (long long)g * kGroup + r0 + lr;
+    float v[8];
+    if (spill) {
+      const float *src = spill + i * spill_cols + blockIdx.x * kTileN + lc;
+      *reinterpret_cast<float4 *>(v) = *reinterpret_cast<const float4 *>(src);
+      *reinterpret_cast<float4 *>(v + 4) = *reinterpret_cast<const float4 *>(src + 4);
+    } else {
+      if (t.d_out % 8 == 0 && n + 7 < t.d_out) {
+        __align__(16) __half r[8];
+        *reinterpret_cast<uint4 *>(r) = *reinterpret_cast<const uint4 *>(W + i * t.d_out + n);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = __half2float(r[e]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = n + e < t.d_out ? __half2float(W[i * t.d_out + n + e]) : 0.f;
+      }
+      if (in_scale) {
+        const float d = in_scale[i];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = __fmul_rn(d, v[e]);
+      }
+    }
+    float *dst = tile + (r0 + lr) * kTilePitch + lc;
+    *reinterpret_cast<float4 *>(dst) = *reinterpret_cast<const float4 *>(v);
+    *reinterpret_cast<float4 *>(dst + 4) = *reinterpret_cast<const float4 *>(v + 4);
+  }
+  __syncthreads();
+  quant_tile<kBits, kQuantParts>(tile, reinterpret_cast<float2 *>(tile + kGroup * kTilePitch), t, nt, g);
+}
+
+template <typename K>
+static bool allow_smem(K kern, int bytes) {
+  // (a per-device attribute; setting it again is a cheap no-op and these calls are offline)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess) return true;
+  (void)cudaGetLastError();
+  return false;
+}
+
+template <typename TQ, int kBits, bool kScaled>
+static int rotate_quantize_typed(const RotateArgs &args, int n_blocks, const TiledOperand &t, cudaStream_t s) {
+  RotateArgs a = args;
+  const auto fused = rotate_tile_kernel<TQ, kBits, false, kScaled>, spilling = rotate_tile_kernel<TQ, kBits, true, kScaled>;
+  const auto quant = quant_tile_kernel<kBits>;
+  if (!allow_smem(fused, kFmaSmemBytes) || !allow_smem(spilling, kFmaSmemBytes) || !allow_smem(quant, kQuantSmemBytes)) return ROSAQ_ERR_CUDA;
+  const int groups = groups_per_tile(t);
+  if (!a.q) {
+    quant<<<dim3(t.n_tiles, groups), kQuantThreads, kQuantSmemBytes, s>>>(nullptr, a.W, a.in_scale, 0, 0, t);
+  } else if (n_blocks == 1 || (a.perm == nullptr && a.dh % kGroup == 0)) {
+    fused<<<dim3(t.n_tiles, groups), kFmaThreads, kFmaSmemBytes, s>>>(a, t);
+  } else {
+    const int tiles_max = a.spill_cols / kTileN, row_tiles = n_blocks * ((a.dh + kBM - 1) / kBM);
+    for (int nt0 = 0; nt0 < t.n_tiles; nt0 += tiles_max) {
+      const int nts = std::min(tiles_max, t.n_tiles - nt0);
+      a.n_base = nt0 * kTileN;
+      spilling<<<dim3(nts, row_tiles), kFmaThreads, kFmaSmemBytes, s>>>(a, t);
+      quant<<<dim3(nts, groups), kQuantThreads, kQuantSmemBytes, s>>>(a.spill, nullptr, nullptr, nt0, a.spill_cols, t);
+    }
+  }
+  return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
+}
+
+// Slab of W' that launch_rotate_quantize wants in `spill`: 16 MB of columns (L2-resident, whatever the weight's size), at
+// least one column tile; 0 when the call needs none.
+size_t rotate_quantize_spill_bytes(int d_in, int d_out, int n_blocks, bool perm) {
+  if (n_blocks <= 1 || (!perm && d_in / n_blocks % kGroup == 0)) return 0;
+  const size_t tile = sizeof(float) * (size_t)d_in * kTileN, most = size_t(16) << 20;
+  const size_t tiles = most / tile < 1 ? 1 : most / tile, all = (size_t)(d_out + kTileN - 1) / kTileN;
+  return tile * (tiles < all ? tiles : all);
+}
+
+int launch_rotate_quantize(const void *q, int q_is_f32, int n_blocks, const int32_t *perm, const int32_t *inv, const __half *W,
+                           const float *in_scale, float *spill, size_t spill_bytes, const TiledOperand &t, cudaStream_t s) {
+  RotateArgs a{};
+  a.q = q, a.perm = perm, a.inv = inv, a.W = W, a.in_scale = in_scale, a.spill = spill;
+  a.d_in = t.d_in, a.d_out = t.d_out, a.dh = q ? t.d_in / n_blocks : t.d_in;
+  a.spill_cols = (int)(spill_bytes / (sizeof(float) * (size_t)t.d_in)) / kTileN * kTileN;
+  auto run = [&](auto f32, auto f16) { return (q && !q_is_f32 ? f16 : f32)(a, n_blocks, t, s); };
   if (t.bits == 3)
-    quant_pack_kernel<3><<<grid, kTileN, 0, s>>>(Wp, t);
-  else
-    quant_pack_kernel<4><<<grid, kTileN, 0, s>>>(Wp, t);
+    return in_scale ? run(rotate_quantize_typed<float, 3, true>, rotate_quantize_typed<__half, 3, true>)
+                    : run(rotate_quantize_typed<float, 3, false>, rotate_quantize_typed<__half, 3, false>);
+  return in_scale ? run(rotate_quantize_typed<float, 4, true>, rotate_quantize_typed<__half, 4, true>)
+                  : run(rotate_quantize_typed<float, 4, false>, rotate_quantize_typed<__half, 4, false>);
+}
+
+// Gram matrix on CUDA cores (fp32 products, fp32 accumulate): exact-product path for fp32 calibration activations and
+// the fallback for shapes the tensor-core kernel does not take.  Only tiles of the lower triangle are computed; an
+// off-diagonal tile is also added, transposed, to the mirrored position (products commute and both chains run over the
+// tokens in the same order, so the mirrored bits are those a tile of its own would produce).
+template <typename T>
+__global__ void __launch_bounds__(kFmaThreads, 2)
+gram_fma_kernel(const T *__restrict__ X, long long ldx, int dh, float *__restrict__ C, int K) {
+  extern __shared__ __align__(16) float tile[];
+  const FmaThread ft;
+  int bi = 0;
+  while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
+  const int bj = blockIdx.x - bi * (bi + 1) / 2;
+  const int i0 = bi * kBM, n0 = bj * kBN;
+  X += (long long)blockIdx.y * dh;
+  C += (long long)blockIdx.y * dh * dh;
+  auto fetch = [&](int k, int c, Raw4<T> &raw) {                     // (dh and ldx are multiples of 8, X is 16-byte aligned)
+    if (k < K && c + 3 < dh) raw.load4(X + (long long)k * ldx + c);
+    else raw.zero();
+  };
+  unsigned long long acc[8][8];
+  fma_tile<T, T, false>(
+      tile, K, ft, [&](int k, int c, Raw4<T> &raw) { fetch(k, i0 + c, raw); },
+      [&](int k, int c, Raw4<T> &raw) { fetch(k, n0 + c, raw); }, [](int) { return 0.f; }, acc);
+  store_tile_smem(tile, ft, acc);
+  __syncthreads();
+  const int c4 = (threadIdx.x & 31) * 4, r_first = threadIdx.x >> 5;
+  auto add4 = [](float *dst, float4 v) {
+    const float4 o = *reinterpret_cast<const float4 *>(dst);
+    *reinterpret_cast<float4 *>(dst) = make_float4(__fadd_rn(o.x, v.x), __fadd_rn(o.y, v.y), __fadd_rn(o.z, v.z), __fadd_rn(o.w, v.w));
+  };
+  if (n0 + c4 < dh)
+    for (int r = r_first; r < kBM && i0 + r < dh; r += 4)
+      add4(C + (long long)(i0 + r) * dh + n0 + c4, *reinterpret_cast<const float4 *>(tile + r * kTilePitch + c4));
+  if (bi != bj && i0 + c4 < dh)
+    for (int r = r_first; r < kBN && n0 + r < dh; r += 4) {
+      const float *tc = tile + c4 * kTilePitch + r;
+      add4(C + (long long)(n0 + r) * dh + i0 + c4, make_float4(tc[0], tc[kTilePitch], tc[2 * kTilePitch], tc[3 * kTilePitch]));
+    }
+}
+
+int launch_cov_fma(const void *X, int x_dtype, long long n_tokens, int d, long long ldx, int n_blocks, float *C,
+                   cudaStream_t s) {
+  const int dh = d / n_blocks, nb = (dh + kBM - 1) / kBM;
+  const dim3 grid(nb * (nb + 1) / 2, n_blocks);
+  if (!allow_smem(gram_fma_kernel<float>, kFmaSmemBytes) || !allow_smem(gram_fma_kernel<__half>, kFmaSmemBytes)) return ROSAQ_ERR_CUDA;
+  for (long long t0 = 0; t0 < n_tokens; t0 += 1ll << 30) {           // (the kernel counts tokens in 32 bits)
+    const int n = (int)std::min(n_tokens - t0, 1ll << 30);
+    if (x_dtype == ROSAQ_F32)
+      gram_fma_kernel<float><<<grid, kFmaThreads, kFmaSmemBytes, s>>>(static_cast<const float *>(X) + t0 * ldx, ldx, dh, C, n);
+    else
+      gram_fma_kernel<__half><<<grid, kFmaThreads, kFmaSmemBytes, s>>>(static_cast<const __half *>(X) + t0 * ldx, ldx, dh, C, n);
+  }
   return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
 }
 

@@ -28,13 +28,40 @@ TiledOperand make_geometry(int d_in, int d_out, int bits, int g_fp16, int g_quan
   return t;
 }
 
-int alloc_blob(TiledOperand *t) {
+// Operands come from the context's pool: mapping fresh device memory costs a call hundreds of microseconds and more
+// (quantizing a per-head 4096 -> 4096 linear and freeing it again: 2.1 ms with cudaMalloc and cudaFree for the operand
+// and for an fp32 W', 0.23 ms with pooled operands and no W', of which 0.2 are kernels).  The pool keeps at most
+// kPoolKeepBytes that nobody uses and gives everything back when the context goes.
+constexpr unsigned long long kPoolKeepBytes = 64ull << 20;
+
+int pool_create(rosaq_ctx *ctx) {
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = ctx->device;
+  int st = cuda_status(cudaMemPoolCreate(&ctx->pool, &props));
+  unsigned long long keep = kPoolKeepBytes;
+  if (st == ROSAQ_OK) st = cuda_status(cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+  return st;
+}
+
+// usable on any stream once the caller has synchronized `s`, which every user of these does before it returns
+int pool_alloc(rosaq_ctx *ctx, void **p, size_t bytes, cudaStream_t s) {
+  return cuda_status(cudaMallocFromPoolAsync(p, bytes, ctx->pool, s));
+}
+
+// work in flight on any stream may still read the memory: like cudaFree on plain memory, wait for the device first
+void pool_free(void *p) {
+  if (!p) return;
+  (void)cudaDeviceSynchronize();
+  (void)cudaFree(p);
+}
+
+int alloc_blob(rosaq_ctx *ctx, TiledOperand *t, cudaStream_t s) {
   void *p = nullptr;
-  size_t bytes = t->bytes > 0 ? (size_t)t->bytes : 16;
-  int st = cuda_status(cudaMalloc(&p, bytes));
-  if (st != ROSAQ_OK) return st;
-  t->blob = static_cast<uint8_t *>(p);
-  return ROSAQ_OK;
+  const int st = pool_alloc(ctx, &p, t->bytes > 0 ? (size_t)t->bytes : 16, s);
+  t->blob = st == ROSAQ_OK ? static_cast<uint8_t *>(p) : nullptr;
+  return st;
 }
 
 int check_quant_args(int d_in, int d_out, int bits, int group, int k_salient) {
@@ -172,7 +199,9 @@ int rosaq_create(rosaq_ctx **out, int device) {
   ctx->pl_sync = nullptr;
   ctx->pf_pairs = 0;
   ctx->pf_flags = nullptr;
-  st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->d_status), 2 * sizeof(int)));   // [1]: scratch flag of argument checks
+  ctx->pool = nullptr;
+  st = pool_create(ctx);
+  if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->d_status), 2 * sizeof(int)));   // [1]: scratch flag of argument checks
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->d_status, 0, 2 * sizeof(int)));
   // the stream-K workspace is taken here, once, so that no linear call ever allocates for it
   if (st == ROSAQ_OK)
@@ -196,6 +225,7 @@ int rosaq_create(rosaq_ctx **out, int device) {
     if (ctx->d_status) (void)cudaFree(ctx->d_status);
     if (ctx->sk_partials) (void)cudaFree(ctx->sk_partials);
     if (ctx->sk_arrive) (void)cudaFree(ctx->sk_arrive);
+    if (ctx->pool) (void)cudaMemPoolDestroy(ctx->pool);
     delete ctx;
     return st;
   }
@@ -216,6 +246,7 @@ int rosaq_destroy(rosaq_ctx *ctx) {
     if (ctx->pf_flags) (void)cudaFree(ctx->pf_flags);
     if (ctx->pl_partials) (void)cudaFree(ctx->pl_partials);
     plan_free_schedules(ctx);
+    if (ctx->pool) (void)cudaMemPoolDestroy(ctx->pool);   // operands that outlive the context keep their memory until they are freed
     (void)cudaGetLastError();
   }
   delete ctx;
@@ -295,38 +326,21 @@ static int quantize_impl(rosaq_ctx *ctx, const void *W, int d_in, int d_out, con
   w->k_salient = k_salient;
   w->device = ctx->device;
   w->t = make_geometry(d_in, d_out, bits, k_salient / kGroup, (d_in - k_salient) / kGroup, 0);
-  float *Wp = nullptr, *Ws = nullptr;
-  const size_t fbytes = sizeof(float) * (size_t)d_in * d_out;
-  st = alloc_blob(&w->t);
-  if (st == ROSAQ_OK && rot && rot->perm) {
-    // the rotate kernels index R and W with perm: reject anything that is not a permutation first
-    int32_t *inv = nullptr;
-    st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&inv), sizeof(int32_t) * (size_t)d_in));
-    if (st == ROSAQ_OK) st = launch_invert_perm(rot->perm, d_in, inv, ctx->d_status + 1, s);
-    if (inv) (void)cudaFree(inv);
-  }
-  if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&Wp), fbytes));
-  if (st == ROSAQ_OK && rot && in_scale) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&Ws), fbytes));
-  if (st == ROSAQ_OK) {
-    const __half *Wh = static_cast<const __half *>(W);
-    if (rot && in_scale) {
-      st = launch_scale_rows(Wh, in_scale, d_in, d_out, Ws, s);
-      if (st == ROSAQ_OK)
-        st = launch_rotate_weights_w32(rot->q, rot->q_dtype == ROSAQ_F32, d_in, rot->n_blocks, rot->perm, Ws, d_out, Wp, s);
-    } else if (rot) {
-      st = launch_rotate_weights(rot->q, rot->q_dtype == ROSAQ_F32, d_in, rot->n_blocks, rot->perm, Wh, d_out, Wp, s);
-    } else if (in_scale) {
-      st = launch_scale_rows(Wh, in_scale, d_in, d_out, Wp, s);
-    } else {
-      st = launch_cast_weights(Wh, d_in, d_out, Wp, s);
-    }
-  }
-  if (st == ROSAQ_OK) st = launch_quant_pack(Wp, w->t, s);
+  // scratch in the context workspace: the inverse of perm (the kernels index R and W with it, so anything that is not
+  // a permutation is rejected first) and, for head blocks in a column order of their own, a bounded slab of W'
+  const size_t inv_bytes = rot && rot->perm ? (sizeof(int32_t) * (size_t)d_in + 255) / 256 * 256 : 0;
+  const size_t spill_bytes = rot ? rotate_quantize_spill_bytes(d_in, d_out, rot->n_blocks, rot->perm != nullptr) : 0;
+  st = alloc_blob(ctx, &w->t, s);
+  if (st == ROSAQ_OK && inv_bytes + spill_bytes > 0) st = ensure_workspace(ctx, inv_bytes + spill_bytes, s);
+  int32_t *inv = inv_bytes ? static_cast<int32_t *>(ctx->ws) : nullptr;
+  if (st == ROSAQ_OK && inv) st = launch_invert_perm(rot->perm, d_in, inv, ctx->d_status + 1, s);
+  if (st == ROSAQ_OK)
+    st = launch_rotate_quantize(rot ? rot->q : nullptr, rot ? rot->q_dtype == ROSAQ_F32 : 1, rot ? rot->n_blocks : 1,
+                                rot ? rot->perm : nullptr, inv, static_cast<const __half *>(W), in_scale,
+                                reinterpret_cast<float *>(static_cast<uint8_t *>(ctx->ws) + inv_bytes), spill_bytes, w->t, s);
   if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(s));
-  if (Wp) (void)cudaFree(Wp);
-  if (Ws) (void)cudaFree(Ws);
   if (st != ROSAQ_OK) {
-    if (w->t.blob) (void)cudaFree(w->t.blob);
+    pool_free(w->t.blob);
     delete w;
     return st;
   }
@@ -374,13 +388,13 @@ int rosaq_weight_import(rosaq_ctx *ctx, int d_in, int d_out, int bits, int group
   w->k_salient = k_salient;
   w->device = ctx->device;
   w->t = make_geometry(d_in, d_out, bits, k_salient / kGroup, (d_in - k_salient) / kGroup, 0);
-  st = alloc_blob(&w->t);
+  st = alloc_blob(ctx, &w->t, s);
   if (st == ROSAQ_OK)
     st = launch_import(w->t, qw, static_cast<const __half *>(scales_f16), static_cast<const __half *>(zeros_f16),
                        static_cast<const __half *>(salient_f16), s);
   if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(s));
   if (st != ROSAQ_OK) {
-    if (w->t.blob) (void)cudaFree(w->t.blob);
+    pool_free(w->t.blob);
     delete w;
     return st;
   }
@@ -392,7 +406,7 @@ int rosaq_weight_free(rosaq_weight *w) {
   if (!w) return ROSAQ_ERR_INVALID_ARG;
   DeviceGuard guard(w->device);
   if (guard.ok && w->t.blob) {
-    (void)cudaFree(w->t.blob);
+    pool_free(w->t.blob);
     (void)cudaGetLastError();
   }
   delete w;
@@ -433,18 +447,18 @@ int rosaq_rotation_create(rosaq_ctx *ctx, const rosaq_rot *rot, rosaq_rotation *
   // pair of SMs share one MMA stream over them
   const int bg = (dh == kGroup && rot->n_blocks % 2 == 0) ? 2 : dh / kGroup;
   r->t = make_geometry(rot->d, rot->d, 4, bg, 0, rot->n_blocks == 1 ? 0 : bg);
-  int st = alloc_blob(&r->t);
+  int st = alloc_blob(ctx, &r->t, s);
   if (st == ROSAQ_OK && rot->perm) {
     // checked first: the epilogues store through col_map, so a perm that is not a permutation is an error
     // code here, never a stray write later
-    st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&r->col_map), sizeof(int32_t) * rot->d));
+    st = pool_alloc(ctx, reinterpret_cast<void **>(&r->col_map), sizeof(int32_t) * rot->d, s);
     if (st == ROSAQ_OK) st = launch_invert_perm(rot->perm, rot->d, r->col_map, ctx->d_status + 1, s);
   }
   if (st == ROSAQ_OK) st = launch_rotation_tiles(static_cast<const __half *>(rot->q), rot->d, rot->n_blocks, r->t, s);
   if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(s));
   if (st != ROSAQ_OK) {
-    if (r->t.blob) (void)cudaFree(r->t.blob);
-    if (r->col_map) (void)cudaFree(r->col_map);
+    pool_free(r->t.blob);
+    pool_free(r->col_map);
     delete r;
     return st;
   }
@@ -456,8 +470,8 @@ int rosaq_rotation_free(rosaq_rotation *r) {
   if (!r) return ROSAQ_ERR_INVALID_ARG;
   DeviceGuard guard(r->device);
   if (guard.ok) {
-    if (r->t.blob) (void)cudaFree(r->t.blob);
-    if (r->col_map) (void)cudaFree(r->col_map);
+    pool_free(r->t.blob);
+    pool_free(r->col_map);
     (void)cudaGetLastError();
   }
   delete r;

@@ -245,6 +245,7 @@ struct rosaq_ctx {
   int *d_status;       // device status word (0 or ROSAQ_ERR_TIMEOUT)
   void *ws;            // rotated-activation workspace
   size_t ws_bytes;
+  cudaMemPool_t pool;  // memory of the weights and rotations
   long long wait_limit;
   int impl;            // 0 tensor-core, 1 CUDA-core, 2 tensor-core with CTA pairs, 3 tensor-core without stream-K,
                        // 4 persistent launch for every call, 5 prefill tiles for every weight
@@ -301,13 +302,9 @@ struct DeviceGuard {
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 // launchers implemented in the other translation units; all return a rosaq_status
-int launch_rotate_weights(const void *q, int q_is_f32, int d_in, int n_blocks, const int32_t *perm,
-                          const __half *W, int d_out, float *Wp, cudaStream_t s);
-int launch_rotate_weights_w32(const void *q, int q_is_f32, int d_in, int n_blocks, const int32_t *perm,
-                              const float *W32, int d_out, float *Wp, cudaStream_t s);
-int launch_scale_rows(const __half *W, const float *in_scale, int d_in, int d_out, float *out, cudaStream_t s);
-int launch_cast_weights(const __half *W, int d_in, int d_out, float *Wp, cudaStream_t s);
-int launch_quant_pack(const float *Wp, const TiledOperand &t, cudaStream_t s);
+size_t rotate_quantize_spill_bytes(int d_in, int d_out, int n_blocks, bool perm);
+int launch_rotate_quantize(const void *q, int q_is_f32, int n_blocks, const int32_t *perm, const int32_t *inv, const __half *W,
+                           const float *in_scale, float *spill, size_t spill_bytes, const TiledOperand &t, cudaStream_t s);
 int launch_export(const TiledOperand &t, uint32_t *qw, __half *scales, __half *zeros, __half *salient,
                   cudaStream_t s);
 int launch_import(const TiledOperand &t, const uint32_t *qw, const __half *scales, const __half *zeros,
