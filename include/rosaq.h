@@ -104,8 +104,8 @@ int64_t rosaq_set_wait_limit(rosaq_ctx *ctx, int64_t iterations);
  * rosaq_create allocated; again the same sums in another order); 4 = every call of up to 64 tokens runs as
  * ONE persistent launch, the rotation and the linears that consume it included (the kernel of rosaq_plan;
  * for a single call slower than 0, which is why it is not the default -- see rosaq_plan_create);
- * 5 = every weight, at any token count, on the 256-column x 256-token tiles that 0 picks for large batches
- * (rotations and all-fp16 weights stay on the kernels of 0); 6 = calls of 65 ... 1536 tokens as blocks of 128
+ * 5 = every weight and every rotation without a column permutation, at any token count, on the 256-column x 256-token
+ * tiles that 0 picks for large batches; 6 = calls of 65 ... 1536 tokens as blocks of 128
  * tokens, one operation of the persistent launch per block, in one launch (slower than 0 for a single
  * call: it exists to test that form of the launch).
  * Returns the previous value. */
@@ -151,8 +151,8 @@ int rosaq_calib_cov(rosaq_ctx *ctx, const void *X, int x_dtype, int64_t n_tokens
  *   z = clamp(-rint(lo/s), 0, 2^bits-1), stored as +0 when lo >= 0,
  *   code = clamp(rint(w/s) + z, 0, 2^bits-1), all IEEE fp32, ties to even.
  * Allocates the result (*out, release with rosaq_weight_free) from the context's memory pool, which keeps up to 64 MB
- * of freed operands for reuse and is released with the context.  A rotation with a column permutation may grow the
- * context workspace (by at most 16 MB, or one 128-column strip of W' in fp32).  Synchronizes `stream`.
+ * of freed memory for reuse and is released with the context; a rotation with a column permutation takes scratch from
+ * it too (at most 16 MB, or one 128-column strip of W' in fp32).  Synchronizes `stream`.
  * d_in % 128 == 0 required; d_out >= 1 (padded internally to a multiple of 128).
  */
 int rosaq_quantize(rosaq_ctx *ctx, const void *W, int d_in, int d_out, const rosaq_rot *rot,
@@ -216,10 +216,9 @@ int rosaq_rotate(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
  *   r != NULL : x . R goes through the context workspace (grown on demand: this call
  *               may then allocate and synchronize once), then the GEMM stage runs
  * Only the first d_out columns of each y row are written.  ldx, ldy multiples of 8.
- * Any M >= 1.  The kernel is chosen by size: up to 64 tokens the weight-streaming kernels; large batches
- * (more than 256 tokens, when the launch has at least 40 tiles of 256 columns x 256 tokens and 36
- * 128-channel groups of work per pair of SMs) run on those tiles, each shared by two CTAs on adjacent SMs
- * (tcgen05 cta_group::2, one dequantisation of a weight tile per 256 tokens); everything in between one
+ * Any M >= 1.  The kernel is chosen by size: up to 128 tokens the weight-streaming kernels; larger batches run, where an
+ * estimate says that it pays, on tiles of 256 columns x up to 256 tokens shared by two CTAs on adjacent SMs
+ * (tcgen05 cta_group::2, one dequantisation of a weight tile per 256 tokens), else one
  * 128-token tile per CTA.  The choice changes the order of the fp32 sums only; a call gives the same bits
  * every time.  Calls of one context that use the exchange workspace (the large-batch tiles, the
  * equal-share kernel, rosaq_plan_run) must not overlap on the GPU: keep them on one stream.

@@ -337,17 +337,6 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
 constexpr int kPairStages = 6;
 constexpr int kPairStageBytes = 2 * kOperandBytes;      // A rows (or nothing on a diagonal tile) + this CTA's half of B
 
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(1000u)
-      : "memory");
-  return ok != 0;
-}
 // Loads of a CTA pair: the data lands in the issuing CTA's shared memory, the bytes are counted on the
 // leader's barrier (a shared::cluster address), so the leader learns about both halves from one barrier.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, uint32_t lead_bar, int c0, int c1) {
@@ -391,23 +380,6 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-struct PairAbort {
-  volatile int *flag;
-  int *status;
-  long long limit;
-  __device__ __forceinline__ bool set() const { return *flag != 0; }
-  __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) const {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    for (long long it = 0; it < limit; ++it) {
-      if (mbar_try_wait_cluster(bar, parity)) return true;
-      if ((it & 63) == 63 && set()) return false;
-    }
-    *flag = 1;
-    atomicExch(status, (int)ROSAQ_ERR_TIMEOUT);
-    return false;
-  }
-};
-
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCovThreads, 1)
 cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap map2,
                    const CovParams p) {
@@ -422,7 +394,7 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint32_t rank;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  const PairAbort ab{reinterpret_cast<volatile int *>(&misc[1]), p.status, p.wait_limit};
+  const CovAbort ab{reinterpret_cast<volatile int *>(&misc[1]), p.status, p.wait_limit};
 
   // 256 x 256 tile (bi >= bj) of the lower triangle from the pair index bi (bi + 1) / 2 + bj
   const int pair = blockIdx.x >> 1;
@@ -489,7 +461,7 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         for (int back = 1; back <= kPairStages && back <= issued; ++back) {
           const int u = issued - back;
           for (int it = 0; it < kCovDrainPolls; ++it)
-            if (mbar_try_wait_cluster(bar_tma + 8 * (u % kPairStages), (u / kPairStages) & 1)) break;
+            if (mbar_try_wait(bar_tma + 8 * (u % kPairStages), (u / kPairStages) & 1)) break;
         }
       }
     }
@@ -514,7 +486,7 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
       tc_commit_pair(bar_d);
       if (ab.set()) {  // MMAs already issued must retire before the tensor memory is given back
         for (int it = 0; it < kCovDrainPolls; ++it)
-          if (mbar_try_wait_cluster(bar_d, 0)) break;
+          if (mbar_try_wait(bar_d, 0)) break;
       }
     }
   } else {

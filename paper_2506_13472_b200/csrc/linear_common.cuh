@@ -114,36 +114,22 @@ struct Abort {
   volatile int *flag;     // shared
   int *status;            // global
   long long limit;
-  bool cluster_scope;     // barriers also receive arrivals from the peer CTA of a pair
   __device__ __forceinline__ bool set() const { return *flag != 0; }
   __device__ __forceinline__ void raise() const {
     *flag = 1;
     atomicExch(status, (int)ROSAQ_ERR_TIMEOUT);
   }
-  // false when the wait gave up (or somebody else already did)
-  __device__ __forceinline__ bool poll(uint32_t bar, uint32_t parity) const {
-    return cluster_scope ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity);
-  }
-  // barriers that only this CTA's threads and copies feed: CTA scope whatever the mode
-  __device__ __forceinline__ bool wait_local(uint32_t bar, uint32_t parity) const {
-    if (mbar_try_wait(bar, parity)) return true;
-    for (long long it = 0; it < limit; ++it) {
-      if (mbar_try_wait(bar, parity)) return true;
-      if ((it & 63) == 63 && set()) return false;
-    }
-    raise();
-    return false;
-  }
-  // one cluster-scope poll per warp instead of thirty-two, verdict broadcast (also the warp-level sync)
+  // one poll per warp instead of thirty-two, verdict broadcast (also the warp-level sync)
   __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity) const {
     int ok = 1;
     if ((threadIdx.x & 31) == 0) ok = wait(bar, parity) ? 1 : 0;
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
   }
+  // false when the wait gave up (or somebody else already did)
   __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) const {
-    if (poll(bar, parity)) return true;
+    if (mbar_try_wait(bar, parity)) return true;
     for (long long it = 0; it < limit; ++it) {
-      if (poll(bar, parity)) return true;
+      if (mbar_try_wait(bar, parity)) return true;
       if ((it & 63) == 63 && set()) return false;
     }
     raise();

@@ -264,7 +264,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const bool is_lead = rank == 0;
   const int cta = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;   // entry of the schedule
   const int s_begin = p.seg_begin[cta], s_end = p.seg_begin[cta + 1];
-  const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit, kPair};
+  const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit};
   const int tile_mul = kPair ? 2 : 1;                          // this CTA's column tile of a piece: tile_mul * tile + rank
 
   if (threadIdx.x == 0) {
@@ -333,7 +333,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
           uint32_t idx = (idx4 >> (8 * team)) & 0xffu;
           for (int sub = 0; sub < nsub; ++sub) {
             const int slot = team * NWT + (int)idx;
-            if (!ab.wait_local(bar_w_empty + 8 * slot, ((lap4 >> team) & 1u) ^ 1u)) {
+            if (!ab.wait(bar_w_empty + 8 * slot, ((lap4 >> team) & 1u) ^ 1u)) {
               live = false;
               break;
             }
@@ -405,7 +405,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         for (int back = 1; back <= NS && back <= gc; ++back) {
           const int u = gc - back;
           for (int it = 0; it < kDrainPolls; ++it)
-            if (ab.poll(bar_a_full + 8 * (u % NS), (u / NS) & 1)) break;
+            if (mbar_try_wait(bar_a_full + 8 * (u % NS), (u / NS) & 1)) break;
         }
       }
     }
@@ -467,7 +467,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         if (kPair) tc_commit_mc(bar_drain + 8 * me, 1);
         else tc_commit(bar_drain + 8 * me);
         for (int it = 0; it < kDrainPolls; ++it)
-          if (ab.poll(bar_drain + 8 * me, 0)) break;
+          if (mbar_try_wait(bar_drain + 8 * me, 0)) break;
       }
     }
   } else if (warp >= kPlFirstDequantWarp && warp < kPlFirstEpiWarp) {
@@ -496,7 +496,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         const uint32_t my_s_empty = bar_s_empty + 8 * st, my_a_full = bar_a_full + 8 * st;
         bool got = ab.wait(my_s_empty, (use & 1u) ^ 1u);
         for (int sub = 0; sub < nsub && ok; ++sub, rw.advance(NWT)) {
-          got = got && ab.wait_local(my_full + 8 * rw.idx, rw.lap);
+          got = got && ab.wait(my_full + 8 * rw.idx, rw.lap);
           got = __all_sync(0xffffffffu, got);        // the TMEM instructions below need the whole warp
           if (!got) {
             ok = false;

@@ -1,4 +1,5 @@
-// The GEMM stage  y = x . W^  (Eq. 3) for prefill-sized batches: more than 128 tokens.
+// The GEMM stage  y = x . W^  (Eq. 3; x . R of Eq. 2 / Eq. 6 is the same contraction) for prefill-sized batches: more than
+// 128 tokens.
 //
 // Why another kernel.  With a few hundred tokens the stage is bound by the tensor pipe, not by the weight
 // stream, and what counts is how many tokens share one dequantisation of a weight tile and how often an
@@ -6,34 +7,45 @@
 // cycles, 128 for N = 256; 55 for N = 64 is 58 %), a weight tile dequantised for 128 tokens costs as many
 // instructions as one dequantised for 256, and a CTA that multiplies 128 columns with 256 tokens on its own
 // pulls 64 KB of activations per 128-channel group.  Here two CTAs of a cluster (adjacent SMs) share a
-// 256-column x 256-token tile as a cta_group::2 pair: rank r dequantises column tile 2 c + r into its own
-// tensor memory (the A operand, 128 lanes each) and loads 128 of the 256 token rows (its half of the B
-// operand, 32 KB per group), the leader issues M = 256, N = 256 MMAs for both, and each CTA ends up with the
-// accumulator of its own 128 columns for all 256 tokens.  A weight tile is dequantised once per 256 tokens.
+// tile of 256 columns x NT <= 256 tokens as a cta_group::2 pair: rank r dequantises column tile 2 c + r into its own
+// tensor memory (the A operand, 128 lanes each) and loads half of the token rows (its half of the B
+// operand), the leader issues M = 256, N = NT MMAs for both, and each CTA ends up with the
+// accumulator of its own 128 columns for all NT tokens.  A weight tile is dequantised once per 256 tokens.
+// Several weights that multiply the same activations (q/k/v, gate/up) run in one launch, their column pairs side by side.
 //
-// Work is cut the stream-K way: the list of (tile, 128-channel group) units, token blocks of one column pair
-// next to each other so that the second one finds the packed weights in L2, is cut into one contiguous range
-// of equal length per pair of CTAs (a 13B projection at 512 tokens is 108 tiles for 74 pairs: whole tiles
-// would take two rounds, equal ranges take 1.46).  A pair therefore holds at most one tile without its first
-// groups -- the first piece of its range: it stores that partial tile (fp32) in its own slot of a workspace
-// and raises its flag -- then whole tiles, and at the end of its range possibly a tile without its last groups:
-// it owns that tile, waits for the flags of the pairs that hold the rest (they went through it at the
-// start of their ranges, long before), adds their partial tiles in ascending K order and writes y.  A flag
-// has one writer and one reader, which puts it back to zero once the partial tile is in its shared memory:
-// every launch, replays of a captured launch included, starts from zero flags.  The launch is cooperative:
-// every pair is resident, and a pair only ever waits for work that other pairs do first in their ranges.
+// All-fp16 operands (rotations) need no dequantisation: a fp16 tile lies in memory as the tensor core reads it (K-major,
+// no swizzle), so both operands come straight from shared memory, the launch has no dequantisation warps, and the tensor
+// memory they would fill holds a second accumulator.  (4096 -> 4096 dense rotation, 1900 tokens: 88 us through tensor
+// memory, 57 so, 80 on the per-call kernel.)
 //
-// Per CTA: warp 0 = weight-tile producer (bulk copies; one sub-ring of slots per dequantisation team),
-// 1 = activation producer (TMA, bytes of both CTAs counted on the leader's barrier), 2 = MMA issuer (leader
-// only; also owns the tensor memory), 4..19 = four dequantisation teams (group j of the CTA's stream goes
-// to team and operand buffer j mod 4), 20..27 = epilogue (two warps per TMEM lane quadrant, 128 tokens
-// each).  Tensor memory: accumulator in columns 0..255, four operand buffers of 64 columns behind it, so the
-// accumulator is single: the epilogue of a tile (about a microsecond) is not overlapped with the next
-// tile's MMAs, only with its copies and its dequantisation.  Loads carry no cluster multicast.
+// Work is cut in one of two ways (prefill_choose):
+//   * S > 0: a cluster of S pairs per tile, each with 1 / S of the groups.  The partial rows meet in distributed shared memory
+//     (two cluster barriers, 2-3 us).  Used while all clusters are resident at once.
+//   * S = 0, equal shares: the list of (tile, 128-channel group) units, token blocks of one column pair
+//     next to each other so that the second one finds the packed weights in L2, is cut into one contiguous range
+//     of equal length per pair (a 13B projection at 512 tokens is 108 tiles for 74 pairs: whole tiles
+//     would take two rounds, equal ranges take 1.46).  The first piece of a range can be the end of a tile; its partial tile
+//     (fp32) goes to a workspace and a flag is raised.  The last piece can be a tile without its last groups: the pairs that
+//     hold it so ("closers") each finish a share of its token rows: they store the other rows of their own partial tile, wait
+//     for the flags of the other holders, fetch their rows with bulk copies and add them.  A flag counts the readers that
+//     have yet to fetch; the last one puts it back to zero, so every launch, replays of a captured launch included, starts
+//     from zero flags.  The launch is cooperative: closers wait for one another, so every pair must be resident.  A
+//     handshake through L2 costs 3 us from the flag's store to the reader, the whole exchange about 8.
+// In both, sums are added in a fixed order: the same bits on every run.
+//
+// Per CTA: warp 0 = weight-tile producer (bulk copies; one sub-ring of slots per dequantisation team; for an fp16 operand the
+// producer of both operands), 1 = activation producer (TMA, bytes of both CTAs counted on the leader's barrier),
+// 2 = MMA issuer (leader only; also owns the tensor memory), 4..19 = four dequantisation teams (group j of the CTA's stream
+// goes to team and operand buffer j mod 4), the last eight = epilogue (two warps per TMEM lane quadrant, alternate blocks of
+// sixteen tokens).  Tensor memory: accumulator in columns 0..255, four operand buffers of 64 columns behind it, so the
+// accumulator of a quantized weight is single: the epilogue therefore rounds a finished tile into registers (64 of them, which
+// setmaxnreg takes from the other warps), gives the accumulator back and only then stores.  Loads carry no cluster
+// multicast.
 // Every wait is bounded; a CTA that gives up records ROSAQ_ERR_TIMEOUT, lets its copies and MMAs in flight
 // finish, frees its tensor memory and returns.
 #include <cuda.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "linear_common.cuh"
@@ -43,33 +55,56 @@ namespace rosaq {
 namespace {
 
 constexpr int kPfTmemCols = 512;
-constexpr int kPfTokens = 256;                      // tokens per tile = N of the MMA
-constexpr int kPfRows = kPfTokens / 2;              // token rows a CTA keeps in shared memory
+constexpr int kPfMaxTokens = 256;                   // most tokens per tile = N of the MMA
 constexpr int kPfStages = 4;                        // operand buffers, each with its activation slot
 constexpr int kPfTeams = 4;
 constexpr int kPfFirstDequantWarp = 4, kPfFirstEpiWarp = kPfFirstDequantWarp + 4 * kPfTeams;
 constexpr int kPfEpiThreads = 256;
 constexpr int kPfThreads = kPfFirstEpiWarp * 32 + kPfEpiThreads;   // 896
-constexpr int kPfXSlotBytes = kPfRows * 256;        // 128 tokens x 128 channels of fp16
-constexpr int kPfNW = 8;                            // weight slots: two per team
-constexpr int kPfSmemBytes = 1024 + kPfStages * kPfXSlotBytes + kPfNW * kWSlotBytes + 8 * (2 * kPfNW + 2 * kPfStages + 5) + 16;
+// Registers: 72 per thread at launch; 128 x 40 + 512 x 64 + 256 x 104 = 896 x 72.
+constexpr int kPfRegsLaunch = 72, kPfRegsRoles = 40, kPfRegsDequant = 64, kPfRegsEpi = 104;
+static_assert(128 * kPfRegsRoles + kPfTeams * kTeamThreads * kPfRegsDequant + kPfEpiThreads * kPfRegsEpi == kPfThreads * kPfRegsLaunch,
+              "the warpgroups share the registers of the launch");
+constexpr int kPfMaxNW = 16;                        // weight slots (a multiple of the teams)
+constexpr int kPfMaxSmemBytes = 227 * 1024;
+constexpr int kPfMaxProblems = 4;
+constexpr int kPfMaxSplits = 4;                     // pairs in a cluster (eight CTAs: the portable limit)
+constexpr int kDenseBits = 16;                      // an operand without quantized groups
+constexpr int kPdEpiWarp = 4, kPdThreads = kPdEpiWarp * 32 + kPfEpiThreads;   // 384
+constexpr int kPdMaxStages = 8;                     // stages of 64 channels
+constexpr int kPdABytes = kFp16TileBytes / 2;       // 64 channels x 128 columns
 
 struct alignas(64) PfParams {
   CUtensorMap xmap;
-  const uint8_t *blob;
-  __half *y;
-  long long tile_stride, ldy;
-  int d_out, n_tiles, g_fp16, groups;
-  int n_col_pairs, n_tok_blocks, M;
+  CUtensorMap wmap[kPfMaxProblems];                 // all-fp16 operands: the blob as rows of 128 bytes
+  int n_prob;
+  int pair_start[kPfMaxProblems + 1];
+  const uint8_t *blob[kPfMaxProblems];
+  __half *y[kPfMaxProblems];
+  long long ldy[kPfMaxProblems];
+  int d_out[kPfMaxProblems], n_tiles[kPfMaxProblems];
+  long long tile_stride;
+  int g_fp16, groups, block_groups;
+  int n_tok_blocks, M;
+  int NT;                     // tokens per tile (a multiple of 32); a CTA keeps NT / 2 rows of x in shared memory
+  int NW;                     // weight slots; all-fp16 operands: stages
   int units;                  // (column pairs x token blocks) x groups
-  float *partials;            // [pair][rank][256 tokens][128 columns]
-  unsigned *flags;            // [pair][rank]: 1 while the slot holds a partial tile that nobody has fetched yet
+  int S;
+  float *partials;            // [pair][2][rank][NT tokens][128 columns]: of the first and of the last piece of a range
+  unsigned *flags;            // [pair][2][rank]: readers that still have to fetch from the slot
   int *status;
   long long wait_limit;
 };
 
 __device__ __forceinline__ int pf_range_begin(int pair, int n_pairs, int units) {
   return (int)(((long long)pair * units) / n_pairs);
+}
+// the pair whose range holds unit u
+__device__ __forceinline__ int pf_owner(int u, int n_pairs, int units) {
+  int q = (int)(((long long)u * n_pairs) / units);
+  while (q + 1 < n_pairs && pf_range_begin(q + 1, n_pairs, units) <= u) ++q;
+  while (q > 0 && pf_range_begin(q, n_pairs, units) > u) --q;
+  return q;
 }
 // next piece of the range [u, end): groups [g0, g1) of work item wk; false when the range is used up
 __device__ __forceinline__ bool pf_next_piece(int &u, int end, int G, int &wk, int &g0, int &g1) {
@@ -81,6 +116,14 @@ __device__ __forceinline__ bool pf_next_piece(int &u, int end, int G, int &wk, i
   u += len;
   return true;
 }
+// weight and column pair of work item wk
+__device__ __forceinline__ int pf_problem(const PfParams &p, int wk, int &col_pair) {
+  col_pair = wk / p.n_tok_blocks;
+  int prob = 0;
+  while (prob + 1 < p.n_prob && col_pair >= p.pair_start[prob + 1]) ++prob;
+  col_pair -= p.pair_start[prob];
+  return prob;
+}
 // the 256 epilogue threads agree on whether to go on (all of them always come here)
 __device__ __forceinline__ bool pf_epi_vote(bool v) {
   uint32_t r;
@@ -91,61 +134,143 @@ __device__ __forceinline__ bool pf_epi_vote(bool v) {
       : "memory");
   return r != 0;
 }
-__device__ __forceinline__ unsigned pf_ld_acquire(const unsigned *ptr) {
+__device__ __forceinline__ unsigned pf_ld_relaxed(const unsigned *ptr) {
   unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
   return v;
 }
-
-// sixteen tokens t0 .. of one output column, rounded once, rows past M left alone
-__device__ __forceinline__ void pf_store_rows(const uint32_t *v, __half *y_col, int t0, int M, long long ldy, bool n_ok) {
-  __half *yp = y_col + (long long)t0 * ldy;
-  if (n_ok && t0 + 16 <= M) {
+template <int kRegs>
+__device__ __forceinline__ void reg_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs));
+}
+template <int kRegs>
+__device__ __forceinline__ void reg_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
+}
+// The fp16 tile of an operand (16-byte chunks of eight channels, column by column) is a K-major operand without swizzle:
+// eight columns 128 bytes apart from the next eight, the next eight channels kTileN * 16 bytes further.
+__device__ __forceinline__ uint64_t make_a_desc(uint32_t smem_addr) {
+  return (uint64_t)((smem_addr >> 4) & 0x3fff) | ((uint64_t)(kTileN * 16 >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
+}
+// four MMAs = 64 channels; A advances by two chunks (4096 bytes) per MMA, B by 32 bytes inside a swizzle row
+__device__ __forceinline__ void tc_mma4_ss_pair(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 ta, tb;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "add.u64 ta, %1, 256;\n\tadd.u64 tb, %2, 2;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t"
+      "add.u64 ta, %1, 512;\n\tadd.u64 tb, %2, 4;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t"
+      "add.u64 ta, %1, 768;\n\tadd.u64 tb, %2, 6;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t}" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ uint32_t pf_pack(uint32_t lo, uint32_t hi) {          // two fp32 bit patterns, each rounded once
+  __half2 r = __floats2half2_rn(__uint_as_float(lo), __uint_as_float(hi));
+  return *reinterpret_cast<uint32_t *>(&r);
+}
+// Writes sixteen tokens t0 .. of 32 columns n0 .. (a warp): h[j] = tokens 2 j, 2 j + 1 of this lane's column.  When the
+// warp's columns are all there, three rounds of exchange between lanes turn the columns into rows of eight, so that a
+// lane writes 16 bytes twice instead of 2 bytes sixteen times.
+__device__ __forceinline__ void pf_store_block(const uint32_t *h, __half *y, int n0, int d_out, int t0, int M, long long ldy, int lane) {
+  if (n0 + 32 <= d_out) {
+    uint32_t r[8];
+    const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
 #pragma unroll
-    for (int e = 0; e < 16; ++e, yp += ldy) *yp = __float2half_rn(__uint_as_float(v[e]));
-  } else if (n_ok) {
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t o = __shfl_xor_sync(0xffffffffu, h[j], 1);
+      r[j] = __byte_perm(h[j], o, b0 ? 0x3276 : 0x5410);       // token 2 j + b0, two columns
+    }
+    uint32_t e[4][2];
 #pragma unroll
-    for (int e = 0; e < 16; ++e, yp += ldy)
-      if (t0 + e < M) *yp = __float2half_rn(__uint_as_float(v[e]));
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t o = __shfl_xor_sync(0xffffffffu, b1 ? r[2 * q] : r[2 * q + 1], 2);
+      e[q][0] = b1 ? o : r[2 * q], e[q][1] = b1 ? r[2 * q + 1] : o;
+    }
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      uint32_t o[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) o[k] = __shfl_xor_sync(0xffffffffu, b2 ? e[2 * m][k] : e[2 * m + 1][k], 4);
+      const uint4 v = b2 ? make_uint4(o[0], o[1], e[2 * m + 1][0], e[2 * m + 1][1]) : make_uint4(e[2 * m][0], e[2 * m][1], o[0], o[1]);
+      const int tok = t0 + 8 * m + (lane & 7);
+      if (tok < M) *reinterpret_cast<uint4 *>(y + (long long)tok * ldy + n0 + (lane & 24)) = v;
+    }
+    return;
+  }
+  if (n0 + lane >= d_out) return;
+  __half *yp = y + (long long)t0 * ldy + n0 + lane;
+#pragma unroll
+  for (int j = 0; j < 8; ++j, yp += 2 * ldy) {
+    if (t0 + 2 * j < M) *yp = __ushort_as_half((unsigned short)(h[j] & 0xffffu));
+    if (t0 + 2 * j + 1 < M) yp[ldy] = __ushort_as_half((unsigned short)(h[j] >> 16));
   }
 }
+// the two cluster barriers around the exchange of a split tile, for the warps that have no part in it
+__device__ __forceinline__ void pf_join_exchange() {
+  cluster_arrive();
+  cluster_wait();
+  cluster_arrive();
+  cluster_wait();
+}
 
+// kBits: 3 or 4, or kDenseBits for an operand without quantized groups.
 template <int kBits>
-__global__ void __launch_bounds__(kPfThreads, 1)
+__global__ void __launch_bounds__(kBits == kDenseBits ? kPdThreads : kPfThreads, 1)
 linear_prefill_kernel(const __grid_constant__ PfParams p) {
+  constexpr bool kDense = kBits == kDenseBits;
+  constexpr int kFirstEpi = kDense ? kPdEpiWarp : kPfFirstEpiWarp;
+  constexpr int kAcc = kDense ? 2 : 1;                         // accumulators
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const int NT = p.NT, rows = NT >> 1, NW = p.NW;
+  // quantized: kPfStages activation slots of a group (128 channels), then NW weight slots;
+  // dense: NW stages of half a group, the weights' 64 channels x 128 columns and the activations' behind them
+  const uint32_t x_slot_bytes = (uint32_t)rows * (kDense ? 128u : 256u);
+  const uint32_t d_stage_bytes = kPdABytes + x_slot_bytes;
   const uint32_t x_ring = base;
-  const uint32_t w_ring = x_ring + kPfStages * kPfXSlotBytes;
-  const uint32_t bars = w_ring + kPfNW * kWSlotBytes;
-  const uint32_t bar_w_full = bars, bar_w_empty = bar_w_full + 8 * kPfNW;
-  const uint32_t bar_a_full = bar_w_empty + 8 * kPfNW;         // operand buffers written + activation slots landed (leader's)
+  const uint32_t w_ring = x_ring + kPfStages * x_slot_bytes;
+  const uint32_t ring_bytes = kDense ? NW * d_stage_bytes : kPfStages * x_slot_bytes;
+  const uint32_t bars = kDense ? base + NW * d_stage_bytes : w_ring + NW * kWSlotBytes;
+  const uint32_t bar_w_full = bars, bar_w_empty = bar_w_full + 8 * NW;     // dense: a stage's copies (leader's) / its MMAs done
+  const uint32_t bar_a_full = bar_w_empty + 8 * NW;            // operand buffers written + activation slots landed (leader's)
   const uint32_t bar_s_empty = bar_a_full + 8 * kPfStages;     // stage consumed by its MMAs (both CTAs)
-  const uint32_t bar_d_full = bar_s_empty + 8 * kPfStages;     // accumulator complete (both CTAs)
-  const uint32_t bar_d_empty = bar_d_full + 8;                 // accumulator drained by both CTAs (leader's)
-  const uint32_t bar_drain = bar_d_empty + 8;
-  const uint32_t bar_merge = bar_drain + 8;                    // a partial tile has landed in the activation ring
-  const uint32_t misc = bar_drain + 16;                        // [0] TMEM base, [1] abort flag
+  const uint32_t bar_d_full = bar_s_empty + 8 * kPfStages;     // accumulators complete (both CTAs)
+  const uint32_t bar_d_empty = bar_d_full + 16;                // accumulators drained by both CTAs (leader's)
+  const uint32_t bar_drain = bar_d_empty + 16;
+  const uint32_t bar_merge = bar_drain + 8;                    // partial tiles have landed in the ring
+  const uint32_t misc = bar_merge + 8;                         // [0] TMEM base, [1] abort flag
   uint32_t *misc_ptr = reinterpret_cast<uint32_t *>(smem_raw + (misc - smem_u32(smem_raw)));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = blockIdx.x & 1u;                       // position in the pair; 0 = leader
   const bool is_lead = rank == 0;
   const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
-  const int u_begin = pf_range_begin(pair, n_pairs, p.units), u_end = pf_range_begin(pair + 1, n_pairs, p.units);
-  const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit, true};
+  const int S = p.S, G = p.groups;
+  const int split = S > 1 ? pair % S : 0;                      // this pair's position in its cluster
+  const uint32_t lead = 2u * (uint32_t)split, pair_mask = 3u << lead;   // cluster rank of the pair's leader; its two CTAs
+  int u_begin, u_end;
+  if (S > 0) {
+    const int wk0 = (pair / S) * G;
+    u_begin = wk0 + G * split / S, u_end = wk0 + G * (split + 1) / S;
+  } else {
+    u_begin = pf_range_begin(pair, n_pairs, p.units), u_end = pf_range_begin(pair + 1, n_pairs, p.units);
+  }
+  const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit};
+  grid_dep_launch_dependents();
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kPfNW; ++i) {
+    for (int i = 0; i < NW; ++i) {
       mbar_init(bar_w_full + 8 * i, 1);
-      mbar_init(bar_w_empty + 8 * i, kTeamThreads);
+      mbar_init(bar_w_empty + 8 * i, kDense ? 1 : kTeamThreads);
     }
     for (int i = 0; i < kPfStages; ++i) {
       mbar_init(bar_a_full + 8 * i, 2 * (kTeamThreads / 32) + 1);   // a team's warps in both CTAs + the activation copies
       mbar_init(bar_s_empty + 8 * i, 1);
     }
-    mbar_init(bar_d_full, 1);
-    mbar_init(bar_d_empty, 2 * (kPfEpiThreads / 32));          // one arrival per epilogue warp of both CTAs
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar_d_full + 8 * i, 1);
+      mbar_init(bar_d_empty + 8 * i, 2 * (kPfEpiThreads / 32));     // one arrival per epilogue warp of both CTAs
+    }
     mbar_init(bar_drain, 1);
     mbar_init(bar_merge, 1);
     misc_ptr[1] = 0;
@@ -159,137 +284,187 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
   cluster_wait();
   tc_fence_after();
   const uint32_t tmem = misc_ptr[0];
-  const uint32_t a_col0 = kPfTokens;                           // operand buffers follow the accumulator
-  const int qbytes = quant_tile_bytes(kBits);
-  const int G = p.groups;
+  const uint32_t a_col0 = kPfMaxTokens;                        // operand buffers follow the accumulator
 
-  if (warp == 0) {
-    // ---------------- weight-tile producer
-    if (lane == 0) {
-      constexpr int NWT = kPfNW / kPfTeams;
-      uint32_t idx4 = 0, lap4 = 0;
-      unsigned long long fills4 = 0;
-      int j = 0;
-      bool live = true;
-      int u = u_begin, wk, g0, g1;
-      while (live && !ab.set() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
-        // (the second CTA of a pair on an odd last tile streams that tile again; its results are dropped)
-        int my_tile = 2 * (wk / p.n_tok_blocks) + (int)rank;
-        if (my_tile >= p.n_tiles) my_tile = p.n_tiles - 1;
-        const uint8_t *tile_base = p.blob + (long long)my_tile * p.tile_stride;
-        for (int g = g0; g < g1 && live; ++g, ++j) {
-          const bool f16 = g < p.g_fp16;
-          const uint8_t *src = tile_base + (f16 ? (long long)g * kFp16TileBytes
-                                                : (long long)p.g_fp16 * kFp16TileBytes + (long long)(g - p.g_fp16) * qbytes);
-          const int nsub = f16 ? 4 : 1;
-          const uint32_t bytes = f16 ? kFp16SubBytes : qbytes;
-          const int team = j & (kPfTeams - 1);
-          uint32_t idx = (idx4 >> (8 * team)) & 0xffu;
-          for (int sub = 0; sub < nsub; ++sub) {
-            const int slot = team * NWT + (int)idx;
-            if (!ab.wait_local(bar_w_empty + 8 * slot, ((lap4 >> team) & 1u) ^ 1u)) {
+  // (what comes before the roles join again stays inside each role: the warps have different numbers of registers)
+  if (warp < 4) {
+    if (!kDense) reg_dec<kPfRegsRoles>();
+    if (kDense && warp == 0) {
+      // ---------------- dense producer: per stage this CTA's half of both operands, all bytes counted on the leader's barrier
+      if (lane == 0) {
+        grid_dep_wait();                                       // x may be the previous kernel's output
+        int issued = 0;
+        Ring rs{0, 0};
+        bool live = true;
+        int u = u_begin, wk, g0, g1;
+        while (live && !ab.set() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
+          int col_pair;
+          const int prob = pf_problem(p, wk, col_pair);
+          const int my_tile = min(2 * col_pair + (int)rank, p.n_tiles[prob] - 1);
+          const int a_row0 = (int)((long long)my_tile * p.tile_stride >> 7);     // rows of 128 bytes
+          const int tok0 = (wk % p.n_tok_blocks) * NT + (int)rank * rows;
+          // block-diagonal operand: the pair of column tiles multiplies the channels of its own diagonal block
+          const int g_block0 = p.block_groups > 0 ? (2 * col_pair / p.block_groups) * p.block_groups : 0;
+          for (int h = 2 * g0; h < 2 * g1; ++h, ++issued, rs.advance(NW)) {
+            if (!ab.wait(bar_w_empty + 8 * rs.idx, rs.lap ^ 1u)) {
               live = false;
               break;
             }
-            mbar_arrive_expect_tx(bar_w_full + 8 * slot, bytes);
-            bulk_copy_g2s(w_ring + slot * kWSlotBytes, src + (long long)sub * kFp16SubBytes, bytes, bar_w_full + 8 * slot);
-            fills4 += 1ull << (16 * team);
-            if (++idx == (uint32_t)NWT) {
-              idx = 0;
-              lap4 ^= 1u << team;
+            if (is_lead) mbar_arrive_expect_tx(bar_w_full + 8 * rs.idx, 2 * d_stage_bytes);
+            const uint32_t bar = map_to_rank(bar_w_full + 8 * rs.idx, lead), dst = base + rs.idx * d_stage_bytes;
+            tma_load_2d_pair(dst, &p.wmap[prob], bar, 0, a_row0 + h * (kPdABytes / 128));
+            tma_load_3d_pair(dst + kPdABytes, &p.xmap, bar, tok0, 2 * g_block0 + h);
+          }
+        }
+        // (the leader's barriers count the copies of both CTAs, and the peer stays until the cluster barrier
+        // at the end of the kernel, which the leader reaches after this drain)
+        if (ab.set() && is_lead) {
+          for (int back = 1; back <= NW && back <= issued; ++back) {
+            const int k = issued - back;
+            for (int it = 0; it < kDrainPolls; ++it)
+              if (mbar_try_wait(bar_w_full + 8 * (k % NW), (k / NW) & 1)) break;
+          }
+        }
+      }
+    } else if (!kDense && warp == 0) {
+      // ---------------- weight-tile producer
+      if (lane == 0) {
+        const int NWT = NW / kPfTeams, qbytes = quant_tile_bytes(kBits);
+        uint32_t idx4 = 0, lap4 = 0;
+        unsigned long long fills4 = 0;
+        int j = 0;
+        bool live = true;
+        int u = u_begin, wk, g0, g1;
+        while (live && !ab.set() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
+          // (the second CTA of a pair on an odd last tile streams that tile again; its results are dropped)
+          int col_pair;
+          const int prob = pf_problem(p, wk, col_pair);
+          const int my_tile = min(2 * col_pair + (int)rank, p.n_tiles[prob] - 1);
+          const uint8_t *tile_base = p.blob[prob] + (long long)my_tile * p.tile_stride;
+          for (int g = g0; g < g1 && live; ++g, ++j) {
+            const bool f16 = g < p.g_fp16;
+            const uint8_t *src = tile_base + (f16 ? (long long)g * kFp16TileBytes
+                                                  : (long long)p.g_fp16 * kFp16TileBytes + (long long)(g - p.g_fp16) * qbytes);
+            const int nsub = f16 ? 4 : 1;
+            const uint32_t bytes = f16 ? kFp16SubBytes : qbytes;
+            const int team = j & (kPfTeams - 1);
+            uint32_t idx = (idx4 >> (8 * team)) & 0xffu;
+            for (int sub = 0; sub < nsub; ++sub) {
+              const int slot = team * NWT + (int)idx;
+              if (!ab.wait(bar_w_empty + 8 * slot, ((lap4 >> team) & 1u) ^ 1u)) {
+                live = false;
+                break;
+              }
+              mbar_arrive_expect_tx(bar_w_full + 8 * slot, bytes);
+              bulk_copy_g2s(w_ring + slot * kWSlotBytes, src + (long long)sub * kFp16SubBytes, bytes, bar_w_full + 8 * slot);
+              fills4 += 1ull << (16 * team);
+              if (++idx == (uint32_t)NWT) {
+                idx = 0;
+                lap4 ^= 1u << team;
+              }
+            }
+            idx4 = (idx4 & ~(0xffu << (8 * team))) | (idx << (8 * team));
+          }
+        }
+        if (ab.set()) {  // let copies already in flight land before the CTA goes away
+          for (int team = 0; team < kPfTeams; ++team) {
+            const int f = (int)((fills4 >> (16 * team)) & 0xffffu);
+            for (int back = 1; back <= NWT && back <= f; ++back) {
+              const int k = f - back;
+              for (int it = 0; it < kDrainPolls; ++it)
+                if (mbar_try_wait(bar_w_full + 8 * (team * NWT + k % NWT), (k / NWT) & 1)) break;
             }
           }
-          idx4 = (idx4 & ~(0xffu << (8 * team))) | (idx << (8 * team));
         }
       }
-      if (ab.set()) {  // let copies already in flight land before the CTA goes away
-        for (int team = 0; team < kPfTeams; ++team) {
-          const int f = (int)((fills4 >> (16 * team)) & 0xffffu);
-          for (int back = 1; back <= NWT && back <= f; ++back) {
-            const int u = f - back;
+    } else if (!kDense && warp == 1) {
+      // ---------------- activation producer: this CTA's half of the token rows of every group
+      if (lane == 0) {
+        grid_dep_wait();                                       // x may be the previous kernel's output
+        int gc = 0;
+        Ring rs{0, 0};
+        bool live = true;
+        int u = u_begin, wk, g0, g1;
+        while (live && !ab.set() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
+          const int tok0 = (wk % p.n_tok_blocks) * NT + (int)rank * rows;
+          for (int g = g0; g < g1; ++g, ++gc, rs.advance(kPfStages)) {
+            const int slot = rs.idx;
+            if (!ab.wait(bar_s_empty + 8 * slot, rs.lap ^ 1u)) {
+              live = false;
+              break;
+            }
+            // all bytes are counted on the leader's barrier
+            if (is_lead) mbar_arrive_expect_tx(bar_a_full + 8 * slot, 2 * x_slot_bytes);
+            tma_load_3d_pair(x_ring + slot * x_slot_bytes, &p.xmap, map_to_rank(bar_a_full + 8 * slot, lead), tok0, 2 * g);
+          }
+        }
+        if (ab.set() && is_lead) {
+          for (int back = 1; back <= kPfStages && back <= gc; ++back) {
+            const int k = gc - back;
             for (int it = 0; it < kDrainPolls; ++it)
-              if (mbar_try_wait(bar_w_full + 8 * (team * NWT + u % NWT), (u / NWT) & 1)) break;
+              if (mbar_try_wait(bar_a_full + 8 * (k % kPfStages), (k / kPfStages) & 1)) break;
           }
         }
       }
-    }
-  } else if (warp == 1) {
-    // ---------------- activation producer: this CTA's 128 token rows of every group
-    if (lane == 0) {
-      int gc = 0;
-      Ring rs{0, 0};
-      bool live = true;
-      int u = u_begin, wk, g0, g1;
-      while (live && !ab.set() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
-        const int tok0 = (wk % p.n_tok_blocks) * kPfTokens + (int)rank * kPfRows;
-        for (int g = g0; g < g1; ++g, ++gc, rs.advance(kPfStages)) {
-          const int slot = rs.idx;
-          if (!ab.wait(bar_s_empty + 8 * slot, rs.lap ^ 1u)) {
-            live = false;
-            break;
-          }
-          // all bytes are counted on the leader's barrier
-          if (is_lead) mbar_arrive_expect_tx(bar_a_full + 8 * slot, 2 * kPfXSlotBytes);
-          tma_load_3d_pair(x_ring + slot * kPfXSlotBytes, &p.xmap, map_to_rank(bar_a_full + 8 * slot, 0), tok0, 2 * g);
-        }
-      }
-      // (the leader's barriers count the copies of both CTAs, and the peer stays until the cluster barrier
-      // at the end of the kernel, which the leader reaches after this drain)
-      if (ab.set() && is_lead) {
-        for (int back = 1; back <= kPfStages && back <= gc; ++back) {
-          const int u = gc - back;
-          for (int it = 0; it < kDrainPolls; ++it)
-            if (ab.poll(bar_a_full + 8 * (u % kPfStages), (u / kPfStages) & 1)) break;
-        }
-      }
-    }
-  } else if (warp == 2) {
-    // ---------------- MMA issuer (leader): per group one wait, eight MMAs of 256 x 256 x 16, one commit
-    if (lane == 0 && is_lead) {
-      const uint32_t idesc = (1u << 4) | ((uint32_t)(kPfTokens >> 3) << 17) | (16u << 24);
-      const uint64_t desc0 = make_b_desc(x_ring);
-      constexpr uint32_t x_slot16 = kPfXSlotBytes >> 4, half16 = (uint32_t)(kPfRows * 128) >> 4;
-      Ring rs{0, 0};
-      int n_done = 0;
-      bool live = true, issued = false;
-      int u = u_begin, wk, g0, g1;
-      for (; live && pf_next_piece(u, u_end, G, wk, g0, g1); ++n_done) {
-        if (!ab.wait(bar_d_empty, (uint32_t)(n_done & 1) ^ 1u)) break;   // the previous piece has been drained
-        tc_fence_after();
-        uint32_t accumulate = 0;
-        for (int g = g0; g < g1; ++g, rs.advance(kPfStages)) {
-          const int st = rs.idx;
-          if (!ab.wait(bar_a_full + 8 * st, rs.lap)) {
-            live = false;
-            break;
-          }
+    } else if (warp == 2) {
+      // ---------------- MMA issuer (leader): per group one wait, eight MMAs of 256 x NT x 16, one commit (dense: half a group)
+      if (lane == 0 && is_lead) {
+        const uint32_t idesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | (16u << 24);
+        const uint64_t desc0 = make_b_desc(kDense ? base + kPdABytes : x_ring), adesc0 = make_a_desc(base);
+        const uint32_t slot16 = (kDense ? d_stage_bytes : x_slot_bytes) >> 4, half16 = (uint32_t)(rows * 128) >> 4;
+        Ring rs{0, 0};
+        int n_done = 0;
+        bool live = true, issued = false;
+        int u = u_begin, wk, g0, g1;
+        for (; live && pf_next_piece(u, u_end, G, wk, g0, g1); ++n_done) {
+          const int buf = kDense ? n_done & 1 : 0;
+          if (!ab.wait(bar_d_empty + 8 * buf, (uint32_t)((n_done / kAcc) & 1) ^ 1u)) break;   // the last piece in it has been drained
           tc_fence_after();
-          const uint64_t b0 = desc0 + (uint64_t)(st * x_slot16);
-          tc_mma8_ts_pair(tmem, tmem + a_col0 + st * 64, b0, b0 + (uint64_t)half16, idesc, accumulate);
-          tc_commit_mc(bar_s_empty + 8 * st, 3);               // frees the stage in both CTAs
-          accumulate = 1;
-          issued = true;
+          const uint32_t d_tmem = tmem + buf * kPfMaxTokens;
+          uint32_t accumulate = 0;
+          const int n = (g1 - g0) * (kDense ? 2 : 1);
+          for (int i = 0; i < n; ++i, rs.advance(kDense ? NW : kPfStages)) {
+            const int st = rs.idx;
+            if (!ab.wait((kDense ? bar_w_full : bar_a_full) + 8 * st, rs.lap)) {
+              live = false;
+              break;
+            }
+            tc_fence_after();
+            const uint64_t b0 = desc0 + (uint64_t)(st * slot16);
+            if (kDense) {
+              tc_mma4_ss_pair(d_tmem, adesc0 + (uint64_t)(st * slot16), b0, idesc, accumulate);
+              tc_commit_mc(bar_w_empty + 8 * st, pair_mask);   // frees the stage in both CTAs
+            } else {
+              tc_mma8_ts_pair(d_tmem, tmem + a_col0 + st * 64, b0, b0 + (uint64_t)half16, idesc, accumulate);
+              tc_commit_mc(bar_s_empty + 8 * st, pair_mask);
+            }
+            accumulate = 1;
+            issued = true;
+          }
+          if (!live) break;
+          tc_commit_mc(bar_d_full + 8 * buf, pair_mask);
         }
-        if (!live) break;
-        tc_commit_mc(bar_d_full, 3);
-      }
-      if (ab.set() && issued) {  // MMAs already issued must retire before the tensor memory is given back
-        tc_commit_mc(bar_drain, 1);
-        for (int it = 0; it < kDrainPolls; ++it)
-          if (ab.poll(bar_drain, 0)) break;
+        if (ab.set() && issued) {  // MMAs already issued must retire before the tensor memory is given back
+          tc_commit_mc(bar_drain, 1u << lead);
+          for (int it = 0; it < kDrainPolls; ++it)
+            if (mbar_try_wait(bar_drain, 0)) break;
+        }
       }
     }
-  } else if (warp >= kPfFirstDequantWarp && warp < kPfFirstEpiWarp) {
+    __syncwarp();
+    if (S > 1) pf_join_exchange();
+  } else if (!kDense && warp < kFirstEpi) {
     // ---------------- dequantisation: group j of the CTA's stream goes to team and operand buffer j mod 4
+    reg_dec<kPfRegsDequant>();
     const int quad = warp & 3;
     const int team = (warp - kPfFirstDequantWarp) >> 2;
     const int n = quad * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-    constexpr int NWT = kPfNW / kPfTeams;
+    const int NWT = NW / kPfTeams;
     const uint32_t my_ring = w_ring + team * NWT * kWSlotBytes, my_full = bar_w_full + 8 * team * NWT,
                    my_empty = bar_w_empty + 8 * team * NWT;
     const uint32_t a_addr = lane_addr + a_col0 + team * 64;
-    const uint32_t my_s_empty = bar_s_empty + 8 * team, my_a_full = bar_a_full + 8 * team;
+    const uint32_t my_s_empty = bar_s_empty + 8 * team, my_a_full = map_to_rank(bar_a_full + 8 * team, lead);
     Ring rw{0, 0};
     bool ok = true;
     int j0 = 0;                                      // position of the tile's first group in the CTA's stream
@@ -301,142 +476,238 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
         const int nsub = f16 ? 4 : 1;
         bool got = ab.wait(my_s_empty, (use & 1u) ^ 1u);
         for (int sub = 0; sub < nsub && ok; ++sub, rw.advance(NWT)) {
-          got = got && ab.wait_local(my_full + 8 * rw.idx, rw.lap);
+          got = got && ab.wait(my_full + 8 * rw.idx, rw.lap);
           got = __all_sync(0xffffffffu, got);        // the TMEM instructions below need the whole warp
           if (!got) {
             ok = false;
             break;
           }
           tc_fence_after();
-          dequant_unit<kBits>(f16, my_ring + rw.idx * kWSlotBytes, n, a_addr, sub, my_empty + 8 * rw.idx);
+          dequant_unit<kDense ? 4 : kBits>(f16, my_ring + rw.idx * kWSlotBytes, n, a_addr, sub, my_empty + 8 * rw.idx);
         }
         tc_wait_st();
         if (!ok) break;
         tc_fence_before();
         __syncwarp();                                // one arrival per warp, on the leader's barrier
-        if (lane == 0) mbar_arrive_cluster(map_to_rank(my_a_full, 0));
+        if (lane == 0) mbar_arrive_cluster(my_a_full);
       }
       j0 += g1 - g0;
     }
-  } else if (warp >= kPfFirstEpiWarp) {
-    // ---------------- epilogue: thread = (output column n of this CTA's tile = TMEM lane, 128 of the 256
-    // tokens = TMEM columns); a warp's store covers 32 consecutive columns of one token row
+    if (S > 1) pf_join_exchange();
+  } else if (warp >= kFirstEpi) {
+    // ---------------- epilogue: thread = (output column n of this CTA's tile = TMEM lane, every other block of sixteen
+    // tokens = TMEM columns)
+    if (!kDense) reg_inc<kPfRegsEpi>();
     const int quad = warp & 3;
     const int n = quad * 32 + lane;
-    const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-    const int c_begin = ((warp - kPfFirstEpiWarp) >> 2) * kPfRows;
-    const bool lead = threadIdx.x == kPfFirstEpiWarp * 32;
-    constexpr long long kSlotFloats = (long long)kPfTokens * kTileN;             // one CTA's partial tile
-    float *const my_slot = p.partials + (long long)(2 * pair + (int)rank) * kSlotFloats + n;
-    int n_done = 0;
-    uint32_t merge_phase = 0;
-    int u = u_begin, wk, g0, g1;
-    for (; pf_next_piece(u, u_end, G, wk, g0, g1); ++n_done) {
-      const bool have_d = ab.wait(bar_d_full, (uint32_t)(n_done & 1));
-      if (!pf_epi_vote(have_d && !ab.set())) break;
-      tc_fence_after();
-      const int tile = 2 * (wk / p.n_tok_blocks) + (int)rank;
-      const int n_glob = tile * kTileN + n;
-      const bool n_ok = tile < p.n_tiles && n_glob < p.d_out;
-      const int tok0 = (wk % p.n_tok_blocks) * kPfTokens;
-      if (g0 > 0) {
-        // a tile without its first groups: store the partial tile, then raise this CTA's flag
-        for (int c0 = c_begin; c0 < c_begin + kPfRows && tok0 + c0 < p.M; c0 += 16) {
-          uint32_t v[16];
-          tmem_ld16(lane_addr + c0, v);
-          tc_wait_ld();
-          float *dp = my_slot + (long long)c0 * kTileN;
+    const int hf = (warp - kFirstEpi) >> 2;
+    const bool epi_lead = threadIdx.x == kFirstEpi * 32;
+    const long long slot_floats = (long long)NT * kTileN;                        // one CTA's partial tile
+    auto slot_of = [&](int pr, int which) { return p.partials + ((long long)pr * 4 + which * 2 + (int)rank) * slot_floats; };
+    auto flag_of = [&](int pr, int which) { return p.flags + pr * 4 + which * 2 + (int)rank; };
+    uint32_t lane_addr = 0;
+    // blocks [b0, b1) of the accumulator -> a partial tile
+    auto store_partial = [&](float *slot, int b0, int b1) {
+      for (int bk = b0 + hf; bk < b1; bk += 2) {
+        uint32_t v[16];
+        tmem_ld16(lane_addr + bk * 16, v);
+        tc_wait_ld();
+        float *dp = slot + (long long)bk * 16 * kTileN + n;
 #pragma unroll
-          for (int e = 0; e < 16; ++e) dp[e * kTileN] = __uint_as_float(v[e]);
-        }
+        for (int e = 0; e < 16; ++e) dp[e * kTileN] = __uint_as_float(v[e]);
+      }
+    };
+    auto raise_flag = [&](unsigned *flag, int readers) {
+      pf_epi_vote(true);                                       // all stores of the CTA are issued ...
+      if (epi_lead) {
+        __threadfence();                                       // ... and ordered before the flag (cumulative fence)
+        asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(flag), "r"((unsigned)readers) : "memory");
+      }
+    };
+    if (S <= 1) grid_dep_wait();   // y, the partial tiles and the flags may still be in use by the previous kernel
+    int n_done = 0;
+    int u = u_begin, wk, g0, g1;
+    for (; S <= 1 && pf_next_piece(u, u_end, G, wk, g0, g1); ++n_done) {
+      const int buf = kDense ? n_done & 1 : 0;
+      lane_addr = tmem + ((uint32_t)(quad * 32) << 16) + buf * kPfMaxTokens;
+      auto release = [&]() {                                   // the accumulator is free for the next piece but one (dense: two)
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_to_rank(bar_d_empty, 0));
-        __threadfence();
-        pf_epi_vote(true);
-        if (lead) {
-          __threadfence();
-          atomicExch(p.flags + 2 * pair + (int)rank, 1u);
+        if (lane == 0) mbar_arrive_cluster(map_to_rank(bar_d_empty + 8 * buf, lead));
+      };
+      const bool have_d = ab.wait(bar_d_full + 8 * buf, (uint32_t)((n_done / kAcc) & 1));
+      if (!pf_epi_vote(have_d && !ab.set())) break;
+      tc_fence_after();
+      int col_pair;
+      const int prob = pf_problem(p, wk, col_pair);
+      const int tile = 2 * col_pair + (int)rank;
+      const int d_out = tile < p.n_tiles[prob] ? p.d_out[prob] : 0;              // (a tile that is not there writes nothing)
+      const int n0 = tile * kTileN + quad * 32;
+      __half *const y = p.y[prob];
+      const long long ldy = p.ldy[prob];
+      const int tok0 = (wk % p.n_tok_blocks) * NT;
+      const int n_blk = (min(NT, p.M - tok0) + 15) >> 4;       // blocks of sixteen tokens in this tile
+      // the pairs `first` .. `last` hold the tile's groups, ascending K
+      const int first = S > 0 || g0 == 0 ? pair : pf_owner(wk * G, n_pairs, p.units);
+      const int last = S > 0 || g1 == G ? pair : pf_owner(wk * G + G - 1, n_pairs, p.units);
+      const int closers = last - first;                        // all holders but the last share the tile's token rows
+      if (closers == 0) {
+        // the whole tile is here: round it into registers, give the accumulator back, then store
+        uint32_t h[8][8];
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+          uint32_t v[2][16];
+#pragma unroll
+          for (int k = 0; k < 2; ++k)
+            if (hf + 2 * (i + k) < n_blk) tmem_ld16(lane_addr + (hf + 2 * (i + k)) * 16, v[k]);
+          tc_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) h[i + k][j] = pf_pack(v[k][2 * j], v[k][2 * j + 1]);
         }
+        release();
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (hf + 2 * i < n_blk) pf_store_block(h[i], y, n0, d_out, tok0 + (hf + 2 * i) * 16, p.M, ldy, lane);
         continue;
       }
-      // the tile's first groups are here: this CTA writes y.  The pairs pair + 1 .. last hold the tile's other groups.
-      int last = pair;
-      if (g1 < G) {
-        const int uu = wk * G + G - 1;                         // the tile's last unit
-        last = (int)(((long long)uu * n_pairs) / p.units);
-        while (last + 1 < n_pairs && pf_range_begin(last + 1, n_pairs, p.units) <= uu) ++last;
-        while (last > pair && pf_range_begin(last, n_pairs, p.units) > uu) --last;
-        bool got = true;
-        if (lead) {
-          for (int h = pair + 1; h <= last && got; ++h) {
-            const unsigned *f = p.flags + 2 * h + (int)rank;
-            got = false;
-            for (long long it = 0; it < ab.limit && !got; ++it) {
-              got = pf_ld_acquire(f) != 0u;
-              if (!got && (it & 15) == 15) {
-                if (ab.set()) break;
-                __nanosleep(64);
-              }
-            }
-          }
-          if (!got && !ab.set()) ab.raise();
-        }
-        if (!pf_epi_vote(got && !ab.set())) break;
+      if (pair == last) {
+        // the first piece of this range: its partial tile goes to the workspace
+        store_partial(slot_of(pair, 0), 0, n_blk);
+        release();
+        raise_flag(flag_of(pair, 0), closers);
+        continue;
       }
-      // The other holders' partial tiles, in ascending K order.  This is the last piece of the range, so the
-      // activation ring (4 x 32 KB = one partial tile of this CTA) is free: a partial tile comes in as four bulk
-      // copies and is added to the accumulator in tensor memory from shared memory -- read straight from L2,
-      // sixteen loads at a time per thread, a tile took 6 us.
+      int b0 = 0, b1 = n_blk;                                  // the blocks of token rows this pair finishes
+      const int mine = pair - first;
+      if (closers > 1) {
+        b0 = n_blk * mine / closers, b1 = n_blk * (mine + 1) / closers;
+        store_partial(slot_of(pair, 1), 0, b0);
+        store_partial(slot_of(pair, 1), b1, n_blk);
+        raise_flag(flag_of(pair, 1), closers - 1);
+      }
+      // This is the last piece of the range, so the ring is free: the other holders' rows come in as bulk copies, about a
+      // whole tile in all (read straight from L2, sixteen loads at a time per thread, a tile took 6 us), and are added in
+      // ascending order of the holders.
+      const uint32_t share_bytes = (uint32_t)(b1 - b0) * 16 * kTileN * 4;
+      const int fit = share_bytes > 0 ? (int)(ring_bytes / share_bytes) : closers;   // holders per round; the ring holds a whole tile
       bool alive = true;
-      for (int h = pair + 1; h <= last && alive; ++h) {
-        if (lead) {
-          const float *src = p.partials + (long long)(2 * h + (int)rank) * kSlotFloats;
-          mbar_arrive_expect_tx(bar_merge, (uint32_t)(kSlotFloats * sizeof(float)));
-          for (int q = 0; q < kPfStages; ++q)
-            bulk_copy_g2s(x_ring + q * kPfXSlotBytes, src + (long long)q * (kPfXSlotBytes / 4), kPfXSlotBytes, bar_merge);
+      uint32_t phase = 0;
+      for (int h0 = 0; h0 < closers && alive; h0 += fit) {
+        const int h1 = min(closers, h0 + fit);                 // others: 0 .. closers - 1 = holders without `pair`
+        if (warp == kFirstEpi) {
+          // a lane per holder: the flags are polled and the copies issued side by side
+          if (lane == 0) mbar_arrive_expect_tx(bar_merge, share_bytes * (uint32_t)(h1 - h0));
+          __syncwarp();
+          for (int o0 = h0; o0 < h1; o0 += 32) {
+            const int o = o0 + lane, h = first + o + (o >= mine ? 1 : 0), which = h == last ? 0 : 1;
+            bool got = o >= h1;
+            for (long long it = 0; it < ab.limit; ++it) {
+              if (!got) got = pf_ld_relaxed(flag_of(h, which)) != 0u;
+              if (__all_sync(0xffffffffu, got)) break;         // (together: divergent lanes would fence and copy one after the other)
+              if ((it & 15) == 15 && __any_sync(0xffffffffu, ab.set())) break;
+            }
+            if (!__all_sync(0xffffffffu, got)) {
+              if (!got && !ab.set()) ab.raise();
+              break;
+            }
+            __threadfence();                                   // acquires what the flags announce ...
+            asm volatile("fence.proxy.async;" ::: "memory");   // ... written by generic stores, read by the copy engine
+            if (o < h1 && share_bytes > 0)
+              bulk_copy_g2s(base + (uint32_t)(o - h0) * share_bytes, slot_of(h, which) + (long long)b0 * 16 * kTileN, share_bytes, bar_merge);
+          }
+          __syncwarp();
         }
-        const bool landed = ab.wait_local(bar_merge, merge_phase);
-        merge_phase ^= 1u;
-        if (lead && landed) p.flags[2 * h + (int)rank] = 0u;    // fetched: the slot is free for the next launch
+        const bool landed = ab.wait(bar_merge, phase);
+        phase ^= 1u;
+        if (warp == kFirstEpi && landed && !ab.set())
+          for (int o = h0 + lane; o < h1; o += 32) {           // fetched: one reader less
+            const int h = first + o + (o >= mine ? 1 : 0);
+            atomicSub(flag_of(h, h == last ? 0 : 1), 1u);
+          }
         if (!pf_epi_vote(landed && !ab.set())) {
           alive = false;
           break;
         }
-        for (int c0 = c_begin; c0 < c_begin + kPfRows && tok0 + c0 < p.M; c0 += 16) {
+        const bool final_round = h1 == closers;
+        for (int bk = b0 + hf; bk < b1; bk += 2) {
           uint32_t v[16];
-          tmem_ld16(lane_addr + c0, v);
-          const uint32_t sp = x_ring + (uint32_t)((c0 * kTileN + n) * 4);
-          float w[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) w[e] = __uint_as_float(lds32(sp + e * kTileN * 4));
+          tmem_ld16(lane_addr + bk * 16, v);
           tc_wait_ld();
+          for (int o = 0; o < h1 - h0; ++o) {
+            const uint32_t sp = base + (uint32_t)o * share_bytes + (uint32_t)(((bk - b0) * 16 * kTileN + n) * 4);
 #pragma unroll
-          for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__fadd_rn(__uint_as_float(v[e]), w[e]));
-          tmem_st16(lane_addr + c0, v);
+            for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__fadd_rn(__uint_as_float(v[e]), __uint_as_float(lds32(sp + e * kTileN * 4))));
+          }
+          if (final_round) {
+            uint32_t h[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) h[j] = pf_pack(v[2 * j], v[2 * j + 1]);
+            pf_store_block(h, y, n0, d_out, tok0 + bk * 16, p.M, ldy, lane);
+          } else {
+            tmem_st16(lane_addr + bk * 16, v);
+          }
         }
-        tc_wait_st();
-        pf_epi_vote(true);                                     // everybody has read the tile: the next one may land
+        if (!final_round) {
+          tc_wait_st();
+          pf_epi_vote(true);                                   // everybody has read the rows: the next ones may land
+        }
       }
       if (!alive) break;
-      // (the load of the next sixteen tokens is in flight while these are rounded and stored)
-      __half *y_col = p.y + (n_ok ? n_glob : 0);
-      const int c_end = min(c_begin + kPfRows, ((p.M - tok0 + 15) / 16) * 16);
-      uint32_t va[16], vb[16];
-      if (c_begin < c_end) tmem_ld16(lane_addr + c_begin, va);
-      for (int c0 = c_begin; c0 < c_end; c0 += 32) {
-        tc_wait_ld();
-        if (c0 + 16 < c_end) tmem_ld16(lane_addr + c0 + 16, vb);
-        pf_store_rows(va, y_col, tok0 + c0, p.M, p.ldy, n_ok);
-        if (c0 + 16 < c_end) {
+      release();
+    }
+    if (S > 1) {
+      // The pairs of a cluster hold the same tile: each finishes the token blocks of its share.  Everybody sends the rows of
+      // the others' shares into their shared memory (over the rings, hence the first barrier), then adds what came to its
+      // own accumulator, in ascending order of the pairs.  All threads take the barriers whatever happened before.
+      bool have = ab.wait(bar_d_full, 0);
+      have = __all_sync(0xffffffffu, have && !ab.set());
+      tc_fence_after();
+      pf_next_piece(u, u_end, G, wk, g0, g1);
+      int col_pair;
+      const int prob = pf_problem(p, wk, col_pair);
+      const int tok0 = (wk % p.n_tok_blocks) * NT;
+      const int n_blk = (min(NT, p.M - tok0) + 15) >> 4;       // blocks of sixteen tokens
+      const int max_blk = (n_blk + S - 1) / S;                 // blocks of the largest share
+      lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
+      cluster_arrive();
+      cluster_wait();
+      if (have) {
+        for (int bk = hf; bk < n_blk; bk += 2) {
+          const int o = ((bk + 1) * S - 1) / n_blk;            // the pair that finishes block bk
+          if (o == split) continue;
+          const int from = split < o ? split : split - 1;
+          const uint32_t dst = map_to_rank(base + (uint32_t)(((from * max_blk + bk - n_blk * o / S) * 16 * kTileN + n) * 4), 2u * (uint32_t)o + rank);
+          uint32_t v[16];
+          tmem_ld16(lane_addr + bk * 16, v);
           tc_wait_ld();
-          if (c0 + 32 < c_end) tmem_ld16(lane_addr + c0 + 32, va);
-          pf_store_rows(vb, y_col, tok0 + c0 + 16, p.M, p.ldy, n_ok);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) st_cluster_u32(dst + e * kTileN * 4, v[e]);
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(map_to_rank(bar_d_empty, 0));
+      cluster_arrive();                                        // releases my rows, acquires everybody's
+      cluster_wait();
+      if (have && !ab.set()) {
+        grid_dep_wait();                                       // y may still be in use by the previous kernel
+        const int tile = 2 * col_pair + (int)rank;
+        const int d_out = tile < p.n_tiles[prob] ? p.d_out[prob] : 0;
+        const int b0 = n_blk * split / S, b1 = n_blk * (split + 1) / S;
+        for (int bk = b0 + hf; bk < b1; bk += 2) {
+          uint32_t v[16];
+          tmem_ld16(lane_addr + bk * 16, v);
+          tc_wait_ld();
+          for (int from = 0; from < S - 1; ++from) {
+            const uint32_t sp = base + (uint32_t)(((from * max_blk + bk - b0) * 16 * kTileN + n) * 4);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__fadd_rn(__uint_as_float(v[e]), __uint_as_float(lds32(sp + e * kTileN * 4))));
+          }
+          uint32_t h[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) h[j] = pf_pack(v[2 * j], v[2 * j + 1]);
+          pf_store_block(h, p.y[prob], tile * kTileN + quad * 32, d_out, tok0 + bk * 16, p.M, p.ldy[prob], lane);
+        }
+      }
     }
   }
 
@@ -467,9 +738,11 @@ EncodeTiledFn prefill_encode_fn() {
   return fn;
 }
 
-int prefill_set_attrs(void (*kern)(PfParams)) {
+typedef void (*PrefillKernel)(PfParams);
+
+int prefill_set_attrs(PrefillKernel kern) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmemBytes) != cudaSuccess) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfMaxSmemBytes) != cudaSuccess) {
     (void)cudaGetLastError();
     return ROSAQ_ERR_CUDA;
   }
@@ -477,114 +750,172 @@ int prefill_set_attrs(void (*kern)(PfParams)) {
 }
 
 std::mutex g_pf_mu;
-bool g_pf_attr_done[64] = {};                                // per device, both code widths at once
+bool g_pf_attr_done[64] = {};                                // per device, all kernels at once
 
 int prefill_prepare_device() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return ROSAQ_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_pf_mu);
   if (!g_pf_attr_done[dev]) {
-    if (prefill_set_attrs(linear_prefill_kernel<4>) != ROSAQ_OK || prefill_set_attrs(linear_prefill_kernel<3>) != ROSAQ_OK)
+    if (prefill_set_attrs(linear_prefill_kernel<4>) != ROSAQ_OK || prefill_set_attrs(linear_prefill_kernel<3>) != ROSAQ_OK ||
+        prefill_set_attrs(linear_prefill_kernel<kDenseBits>) != ROSAQ_OK)
       return ROSAQ_ERR_CUDA;
     g_pf_attr_done[dev] = true;
   }
   return ROSAQ_OK;
 }
 
-void prefill_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, int n_pairs, cudaStream_t s) {
-  cfg->gridDim = dim3(2 * n_pairs);
-  cfg->blockDim = dim3(kPfThreads);
-  cfg->dynamicSmemBytes = kPfSmemBytes;
-  cfg->stream = s;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeCooperative;               // all pairs resident: the waits between pairs cannot starve
-  attr[1].val.cooperative = 1;
-  cfg->attrs = attr;
-  cfg->numAttrs = 2;
+size_t prefill_smem(bool dense, int NT, int NW) {
+  const size_t rings = dense ? (size_t)NW * (kPdABytes + (NT / 2) * 128) : (size_t)kPfStages * (NT / 2) * 256 + (size_t)NW * kWSlotBytes;
+  return 1024 + rings + 8 * (2 * NW + 2 * kPfStages + 6) + 16;
 }
 
-// pairs of CTAs that the device keeps resident at once (an SM without a free neighbour in its GPC cannot
-// host half a pair); 0 when the query fails
-int prefill_pairs(rosaq_ctx *ctx) {
-  if (ctx->pf_pairs > 0) return ctx->pf_pairs;
+void prefill_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, int n_pairs, int S, int threads, size_t smem, cudaStream_t s) {
+  cfg->gridDim = dim3(2 * n_pairs);
+  cfg->blockDim = dim3(threads);
+  cfg->dynamicSmemBytes = smem;
+  cfg->stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = S > 0 ? 2 * S : 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the prologue runs under the previous kernel's tail
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[2].id = cudaLaunchAttributeCooperative;               // equal shares: pairs wait for one another, all must be resident
+  attr[2].val.cooperative = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = S > 0 ? 2 : 3;
+}
+
+// Clusters of S pairs that the device keeps resident at once (a cluster lives inside one GPC, so larger ones leave SMs over);
+// 0 when the query fails
+int prefill_clusters(rosaq_ctx *ctx, int S) {
+  if (ctx->pf_clusters[S - 1] > 0) return ctx->pf_clusters[S - 1];
   if (prefill_prepare_device() != ROSAQ_OK) return 0;
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr[2];
-  prefill_config(&cfg, attr, ctx->sm_count / 2, nullptr);
+  cudaLaunchAttribute attr[3];
+  prefill_config(&cfg, attr, S * (ctx->sm_count / (2 * S)), S, kPfThreads, kPfMaxSmemBytes, nullptr);
   cfg.numAttrs = 1;                                          // (the cluster shape only)
   int clusters = 0;
   if (cudaOccupancyMaxActiveClusters(&clusters, linear_prefill_kernel<4>, &cfg) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
   }
-  if (clusters > ctx->sm_count / 2) clusters = ctx->sm_count / 2;
-  ctx->pf_pairs = clusters;
+  clusters = std::min(clusters, ctx->sm_count / (2 * S));
+  ctx->pf_clusters[S - 1] = clusters;
   return clusters;
-}
-
-int prefill_launch(void (*kern)(PfParams), const PfParams &p, int n_pairs, cudaStream_t s) {
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr[2];
-  prefill_config(&cfg, attr, n_pairs, s);
-  if (cudaLaunchKernelEx(&cfg, kern, p) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return ROSAQ_ERR_CUDA;
-  }
-  return ROSAQ_OK;
 }
 
 }  // namespace
 
-// Shapes this kernel takes: a dense operand with quantized groups (a weight), no column map.
+// Operands this kernel takes: any whose adjacent column tiles multiply the same channels; outputs in column order.
 bool prefill_supported(const TiledOperand &t, const int32_t *col_map) {
-  return t.block_groups == 0 && t.g_quant > 0 && col_map == nullptr && (t.bits == 3 || t.bits == 4);
+  return t.block_groups % 2 == 0 && groups_per_tile(t) > 0 && (t.block_groups == 0 || t.g_quant == 0) && col_map == nullptr &&
+         (t.bits == 3 || t.bits == 4);
 }
 
-int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t, __half *y,
-                          long long ldy, cudaStream_t s) {
+// How a launch is cut, and about how long it takes (us).  The figures are a fit to 7B and 13B shapes and smaller ones at
+// 65 ... 1900 tokens: a launch costs about 5.5 us + 0.016 per token of a tile, an exchange in a cluster of more than four
+// CTAs 0.012 per token more, the exchange through L2 7; a group takes a pair 0.3 us + 0.0008 per token, and more the more
+// pairs run (they share the L2 and the power limit).
+PrefillCut prefill_choose(rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts) {
+  const int G = groups_per_tile(*ts[0]);
+  long long col_pairs = 0;
+  for (int i = 0; i < n; ++i) col_pairs += (ts[i]->n_tiles + 1) / 2;
+  PrefillCut best;
+  const int blocks = (M + kPfMaxTokens - 1) / kPfMaxTokens;
+  best.NT = ((M + blocks - 1) / blocks + 31) / 32 * 32;
+  best.n_tok_blocks = (M + best.NT - 1) / best.NT;
+  const double NT = best.NT, tiles = (double)col_pairs * best.n_tok_blocks;
+  const double dense = ts[0]->g_quant == 0 ? 2.0 : 0.0;
+  auto group_us = [&](double pairs) { return 0.3 + 0.0008 * NT + (0.0011 + 0.0000133 * NT) * pairs; };
+  const double pairs = prefill_clusters(ctx, 1), units = tiles * G;
+  best.S = 0;
+  best.us = 12.5 + 0.026 * NT + dense + units / (pairs > 0 ? pairs : 1) * group_us(std::min(pairs, units));
+  for (int S = 1; S <= kPfMaxSplits && S <= G; ++S) {
+    const int res = prefill_clusters(ctx, S);
+    if (res < 1 || tiles > res) continue;                    // (a second round of clusters costs more than equal shares)
+    const double us = 5.5 + 0.016 * NT + (S > 2 ? 0.012 * NT : 0.0) + dense + (double)((G + S - 1) / S) * group_us(tiles * S);
+    if (us < best.us) best.us = us, best.S = S;
+  }
+  return best;
+}
+
+// n weights of identical geometry applied to the same activations in one launch
+int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const TiledOperand *const *ts,
+                          __half *const *ys, const long long *ldys, const PrefillCut &cut, cudaStream_t s) {
   EncodeTiledFn encode = prefill_encode_fn();
   if (!encode) return ROSAQ_ERR_CUDA;
-  if (!prefill_supported(t, nullptr) || M < 1) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
-  const int max_pairs = prefill_pairs(ctx);
+  if (n < 1 || n > kPfMaxProblems) return ROSAQ_ERR_INVALID_ARG;
+  const TiledOperand &t = *ts[0];
+  if (!prefill_supported(t, nullptr) || M < 1 || (n > 1 && t.block_groups > 0)) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
+  const int max_pairs = prefill_clusters(ctx, 1);
   if (max_pairs < 1) return ROSAQ_ERR_CUDA;
   PfParams p{};
-  // {64 channels, tokens, 64-channel block} view of the row-major activations, box = one group (two blocks) of
-  // 128 tokens; rows past M are zero-filled by the copy
+  p.n_prob = n;
+  int col_pairs = 0;
+  for (int i = 0; i < n; ++i) {
+    const TiledOperand &ti = *ts[i];
+    if (ti.d_in != t.d_in || ti.g_fp16 != t.g_fp16 || ti.g_quant != t.g_quant || ti.block_groups != t.block_groups ||
+        (t.g_quant > 0 && ti.bits != t.bits))
+      return ROSAQ_ERR_INVALID_ARG;
+    p.pair_start[i] = col_pairs;
+    p.blob[i] = ti.blob, p.y[i] = ys[i], p.ldy[i] = ldys[i], p.d_out[i] = ti.d_out, p.n_tiles[i] = ti.n_tiles;
+    col_pairs += (ti.n_tiles + 1) / 2;
+  }
+  p.pair_start[n] = col_pairs;
+  p.tile_stride = t.tile_stride;
+  p.g_fp16 = t.g_fp16;
+  p.groups = groups_per_tile(t);
+  p.block_groups = t.block_groups;
+  p.M = M;
+  p.NT = cut.NT;
+  p.n_tok_blocks = cut.n_tok_blocks;
+  p.S = cut.S;
+  const bool dense = t.g_quant == 0;
+  const size_t budget = kPfMaxSmemBytes - 2048;
+  if (dense) {
+    p.NW = (int)std::min<size_t>(kPdMaxStages, budget / (kPdABytes + (p.NT / 2) * 128));
+  } else {
+    p.NW = std::min(kPfMaxNW, (int)((budget - kPfStages * (p.NT / 2) * 256) / kWSlotBytes) / kPfTeams * kPfTeams);
+  }
+  // {64 channels, tokens, 64-channel block} view of the row-major activations, box = a group (two blocks; dense: one) of
+  // NT / 2 tokens; rows past M are zero-filled by the copy
   const cuuint64_t dims[3] = {64, (cuuint64_t)M, (cuuint64_t)(t.d_in / 64)};
   const cuuint64_t strides[2] = {(cuuint64_t)ldx * sizeof(__half), 128};
-  const cuuint32_t box[3] = {64, (cuuint32_t)kPfRows, 2};
+  const cuuint32_t box[3] = {64, (cuuint32_t)(p.NT / 2), dense ? 1u : 2u};
   const cuuint32_t estr[3] = {1, 1, 1};
   if (encode(&p.xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half *>(x), dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return ROSAQ_ERR_CUDA;
-  p.blob = t.blob;
-  p.y = y;
-  p.tile_stride = t.tile_stride;
-  p.ldy = ldy;
-  p.d_out = t.d_out;
-  p.n_tiles = t.n_tiles;
-  p.g_fp16 = t.g_fp16;
-  p.groups = groups_per_tile(t);
-  p.n_col_pairs = (t.n_tiles + 1) / 2;
-  p.n_tok_blocks = (M + kPfTokens - 1) / kPfTokens;
-  p.M = M;
-  const long long units = (long long)p.n_col_pairs * p.n_tok_blocks * p.groups;
+  for (int i = 0; i < n && dense; ++i) {
+    const cuuint64_t wdims[2] = {64, (cuuint64_t)(ts[i]->bytes / 128)}, wstrides[1] = {128};
+    const cuuint32_t wbox[2] = {64, kPdABytes / 128}, west[2] = {1, 1};
+    if (encode(&p.wmap[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ts[i]->blob, wdims, wstrides, wbox, west, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return ROSAQ_ERR_CUDA;
+  }
+  const long long tiles = (long long)col_pairs * p.n_tok_blocks, units = tiles * p.groups;
   if (units < 1 || units > (1ll << 30)) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
   p.units = (int)units;
-  const int n_pairs = units < max_pairs ? (int)units : max_pairs;
-  // one slot of 2 x 256 x 128 floats per pair, in the workspace of the persistent launch (launches of one
+  const int n_pairs = p.S > 0 ? (int)tiles * p.S : (int)std::min<long long>(units, max_pairs);
+  // two slots of 2 x NT x 128 floats per pair, in the workspace of the persistent launch (launches of one
   // context do not overlap on the GPU)
-  if (ctx->pl_partial_bytes < (size_t)n_pairs * 2 * kPfTokens * kTileN * sizeof(float)) return ROSAQ_ERR_ALLOC;
+  if (p.S == 0 && ctx->pl_partial_bytes < (size_t)n_pairs * 4 * p.NT * kTileN * sizeof(float)) return ROSAQ_ERR_ALLOC;
   p.partials = ctx->pl_partials;
   p.flags = ctx->pf_flags;
   p.status = ctx->d_status;
   p.wait_limit = ctx->wait_limit;
-  return t.bits == 4 ? prefill_launch(linear_prefill_kernel<4>, p, n_pairs, s)
-                     : prefill_launch(linear_prefill_kernel<3>, p, n_pairs, s);
+  const PrefillKernel kern = dense ? linear_prefill_kernel<kDenseBits> : (t.bits == 3 ? linear_prefill_kernel<3> : linear_prefill_kernel<4>);
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[3];
+  prefill_config(&cfg, attr, n_pairs, p.S, dense ? kPdThreads : kPfThreads, prefill_smem(dense, p.NT, p.NW), s);
+  if (cudaLaunchKernelEx(&cfg, kern, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return ROSAQ_ERR_CUDA;
+  }
+  return ROSAQ_OK;
 }
 
 }  // namespace rosaq

@@ -22,6 +22,7 @@
 // status word, stops issuing work, still joins the cluster barriers, frees its TMEM and returns.
 #include <cuda.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "linear_common.cuh"
@@ -95,7 +96,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
   __half *const y_out = p.y[prob];
   const long long ldy = p.ldy[prob];
   const int g_begin = p.g_bounds[split], g_end = p.g_bounds[split + 1];
-  const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit, kPair};
+  const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit};
   const uint32_t pair_x = kPair ? (blockIdx.x & 1u) : 0u;      // 0 = leader of the pair
   const uint32_t lead_rank = kPair ? 2u * (uint32_t)split : 0u;   // cluster rank of this pair's leader
   const bool is_lead = pair_x == 0;
@@ -150,7 +151,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         const uint32_t bytes = f16 ? kFp16SubBytes : qbytes;
         for (int sub = 0; sub < nsub; ++sub, ++uc, rw.advance(p.NW)) {
           const int slot = rw.idx;
-          if (!ab.wait_local(bar_w_empty + 8 * slot, rw.lap ^ 1u)) break;
+          if (!ab.wait(bar_w_empty + 8 * slot, rw.lap ^ 1u)) break;
           mbar_arrive_expect_tx(bar_w_full + 8 * slot, bytes);
           bulk_copy_g2s(w_ring + slot * kWSlotBytes, src + (long long)sub * kFp16SubBytes, bytes, bar_w_full + 8 * slot);
         }
@@ -195,7 +196,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         for (int back = 1; back <= p.NA && back <= gc; ++back) {
           const int u = gc - back;
           for (int it = 0; it < kDrainPolls; ++it)
-            if (ab.poll(bar_copy + 8 * (u % p.NA), (u / p.NA) & 1)) break;
+            if (mbar_try_wait(bar_copy + 8 * (u % p.NA), (u / p.NA) & 1)) break;
         }
       }
     }
@@ -227,7 +228,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
       else tc_commit(bar_d_full);
       if (ab.set()) {  // MMAs already issued must retire before the tensor memory is given back
         for (int it = 0; it < kDrainPolls; ++it)
-          if (ab.poll(bar_d_full, 0)) break;
+          if (mbar_try_wait(bar_d_full, 0)) break;
       }
     }
   } else {
@@ -257,7 +258,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         // A parity wait must not be a whole phase early.  The previous fill of this slot may belong to
         // the other team, which can lag by a group: first see that fill released (the same phase the
         // producer waits for), only then wait for the new one.
-        got = got && ab.wait_local(bar_w_empty + 8 * slot, rw.lap ^ 1u) && ab.wait_local(bar_w_full + 8 * slot, rw.lap);
+        got = got && ab.wait(bar_w_empty + 8 * slot, rw.lap ^ 1u) && ab.wait(bar_w_full + 8 * slot, rw.lap);
         got = __all_sync(0xffffffffu, got);        // the TMEM instructions below need the whole warp
         if (!got) {
           ok = false;
@@ -460,7 +461,7 @@ linear_sk_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
   const int u_begin = p.bounds[cta], n_units = p.bounds[cta + 1] - u_begin;
   const int tile0 = u_begin / p.G, g0 = u_begin - tile0 * p.G;
   const int len0 = n_units < p.G - g0 ? n_units : p.G - g0;    // entries of the first tile; the rest start the next tile
-  const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit, false};
+  const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit};
 
   grid_dep_launch_dependents();
 
@@ -504,7 +505,7 @@ linear_sk_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
         bool live = true;
         for (int sub = 0; sub < nsub; ++sub, ++uc, rw.advance(p.NW)) {
           const int slot = rw.idx;
-          if (!ab.wait_local(bar_w_empty + 8 * slot, rw.lap ^ 1u)) {
+          if (!ab.wait(bar_w_empty + 8 * slot, rw.lap ^ 1u)) {
             live = false;
             break;
           }
@@ -612,7 +613,7 @@ linear_sk_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
         const int slot = rw.idx;
         // first see the slot's previous fill released (it may belong to the other team, which can lag by
         // an entry), then wait for the new one: a parity wait must not be a whole phase early
-        got = got && ab.wait_local(bar_w_empty + 8 * slot, rw.lap ^ 1u) && ab.wait_local(bar_w_full + 8 * slot, rw.lap);
+        got = got && ab.wait(bar_w_empty + 8 * slot, rw.lap ^ 1u) && ab.wait(bar_w_full + 8 * slot, rw.lap);
         got = __all_sync(0xffffffffu, got);
         if (!got) {
           ok = false;
@@ -804,6 +805,66 @@ bool sk_bounds(int T, int G, int g_fp16, int P, int *bounds) {
 constexpr bool kUsePdl = true;
 constexpr int kSkTileRatio = 2;
 
+// K splits of the cluster kernel: fill about two CTAs per SM.  Cluster launches place a little less than two CTAs per SM
+// (more than about 2 x SMs - 32 CTAs spill into a second wave), and six splits measured faster than eight on the 32-tile
+// shapes: the exchange grows with the cluster.
+static int linear_tc_splits(const rosaq_ctx *ctx, long long tiles, int G, int most) {
+  const int S = (int)((2 * ctx->sm_count - 32) / (tiles > 0 ? tiles : 1));
+  return std::min(G, S < 1 ? 1 : (S > most ? most : S));
+}
+
+// Moves the columns of every row of y in place: column p goes to col_map[p].  A CTA takes a row into shared memory and writes
+// it back in order: 4 d bytes per row at the copy rate, against a scatter of 2-byte stores in a kernel's epilogue.
+__global__ void __launch_bounds__(256) permute_rows_kernel(__half *__restrict__ y, long long ldy, int d, const int32_t *__restrict__ col_map) {
+  extern __shared__ __align__(16) __half row[];
+  grid_dep_launch_dependents();
+  __half *yr = y + (long long)blockIdx.x * ldy;
+  const int d8 = d >> 3;                                     // (d is a multiple of 128)
+  grid_dep_wait();                                           // y is the previous kernel's output
+  for (int i = threadIdx.x; i < d8; i += blockDim.x) {
+    const uint4 v = reinterpret_cast<const uint4 *>(yr)[i];
+    const int4 c0 = __ldg(reinterpret_cast<const int4 *>(col_map) + 2 * i), c1 = __ldg(reinterpret_cast<const int4 *>(col_map) + 2 * i + 1);
+    const __half *h = reinterpret_cast<const __half *>(&v);
+    row[c0.x] = h[0], row[c0.y] = h[1], row[c0.z] = h[2], row[c0.w] = h[3];
+    row[c1.x] = h[4], row[c1.y] = h[5], row[c1.z] = h[6], row[c1.w] = h[7];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < d8; i += blockDim.x) reinterpret_cast<uint4 *>(yr)[i] = reinterpret_cast<const uint4 *>(row)[i];
+}
+
+int launch_permute_rows(__half *y, int M, long long ldy, int d, const int32_t *col_map, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(M);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = sizeof(__half) * (size_t)d;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, permute_rows_kernel, y, ldy, d, col_map) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return ROSAQ_ERR_CUDA;
+  }
+  return ROSAQ_OK;
+}
+
+// About how long launch_linear_tc_multi takes (us) for more than 128 tokens: 0.9 us per group of a CTA's share (fp16 1.3), two
+// CTAs per SM; a last round that is not full is shorter, its CTAs having an SM to themselves.
+double linear_tc_estimate(const rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts) {
+  const TiledOperand &t = *ts[0];
+  long long tiles = 0;
+  for (int i = 0; i < n; ++i) tiles += ts[i]->n_tiles;
+  tiles *= (M + 127) / 128;
+  const int G = groups_per_tile(t);
+  const int S = linear_tc_splits(ctx, tiles, G, 6);
+  const double rounds = (double)tiles * S / (2.0 * ctx->sm_count), whole = (double)(long long)rounds, part = rounds - whole;
+  const double full = rounds <= 1.0 ? 1.0 : whole + (part > 0 ? 0.65 + 0.4 * part : 0.0);
+  const bool dense = t.g_quant == 0;
+  return (dense ? 7.0 : 5.5) + full * ((G + S - 1) / S) * (dense ? 1.3 : 0.9);
+}
+
 static int launch_linear_sk(const rosaq_ctx *ctx, const __half *x, long long ldx, const TiledOperand &t, const SkParams &q,
                             int P, cudaStream_t s) {
   EncodeTiledFn encode = encode_tiled_fn();
@@ -937,17 +998,10 @@ int launch_linear_tc_multi(const rosaq_ctx *ctx, const __half *x, int M, long lo
     p.NW = nw > 10 ? 10 : nw;
   }
 
-  // K splits: fill about two CTAs per SM; each split gets a contiguous range of groups of roughly
-  // equal cost
+  // K splits; each split gets a contiguous range of groups of roughly equal cost
   const int tiles = n_tiles_all * m_tiles;
-  // (measured: cluster launches place a little less than two CTAs per SM; asking for more than about
-  // 2 x SMs - 32 CTAs spills into a second wave)
-  int S = (2 * ctx->sm_count - 32) / (tiles > 0 ? tiles : 1);
   const int max_splits = pair ? kMaxSplits / 2 : kMaxSplits;    // a cluster holds the S splits of both CTAs of a pair
-  // (six splits measured faster than eight on the 32-tile shapes: the exchange grows with the cluster)
-  const int auto_cap = pair ? max_splits : 6;
-  S = S < 1 ? 1 : (S > auto_cap ? auto_cap : S);
-  if (S > G) S = G;
+  const int S = linear_tc_splits(ctx, tiles, G, pair ? max_splits : 6);
   p.S = S;
   {
     // bound sp is the first group whose

@@ -39,15 +39,34 @@ int pool_create(rosaq_ctx *ctx) {
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = ctx->device;
-  int st = cuda_status(cudaMemPoolCreate(&ctx->pool, &props));
+  MemPool *pool = new (std::nothrow) MemPool();
+  if (!pool) return ROSAQ_ERR_ALLOC;
+  int st = cuda_status(cudaMemPoolCreate(&pool->handle, &props));
+  if (st != ROSAQ_OK) {
+    delete pool;
+    return st;
+  }
+  ctx->pool = pool;
   unsigned long long keep = kPoolKeepBytes;
-  if (st == ROSAQ_OK) st = cuda_status(cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
-  return st;
+  return cuda_status(cudaMemPoolSetAttribute(pool->handle, cudaMemPoolAttrReleaseThreshold, &keep));
+}
+
+// The context and every operand hold the pool: it is destroyed when nothing is allocated from it any more, also when
+// operands outlive their context.
+void pool_release(MemPool *pool) {
+  if (pool && pool->users.fetch_sub(1) == 1) {
+    (void)cudaMemPoolDestroy(pool->handle);
+    delete pool;
+  }
+}
+MemPool *pool_hold(rosaq_ctx *ctx) {
+  ctx->pool->users.fetch_add(1);
+  return ctx->pool;
 }
 
 // usable on any stream once the caller has synchronized `s`, which every user of these does before it returns
 int pool_alloc(rosaq_ctx *ctx, void **p, size_t bytes, cudaStream_t s) {
-  return cuda_status(cudaMallocFromPoolAsync(p, bytes, ctx->pool, s));
+  return cuda_status(cudaMallocFromPoolAsync(p, bytes, ctx->pool->handle, s));
 }
 
 // work in flight on any stream may still read the memory: like cudaFree on plain memory, wait for the device first
@@ -89,8 +108,8 @@ int ensure_workspace(rosaq_ctx *ctx, size_t bytes, cudaStream_t s) {
   return ROSAQ_OK;
 }
 
-constexpr int kPrefillMinTiles = 40, kPrefillMinUnits = 36;
 constexpr int kBlockTokens = 128;
+constexpr int kScatterTokens = 16;
 
 int run_ops(rosaq_ctx *ctx, int M, int n, const PlanOp *ops, cudaStream_t s);
 
@@ -108,21 +127,38 @@ int run_token_blocks(rosaq_ctx *ctx, const __half *x, int M, long long ldx, cons
   return run_ops(ctx, std::min(M, kBlockTokens), nb, ops, s);
 }
 
+// n weights of identical geometry on the same activations (n > 1: no column map)
+int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const TiledOperand *const *ts, const int32_t *col_map,
+             __half *const *ys, const long long *ldys, cudaStream_t s) {
+  if (ctx->impl == 1) {
+    int st = ROSAQ_OK;
+    for (int i = 0; i < n && st == ROSAQ_OK; ++i) st = launch_linear_simt(ctx, x, M, ldx, *ts[i], col_map, ys[i], ldys[i], s);
+    return st;
+  }
+  if (ctx->impl == 6 && n == 1 && M > 64 && M <= kBlockTokens * kPlanMaxOps)
+    return run_token_blocks(ctx, x, M, ldx, *ts[0], col_map, ys[0], ldys[0], s);
+  // A permuted output (head-wise rotation) is a scatter of 2-byte elements; in column order and then moved inside each row
+  // it is faster from 32 tokens on, the second launch included: d = 5120, 16 tokens 5.9 us scattered and 6.5 so, 32: 7.6
+  // and 6.8, 64: 12.5 and 7.5, 512: 38.8 and 12.6, 1900: 97.9 and 31.6.
+  if (ctx->impl == 0 && n == 1 && col_map && M > kScatterTokens && ts[0]->d_out <= kPermuteMaxColumns) {
+    const int st = run_gemm(ctx, x, M, ldx, n, ts, nullptr, ys, ldys, s);
+    return st == ROSAQ_OK ? launch_permute_rows(ys[0], M, ldys[0], ts[0]->d_out, col_map, s) : st;
+  }
+  // More than 128 tokens may run on 256-column tiles shared by pairs of CTAs, one dequantisation per 256 tokens; the
+  // estimates of the two kernels decide.  Per-call kernel / pairs, measured (us): 4096 -> 4096 at 200 tokens 13.4 / 15.8, at
+  // 768 33.6 / 31.3; 4096 -> 3 x 4096 at 200 30.5 / 27.0, at 1900 180 / 172; 4096 -> 2 x 11008 at 200 53.7 / 46.0, at 1900
+  // 338 / 288; 11008 -> 4096 at 200 25.3 / 28.3, at 768 92.8 / 61.2; 5120 x 5120 rotation at 200 21.3 / 18.8, at 1900 157 / 89.
+  if (prefill_supported(*ts[0], col_map) && (ctx->impl == 5 || (ctx->impl == 0 && M > 128))) {
+    const PrefillCut cut = prefill_choose(ctx, M, n, ts);
+    if (ctx->impl == 5 || cut.us < 0.97 * linear_tc_estimate(ctx, M, n, ts)) return launch_linear_prefill(ctx, x, M, ldx, n, ts, ys, ldys, cut, s);
+  }
+  return launch_linear_tc_multi(ctx, x, M, ldx, n, ts, col_map, ys, ldys, s);
+}
+
 int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t, const int32_t *col_map,
              __half *y, long long ldy, cudaStream_t s) {
-  if (ctx->impl == 1) return launch_linear_simt(ctx, x, M, ldx, t, col_map, y, ldy, s);
-  if (ctx->impl == 6 && M > 64 && M <= kBlockTokens * kPlanMaxOps) return run_token_blocks(ctx, x, M, ldx, t, col_map, y, ldy, s);
-  // Large batches of tokens run a weight on 256-column x 256-token tiles shared by pairs of CTAs -- where
-  // the launch is long enough to pay for the exchange of the tiles that two pairs share: at least
-  // kPrefillMinTiles tiles and kPrefillMinUnits 128-channel groups per pair of SMs (measured against the
-  // per-call kernel on the 7B and 13B shapes at 256 ... 2048 tokens).
-  if (prefill_supported(t, col_map) && (ctx->impl == 5 || (ctx->impl == 0 && M > 256))) {
-    const long long tiles = (long long)((t.n_tiles + 1) / 2) * ((M + 255) / 256);
-    const long long units = tiles * groups_per_tile(t);
-    if (ctx->impl == 5 || (tiles >= kPrefillMinTiles && units >= (long long)kPrefillMinUnits * (ctx->sm_count / 2)))
-      return launch_linear_prefill(ctx, x, M, ldx, t, y, ldy, s);
-  }
-  return launch_linear_tc(ctx, x, M, ldx, t, col_map, y, ldy, s);
+  const TiledOperand *ts[1] = {&t};
+  return run_gemm(ctx, x, M, ldx, 1, ts, col_map, &y, &ldy, s);
 }
 
 // The persistent launch (rosaq_plan) pays off when a list is long: it saves a launch, a pipeline fill and a
@@ -197,7 +233,7 @@ int rosaq_create(rosaq_ctx **out, int device) {
   ctx->pl_partials = nullptr;
   ctx->pl_partial_bytes = 0;
   ctx->pl_sync = nullptr;
-  ctx->pf_pairs = 0;
+  for (int i = 0; i < 4; ++i) ctx->pf_clusters[i] = 0;
   ctx->pf_flags = nullptr;
   ctx->pool = nullptr;
   st = pool_create(ctx);
@@ -210,8 +246,8 @@ int rosaq_create(rosaq_ctx **out, int device) {
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->sk_arrive, 0, rosaq::kSkCounterInts * sizeof(int)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pl_sync), rosaq::kPlSyncWords * sizeof(unsigned)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));
-  if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pf_flags), (size_t)ctx->sm_count * sizeof(unsigned)));
-  if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pf_flags, 0, (size_t)ctx->sm_count * sizeof(unsigned)));
+  if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pf_flags), (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
+  if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pf_flags, 0, (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
   // the partial tiles of a launch whose CTAs all share tiles at both ends of two phases (grown if a plan needs more)
   if (st == ROSAQ_OK) {
     const size_t bytes = (size_t)4 * ctx->sk_ctas * rosaq::kSkPartialBytes;
@@ -225,7 +261,7 @@ int rosaq_create(rosaq_ctx **out, int device) {
     if (ctx->d_status) (void)cudaFree(ctx->d_status);
     if (ctx->sk_partials) (void)cudaFree(ctx->sk_partials);
     if (ctx->sk_arrive) (void)cudaFree(ctx->sk_arrive);
-    if (ctx->pool) (void)cudaMemPoolDestroy(ctx->pool);
+    pool_release(ctx->pool);
     delete ctx;
     return st;
   }
@@ -246,7 +282,7 @@ int rosaq_destroy(rosaq_ctx *ctx) {
     if (ctx->pf_flags) (void)cudaFree(ctx->pf_flags);
     if (ctx->pl_partials) (void)cudaFree(ctx->pl_partials);
     plan_free_schedules(ctx);
-    if (ctx->pool) (void)cudaMemPoolDestroy(ctx->pool);   // operands that outlive the context keep their memory until they are freed
+    pool_release(ctx->pool);
     (void)cudaGetLastError();
   }
   delete ctx;
@@ -271,7 +307,7 @@ int rosaq_last_status(rosaq_ctx *ctx, void *stream) {
     if (st != ROSAQ_OK) return st;
     st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));
     if (st != ROSAQ_OK) return st;
-    st = cuda_status(cudaMemset(ctx->pf_flags, 0, (size_t)ctx->sm_count * sizeof(unsigned)));
+    st = cuda_status(cudaMemset(ctx->pf_flags, 0, (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
     if (st != ROSAQ_OK) return st;
   }
   return host;
@@ -325,22 +361,26 @@ static int quantize_impl(rosaq_ctx *ctx, const void *W, int d_in, int d_out, con
   w->group = group;
   w->k_salient = k_salient;
   w->device = ctx->device;
+  w->pool = pool_hold(ctx);
   w->t = make_geometry(d_in, d_out, bits, k_salient / kGroup, (d_in - k_salient) / kGroup, 0);
-  // scratch in the context workspace: the inverse of perm (the kernels index R and W with it, so anything that is not
+  // scratch, from the pool: the inverse of perm (the kernels index R and W with it, so anything that is not
   // a permutation is rejected first) and, for head blocks in a column order of their own, a bounded slab of W'
   const size_t inv_bytes = rot && rot->perm ? (sizeof(int32_t) * (size_t)d_in + 255) / 256 * 256 : 0;
   const size_t spill_bytes = rot ? rotate_quantize_spill_bytes(d_in, d_out, rot->n_blocks, rot->perm != nullptr) : 0;
   st = alloc_blob(ctx, &w->t, s);
-  if (st == ROSAQ_OK && inv_bytes + spill_bytes > 0) st = ensure_workspace(ctx, inv_bytes + spill_bytes, s);
-  int32_t *inv = inv_bytes ? static_cast<int32_t *>(ctx->ws) : nullptr;
+  void *scratch = nullptr;
+  if (st == ROSAQ_OK && inv_bytes + spill_bytes > 0) st = pool_alloc(ctx, &scratch, inv_bytes + spill_bytes, s);
+  int32_t *inv = inv_bytes ? static_cast<int32_t *>(scratch) : nullptr;
   if (st == ROSAQ_OK && inv) st = launch_invert_perm(rot->perm, d_in, inv, ctx->d_status + 1, s);
   if (st == ROSAQ_OK)
     st = launch_rotate_quantize(rot ? rot->q : nullptr, rot ? rot->q_dtype == ROSAQ_F32 : 1, rot ? rot->n_blocks : 1,
                                 rot ? rot->perm : nullptr, inv, static_cast<const __half *>(W), in_scale,
-                                reinterpret_cast<float *>(static_cast<uint8_t *>(ctx->ws) + inv_bytes), spill_bytes, w->t, s);
+                                reinterpret_cast<float *>(static_cast<uint8_t *>(scratch) + inv_bytes), spill_bytes, w->t, s);
+  if (scratch) (void)cudaFreeAsync(scratch, s);
   if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(s));
   if (st != ROSAQ_OK) {
     pool_free(w->t.blob);
+    pool_release(w->pool);
     delete w;
     return st;
   }
@@ -387,6 +427,7 @@ int rosaq_weight_import(rosaq_ctx *ctx, int d_in, int d_out, int bits, int group
   w->group = group;
   w->k_salient = k_salient;
   w->device = ctx->device;
+  w->pool = pool_hold(ctx);
   w->t = make_geometry(d_in, d_out, bits, k_salient / kGroup, (d_in - k_salient) / kGroup, 0);
   st = alloc_blob(ctx, &w->t, s);
   if (st == ROSAQ_OK)
@@ -395,6 +436,7 @@ int rosaq_weight_import(rosaq_ctx *ctx, int d_in, int d_out, int bits, int group
   if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(s));
   if (st != ROSAQ_OK) {
     pool_free(w->t.blob);
+    pool_release(w->pool);
     delete w;
     return st;
   }
@@ -405,8 +447,9 @@ int rosaq_weight_import(rosaq_ctx *ctx, int d_in, int d_out, int bits, int group
 int rosaq_weight_free(rosaq_weight *w) {
   if (!w) return ROSAQ_ERR_INVALID_ARG;
   DeviceGuard guard(w->device);
-  if (guard.ok && w->t.blob) {
+  if (guard.ok) {
     pool_free(w->t.blob);
+    pool_release(w->pool);
     (void)cudaGetLastError();
   }
   delete w;
@@ -441,6 +484,7 @@ int rosaq_rotation_create(rosaq_ctx *ctx, const rosaq_rot *rot, rosaq_rotation *
   if (!r) return ROSAQ_ERR_ALLOC;
   r->d = rot->d;
   r->device = ctx->device;
+  r->pool = pool_hold(ctx);
   r->col_map = nullptr;
   // 128-channel head blocks are stored in pairs, as 256 x 256 blocks with zero off-diagonal quarters (2 MB
   // instead of 1 MB at d = 4096): two adjacent column tiles then multiply the same channels, which lets a
@@ -459,6 +503,7 @@ int rosaq_rotation_create(rosaq_ctx *ctx, const rosaq_rot *rot, rosaq_rotation *
   if (st != ROSAQ_OK) {
     pool_free(r->t.blob);
     pool_free(r->col_map);
+    pool_release(r->pool);
     delete r;
     return st;
   }
@@ -472,6 +517,7 @@ int rosaq_rotation_free(rosaq_rotation *r) {
   if (guard.ok) {
     pool_free(r->t.blob);
     pool_free(r->col_map);
+    pool_release(r->pool);
     (void)cudaGetLastError();
   }
   delete r;
@@ -569,16 +615,11 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
     xin = static_cast<const __half *>(ctx->ws);
     ld = r->d;
   }
-  if (ctx->impl == 1) {
-    for (int i = 0; i < n && st == ROSAQ_OK; ++i)
-      st = launch_linear_simt(ctx, xin, M, ld, w[i]->t, nullptr, static_cast<__half *>(y[i]), ldy[i], s);
-    return st;
-  }
   const TiledOperand *ts[4];
   __half *ys[4];
   long long ldys[4];
   for (int i = 0; i < n; ++i) ts[i] = &w[i]->t, ys[i] = static_cast<__half *>(y[i]), ldys[i] = ldy[i];
-  return launch_linear_tc_multi(ctx, xin, M, ld, n, ts, nullptr, ys, ldys, s);
+  return run_gemm(ctx, xin, M, ld, n, ts, nullptr, ys, ldys, s);
 }
 
 int rosaq_plan_create(rosaq_ctx *ctx, int M, int n_ops, const rosaq_op *ops, rosaq_plan **out) {

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <vector>
 
 #include "rosaq.h"
@@ -166,6 +167,7 @@ __device__ __forceinline__ void load_quant_tile_column(const uint8_t *tile, int 
 }  // namespace rosaq
 
 namespace rosaq {
+constexpr int kPfFlagsPerSm = 2;                    // prefill tiles: two partial-tile slots per CTA
 constexpr int kSkMaxCtas = 320;                     // stream-K grid limit (two CTAs per SM)
 constexpr int kSkCounterInts = 1024;                // arrival counters (one per column tile of a launch)
 constexpr size_t kSkPartialBytes = 128 * 64 * sizeof(float);   // one partial tile: 128 columns x 64 tokens
@@ -239,13 +241,20 @@ struct PlanLaunch {
 };
 }  // namespace rosaq
 
+namespace rosaq {
+struct MemPool {
+  cudaMemPool_t handle = nullptr;
+  std::atomic<int> users{1};          // the context and the operands that live in it
+};
+}  // namespace rosaq
+
 struct rosaq_ctx {
   int device;
   int sm_count;
   int *d_status;       // device status word (0 or ROSAQ_ERR_TIMEOUT)
   void *ws;            // rotated-activation workspace
   size_t ws_bytes;
-  cudaMemPool_t pool;  // memory of the weights and rotations
+  rosaq::MemPool *pool;   // memory of the weights and rotations
   long long wait_limit;
   int impl;            // 0 tensor-core, 1 CUDA-core, 2 tensor-core with CTA pairs, 3 tensor-core without stream-K,
                        // 4 persistent launch for every call, 5 prefill tiles for every weight
@@ -263,13 +272,14 @@ struct rosaq_ctx {
   unsigned *pl_sync;                             // counters, zero between launches
   std::vector<rosaq::PlanSchedule *> pl_schedules;   // one per geometry seen, owned
   // prefill tiles (pairs of CTAs; the partial tiles of a launch live in pl_partials)
-  int pf_pairs;                                  // pairs the device keeps resident at once (0 until first asked for)
-  unsigned *pf_flags;                            // [pair][rank]: a partial tile is stored and not yet fetched; zero between launches
+  int pf_clusters[4];                            // clusters of 1 .. 4 pairs the device keeps resident at once (0 until first asked for)
+  unsigned *pf_flags;                            // [pair][2][rank]: readers that have yet to fetch a partial tile; zero between launches
 };
 
 struct rosaq_weight {
   rosaq::TiledOperand t;
   int group, k_salient, device;
+  rosaq::MemPool *pool;
 };
 
 struct rosaq_plan {
@@ -282,6 +292,7 @@ struct rosaq_rotation {
   rosaq::TiledOperand t;
   int32_t *col_map;    // device [d] or nullptr: rotated column p is stored at position col_map[p]
   int d, device;
+  rosaq::MemPool *pool;
 };
 
 namespace rosaq {
@@ -322,10 +333,19 @@ int launch_linear_tc(const rosaq_ctx *ctx, const __half *x, int M, long long ldx
 int launch_linear_tc_multi(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n,
                            const TiledOperand *const *ts, const int32_t *col_map, __half *const *ys,
                            const long long *ldys, cudaStream_t s);
+double linear_tc_estimate(const rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts);
+constexpr int kPermuteMaxColumns = 24576;            // a row in 48 KB of shared memory
+int launch_permute_rows(__half *y, int M, long long ldy, int d, const int32_t *col_map, cudaStream_t s);
 
 bool prefill_supported(const TiledOperand &t, const int32_t *col_map);
-int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t, __half *y,
-                          long long ldy, cudaStream_t s);
+struct PrefillCut {
+  int NT = 0, n_tok_blocks = 0;   // tokens per tile
+  int S = 0;                      // > 0: a cluster of S pairs per tile; 0: equal shares of the whole launch
+  double us = 0;                  // estimate
+};
+PrefillCut prefill_choose(rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts);
+int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const TiledOperand *const *ts,
+                          __half *const *ys, const long long *ldys, const PrefillCut &cut, cudaStream_t s);
 
 int plan_build_schedule(const std::vector<PlanGeom> &ops, int n_ctas, const int *cost, PlanSchedule *out);
 int plan_ctas(rosaq_ctx *ctx);

@@ -1,0 +1,105 @@
+"""The prefill tiles (implementation 5) in each way a launch can be cut: a cluster of one to four pairs of CTAs per tile,
+equal shares with the exchange through L2 (two and more holders of a tile), the all-fp16 operand, several weights in one
+launch; ragged token counts and widths; and the head-wise rotation written in column order and moved inside its rows.
+Sampled columns against the oracle, every column against the per-call kernels (implementation 3: the same sums in another
+order, one rounding to fp16: 2e-4 as elsewhere), the same bits again, also when a captured launch is replayed on other input."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import rosaq_oracle as orc
+from paper_2506_13472_b200 import binding as rb
+from paper_2506_13472_b200 import synth
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = rb.Context(0)
+    yield c
+    c.close()
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def same(a, b):
+    return torch.equal(a.view(torch.int16), b.view(torch.int16))
+
+
+@pytest.mark.parametrize("M,d_in,widths,bits", [
+    (200, 1024, [384], 4),              # a cluster of several pairs per tile
+    (255, 896, [1160], 3),              # ragged tokens, a last tile without a second column tile, groups that do not divide evenly
+    (33, 1152, [6000], 4),              # narrow token tile, one pair per tile
+    (300, 384, [512, 200, 136], 4),     # three weights, two token blocks
+    (520, 1024, [11008, 1000], 3),      # equal shares
+    (260, 2048, [10496], 4),            # equal shares, many holders of a tile
+])
+def test_prefill_cuts(ctx, M, d_in, widths, bits):
+    Ws = [synth.weights(d_in, n, seed=91, key=f"cut{n}", outlier_frac=0.01) for n in widths]
+    ws = [ctx.quantize(dev(W), None, bits=bits, k_salient=128) for W in Ws]
+    rng = synth.rng_for(91, "x", M, d_in)
+    xa, xb = (dev(rng.standard_normal((M, d_in)).astype(np.float16)) for _ in range(2))
+    bufs = [torch.full((M + 1, n + 16), 7.0, dtype=torch.float16, device="cuda") for n in widths]
+    outs = [b[:M, :n] for b, n in zip(bufs, widths)]
+    ctx.set_linear_impl(3)
+    ref = [y.clone() for y in ctx.linear_multi(xa, ws)]
+    ctx.set_linear_impl(5)
+    try:
+        got = [y.clone() for y in ctx.linear_multi(xa, ws, outs=outs)]
+        for b, n in zip(bufs, widths):
+            assert torch.all(b[M:] == 7.0) and torch.all(b[:, n:] == 7.0)              # nothing written outside
+        want_b = [y.clone() for y in ctx.linear_multi(xb, ws)]
+        x = xa.clone()
+        ys = [torch.empty((M, n), dtype=torch.float16, device="cuda") for n in widths]
+        side = torch.cuda.Stream()
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side):
+            for _ in range(2):                                                           # chained launches
+                ctx.linear_multi(x, ws, outs=ys)
+        for src, want in ((xa, got), (xb, want_b), (xa, got)):
+            x.copy_(src)
+            torch.cuda.synchronize()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert all(same(y, w) for y, w in zip(ys, want))
+    finally:
+        ctx.set_linear_impl(0)
+    assert ctx.last_status() == rb.ROSAQ_OK
+    for y, r, W, n in zip(got, ref, Ws, widths):
+        assert H.rel_fro(y.cpu().numpy(), r.cpu().numpy()) <= 2e-4
+        cols = synth.sample_columns(n, 24, 91, f"cut{n}")
+        qd = H.oracle_quantized(W, None, None, bits, 128, cols=cols)
+        assert H.rel_fro(y.cpu().numpy()[:, cols], orc.forward(xa.cpu().numpy(), qd, None)) <= H.REL_TOL_Y
+
+
+@pytest.mark.parametrize("M", [5, 200, 300])
+@pytest.mark.parametrize("d,heads", [(512, 1), (640, 1), (512, 4), (384, 3), (768, 2)])
+def test_rotations_at_prefill_sizes(ctx, M, d, heads):
+    """Dense and head-wise rotations, with and without a column order: heads of 128 channels in pairs, an odd number of them
+    (not a pair's operand), heads of three groups.  Implementations 5 and 0 against the oracle; untouched columns."""
+    rng = synth.rng_for(92, "rot", d, heads)
+    dh = d // heads
+    Rb = np.stack([synth.orthogonal_qr(dh, rng) for _ in range(heads)]).astype(np.float16)
+    x = rng.standard_normal((M, d)).astype(np.float16)
+    for perm in (None, rng.permutation(d).astype(np.int32)):
+        rot = ctx.rotation_create(dev(Rb if heads > 1 else Rb[0]), None if perm is None else dev(perm))
+        full = np.zeros((d, d))
+        for h in range(heads):
+            full[h * dh:(h + 1) * dh, h * dh:(h + 1) * dh] = Rb[h].astype(np.float64)
+        ref = x.astype(np.float64) @ (full if perm is None else full[:, perm])
+        for impl in (0, 5):
+            ctx.set_linear_impl(impl)
+            try:
+                buf = torch.full((M, d + 8), 7.0, dtype=torch.float16, device="cuda")
+                ctx.rotate(dev(x), rot, out=buf[:, :d])
+                assert torch.all(buf[:, d:] == 7.0)
+                assert H.rel_fro(buf[:, :d].cpu().numpy(), ref) <= 1e-3
+            finally:
+                ctx.set_linear_impl(0)
+        rot.free()
+    assert ctx.last_status() == rb.ROSAQ_OK
