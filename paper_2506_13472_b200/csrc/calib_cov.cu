@@ -12,6 +12,11 @@
 // directly by it or its sibling.  The other tiles add themselves to C and their transpose to the
 // mirrored position.  Both triangles are therefore written and C stays exactly symmetric.
 //
+// When the tiles are few (small d, or head-wise blocks: 32 tiles of 128 x 128 for 148 SMs) the tokens are
+// split over a cluster of up to eight CTAs per tile: each accumulates its range, the partial tiles meet in distributed
+// shared memory, every CTA adds a share of the rows in order of the splits (a call gives the same bits every time) and
+// updates C there.
+//
 // fp32 activations (and blocks narrower than 64 channels) keep the CUDA-core path of quantize.cu,
 // whose products are exact.
 //
@@ -22,6 +27,7 @@
 #include <mutex>
 
 #include "rosaq_internal.cuh"
+#include "cov_common.cuh"
 
 namespace rosaq {
 
@@ -42,6 +48,7 @@ struct CovParams {
   int dh, bn;                  // block edge; tile columns (MMA N): 256, or 128 for narrow blocks
   int use3d;                   // the 3-D maps are valid (channel count a multiple of 64)
   long long n_tokens;
+  int splits;                  // CTAs (pairs) of a cluster that share a tile's tokens: 1, 2, 4 or 8
   int *status;
   long long wait_limit;
 };
@@ -125,6 +132,23 @@ struct CovAbort {
   }
 };
 
+// One row of the accumulator (lane = row), bn columns, to shared memory
+__device__ __forceinline__ void cov_stage_row(uint32_t lane_addr, float *row, int bn) {
+  for (int c0 = 0; c0 < bn; c0 += 32) {
+    uint32_t v[32];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                   : "=r"(v[8 * q]), "=r"(v[8 * q + 1]), "=r"(v[8 * q + 2]), "=r"(v[8 * q + 3]), "=r"(v[8 * q + 4]), "=r"(v[8 * q + 5]),
+                     "=r"(v[8 * q + 6]), "=r"(v[8 * q + 7])
+                   : "r"(lane_addr + c0 + 8 * q)
+                   : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int e = 0; e < 32; ++e) row[c0 + e] = __uint_as_float(v[e]);
+  }
+}
+
 __global__ void __launch_bounds__(kCovThreads, 1)
 cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap map2,
               const __grid_constant__ CUtensorMap map4, const CovParams p) {
@@ -152,7 +176,10 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
   const int b_boxes = p.bn / 64;
   // on a diagonal tile operand A is the slice of B that holds row block bi
   const uint32_t a_in_b = diag ? (uint32_t)((bi % ratio) * kOperandBytes) : 0u;
-  const int n_stages_total = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
+  const int Z = p.splits, z = blockIdx.z;
+  const int n_stages_all = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
+  const int s_begin = (int)((long long)n_stages_all * z / Z), n_stages_total = (int)((long long)n_stages_all * (z + 1) / Z) - s_begin;
+  cov_grid_dep_launch();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kCovStages; ++i) {
@@ -177,12 +204,13 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
 
   if (warp == 0) {
     if (lane == 0) {
+      cov_grid_dep_wait();                           // X may be the previous kernel's output
       int issued = 0, idx = 0;
       uint32_t lap = 0;
       for (int s = 0; s < n_stages_total && !ab.set(); ++s, ++issued) {
         if (!ab.wait(bar_empty + 8 * idx, lap ^ 1u)) break;
         const uint32_t dst = base + idx * kStageBytes;
-        const int tok = s * kCovTokens;
+        const int tok = (s_begin + s) * kCovTokens;
         mbar_arrive_expect_tx(bar_full + 8 * idx, (uint32_t)((diag ? 0 : 2) + b_boxes) * kBoxBytes);
         if (p.use3d) {
           if (!diag) tma_load_3d(dst, &map2, bar_full + 8 * idx, tok, col_a >> 6);
@@ -237,21 +265,18 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
     have = __all_sync(0xffffffffu, have && !ab.set());
     float *stage = reinterpret_cast<float *>(gen);    // [128][bn + 1] fp32, reuses the operand ring
     const int pitch = p.bn + 1;
+    cov_grid_dep_wait();                              // C may still be in use by the previous kernel
     if (have) {
       tc_fence_after();
-      const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-      for (int c0 = 0; c0 < p.bn; c0 += 8) {
-        uint32_t v[8];
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                     : "r"(lane_addr + c0)
-                     : "memory");
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int e = 0; e < 8; ++e) stage[row * pitch + c0 + e] = __uint_as_float(v[e]);
-      }
+      cov_stage_row(tmem + ((uint32_t)(quad * 32) << 16), stage + row * pitch, p.bn);
     }
-    asm volatile("bar.sync 1, 128;" ::: "memory");    // the four epilogue warps
+    cov_epi_bar();
+    const int r_begin = kCovTile * z / Z, r_end = kCovTile * (z + 1) / Z;   // rows of the tile that this CTA finishes
+    if (Z > 1) {
+      cov_cluster_sync();                             // every partial tile is staged
+      if (!ab.set()) cov_sum_rows(smem_u32(stage), stage, pitch, p.bn, r_begin, r_end, Z, 1, 0u, (int)threadIdx.x - 64, 128);
+      cov_epi_bar();
+    }
     if (!ab.set()) {
       const int tid = threadIdx.x - 64;               // 0..127
       float *Cb = p.C + (long long)h * p.dh * p.dh;
@@ -259,13 +284,13 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
       // C[i0 + r][j0 + c] += tile[r][c]: a warp touches 32 consecutive floats of one row of C
       // The update of C is latency-bound (read-modify-write through L2), so each thread keeps eight
       // independent 16-byte loads in flight.  Direct part: C[i0 + r][j0 + 4 q .. + 3] += tile[r][4 q .. + 3].
-      const int n_rows = min(kCovTile, p.dh - i0), n_cols = min(p.bn, p.dh - j0);   // both multiples of 8
+      const int n_rows = min(r_end, p.dh - i0), n_cols = min(p.bn, p.dh - j0);   // both multiples of 8
       {
         const int quads = p.bn >> 2, sets = 128 / quads;   // 64 x 2 or 32 x 4 (column quads x interleaved row sets)
         const int q = tid % quads, r_first = tid / quads;
         if (4 * q < n_cols) {
           float *dst = Cb + (long long)i0 * p.dh + j0 + 4 * q;
-          for (int r0 = r_first; r0 < n_rows; r0 += 8 * sets) {
+          for (int r0 = r_begin + r_first; r0 < n_rows; r0 += 8 * sets) {
             float4 old[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -288,20 +313,21 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
       }
       // mirror: C[j0 + c][i0 + 4 q .. + 3] += tile[4 q .. + 3][c]
       if (!diag) {
-        const int q = tid & 31, c_first = tid >> 5;       // 32 row quads of the tile x 4 interleaved column sets
+        const int n_quads = (r_end - r_begin) / 4, sets = 128 / n_quads;      // row quads of the share x interleaved column sets
+        const int q = r_begin / 4 + tid % n_quads, c_first = tid / n_quads;
         if (4 * q < n_rows) {
           float *dst = Cb + (long long)j0 * p.dh + i0 + 4 * q;
-          for (int c0 = c_first; c0 < n_cols; c0 += 32) {
+          for (int c0 = c_first; c0 < n_cols; c0 += 8 * sets) {
             float4 old[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              const int c = c0 + 4 * e;
+              const int c = c0 + sets * e;
               old[e] = c < n_cols ? __ldcg(reinterpret_cast<const float4 *>(dst + (long long)c * p.dh))
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              const int c = c0 + 4 * e;
+              const int c = c0 + sets * e;
               if (c < n_cols) {
                 const float *t = stage + (4 * q) * pitch + c;
                 *reinterpret_cast<float4 *>(dst + (long long)c * p.dh) =
@@ -315,6 +341,11 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
     }
   }
 
+  __syncwarp();
+  if (Z > 1) {
+    if (warp < 2) cov_cluster_sync();                 // (the epilogue warps are past this one)
+    cov_cluster_sync();                               // nobody reads this CTA's tile any more
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -358,10 +389,10 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t smem_addr, uint32_t ran
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint32_t lead) {
   asm volatile(
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"((unsigned short)3)
+      "h"((unsigned short)(3u << lead))
       : "memory");
 }
 __device__ __forceinline__ void tc_mma4_ss_pair(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
@@ -376,11 +407,7 @@ __device__ __forceinline__ void tc_mma4_ss_pair(uint32_t d_tmem, uint64_t a, uin
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCovThreads, 1)
+__global__ void __launch_bounds__(kCovThreads, 1)
 cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap map2,
                    const CovParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -392,8 +419,8 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   const uint32_t bar_empty = smem_u32(&bars[kPairStages]);           // stage free again (multicast commit)
   const uint32_t bar_d = smem_u32(&bars[2 * kPairStages]);           // accumulators final (multicast commit)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint32_t rank;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  // a cluster of 2 Z CTAs: ranks 2 z, 2 z + 1 are the pair with split z of the tokens
+  const uint32_t rank = blockIdx.x & 1u, lead = 2u * blockIdx.z;
   const CovAbort ab{reinterpret_cast<volatile int *>(&misc[1]), p.status, p.wait_limit};
 
   // 256 x 256 tile (bi >= bj) of the lower triangle from the pair index bi (bi + 1) / 2 + bj
@@ -405,7 +432,10 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   const bool diag = bi == bj;
   const int i0 = bi * 256 + (int)rank * kCovTile, j0 = bj * 256;
   const int col_a = h * p.dh + i0, col_b = h * p.dh + j0 + (int)rank * kCovTile;
-  const int n_stages_total = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
+  const int Z = p.splits, z = blockIdx.z;
+  const int n_stages_all = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
+  const int s_begin = (int)((long long)n_stages_all * z / Z), n_stages_total = (int)((long long)n_stages_all * (z + 1) / Z) - s_begin;
+  cov_grid_dep_launch();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kPairStages; ++i) {
@@ -425,20 +455,21 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();                                // the peer's barriers and tensor memory exist
+  cov_cluster_sync();                                // the peer's barriers and tensor memory exist
   tc_fence_after();
   const uint32_t tmem = misc[0];
 
   if (warp == 0) {
     if (lane == 0) {
-      const uint32_t lead_tma = map_to_rank(bar_tma, 0);     // the leader's barriers, as cluster addresses
+      cov_grid_dep_wait();                                   // X may be the previous kernel's output
+      const uint32_t lead_tma = map_to_rank(bar_tma, lead);  // the leader's barriers, as cluster addresses
       const uint32_t stage_bytes = diag ? kOperandBytes : kPairStageBytes;
       int issued = 0, idx = 0;
       uint32_t lap = 0;
       for (int s = 0; s < n_stages_total && !ab.set(); ++s, ++issued) {
         if (!ab.wait(bar_empty + 8 * idx, lap ^ 1u)) break;
         const uint32_t dst = base + idx * kPairStageBytes;
-        const int tok = s * kCovTokens;
+        const int tok = (s_begin + s) * kCovTokens;
         if (rank == 0) mbar_arrive_expect_tx(bar_tma + 8 * idx, 2 * stage_bytes);   // both CTAs' bytes
         const uint32_t lb = lead_tma + 8 * idx;
         if (p.use3d) {
@@ -480,10 +511,10 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         const uint64_t a = diag ? b : make_mn_desc(b_addr - kOperandBytes);
         tc_mma4_ss_pair(tmem, a, b, idesc, accumulate);
         accumulate = 1;
-        tc_commit_pair(bar_empty + 8 * idx);
+        tc_commit_pair(bar_empty + 8 * idx, lead);
         if (++idx == kPairStages) idx = 0, lap ^= 1u;
       }
-      tc_commit_pair(bar_d);
+      tc_commit_pair(bar_d, lead);
       if (ab.set()) {  // MMAs already issued must retire before the tensor memory is given back
         for (int it = 0; it < kCovDrainPolls; ++it)
           if (mbar_try_wait(bar_d, 0)) break;
@@ -497,32 +528,29 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
     have = __all_sync(0xffffffffu, have && !ab.set());
     float *stage = reinterpret_cast<float *>(gen);    // [128][257] fp32, reuses the operand ring
     constexpr int pitch = 257;
+    cov_grid_dep_wait();                              // C may still be in use by the previous kernel
     if (have) {
       tc_fence_after();
-      const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-      for (int c0 = 0; c0 < 256; c0 += 8) {
-        uint32_t v[8];
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                     : "r"(lane_addr + c0)
-                     : "memory");
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int e = 0; e < 8; ++e) stage[row * pitch + c0 + e] = __uint_as_float(v[e]);
-      }
+      cov_stage_row(tmem + ((uint32_t)(quad * 32) << 16), stage + row * pitch, 256);
     }
-    asm volatile("bar.sync 1, 128;" ::: "memory");    // the four epilogue warps
+    cov_epi_bar();
+    const int r_begin = kCovTile * z / Z, r_end = kCovTile * (z + 1) / Z;   // rows of the tile that this CTA finishes
+    if (Z > 1) {
+      cov_cluster_sync();                             // every partial tile is staged
+      if (!ab.set()) cov_sum_rows(smem_u32(stage), stage, pitch, 256, r_begin, r_end, Z, 2, rank, (int)threadIdx.x - 64, 128);
+      cov_epi_bar();
+    }
     if (!ab.set() && i0 < p.dh) {
       const int tid = threadIdx.x - 64;               // 0..127
       float *Cb = p.C + (long long)h * p.dh * p.dh;
-      const int n_rows = min(kCovTile, p.dh - i0), n_cols = min(256, p.dh - j0);   // both multiples of 8
+      const int n_rows = min(r_end, p.dh - i0), n_cols = min(256, p.dh - j0);   // both multiples of 8
       // The update of C is latency-bound (read-modify-write through L2), so each thread keeps eight
       // independent 16-byte loads in flight.  Direct part: C[i0 + r][j0 + 4 q .. + 3] += tile[r][4 q .. + 3].
       {
         const int q = tid & 63, r_first = tid >> 6;       // 64 column quads x 2 interleaved row sets
         if (4 * q < n_cols) {
           float *dst = Cb + (long long)i0 * p.dh + j0 + 4 * q;
-          for (int r0 = r_first; r0 < n_rows; r0 += 16) {
+          for (int r0 = r_begin + r_first; r0 < n_rows; r0 += 16) {
             float4 old[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -545,20 +573,21 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
       }
       // mirror: C[j0 + c][i0 + 4 q .. + 3] += tile[4 q .. + 3][c]
       if (!diag) {
-        const int q = tid & 31, c_first = tid >> 5;       // 32 row quads of the tile x 4 interleaved column sets
+        const int n_quads = (r_end - r_begin) / 4, sets = 128 / n_quads;      // row quads of the share x interleaved column sets
+        const int q = r_begin / 4 + tid % n_quads, c_first = tid / n_quads;
         if (4 * q < n_rows) {
           float *dst = Cb + (long long)j0 * p.dh + i0 + 4 * q;
-          for (int c0 = c_first; c0 < n_cols; c0 += 32) {
+          for (int c0 = c_first; c0 < n_cols; c0 += 8 * sets) {
             float4 old[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              const int c = c0 + 4 * e;
+              const int c = c0 + sets * e;
               old[e] = c < n_cols ? __ldcg(reinterpret_cast<const float4 *>(dst + (long long)c * p.dh))
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              const int c = c0 + 4 * e;
+              const int c = c0 + sets * e;
               if (c < n_cols) {
                 const float *t = stage + (4 * q) * pitch + c;
                 *reinterpret_cast<float4 *>(dst + (long long)c * p.dh) =
@@ -572,9 +601,11 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
     }
   }
 
+  __syncwarp();
+  if (Z > 1 && warp < 2) cov_cluster_sync();         // (the epilogue warps are past this one)
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();                                // neither CTA leaves while the pair's MMAs may touch it
+  cov_cluster_sync();                                // neither CTA leaves while the pair's MMAs may touch it
   if (warp == 1) {
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kCovTmemCols) : "memory");
@@ -605,7 +636,7 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
   const int dh = d / n_blocks;
   EncodeTiledFn encode = cov_encode_fn();
   if (x_dtype != ROSAQ_F16 || dh < 64 || !encode || n_tokens > 0x7fffffffll)
-    return launch_cov_fma(X, x_dtype, n_tokens, d, ldx, n_blocks, C, s);
+    return launch_cov_fma(ctx->sm_count, X, x_dtype, n_tokens, d, ldx, n_blocks, C, s);
 
   CUtensorMap xmap;
   {
@@ -658,8 +689,23 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
   const int n_row_blocks = (dh + kCovTile - 1) / kCovTile, ratio = p.bn / kCovTile;
   int tiles = 0;
   for (int bi = 0; bi < n_row_blocks; ++bi) tiles += bi / ratio + 1;
-  if (dh >= 512) {
-    // wide blocks: 256 x 256 tiles on CTA pairs
+  // Single CTAs with 128 x 256 tiles, or pairs with 256 x 256 tiles (half the loads per product).  A stage of 64 tokens
+  // costs either the same time, so what counts is the number of stages in a row: with the tokens split as far as SMs,
+  // cluster size and tokens (four stages each) allow, pairs are taken unless they leave the chip emptier (512 ... 896 channels).
+  const int nb2 = (dh + 255) / 256, pair_tiles = nb2 * (nb2 + 1) / 2;
+  const long long stages = (n_tokens + kCovTokens - 1) / kCovTokens;
+  // (a cluster lives inside one GPC and these CTAs fill an SM: about 7/8 of the SMs can hold clusters of four, 3/4 of eight;
+  // 2048 channels as 36 clusters of four run in two rounds, 47.8 us against 35.5 unsplit)
+  auto splits = [&](long long ctas, int ctas_per_split) {
+    int z = 1;
+    for (int c : {2, 4, 8}) {
+      const int slots = c == 2 ? ctx->sm_count : (c == 4 ? ctx->sm_count * 7 / 8 : ctx->sm_count * 3 / 4);
+      if (c > ctas_per_split && cov_splits(ctas, slots, stages / 4, c / ctas_per_split) == c / ctas_per_split) z = c / ctas_per_split;
+    }
+    return z;
+  };
+  const int z1 = splits((long long)tiles * n_blocks, 1), z2 = splits(2ll * pair_tiles * n_blocks, 2);
+  if (dh >= 512 && z2 >= z1) {
     const size_t smem2 = 1024 + (size_t)kPairStages * kPairStageBytes;
     static bool attr2_done_all[64] = {};
     bool &attr2_done = attr2_done_all[ctx->device];
@@ -670,14 +716,11 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
       }
       attr2_done = true;
     }
-    const int nb2 = (dh + 255) / 256;
-    dim3 grid2(2 * (nb2 * (nb2 + 1) / 2), n_blocks);
-    cov_tc_pair_kernel<<<grid2, kCovThreads, smem2, s>>>(xmap, map2, p);
-    return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
+    p.splits = z2;
+    return cov_launch(cov_tc_pair_kernel, dim3(2 * pair_tiles, n_blocks, z2), kCovThreads, smem2, 2, z2, s, xmap, map2, p);
   }
-  dim3 grid(tiles, n_blocks);
-  cov_tc_kernel<<<grid, kCovThreads, smem, s>>>(xmap, map2, map4, p);
-  return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
+  p.splits = z1;
+  return cov_launch(cov_tc_kernel, dim3(tiles, n_blocks, z1), kCovThreads, smem, 1, z1, s, xmap, map2, map4, p);
 }
 
 }  // namespace rosaq

@@ -9,6 +9,7 @@
 #include <algorithm>
 
 #include "rosaq_internal.cuh"
+#include "cov_common.cuh"
 
 namespace rosaq {
 
@@ -430,14 +431,19 @@ int launch_rotate_quantize(const void *q, int q_is_f32, int n_blocks, const int3
 // tokens in the same order, so the mirrored bits are those a tile of its own would produce).
 template <typename T>
 __global__ void __launch_bounds__(kFmaThreads, 2)
-gram_fma_kernel(const T *__restrict__ X, long long ldx, int dh, float *__restrict__ C, int K) {
+gram_fma_kernel(const T *__restrict__ X, long long ldx, int dh, float *__restrict__ C, int n_tokens, int Z) {
   extern __shared__ __align__(16) float tile[];
   const FmaThread ft;
   int bi = 0;
   while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
   const int bj = blockIdx.x - bi * (bi + 1) / 2;
   const int i0 = bi * kBM, n0 = bj * kBN;
-  X += (long long)blockIdx.y * dh;
+  // split z of the tokens (a cluster shares the tile), cut at multiples of the K step
+  const int z = blockIdx.z, steps = (n_tokens + kBK - 1) / kBK;
+  const int t0 = (int)((long long)steps * z / Z) * kBK, K = min(n_tokens, (int)((long long)steps * (z + 1) / Z) * kBK) - t0;
+  cov_grid_dep_launch();
+  cov_grid_dep_wait();
+  X += (long long)t0 * ldx + (long long)blockIdx.y * dh;
   C += (long long)blockIdx.y * dh * dh;
   auto fetch = [&](int k, int c, Raw4<T> &raw) {                     // (dh and ldx are multiples of 8, X is 16-byte aligned)
     if (k < K && c + 3 < dh) raw.load4(X + (long long)k * ldx + c);
@@ -449,34 +455,47 @@ gram_fma_kernel(const T *__restrict__ X, long long ldx, int dh, float *__restric
       [&](int k, int c, Raw4<T> &raw) { fetch(k, n0 + c, raw); }, [](int) { return 0.f; }, acc);
   store_tile_smem(tile, ft, acc);
   __syncthreads();
+  const int r_begin = kBM * z / Z, r_end = kBM * (z + 1) / Z;        // rows of the tile that this CTA finishes
+  if (Z > 1) {
+    cov_cluster_sync();
+    cov_sum_rows((uint32_t)__cvta_generic_to_shared(tile), tile, kTilePitch, kBN, r_begin, r_end, Z, 1, 0u, threadIdx.x, kFmaThreads);
+    __syncthreads();
+  }
   const int c4 = (threadIdx.x & 31) * 4, r_first = threadIdx.x >> 5;
   auto add4 = [](float *dst, float4 v) {
     const float4 o = *reinterpret_cast<const float4 *>(dst);
     *reinterpret_cast<float4 *>(dst) = make_float4(__fadd_rn(o.x, v.x), __fadd_rn(o.y, v.y), __fadd_rn(o.z, v.z), __fadd_rn(o.w, v.w));
   };
   if (n0 + c4 < dh)
-    for (int r = r_first; r < kBM && i0 + r < dh; r += 4)
+    for (int r = r_begin + r_first; r < r_end && i0 + r < dh; r += 4)
       add4(C + (long long)(i0 + r) * dh + n0 + c4, *reinterpret_cast<const float4 *>(tile + r * kTilePitch + c4));
-  if (bi != bj && i0 + c4 < dh)
-    for (int r = r_first; r < kBN && n0 + r < dh; r += 4) {
-      const float *tc = tile + c4 * kTilePitch + r;
-      add4(C + (long long)(n0 + r) * dh + i0 + c4, make_float4(tc[0], tc[kTilePitch], tc[2 * kTilePitch], tc[3 * kTilePitch]));
+  // mirror: the share's rows, four at a time, x all columns
+  const int n_quads = (r_end - r_begin) / 4, m4 = r_begin + 4 * (threadIdx.x % n_quads);
+  if (bi != bj && i0 + m4 < dh)
+    for (int r = threadIdx.x / n_quads; r < kBN && n0 + r < dh; r += kFmaThreads / n_quads) {
+      const float *tc = tile + m4 * kTilePitch + r;
+      add4(C + (long long)(n0 + r) * dh + i0 + m4, make_float4(tc[0], tc[kTilePitch], tc[2 * kTilePitch], tc[3 * kTilePitch]));
     }
+  if (Z > 1) cov_cluster_sync();                                     // nobody reads this CTA's tile any more
 }
 
-int launch_cov_fma(const void *X, int x_dtype, long long n_tokens, int d, long long ldx, int n_blocks, float *C,
+int launch_cov_fma(int sm_count, const void *X, int x_dtype, long long n_tokens, int d, long long ldx, int n_blocks, float *C,
                    cudaStream_t s) {
   const int dh = d / n_blocks, nb = (dh + kBM - 1) / kBM;
   const dim3 grid(nb * (nb + 1) / 2, n_blocks);
   if (!allow_smem(gram_fma_kernel<float>, kFmaSmemBytes) || !allow_smem(gram_fma_kernel<__half>, kFmaSmemBytes)) return ROSAQ_ERR_CUDA;
   for (long long t0 = 0; t0 < n_tokens; t0 += 1ll << 30) {           // (the kernel counts tokens in 32 bits)
     const int n = (int)std::min(n_tokens - t0, 1ll << 30);
-    if (x_dtype == ROSAQ_F32)
-      gram_fma_kernel<float><<<grid, kFmaThreads, kFmaSmemBytes, s>>>(static_cast<const float *>(X) + t0 * ldx, ldx, dh, C, n);
-    else
-      gram_fma_kernel<__half><<<grid, kFmaThreads, kFmaSmemBytes, s>>>(static_cast<const __half *>(X) + t0 * ldx, ldx, dh, C, n);
+    // (two CTAs fit an SM; a split keeps at least 64 tokens)
+    const int Z = cov_splits((long long)grid.x * grid.y, 2 * sm_count, n / 64, 8);
+    const dim3 g(grid.x, grid.y, Z);
+    const int st = x_dtype == ROSAQ_F32 ? cov_launch(gram_fma_kernel<float>, g, kFmaThreads, kFmaSmemBytes, 1, Z, s,
+                                                     static_cast<const float *>(X) + t0 * ldx, ldx, dh, C, n, Z)
+                                        : cov_launch(gram_fma_kernel<__half>, g, kFmaThreads, kFmaSmemBytes, 1, Z, s,
+                                                     static_cast<const __half *>(X) + t0 * ldx, ldx, dh, C, n, Z);
+    if (st != ROSAQ_OK) return st;
   }
-  return cudaGetLastError() == cudaSuccess ? ROSAQ_OK : ROSAQ_ERR_CUDA;
+  return ROSAQ_OK;
 }
 
 // =====================================================================================

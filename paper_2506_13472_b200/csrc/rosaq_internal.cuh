@@ -322,7 +322,7 @@ int launch_import(const TiledOperand &t, const uint32_t *qw, const __half *scale
                   const __half *salient, cudaStream_t s);
 int launch_rotation_tiles(const __half *q, int d, int n_blocks, const TiledOperand &t, cudaStream_t s);
 int launch_invert_perm(const int32_t *perm, int d, int32_t *inv, int *bad, cudaStream_t s);
-int launch_cov_fma(const void *X, int x_dtype, long long n_tokens, int d, long long ldx, int n_blocks, float *C,
+int launch_cov_fma(int sm_count, const void *X, int x_dtype, long long n_tokens, int d, long long ldx, int n_blocks, float *C,
                    cudaStream_t s);
 int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tokens, int d, long long ldx,
                int n_blocks, float *C, cudaStream_t s);

@@ -1,0 +1,45 @@
+"""rosaq_calib_cov where few tiles make a cluster of CTAs share each tile's tokens: every split count of the three kernels
+(pairs, single CTAs, fp32), ragged tokens and widths, two accumulated calls, the same bits on a second run."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import rosaq_oracle as orc
+from paper_2506_13472_b200 import binding as rb
+from paper_2506_13472_b200 import synth
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,n_tokens,d,n_blocks", [
+    (np.float16, 2100, 512, 1),       # single CTAs, 8 splits
+    (np.float16, 1030, 768, 1),       # 4 splits (tokens), columns past the last whole tile
+    (np.float16, 1500, 1032, 1),      # pairs, 4 splits, d no multiple of 64
+    (np.float16, 600, 1288, 1),       # pairs, 2 splits
+    (np.float16, 2049, 640, 5),       # head blocks of 128, 8 splits
+    (np.float16, 515, 1024, 2),       # two blocks of 512
+    (np.float32, 1001, 256, 1),       # fp32, 8 splits, mirrored shares
+    (np.float32, 300, 384, 3),        # 4 splits
+    (np.float16, 700, 96, 2),         # narrow blocks on the fp32 kernel
+    (np.float32, 70, 136, 1)])        # one split
+def test_calib_cov_splits(dtype, n_tokens, d, n_blocks):
+    X = synth.ActivationLaw(d, 1.0, seed=47, key=f"covs{d}").sample(n_tokens, "X", dtype)
+    dh, half = d // n_blocks, n_tokens // 2 // 8 * 8
+    Xd = torch.from_numpy(X).cuda()
+    ctx = rb.Context(0)
+    try:
+        runs = []
+        for _ in range(2):
+            Cg = torch.zeros((n_blocks, dh, dh), dtype=torch.float32, device="cuda")
+            ctx.calib_cov(Xd, Cg, n_blocks)
+            ctx.calib_cov(Xd[half:], Cg, n_blocks)
+            runs.append(Cg.cpu().numpy())
+        assert ctx.last_status() == rb.ROSAQ_OK
+    finally:
+        ctx.close()
+    assert np.array_equal(runs[0].view(np.uint32), runs[1].view(np.uint32))
+    Cref = orc.cov(X, n_blocks).reshape(n_blocks, dh, dh) + orc.cov(X[half:], n_blocks).reshape(n_blocks, dh, dh)
+    got = runs[0].astype(np.float64)
+    assert np.all(np.abs(got - Cref) <= H.cov_tolerance(Cref, n_tokens) + 1e-30)
+    assert np.array_equal(got, np.swapaxes(got, -1, -2))
