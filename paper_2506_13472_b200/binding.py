@@ -43,6 +43,7 @@ class _Op(C.Structure):
                 ("y", C.c_void_p), ("ldy", C.c_int64)]
 
 
+_ARRAYS = [(C.c_void_p * n, C.c_int64 * n) for n in range(5)]   # argument arrays of rosaq_linear_multi
 _lib = None
 
 
@@ -103,13 +104,28 @@ def _check(status, where):
         raise RosaqError(status, where)
 
 
-def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+# The calls of a decode step are a few microseconds each, so their marshalling is kept short: the raw handle of the current
+# stream (0.1 us; torch.cuda.current_stream() builds an object, 3.3 us), plain integers for pointers, outputs from the
+# input's own new_empty (1.5 us, torch.empty 2.5 us).
+_raw_stream = torch._C._cuda_getCurrentRawStream if hasattr(torch._C, "_cuda_getCurrentRawStream") else (
+    lambda device: torch.cuda.current_stream(device).cuda_stream)
+
+
+def _stream(stream, device):
+    """The cudaStream_t to launch on: the given torch stream, else the current one of the context's device."""
+    return _raw_stream(device) if stream is None else stream.cuda_stream
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+def _act(x):
+    """(rows, row stride) of an fp16 CUDA activation matrix with contiguous rows."""
+    assert x.is_cuda and x.dtype is torch.float16 and x.dim() == 2
+    ld, inner = x.stride()
+    assert inner == 1
+    return x.shape[0], ld
 
 
 def _dt(t):
@@ -179,7 +195,7 @@ class Context:
             pass
 
     def last_status(self, stream=None):
-        return lib().rosaq_last_status(self._h, _stream(stream))
+        return lib().rosaq_last_status(self._h, _stream(stream, self.device))
 
     def set_wait_limit(self, iterations):
         return lib().rosaq_set_wait_limit(self._h, int(iterations))
@@ -193,7 +209,7 @@ class Context:
         assert X.is_cuda and C_out.is_cuda and C_out.dtype == torch.float32 and C_out.is_contiguous()
         assert X.dim() == 2 and X.stride(1) == 1
         _check(lib().rosaq_calib_cov(self._h, _ptr(X), _dt(X), X.shape[0], X.shape[1], X.stride(0), n_blocks,
-                                     _ptr(C_out), _stream(stream)), "rosaq_calib_cov")
+                                     _ptr(C_out), _stream(stream, self.device)), "rosaq_calib_cov")
         return C_out
 
     # -- Eq. 3
@@ -205,57 +221,59 @@ class Context:
         if in_scale is None:
             _check(lib().rosaq_quantize(self._h, _ptr(W), W.shape[0], W.shape[1],
                                         None if rot is None else C.byref(rot), bits, group, k_salient, C.byref(h),
-                                        _stream(stream)), "rosaq_quantize")
+                                        _stream(stream, self.device)), "rosaq_quantize")
         else:
             assert in_scale.is_cuda and in_scale.dtype == torch.float32 and in_scale.numel() == W.shape[0]
             _check(lib().rosaq_quantize_scaled(self._h, _ptr(W), W.shape[0], W.shape[1],
                                                None if rot is None else C.byref(rot), _ptr(in_scale.contiguous()), bits, group,
-                                               k_salient, C.byref(h), _stream(stream)), "rosaq_quantize_scaled")
+                                               k_salient, C.byref(h), _stream(stream, self.device)), "rosaq_quantize_scaled")
         return Weight(self, h)
 
     def weight_import(self, d_in, d_out, bits, group, k_salient, qw, scales, zeros, salient, stream=None):
         h = C.c_void_p()
         _check(lib().rosaq_weight_import(self._h, d_in, d_out, bits, group, k_salient, _ptr(qw), _ptr(scales),
-                                         _ptr(zeros), _ptr(salient), C.byref(h), _stream(stream)),
+                                         _ptr(zeros), _ptr(salient), C.byref(h), _stream(stream, self.device)),
                "rosaq_weight_import")
         return Weight(self, h)
 
     def rotation_create(self, q, perm=None, stream=None):
         rot = _rot_struct(q, perm)
         h = C.c_void_p()
-        _check(lib().rosaq_rotation_create(self._h, C.byref(rot), C.byref(h), _stream(stream)),
+        _check(lib().rosaq_rotation_create(self._h, C.byref(rot), C.byref(h), _stream(stream, self.device)),
                "rosaq_rotation_create")
         return Rotation(self, h, rot.d)
 
     def rotate(self, x, rotation, out=None, stream=None):
-        assert x.is_cuda and x.dtype == torch.float16 and x.dim() == 2 and x.stride(1) == 1
+        m, ldx = _act(x)
         if out is None:
-            out = torch.empty((x.shape[0], rotation.d), dtype=torch.float16, device=x.device)
-        _check(lib().rosaq_rotate(self._h, _ptr(x), x.shape[0], x.stride(0), rotation._h, _ptr(out), out.stride(0),
-                                  _stream(stream)), "rosaq_rotate")
+            out = x.new_empty(m, rotation.d)
+        st = lib().rosaq_rotate(self._h, x.data_ptr(), m, ldx, rotation._h, out.data_ptr(), out.stride(0), _stream(stream, self.device))
+        if st:
+            raise RosaqError(st, "rosaq_rotate")
         return out
 
     def linear(self, x, weight, rotation=None, out=None, stream=None):
-        assert x.is_cuda and x.dtype == torch.float16 and x.dim() == 2 and x.stride(1) == 1
+        m, ldx = _act(x)
         if out is None:
-            out = torch.empty((x.shape[0], weight.d_out), dtype=torch.float16, device=x.device)
-        _check(lib().rosaq_linear(self._h, _ptr(x), x.shape[0], x.stride(0),
-                                  None if rotation is None else rotation._h, weight._h, _ptr(out), out.stride(0),
-                                  _stream(stream)), "rosaq_linear")
+            out = x.new_empty(m, weight.d_out)
+        st = lib().rosaq_linear(self._h, x.data_ptr(), m, ldx, None if rotation is None else rotation._h, weight._h, out.data_ptr(),
+                                out.stride(0), _stream(stream, self.device))
+        if st:
+            raise RosaqError(st, "rosaq_linear")
         return out
 
     def linear_multi(self, x, weights, rotation=None, outs=None, stream=None):
         """rosaq_linear_multi: the linears `weights` (same d_in / bits / k_salient) applied to one x in one launch."""
-        assert x.is_cuda and x.dtype == torch.float16 and x.dim() == 2 and x.stride(1) == 1
+        m, ldx = _act(x)
         n = len(weights)
         if outs is None:
-            outs = [torch.empty((x.shape[0], w.d_out), dtype=torch.float16, device=x.device) for w in weights]
-        wa = (C.c_void_p * n)(*[w._h.value for w in weights])
-        ya = (C.c_void_p * n)(*[o.data_ptr() for o in outs])
-        la = (C.c_int64 * n)(*[o.stride(0) for o in outs])
-        _check(lib().rosaq_linear_multi(self._h, _ptr(x), x.shape[0], x.stride(0),
-                                        None if rotation is None else rotation._h, n, wa, ya, la, _stream(stream)),
-               "rosaq_linear_multi")
+            outs = [x.new_empty(m, w.d_out) for w in weights]
+        ptrs, lds = _ARRAYS[n] if n < len(_ARRAYS) else (C.c_void_p * n, C.c_int64 * n)
+        st = lib().rosaq_linear_multi(self._h, x.data_ptr(), m, ldx, None if rotation is None else rotation._h, n,
+                                      ptrs(*[w._h.value for w in weights]), ptrs(*[o.data_ptr() for o in outs]),
+                                      lds(*[o.stride(0) for o in outs]), _stream(stream, self.device))
+        if st:
+            raise RosaqError(st, "rosaq_linear_multi")
         return outs
 
     def set_plan_costs(self, fp16_group, quant_group, tile):
@@ -298,7 +316,7 @@ class Context:
             out = torch.empty((x.shape[0], weight.d_out), dtype=torch.float16, device=x.device)
         _check(lib().rosaq_linear_static(self._h, _ptr(x), x.shape[0], x.stride(0),
                                          None if rotation is None else rotation._h, weight._h, _ptr(out),
-                                         out.stride(0), _stream(stream)), "rosaq_linear_static")
+                                         out.stride(0), _stream(stream, self.device)), "rosaq_linear_static")
         return out
 
 
@@ -323,7 +341,7 @@ class Weight:
         zr = torch.empty_like(sc)
         sal = torch.empty((self.k_salient, self.d_out), dtype=torch.float16, device=dev)
         _check(lib().rosaq_weight_export(self._ctx._h, self._h, _ptr(qw), _ptr(sc), _ptr(zr), _ptr(sal),
-                                         _stream(stream)), "rosaq_weight_export")
+                                         _stream(stream, self._ctx.device)), "rosaq_weight_export")
         return dict(qw=qw, scales=sc, zeros=zr, salient=sal)
 
     def free(self):
@@ -345,7 +363,9 @@ class Plan:
         self._ctx, self._h, self._keep = ctx, handle, keep
 
     def run(self, stream=None):
-        _check(lib().rosaq_plan_run(self._ctx._h, self._h, _stream(stream)), "rosaq_plan_run")
+        st = lib().rosaq_plan_run(self._ctx._h, self._h, _stream(stream, self._ctx.device))
+        if st:
+            raise RosaqError(st, "rosaq_plan_run")
 
     def free(self):
         if self._h:

@@ -428,7 +428,9 @@ int launch_rotate_quantize(const void *q, int q_is_f32, int n_blocks, const int3
 // Gram matrix on CUDA cores (fp32 products, fp32 accumulate): exact-product path for fp32 calibration activations and
 // the fallback for shapes the tensor-core kernel does not take.  Only tiles of the lower triangle are computed; an
 // off-diagonal tile is also added, transposed, to the mirrored position (products commute and both chains run over the
-// tokens in the same order, so the mirrored bits are those a tile of its own would produce).
+// tokens in the same order, so the mirrored bits are those a tile of its own would produce).  With few tiles a cluster of up
+// to eight CTAs shares the tokens of a tile and adds the partial tiles in order: a tile costs 128 cycles per token whatever the
+// width (4096 tokens x 512 channels: 634 us with all tiles of both triangles and a CTA each, 67 so; x 2048: 1003 and 418).
 template <typename T>
 __global__ void __launch_bounds__(kFmaThreads, 2)
 gram_fma_kernel(const T *__restrict__ X, long long ldx, int dh, float *__restrict__ C, int n_tokens, int Z) {
