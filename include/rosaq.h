@@ -93,7 +93,7 @@ int rosaq_last_status(rosaq_ctx *ctx, void *stream);
 int64_t rosaq_set_wait_limit(rosaq_ctx *ctx, int64_t iterations);
 
 /* Selects the rosaq_linear / rosaq_rotate implementation: 0 = tensor-core path
- * (tcgen05 + TMEM; default), 1 = plain CUDA-core path (slow; for debugging and
+ * (tcgen05 + TMEM; up to eight tokens warp-level MMAs on 32-column slices; default), 1 = plain CUDA-core path (slow; for debugging and
  * cross-checks -- it is still a GPU kernel of this library), 2 = tensor-core path with
  * CTA pairs (tcgen05 cta_group::2: two SMs share one MMA stream) wherever the shape allows
  * it (token tile a multiple of 32, an even number of 128-column tiles); the K splits may

@@ -135,6 +135,7 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
     for (int i = 0; i < n && st == ROSAQ_OK; ++i) st = launch_linear_simt(ctx, x, M, ldx, *ts[i], col_map, ys[i], ldys[i], s);
     return st;
   }
+  if (ctx->impl == 0 && linear_small_supported(ctx, M, n, ts)) return launch_linear_small(ctx, x, M, ldx, n, ts, col_map, ys, ldys, s);
   if (ctx->impl == 6 && n == 1 && M > 64 && M <= kBlockTokens * kPlanMaxOps)
     return run_token_blocks(ctx, x, M, ldx, *ts[0], col_map, ys[0], ldys[0], s);
   // A permuted output (head-wise rotation) is a scatter of 2-byte elements; in column order and then moved inside each row

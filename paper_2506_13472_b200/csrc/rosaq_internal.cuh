@@ -337,6 +337,11 @@ double linear_tc_estimate(const rosaq_ctx *ctx, int M, int n, const TiledOperand
 constexpr int kPermuteMaxColumns = 24576;            // a row in 48 KB of shared memory
 int launch_permute_rows(__half *y, int M, long long ldy, int d, const int32_t *col_map, cudaStream_t s);
 
+constexpr int kSmallTokens = 8;                      // most tokens of launch_linear_small
+bool linear_small_supported(const rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts);
+int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const TiledOperand *const *ts,
+                        const int32_t *col_map, __half *const *ys, const long long *ldys, cudaStream_t s);
+
 bool prefill_supported(const TiledOperand &t, const int32_t *col_map);
 struct PrefillCut {
   int NT = 0, n_tok_blocks = 0;   // tokens per tile
