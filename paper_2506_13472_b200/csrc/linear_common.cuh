@@ -125,6 +125,17 @@ struct Abort {
     if ((threadIdx.x & 31) == 0) ok = wait(bar, parity) ? 1 : 0;
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
   }
+  // by a converged warp, which stays converged
+  __device__ __forceinline__ bool wait_all(uint32_t bar, uint32_t parity) const {
+    for (long long it = 0; it <= limit; ++it) {
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+      if ((it & 63) == 63 && set_all()) return false;
+    }
+    if ((threadIdx.x & 31) == 0) raise();
+    __syncwarp();
+    return false;
+  }
+  __device__ __forceinline__ bool set_all() const { return __any_sync(0xffffffffu, set()); }
   // false when the wait gave up (or somebody else already did)
   __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) const {
     if (mbar_try_wait(bar, parity)) return true;

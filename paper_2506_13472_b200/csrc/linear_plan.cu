@@ -28,19 +28,18 @@
 // returns.  The last CTA to leave clears the counters, so the next launch starts from zero whatever
 // happened.
 //
-// One CTA owns an SM.  A tcgen05.mma of 128 x N x 16 costs 55 cycles of the tensor pipe for every N <= 64
-// (measured back to back), eight of them per 128-channel group: 440 cycles, 542 with the group's commit,
-// against 375 cycles for the group's bytes from HBM.  Two CTAs per SM only take turns on that pipe and
-// lengthen each other's dequantise -> MMA -> release chain; one CTA with one issuing thread spent 900
-// cycles per group in place, with TWO issuing threads 700: groups with an even position in the CTA's stream
-// accumulate into one tile, odd ones into another, and the epilogue adds the two.  Instruction issue
-// comes next (1700 warp instructions per group = 430 cycles of the four schedulers), which is why every
-// role walks only over its own groups and the epilogue loops carry no per-element address arithmetic.
-// Warp 0 = weight-tile producer (bulk copies, L2 evict-first; one sub-ring of slots per team), 1 =
-// activation producer (TMA), 2 and 3 = MMA issuers (2 also owns the tensor memory), 4..19 = four
-// dequantisation teams (group j goes to team and operand buffer j mod 4), 20..27 = epilogue (two warps per
-// TMEM lane quadrant, half of the tokens each).  Tensor memory (512 columns): accumulators of piece parity b
-// and issuer i at (2b + i) * 64, operand buffers from 256.
+// One CTA owns an SM.  Per 128-channel group at 64 tokens the tensor pipe needs 8 x 33 cycles, the group's bytes 375 at the HBM
+// rate, the four schedulers about 430 (1700 warp instructions); what paced a CTA before were its single-lane roles.  Measured
+// for the ten operations of a 7B decoder layer (64 tokens / 1 token, us in a graph):
+//   * MMAs issued from a branch on one lane, 57 cycles each, by two threads into two accumulators; weights fed by one lane, which
+//     needed 350 cycles per quantized group and 800 per fp16 group even with idle teams:                          57.1 / 50.7
+//   * weights fed by four lanes, one per team:                                                                    56.5 / 48.3
+//   * and one converged warp that issues the MMAs (14 ... 33 cycles each), one accumulator per piece:              53.3 / 45.5
+// Six operand buffers instead of four: 53.3 / 46.6 (the room comes off the weight ring).
+// Warp 0 = weight-tile producers (bulk copies, L2 evict-first; one sub-ring of slots and one lane per team), 1 =
+// activation producer (TMA), 2 = MMA issuer and owner of the tensor memory, 4..19 = four dequantisation teams (group j goes
+// to team j mod 4), 20..27 = epilogue (two warps per TMEM lane quadrant, half of the tokens each).  Tensor memory
+// (512 columns): the accumulator of piece parity b at 64 b (128 b when they hold 128 tokens), operand buffers behind them.
 #include <cuda.h>
 
 #include <algorithm>
@@ -56,13 +55,14 @@ namespace {
 constexpr int kPlTmemCols = 512;
 constexpr int kPlTeams = 4;                         // dequantisation teams of four warps
 constexpr int kPlStages = kPlTeams;                 // TMEM operand buffers, each with its activation slot: one per team ...
-constexpr int kPlPairStages = 6;                    // ... six in a pair of CTAs (one issuing thread, two accumulators)
+constexpr int kPlPairStages = 6;                    // ... six in a pair of CTAs, whose chain is longer
 constexpr int kPlMaxStages = 6;
 constexpr int kPlTokens = 64;                       // token capacity of an accumulator and of a partial tile
 constexpr int kPlFirstDequantWarp = 4, kPlFirstEpiWarp = kPlFirstDequantWarp + 4 * kPlTeams;
 constexpr int kPlEpiThreads = 256;                  // two warps per TMEM lane quadrant
 constexpr int kPlThreads = kPlFirstEpiWarp * 32 + kPlEpiThreads;   // 896
 constexpr int kPlSmemBytes = 227 * 1024;            // the whole SM
+constexpr int kPollsPerWait = 16;                   // polls of the weight producers per blocking wait of the others
 
 struct PlProblem {
   const uint8_t *blob;
@@ -137,31 +137,24 @@ __device__ __forceinline__ void tmem_ld_chunk(uint32_t taddr, uint32_t *v) {
 // Finishes tokens [c_begin, c_end) of one output column from the accumulator in tensor memory: adds, when
 // `keep`, the partial tiles 1 .. S-1 of the workspace in that order (this CTA's groups come first), rounds
 // once and writes the rows inside [t0, t1).  CH loads from the workspace are in flight per thread.
-// Tokens [c0, c0 + CH) of one column: the sum of the two issuers' accumulators (`both`), or the one that
-// holds the only group of a one-group piece (d_addr then points at it).
+// Tokens [c0, c0 + CH) of one column of the accumulator.
 template <int CH>
-__device__ __forceinline__ void epi_load_acc(uint32_t d_addr, bool both, int c0, float *acc) {
+__device__ __forceinline__ void epi_load_acc(uint32_t d_addr, int c0, float *acc) {
   uint32_t v[CH];
   tmem_ld_chunk<CH>(d_addr + c0, v);
   tc_wait_ld();
 #pragma unroll
   for (int e = 0; e < CH; ++e) acc[e] = __uint_as_float(v[e]);
-  if (both) {
-    tmem_ld_chunk<CH>(d_addr + kPlTokens + c0, v);
-    tc_wait_ld();
-#pragma unroll
-    for (int e = 0; e < CH; ++e) acc[e] = __fadd_rn(acc[e], __uint_as_float(v[e]));
-  }
 }
 
 template <int CH>
-__device__ __forceinline__ void epi_finish(uint32_t d_addr, bool both, int c_begin, int c_end, bool keep, int S, const float *src0,
+__device__ __forceinline__ void epi_finish(uint32_t d_addr, int c_begin, int c_end, bool keep, int S, const float *src0,
                                            long long slot_floats, int M, bool n_ok, int t0, int t1, __half *y_col,
                                            long long ldy) {
   for (int c0 = c_begin; c0 < c_end; c0 += CH) {
     if (c0 >= t1 || c0 + CH <= t0) continue;
     float acc[CH];
-    epi_load_acc<CH>(d_addr, both, c0, acc);
+    epi_load_acc<CH>(d_addr, c0, acc);
     if (keep) {
       // two holders' tiles per round trip to L2 (a round trip costs 1.4 us and more while the weight stream
       // runs, and the readers of this tile wait for it), added in holder order
@@ -205,10 +198,10 @@ __device__ __forceinline__ void epi_finish(uint32_t d_addr, bool both, int c_beg
 
 // Stores tokens [c_begin, c_end) of one column of the accumulator to a partial tile [token][128 columns].
 template <int CH>
-__device__ __forceinline__ void epi_store_partial(uint32_t d_addr, bool both, int c_begin, int c_end, int M, float *dst) {
+__device__ __forceinline__ void epi_store_partial(uint32_t d_addr, int c_begin, int c_end, int M, float *dst) {
   for (int c0 = c_begin; c0 < c_end && c0 < M; c0 += CH) {
     float acc[CH];
-    epi_load_acc<CH>(d_addr, both, c0, acc);
+    epi_load_acc<CH>(d_addr, c0, acc);
     float *dp = dst + c0 * kTileN;
     if (c0 + CH <= M) {
 #pragma unroll
@@ -224,17 +217,15 @@ __device__ __forceinline__ void epi_store_partial(uint32_t d_addr, bool both, in
 // kPair: the CTAs of a cluster of two (ranks 0 and 1, adjacent SMs) run as a cta_group::2 pair on one
 // schedule entry: a piece is then the groups of TWO adjacent column tiles, rank r dequantises tile 2 t + r into
 // its own tensor memory and loads half of the token rows, and the leader (rank 0) issues one M = 256 MMA for
-// both.  An MMA instruction costs the same 55 cycles whether it covers 128 or 256 rows, so the pair needs
-// 222 cycles of each SM's tensor pipe per 128-channel group where a single CTA needs 440 -- less than the
-// 375 cycles the group's bytes take.  Barriers that both CTAs feed live in the leader; its commits are
+// both.  Barriers that both CTAs feed live in the leader; its commits are
 // multicast to both.
 // kMode 2: a single CTA with accumulators of 128 tokens: two of them (one per piece parity) and the four
-// operand buffers fill the tensor memory, so there is one issuing thread, as in a pair; a group then costs
+// operand buffers fill the tensor memory; a group then costs
 // eight MMAs of N = 128 (64 cycles each: the full rate of the pipe) and its dequantisation serves twice the tokens.
 template <int kBits, int kMode>
 __global__ void __launch_bounds__(kPlThreads, 1)
 linear_plan_kernel(const __grid_constant__ PlParams p) {
-  constexpr bool kPair = kMode == 1, kBig = kMode == 2, kOne = kMode != 0;
+  constexpr bool kPair = kMode == 1, kBig = kMode == 2;
   constexpr int kTok = kBig ? 2 * kPlTokens : kPlTokens;       // token capacity of an accumulator
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -242,10 +233,6 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const int MTL = kPair ? MT >> 1 : MT;                        // token rows this CTA keeps in shared memory
   const uint32_t x_slot_bytes = (uint32_t)MTL * 256u;
   const uint32_t x_ring = base;
-  // operand buffers: a single CTA has two issuing threads with an accumulator each per piece parity (256
-  // columns) and one buffer per team; a pair has one issuing thread (an MMA over both SMs costs no more than
-  // one over one) and spends the columns on two more buffers, which hides the longer chain of a pair
-  // (dequantise -> remote arrive -> MMA -> multicast commit)
   constexpr int NS = kPair ? kPlPairStages : kPlStages;
   const uint32_t w_ring = x_ring + NS * x_slot_bytes;
   const uint32_t bars = w_ring + p.NW * kWSlotBytes;
@@ -254,12 +241,12 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const uint32_t bar_s_empty = bar_a_full + 8 * kPlMaxStages;  // stage consumed by its MMAs
   const uint32_t bar_d_full = bar_s_empty + 8 * kPlMaxStages;  // accumulator complete (two accumulators)
   const uint32_t bar_d_empty = bar_d_full + 16;                // accumulator drained
-  const uint32_t bar_drain = bar_d_empty + 16;                 // two: one per issuer
+  const uint32_t bar_drain = bar_d_empty + 16;
   const uint32_t misc = bar_drain + 16;                         // [0] TMEM base, [1] abort flag, [2] last CTA out
   uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
   volatile uint32_t *misc_ptr = reinterpret_cast<volatile uint32_t *>(gen + (misc - base));
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = kPair ? (blockIdx.x & 1u) : 0u;        // position in the pair; 0 = leader
   const bool is_lead = rank == 0;
   const int cta = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;   // entry of the schedule
@@ -278,10 +265,10 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
       mbar_init(bar_s_empty + 8 * i, 1);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(bar_d_full + 8 * i, kOne ? 1 : 2);             // the issuing threads
+      mbar_init(bar_d_full + 8 * i, 1);
       mbar_init(bar_d_empty + 8 * i, (kPair ? 2 : 1) * (kPlEpiThreads / 32));   // one arrival per epilogue warp
-      mbar_init(bar_drain + 8 * i, 1);
     }
+    mbar_init(bar_drain, 1);
     misc_ptr[1] = 0;
     misc_ptr[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -299,64 +286,84 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   }
   tc_fence_after();
   const uint32_t tmem = misc_ptr[0];
-  const uint32_t a_col0 = (kPair ? 2 : 4) * kPlTokens;         // operand buffers follow the accumulators (two of 128 columns when kBig)
+  const uint32_t a_col0 = 2 * kTok;                            // operand buffers follow the two accumulators
   const int qbytes = quant_tile_bytes(kBits);
 
   if (warp == 0) {
-    // ---------------- weight-tile producer: streams every piece of every phase, waits for ring slots only
-    if (lane == 0) {
-      // The ring is split into one sub-ring of NWT slots per dequantisation team (group j of the CTA's stream
-      // belongs to team j mod 4): a sub-ring has one consumer, which takes its slots in order, so a full /
-      // empty pair of barriers per slot is enough.  Positions of the four sub-rings: a byte each in idx4,
-      // a bit each in lap4; fills per team in fills4 (16 bits each, only looked at when giving up).
+    // ---------------- weight-tile producers: stream every piece of every phase, wait for ring slots only.
+    // The ring is split into one sub-ring of NWT slots per dequantisation team (group j of the CTA's stream
+    // belongs to team j mod 4): a sub-ring has one consumer, which takes its slots in order, so a full /
+    // empty pair of barriers per slot is enough.  Lane t feeds the sub-ring of team t and the four lanes step
+    // together, each issuing its next copy if its slot is free: one thread for all four needed 350 cycles per
+    // quantized group and 800 per fp16 group (four copies) next to idle teams, and paced the whole CTA.
+    if (lane < kPlTeams) {
+      constexpr unsigned kLanes = (1u << kPlTeams) - 1;
       const uint64_t pol = policy_evict_first();
       const int NWT = p.NW >> 2;
-      uint32_t idx4 = 0, lap4 = 0;
-      unsigned long long fills4 = 0;
-      int j = 0;
-      bool live = true;
-      for (int si = s_begin; si < s_end && live && !ab.set(); ++si) {
-        const PlanSeg s = load_seg(p.segs + si);
-        const PlProblem &P = p.prob[s.prob];
-        // (the second CTA of a pair on an odd last tile streams that tile again; its results are dropped)
-        int my_tile = tile_mul * s.tile + (int)rank;
-        if (my_tile >= P.n_tiles) my_tile = P.n_tiles - 1;
-        const uint8_t *tile_base = P.blob + (long long)my_tile * P.tile_stride;
-        const int g_fp16 = P.g_fp16;
-        for (int g = s.g_begin; g < s.g_end && live; ++g, ++j) {
-          const bool f16 = g < g_fp16;
-          const uint8_t *src = tile_base + (f16 ? (long long)g * kFp16TileBytes
-                                                : (long long)g_fp16 * kFp16TileBytes + (long long)(g - g_fp16) * qbytes);
-          const int nsub = f16 ? 4 : 1;
-          const uint32_t bytes = f16 ? kFp16SubBytes : qbytes;
-          const int team = j & (kPlTeams - 1);
-          uint32_t idx = (idx4 >> (8 * team)) & 0xffu;
-          for (int sub = 0; sub < nsub; ++sub) {
-            const int slot = team * NWT + (int)idx;
-            if (!ab.wait(bar_w_empty + 8 * slot, ((lap4 >> team) & 1u) ^ 1u)) {
-              live = false;
-              break;
-            }
-            mbar_arrive_expect_tx(bar_w_full + 8 * slot, bytes);
-            bulk_copy_g2s_hint(w_ring + slot * kWSlotBytes, src + (long long)sub * kFp16SubBytes, bytes,
-                               bar_w_full + 8 * slot, pol);
-            fills4 += 1ull << (16 * team);
-            if (++idx == (uint32_t)NWT) {
-              idx = 0;
-              lap4 ^= 1u << team;
-            }
-          }
-          idx4 = (idx4 & ~(0xffu << (8 * team))) | (idx << (8 * team));
+      const int team = lane;
+      int si = s_begin, j0 = 0, g = 0, g_end = 0, g_fp16 = 0, left = 0;    // left: copies of this group after the next one
+      unsigned fills = 0;                                      // (only looked at when giving up)
+      uint32_t bytes = 0;
+      const uint8_t *base = nullptr, *src = nullptr;
+      Ring rw{0, 0};
+      PlanSeg ahead = load_seg(p.segs + (s_begin < s_end ? s_begin : 0));
+      auto seek = [&] {                                        // the team's first group at or after g, in this piece or a later one
+        while (g >= g_end) {
+          if (si == s_end) return false;
+          const PlanSeg s = ahead;
+          if (++si < s_end) ahead = load_seg(p.segs + si);
+          const PlProblem &P = p.prob[s.prob];
+          // (the second CTA of a pair on an odd last tile streams that tile again; its results are dropped)
+          int my_tile = tile_mul * s.tile + (int)rank;
+          if (my_tile >= P.n_tiles) my_tile = P.n_tiles - 1;
+          base = P.blob + (long long)my_tile * P.tile_stride;
+          g_fp16 = P.g_fp16;
+          g = s.g_begin + ((team - j0) & (kPlTeams - 1));
+          g_end = s.g_end;
+          j0 += s.g_end - s.g_begin;
         }
-      }
-      if (ab.set()) {  // let copies already in flight land before the CTA goes away
-        for (int team = 0; team < kPlTeams; ++team) {
-          const int f = (int)((fills4 >> (16 * team)) & 0xffffu);     // (mod 65536: only the last NWT fills matter)
-          for (int back = 1; back <= NWT && back <= f; ++back) {
-            const int u = f - back;
-            for (int it = 0; it < kDrainPolls; ++it)
-              if (mbar_try_wait(bar_w_full + 8 * (team * NWT + u % NWT), (u / NWT) & 1)) break;
+        const bool f16 = g < g_fp16;
+        src = base + (f16 ? (long long)g * kFp16TileBytes : (long long)g_fp16 * kFp16TileBytes + (long long)(g - g_fp16) * qbytes);
+        bytes = f16 ? kFp16SubBytes : qbytes;
+        left = f16 ? 3 : 0;
+        return true;
+      };
+      bool more = seek();
+      long long idle = 0;
+      while (__any_sync(kLanes, more)) {
+        const int slot = team * NWT + rw.idx;
+        const bool go = more && mbar_test_wait(bar_w_empty + 8 * slot, rw.lap ^ 1u);
+        if (go) {
+          mbar_arrive_expect_tx(bar_w_full + 8 * slot, bytes);
+          bulk_copy_g2s_hint(w_ring + slot * kWSlotBytes, src, bytes, bar_w_full + 8 * slot, pol);
+          rw.advance(NWT);
+          ++fills;
+          if (left > 0) {
+            --left;
+            src += kFp16SubBytes;
+          } else {
+            g += kPlTeams;
+            more = seek();
           }
+        }
+        if (__any_sync(kLanes, go)) {
+          idle = 0;
+          continue;
+        }
+        // (a poll here is a few dozen nanoseconds where the other waits block for up to a microsecond)
+        if (++idle > kPollsPerWait * p.wait_limit) {
+          if (lane == 0 && !ab.set()) ab.raise();
+          break;
+        }
+        if ((idle & 63) == 63 && ab.set()) break;
+        __nanosleep(20);
+      }
+      __syncwarp(kLanes);
+      if (ab.set()) {  // let copies already in flight land before the CTA goes away
+        for (int back = 1; back <= NWT && back <= (int)fills; ++back) {
+          const int u = (int)fills - back;
+          for (int it = 0; it < kDrainPolls; ++it)
+            if (mbar_try_wait(bar_w_full + 8 * (team * NWT + u % NWT), (u / NWT) & 1)) break;
         }
       }
     }
@@ -409,33 +416,26 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         }
       }
     }
-  } else if (warp == 2 || warp == 3) {
-    // ---------------- MMA issuers: issuer i takes the groups whose position j in the CTA's stream has
-    // j mod 2 == i (operand buffers i and i + 2) and accumulates them into its own tile; per group one
-    // wait, eight MMAs, one commit.  Every piece is committed by both (an issuer without a group in a
-    // one-group piece arrives by hand), so the epilogue waits for one barrier.
-    if (lane == 0 && is_lead && !(kOne && warp == 3)) {        // (a pair, or a CTA with wide accumulators, has one issuing thread)
-      const int me = warp - 2;
-      constexpr int kStep = kOne ? 1 : 2;                      // issuers that share the stream
+  } else if (warp == 2) {
+    // ---------------- MMA issuer (the whole warp, converged): per group one wait, eight MMAs, one commit
+    if (is_lead) {
       // M = 128 output columns (256 for a pair), N = MT tokens
       const uint32_t idesc = (1u << 4) | ((uint32_t)(MT >> 3) << 17) | ((kPair ? 16u : 8u) << 24);
       const uint64_t desc0 = make_b_desc(x_ring);
       const uint32_t x_slot16 = x_slot_bytes >> 4, half16 = (uint32_t)(MTL * 128) >> 4;
-      int nseg = 0, j = 0;
+      int nseg = 0;
       bool live = true, issued = false;
+      Ring rs{0, 0};
       for (int si = s_begin; si < s_end && live; ++si, ++nseg) {
         const PlanSeg s = load_seg(p.segs + si);
         const int buf = nseg & 1;
-        if (!ab.wait(bar_d_empty + 8 * buf, ((nseg >> 1) & 1) ^ 1u)) break;   // the piece before last has been drained
+        if (!ab.wait_all(bar_d_empty + 8 * buf, ((nseg >> 1) & 1) ^ 1u)) break;   // the piece before last has been drained
         tc_fence_after();
-        const uint32_t d_tmem = tmem + (uint32_t)(kOne ? buf : 2 * buf + me) * kTok;
+        const uint32_t d_tmem = tmem + (uint32_t)buf * kTok;
         uint32_t accumulate = 0;
-        const int g_first = kOne ? s.g_begin : s.g_begin + ((me - j) & 1), j_base = j - s.g_begin;
-        j += s.g_end - s.g_begin;
-        for (int g = g_first; g < s.g_end; g += kStep) {
-          const int j = j_base + g;
-          const int st = j % NS;                               // (a constant: a mask or a multiply)
-          if (!ab.wait(bar_a_full + 8 * st, (uint32_t)(j / NS) & 1u)) {
+        for (int g = s.g_begin; g < s.g_end; ++g, rs.advance(NS)) {
+          const int st = rs.idx;
+          if (!ab.wait_all(bar_a_full + 8 * st, rs.lap)) {
             live = false;
             break;
           }
@@ -452,22 +452,14 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
           issued = true;
         }
         if (!live) break;
-        if (kPair) {
-          if (accumulate) tc_commit_mc(bar_d_full + 8 * buf, 3);
-          else {
-            mbar_arrive_cluster(map_to_rank(bar_d_full + 8 * buf, 0));
-            mbar_arrive_cluster(map_to_rank(bar_d_full + 8 * buf, 1));
-          }
-        } else {
-          if (accumulate) tc_commit(bar_d_full + 8 * buf);
-          else mbar_arrive(bar_d_full + 8 * buf);
-        }
+        if (kPair) tc_commit_mc(bar_d_full + 8 * buf, 3);
+        else tc_commit(bar_d_full + 8 * buf);
       }
-      if (ab.set() && issued) {  // MMAs already issued must retire before the tensor memory is given back
-        if (kPair) tc_commit_mc(bar_drain + 8 * me, 1);
-        else tc_commit(bar_drain + 8 * me);
+      if (ab.set_all() && issued) {  // MMAs already issued must retire before the tensor memory is given back
+        if (kPair) tc_commit_mc(bar_drain, 1);
+        else tc_commit(bar_drain);
         for (int it = 0; it < kDrainPolls; ++it)
-          if (mbar_try_wait(bar_drain + 8 * me, 0)) break;
+          if (mbar_try_wait(bar_drain, 0)) break;
       }
     }
   } else if (warp >= kPlFirstDequantWarp && warp < kPlFirstEpiWarp) {
@@ -528,20 +520,16 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     const int half_tok = MT >> 1;
     const int c_begin = ((warp - kPlFirstEpiWarp) >> 2) * half_tok, c_end = c_begin + half_tok;
     const bool wide = (half_tok & 15) == 0;                    // sixteen tokens per batch, else eight
-    int nseg = 0, j0 = 0;
+    int nseg = 0;
     for (int si = s_begin; si < s_end; ++si, ++nseg) {
       const PlanSeg s = load_seg(p.segs + si);
       const PlProblem &P = p.prob[s.prob];
       const int buf = nseg & 1;
-      // the piece's groups have positions j0 .. in the CTA's stream: even ones went to issuer 0's tile
-      const bool both = !kOne && s.g_end - s.g_begin > 1;
-      const int first_acc = (both || kOne) ? 0 : (j0 & 1);
-      j0 += s.g_end - s.g_begin;
       bool have_d = ab.wait(bar_d_full + 8 * buf, (nseg >> 1) & 1);
       have_d = __all_sync(0xffffffffu, have_d && !ab.set());
       if (!have_d) break;
       tc_fence_after();
-      const uint32_t d_addr = lane_addr + (uint32_t)(kOne ? buf : 2 * buf + first_acc) * kTok;
+      const uint32_t d_addr = lane_addr + (uint32_t)buf * kTok;
       const int n_glob = (tile_mul * s.tile + (int)rank) * kTileN + n;
       const bool n_ok = n_glob < P.d_out;
       const long long out_col = n_ok ? (P.col_map ? P.col_map[n_glob] : n_glob) : 0;
@@ -564,10 +552,10 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
       if (sole || keep) {
         // token rows this piece writes (the schedule counts them in 64ths of the capacity)
         const int t0 = s.tok_begin * (kTok / kPlTokens), t1 = min(s.tok_end * (kTok / kPlTokens), P.m);
-        if (wide) epi_finish<16>(d_addr, both, c_begin, c_end, keep, S, src0, slot_step, P.m, n_ok, t0, t1, y_out + out_col, ldy);
-        else epi_finish<8>(d_addr, both, c_begin, c_end, keep, S, src0, slot_step, P.m, n_ok, t0, t1, y_out + out_col, ldy);
+        if (wide) epi_finish<16>(d_addr, c_begin, c_end, keep, S, src0, slot_step, P.m, n_ok, t0, t1, y_out + out_col, ldy);
+        else epi_finish<8>(d_addr, c_begin, c_end, keep, S, src0, slot_step, P.m, n_ok, t0, t1, y_out + out_col, ldy);
         tc_fence_before();
-        __syncwarp();                                          // one arrival per warp, where the issuers wait
+        __syncwarp();                                          // one arrival per warp, where the issuer waits
         if (lane == 0) {
           if (kPair) mbar_arrive_cluster(map_to_rank(bar_d_empty + 8 * buf, 0));
           else mbar_arrive(bar_d_empty + 8 * buf);
@@ -585,8 +573,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
       // accumulator back, count this CTA in
       {
         float *dst = p.partials + ((long long)tile_mul * (s.slot0 + s.contrib_idx) + rank) * p.slot_floats + n;
-        if (wide) epi_store_partial<16>(d_addr, both, c_begin, c_end, P.m, dst);
-        else epi_store_partial<8>(d_addr, both, c_begin, c_end, P.m, dst);
+        if (wide) epi_store_partial<16>(d_addr, c_begin, c_end, P.m, dst);
+        else epi_store_partial<8>(d_addr, c_begin, c_end, P.m, dst);
       }
       tc_fence_before();
       __syncwarp();
@@ -995,7 +983,7 @@ int plan_prepare(rosaq_ctx *ctx, int M, int n, const PlanOp *ops, PlanLaunch *ou
   if (n < 1 || n > kPlanMaxOps || M < 1 || M > 2 * kPlTokens) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
   std::vector<PlanGeom> geom(n);
   int bits = 0;
-  const bool big = M > kPlTokens;                      // accumulators of 128 tokens, single CTAs, one issuing thread
+  const bool big = M > kPlTokens;                      // accumulators of 128 tokens, single CTAs
   // pairs of CTAs (two adjacent column tiles per MMA) unless an operand's adjacent tiles multiply different
   // channels (a block-diagonal operand with an odd number of groups per block) or pairs are switched off
   bool pair = !big && ctx->pl_mode != 1 && plan_units(ctx, true) > 0;

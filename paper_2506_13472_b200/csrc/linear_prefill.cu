@@ -155,12 +155,12 @@ __device__ __forceinline__ uint64_t make_a_desc(uint32_t smem_addr) {
 // four MMAs = 64 channels; A advances by two chunks (4096 bytes) per MMA, B by 32 bytes inside a swizzle row
 __device__ __forceinline__ void tc_mma4_ss_pair(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\t.reg .b64 ta, tb;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
-      "add.u64 ta, %1, 256;\n\tadd.u64 tb, %2, 2;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t"
-      "add.u64 ta, %1, 512;\n\tadd.u64 tb, %2, 4;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t"
-      "add.u64 ta, %1, 768;\n\tadd.u64 tb, %2, 6;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t}" ::"r"(d_tmem),
+      "{\n\t.reg .pred p, q, e;\n\t.reg .b64 ta, tb;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "add.u64 ta, %1, 256;\n\tadd.u64 tb, %2, 2;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t"
+      "add.u64 ta, %1, 512;\n\tadd.u64 tb, %2, 4;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t"
+      "add.u64 ta, %1, 768;\n\tadd.u64 tb, %2, 6;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], ta, tb, %3, q;\n\t}" ::"r"(d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -241,7 +241,7 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
   const uint32_t misc = bar_merge + 8;                         // [0] TMEM base, [1] abort flag
   uint32_t *misc_ptr = reinterpret_cast<uint32_t *>(smem_raw + (misc - smem_u32(smem_raw)));
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = blockIdx.x & 1u;                       // position in the pair; 0 = leader
   const bool is_lead = rank == 0;
   const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
@@ -408,7 +408,7 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
       }
     } else if (warp == 2) {
       // ---------------- MMA issuer (leader): per group one wait, eight MMAs of 256 x NT x 16, one commit (dense: half a group)
-      if (lane == 0 && is_lead) {
+      if (is_lead) {
         const uint32_t idesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | (16u << 24);
         const uint64_t desc0 = make_b_desc(kDense ? base + kPdABytes : x_ring), adesc0 = make_a_desc(base);
         const uint32_t slot16 = (kDense ? d_stage_bytes : x_slot_bytes) >> 4, half16 = (uint32_t)(rows * 128) >> 4;
@@ -418,14 +418,14 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
         int u = u_begin, wk, g0, g1;
         for (; live && pf_next_piece(u, u_end, G, wk, g0, g1); ++n_done) {
           const int buf = kDense ? n_done & 1 : 0;
-          if (!ab.wait(bar_d_empty + 8 * buf, (uint32_t)((n_done / kAcc) & 1) ^ 1u)) break;   // the last piece in it has been drained
+          if (!ab.wait_all(bar_d_empty + 8 * buf, (uint32_t)((n_done / kAcc) & 1) ^ 1u)) break;   // the last piece in it has been drained
           tc_fence_after();
           const uint32_t d_tmem = tmem + buf * kPfMaxTokens;
           uint32_t accumulate = 0;
           const int n = (g1 - g0) * (kDense ? 2 : 1);
           for (int i = 0; i < n; ++i, rs.advance(kDense ? NW : kPfStages)) {
             const int st = rs.idx;
-            if (!ab.wait((kDense ? bar_w_full : bar_a_full) + 8 * st, rs.lap)) {
+            if (!ab.wait_all((kDense ? bar_w_full : bar_a_full) + 8 * st, rs.lap)) {
               live = false;
               break;
             }
@@ -444,7 +444,7 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
           if (!live) break;
           tc_commit_mc(bar_d_full + 8 * buf, pair_mask);
         }
-        if (ab.set() && issued) {  // MMAs already issued must retire before the tensor memory is given back
+        if (ab.set_all() && issued) {  // MMAs already issued must retire before the tensor memory is given back
           tc_commit_mc(bar_drain, 1u << lead);
           for (int it = 0; it < kDrainPolls; ++it)
             if (mbar_try_wait(bar_drain, 0)) break;

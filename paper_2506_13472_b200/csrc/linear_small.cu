@@ -1,7 +1,7 @@
 // The GEMM stage  y = x' . W^  (Eq. 3; Eq. 6 for a block-diagonal rotation operand) for one to eight tokens.
 //
 // Why another kernel.  At a few tokens a launch of the tcgen05 kernel is bound by its latencies, not by the weight stream: every
-// group is a chain through tensor memory (dequantise, store, barrier, eight MMAs of 55 cycles whatever the token count, commit),
+// group is a chain through tensor memory (dequantise, store, barrier, eight MMAs, commit),
 // and the splits of K meet in a cluster exchange of several microseconds before the next launch can begin.  Here
 //   * a CTA owns a slice of 32 output columns and ALL of K, so nothing is exchanged between CTAs: its eight warps take the
 //     units of K in turn (a unit = a quantized group, or 32 channels of an fp16 group: 2 KB of a slice either way) and the

@@ -34,6 +34,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// the same without blocking
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(src), "r"(bytes), "r"(bar)
@@ -65,26 +77,36 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+      : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem desc]; fp16 inputs, fp32 accumulate.  The MMAs of one unit are
-// emitted as one block of back-to-back instructions sharing their predicates: issued one by one from
-// separate statements they cost the issuing thread about 100 cycles each, in a block about 45.
+// emitted as one block of back-to-back instructions sharing their predicates.
 // A advances by 8 TMEM columns (16 input channels) per MMA; B by 32 bytes inside a 64-channel
 // swizzle row (descriptor address field + 2), b_hi is the descriptor of the second 64-channel half.
+// MMAs and commits are issued by the elected lane of a CONVERGED warp: addresses and descriptors are then computed in uniform
+// registers.  From a branch on one lane they are moved there one by one and an MMA takes 57 cycles to issue whatever its size;
+// this way 128 x N x 16 takes 14 (N = 16), 17 (32) and 33 (64) cycles.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}" : "=r"(ok)::"memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void tc_mma8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_lo, uint64_t b_hi,
                                            uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\t.reg .b64 t;\n\t.reg .b32 a;\n\t"
-      "setp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %4, p;\n\t"
-      "add.u32 a, %1, 8;\n\tadd.u64 t, %2, 2;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 16;\n\tadd.u64 t, %2, 4;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 24;\n\tadd.u64 t, %2, 6;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 32;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [a], %3, %4, q;\n\t"
-      "add.u32 a, %1, 40;\n\tadd.u64 t, %3, 2;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 48;\n\tadd.u64 t, %3, 4;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 56;\n\tadd.u64 t, %3, 6;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t}" ::"r"(d_tmem),
+      "{\n\t.reg .pred p, q, e;\n\t.reg .b64 t;\n\t.reg .b32 a;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %4, p;\n\t"
+      "add.u32 a, %1, 8;\n\tadd.u64 t, %2, 2;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 16;\n\tadd.u64 t, %2, 4;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 24;\n\tadd.u64 t, %2, 6;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 32;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], %3, %4, q;\n\t"
+      "add.u32 a, %1, 40;\n\tadd.u64 t, %3, 2;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 48;\n\tadd.u64 t, %3, 4;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 56;\n\tadd.u64 t, %3, 6;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], t, %4, q;\n\t}" ::"r"(d_tmem),
       "r"(a_tmem), "l"(b_lo), "l"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -102,7 +124,8 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t addr) {
 // commit whose arrival is delivered to the barrier at the same offset in every CTA of `mask`
 __device__ __forceinline__ void tc_commit_mc(uint32_t bar, uint32_t mask) {
   asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(bar),
       "h"((unsigned short)mask)
       : "memory");
 }
@@ -132,16 +155,16 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
 __device__ __forceinline__ void tc_mma8_ts_pair(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_lo, uint64_t b_hi,
                                                 uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\t.reg .b64 t;\n\t.reg .b32 a;\n\t"
-      "setp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %4, p;\n\t"
-      "add.u32 a, %1, 8;\n\tadd.u64 t, %2, 2;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 16;\n\tadd.u64 t, %2, 4;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 24;\n\tadd.u64 t, %2, 6;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 32;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], [a], %3, %4, q;\n\t"
-      "add.u32 a, %1, 40;\n\tadd.u64 t, %3, 2;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 48;\n\tadd.u64 t, %3, 4;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
-      "add.u32 a, %1, 56;\n\tadd.u64 t, %3, 6;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t}" ::"r"(d_tmem),
+      "{\n\t.reg .pred p, q, e;\n\t.reg .b64 t;\n\t.reg .b32 a;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %4, p;\n\t"
+      "add.u32 a, %1, 8;\n\tadd.u64 t, %2, 2;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 16;\n\tadd.u64 t, %2, 4;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 24;\n\tadd.u64 t, %2, 6;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 32;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], %3, %4, q;\n\t"
+      "add.u32 a, %1, 40;\n\tadd.u64 t, %3, 2;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 48;\n\tadd.u64 t, %3, 4;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t"
+      "add.u32 a, %1, 56;\n\tadd.u64 t, %3, 6;\n\t@e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], t, %4, q;\n\t}" ::"r"(d_tmem),
       "r"(a_tmem), "l"(b_lo), "l"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
