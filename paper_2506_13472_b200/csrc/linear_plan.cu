@@ -35,6 +35,8 @@
 //     needed 350 cycles per quantized group and 800 per fp16 group even with idle teams:                          57.1 / 50.7
 //   * weights fed by four lanes, one per team:                                                                    56.5 / 48.3
 //   * and one converged warp that issues the MMAs (14 ... 33 cycles each), one accumulator per piece:              53.3 / 45.5
+//   * the counters of a problem's input polled by a warp of its own, ahead of the activation copies (52.4 / 44.3), and the
+//     launch chained to the one before it (its set-up and first weight copies under that one's tail):               52.5 / 43.9
 // Six operand buffers instead of four: 53.3 / 46.6 (the room comes off the weight ring).
 // Warp 0 = weight-tile producers (bulk copies, L2 evict-first; one sub-ring of slots and one lane per team), 1 =
 // activation producer (TMA), 2 = MMA issuer and owner of the tensor memory, 4..19 = four dequantisation teams (group j goes
@@ -115,15 +117,30 @@ __device__ __forceinline__ PlanSeg load_seg(const PlanSeg *s) {
   return r;
 }
 // waits until *ctr >= target; false when the wait gave up
-__device__ __forceinline__ bool wait_counter(const Abort &ab, const unsigned *ctr, unsigned target) {
+__device__ __forceinline__ bool wait_counter(const Abort &ab, const unsigned *ctr, unsigned target, unsigned pause = 0) {
   for (long long it = 0; it < ab.limit; ++it) {
     if (ld_acquire_u32(ctr) >= target) return true;
+    if (pause) __nanosleep(pause);
     if ((it & 15) == 15) {
       if (ab.set()) return false;
       __nanosleep(64);
     }
   }
   if (ld_acquire_u32(ctr) >= target) return true;
+  ab.raise();
+  return false;
+}
+
+// a count in shared memory that one warp raises and another waits for
+__device__ __forceinline__ void st_flag(uint32_t addr, int v) { asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ bool wait_flag(const Abort &ab, uint32_t addr, int target) {
+  for (long long it = 0; it < kPollsPerWait * ab.limit; ++it) {
+    int v;
+    asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    if (v >= target) return true;
+    if ((it & 63) == 63 && ab.set()) return false;
+    __nanosleep(20);
+  }
   ab.raise();
   return false;
 }
@@ -242,7 +259,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const uint32_t bar_d_full = bar_s_empty + 8 * kPlMaxStages;  // accumulator complete (two accumulators)
   const uint32_t bar_d_empty = bar_d_full + 16;                // accumulator drained
   const uint32_t bar_drain = bar_d_empty + 16;
-  const uint32_t misc = bar_drain + 16;                         // [0] TMEM base, [1] abort flag, [2] last CTA out
+  const uint32_t misc = bar_drain + 16;                         // [0] TMEM base, [1] abort flag, [2] last CTA out, [3] dependencies met
   uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
   volatile uint32_t *misc_ptr = reinterpret_cast<volatile uint32_t *>(gen + (misc - base));
 
@@ -254,6 +271,9 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit};
   const int tile_mul = kPair ? 2 : 1;                          // this CTA's column tile of a piece: tile_mul * tile + rank
 
+  // The launch after this one may set itself up (and fetch its first weights) on SMs that this one has left; everything below
+  // that touches x, y, the workspace or the counters comes after griddepcontrol.wait.
+  grid_dep_launch_dependents();
   if (threadIdx.x == 0) {
     for (int i = 0; i < p.NW; ++i) {
       mbar_init(bar_w_full + 8 * i, 1);
@@ -271,6 +291,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     mbar_init(bar_drain, 1);
     misc_ptr[1] = 0;
     misc_ptr[2] = 0;
+    misc_ptr[3] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -370,7 +391,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   } else if (warp == 1) {
     // ---------------- activation producer
     if (lane == 0) {
-      int gc = 0;
+      grid_dep_wait();
+      int gc = 0, n_deps = 0;
       Ring rs{0, 0};
       int last_prob = -1;
       bool live = true;
@@ -382,7 +404,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
           if (P.dep >= 0) {
             // the input is another problem's output: every tile of it must have been written (by generic
             // stores of other CTAs, read here by the copy engine: hence the proxy fence after the acquire)
-            if (!wait_counter(ab, p.sync + kPlSyncDone + P.dep, P.dep_target)) break;
+            if (!wait_flag(ab, misc + 12, ++n_deps)) break;
             asm volatile("fence.proxy.async;" ::: "memory");
           }
         }
@@ -462,6 +484,22 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
           if (mbar_try_wait(bar_drain, 0)) break;
       }
     }
+  } else if (warp == 3) {
+    // ---------------- dependencies: waits for the counters of the problems that this CTA's pieces read, in their order, ahead of
+    // the activation producer (a counter in L2 is seen two to four microseconds after it was complete)
+    if (lane == 0) {
+      grid_dep_wait();
+      int last_prob = -1, n_deps = 0;
+      for (int si = s_begin; si < s_end && !ab.set(); ++si) {
+        const int prob = load_seg(p.segs + si).prob;
+        if (prob == last_prob) continue;
+        last_prob = prob;
+        const PlProblem &P = p.prob[prob];
+        if (P.dep < 0) continue;
+        if (!wait_counter(ab, p.sync + kPlSyncDone + P.dep, P.dep_target, 200)) break;
+        st_flag(misc + 12, ++n_deps);
+      }
+    }
   } else if (warp >= kPlFirstDequantWarp && warp < kPlFirstEpiWarp) {
     // ---------------- dequantisation: group j of the CTA's stream goes to team and operand buffer j mod 4;
     // a team walks over its own groups only and takes the slots of its own sub-ring in order
@@ -521,6 +559,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     const int c_begin = ((warp - kPlFirstEpiWarp) >> 2) * half_tok, c_end = c_begin + half_tok;
     const bool wide = (half_tok & 15) == 0;                    // sixteen tokens per batch, else eight
     int nseg = 0;
+    grid_dep_wait();
     for (int si = s_begin; si < s_end; ++si, ++nseg) {
       const PlanSeg s = load_seg(p.segs + si);
       const PlProblem &P = p.prob[s.prob];
@@ -860,8 +899,11 @@ static int plan_launch_kernel(K kern, const PlanLaunch &l, const PlParams &q, si
   cfg.blockDim = dim3(kPlThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[3];
   int na = 0;
+  attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[na].val.programmaticStreamSerializationAllowed = 1;
+  ++na;
   attr[na].id = cudaLaunchAttributeCooperative;        // all CTAs resident: the waits between CTAs cannot starve
   attr[na].val.cooperative = 1;
   ++na;
