@@ -161,4 +161,63 @@ struct Ring {
   }
 };
 
+// ---- the weight ring of a CTA with several dequantisation teams
+// The ring is split into one sub-ring of NWT slots per team (group j of the CTA's stream belongs to team j mod teams): a sub-ring
+// has one consumer, which takes its slots in order, so a full / empty pair of barriers per slot is enough.  Lane t feeds the
+// sub-ring of team t; the lanes step together, each issuing its next copy if its slot is free.  (One lane for all teams needed
+// 350 cycles per quantized group and 800 per fp16 group, four copies, next to idle teams, and paced the CTA.)
+struct WeightCopies {
+  const uint8_t *src;        // the team's next copy
+  uint32_t bytes;
+  int left;                  // copies of this group after it
+};
+constexpr int kPollsPerWait = 16;                   // polls here and of flags, per blocking wait of the others
+// next(c): the team's next group into c, false when there is none; to be called by the first kTeams lanes of a warp
+template <int kTeams, bool kEvictFirst, typename Next>
+__device__ __forceinline__ void feed_teams(const Abort &ab, int team, int NWT, uint32_t w_ring, uint32_t bar_full, uint32_t bar_empty, Next next) {
+  constexpr unsigned kLanes = (1u << kTeams) - 1;
+  const uint64_t pol = kEvictFirst ? policy_evict_first() : 0;
+  w_ring += team * NWT * kWSlotBytes, bar_full += 8 * team * NWT, bar_empty += 8 * team * NWT;
+  WeightCopies c{};
+  Ring rw{0, 0};
+  int fills = 0;                                               // (only looked at when giving up)
+  long long idle = 0;
+  bool more = next(c);
+  while (__any_sync(kLanes, more)) {
+    const bool go = more && mbar_test_wait(bar_empty + 8 * rw.idx, rw.lap ^ 1u);
+    if (go) {
+      mbar_arrive_expect_tx(bar_full + 8 * rw.idx, c.bytes);
+      if (kEvictFirst) bulk_copy_g2s_hint(w_ring + rw.idx * kWSlotBytes, c.src, c.bytes, bar_full + 8 * rw.idx, pol);
+      else bulk_copy_g2s(w_ring + rw.idx * kWSlotBytes, c.src, c.bytes, bar_full + 8 * rw.idx);
+      rw.advance(NWT);
+      ++fills;
+      if (c.left > 0) {
+        --c.left;
+        c.src += kFp16SubBytes;
+      } else {
+        more = next(c);
+      }
+    }
+    if (__any_sync(kLanes, go)) {
+      idle = 0;
+      continue;
+    }
+    // (a poll here is a few dozen nanoseconds where the other waits block for up to a microsecond)
+    if (++idle > kPollsPerWait * ab.limit) {
+      if (team == 0 && !ab.set()) ab.raise();
+      break;
+    }
+    if ((idle & 63) == 63 && __any_sync(kLanes, ab.set())) break;
+    __nanosleep(20);
+  }
+  __syncwarp(kLanes);
+  if (ab.set()) {  // let copies already in flight land before the CTA goes away
+    for (int back = 1; back <= NWT && back <= fills; ++back) {
+      const int u = fills - back;
+      for (int it = 0; it < kDrainPolls; ++it)
+        if (mbar_try_wait(bar_full + 8 * (u % NWT), (u / NWT) & 1)) break;
+    }
+  }
+}
+
 }  // namespace rosaq

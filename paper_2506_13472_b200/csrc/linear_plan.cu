@@ -64,7 +64,6 @@ constexpr int kPlFirstDequantWarp = 4, kPlFirstEpiWarp = kPlFirstDequantWarp + 4
 constexpr int kPlEpiThreads = 256;                  // two warps per TMEM lane quadrant
 constexpr int kPlThreads = kPlFirstEpiWarp * 32 + kPlEpiThreads;   // 896
 constexpr int kPlSmemBytes = 227 * 1024;            // the whole SM
-constexpr int kPollsPerWait = 16;                   // polls of the weight producers per blocking wait of the others
 
 struct PlProblem {
   const uint8_t *blob;
@@ -95,17 +94,6 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *ptr) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
   return v;
-}
-__device__ __forceinline__ uint64_t policy_evict_first() {
-  uint64_t pol;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-  return pol;
-}
-__device__ __forceinline__ void bulk_copy_g2s_hint(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar, uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar), "l"(pol)
-      : "memory");
 }
 __device__ __forceinline__ PlanSeg load_seg(const PlanSeg *s) {
   PlanSeg r;
@@ -311,24 +299,14 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const int qbytes = quant_tile_bytes(kBits);
 
   if (warp == 0) {
-    // ---------------- weight-tile producers: stream every piece of every phase, wait for ring slots only.
-    // The ring is split into one sub-ring of NWT slots per dequantisation team (group j of the CTA's stream
-    // belongs to team j mod 4): a sub-ring has one consumer, which takes its slots in order, so a full /
-    // empty pair of barriers per slot is enough.  Lane t feeds the sub-ring of team t and the four lanes step
-    // together, each issuing its next copy if its slot is free: one thread for all four needed 350 cycles per
-    // quantized group and 800 per fp16 group (four copies) next to idle teams, and paced the whole CTA.
+    // ---------------- weight-tile producers: stream every piece of every phase, wait for ring slots only
     if (lane < kPlTeams) {
-      constexpr unsigned kLanes = (1u << kPlTeams) - 1;
-      const uint64_t pol = policy_evict_first();
-      const int NWT = p.NW >> 2;
       const int team = lane;
-      int si = s_begin, j0 = 0, g = 0, g_end = 0, g_fp16 = 0, left = 0;    // left: copies of this group after the next one
-      unsigned fills = 0;                                      // (only looked at when giving up)
-      uint32_t bytes = 0;
-      const uint8_t *base = nullptr, *src = nullptr;
-      Ring rw{0, 0};
+      int si = s_begin, j0 = 0, g = -kPlTeams, g_end = 0, g_fp16 = 0;
+      const uint8_t *base = nullptr;
       PlanSeg ahead = load_seg(p.segs + (s_begin < s_end ? s_begin : 0));
-      auto seek = [&] {                                        // the team's first group at or after g, in this piece or a later one
+      feed_teams<kPlTeams, true>(ab, team, p.NW >> 2, w_ring, bar_w_full, bar_w_empty, [&](WeightCopies &c) {
+        g += kPlTeams;                                         // the team's next group, in this piece or a later one
         while (g >= g_end) {
           if (si == s_end) return false;
           const PlanSeg s = ahead;
@@ -344,59 +322,21 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
           j0 += s.g_end - s.g_begin;
         }
         const bool f16 = g < g_fp16;
-        src = base + (f16 ? (long long)g * kFp16TileBytes : (long long)g_fp16 * kFp16TileBytes + (long long)(g - g_fp16) * qbytes);
-        bytes = f16 ? kFp16SubBytes : qbytes;
-        left = f16 ? 3 : 0;
+        c.src = base + (f16 ? (long long)g * kFp16TileBytes : (long long)g_fp16 * kFp16TileBytes + (long long)(g - g_fp16) * qbytes);
+        c.bytes = f16 ? kFp16SubBytes : qbytes;
+        c.left = f16 ? 3 : 0;
         return true;
-      };
-      bool more = seek();
-      long long idle = 0;
-      while (__any_sync(kLanes, more)) {
-        const int slot = team * NWT + rw.idx;
-        const bool go = more && mbar_test_wait(bar_w_empty + 8 * slot, rw.lap ^ 1u);
-        if (go) {
-          mbar_arrive_expect_tx(bar_w_full + 8 * slot, bytes);
-          bulk_copy_g2s_hint(w_ring + slot * kWSlotBytes, src, bytes, bar_w_full + 8 * slot, pol);
-          rw.advance(NWT);
-          ++fills;
-          if (left > 0) {
-            --left;
-            src += kFp16SubBytes;
-          } else {
-            g += kPlTeams;
-            more = seek();
-          }
-        }
-        if (__any_sync(kLanes, go)) {
-          idle = 0;
-          continue;
-        }
-        // (a poll here is a few dozen nanoseconds where the other waits block for up to a microsecond)
-        if (++idle > kPollsPerWait * p.wait_limit) {
-          if (lane == 0 && !ab.set()) ab.raise();
-          break;
-        }
-        if ((idle & 63) == 63 && ab.set()) break;
-        __nanosleep(20);
-      }
-      __syncwarp(kLanes);
-      if (ab.set()) {  // let copies already in flight land before the CTA goes away
-        for (int back = 1; back <= NWT && back <= (int)fills; ++back) {
-          const int u = (int)fills - back;
-          for (int it = 0; it < kDrainPolls; ++it)
-            if (mbar_try_wait(bar_w_full + 8 * (team * NWT + u % NWT), (u / NWT) & 1)) break;
-        }
-      }
+      });
     }
   } else if (warp == 1) {
-    // ---------------- activation producer
-    if (lane == 0) {
+    // ---------------- activation producer (the whole warp, converged)
+    {
       grid_dep_wait();
       int gc = 0, n_deps = 0;
       Ring rs{0, 0};
       int last_prob = -1;
       bool live = true;
-      for (int si = s_begin; si < s_end && live && !ab.set(); ++si) {
+      for (int si = s_begin; si < s_end && live && !ab.set_all(); ++si) {
         const PlanSeg s = load_seg(p.segs + si);
         const PlProblem &P = p.prob[s.prob];
         if (s.prob != last_prob) {
@@ -404,7 +344,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
           if (P.dep >= 0) {
             // the input is another problem's output: every tile of it must have been written (by generic
             // stores of other CTAs, read here by the copy engine: hence the proxy fence after the acquire)
-            if (!wait_flag(ab, misc + 12, ++n_deps)) break;
+            if (!__all_sync(0xffffffffu, wait_flag(ab, misc + 12, ++n_deps))) break;
             asm volatile("fence.proxy.async;" ::: "memory");
           }
         }
@@ -413,24 +353,27 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         const CUtensorMap *map = &p.xmap[s.prob];
         for (int g = s.g_begin; g < s.g_end; ++g, ++gc, rs.advance(NS)) {
           const int slot = rs.idx;
-          if (!ab.wait(bar_s_empty + 8 * slot, rs.lap ^ 1u)) {
+          if (!ab.wait_all(bar_s_empty + 8 * slot, rs.lap ^ 1u)) {
             live = false;
             break;
           }
           const int k0 = (g_block0 + g) * kGroup;
-          if (kPair) {
-            // each CTA loads its half of the token rows; all bytes are counted on the leader's barrier
-            if (is_lead) mbar_arrive_expect_tx(bar_a_full + 8 * slot, 2 * x_slot_bytes);
-            tma_load_3d_pair(x_ring + slot * x_slot_bytes, map, map_to_rank(bar_a_full + 8 * slot, 0), (int)rank * MTL, k0 >> 6);
-          } else {
-            mbar_arrive_expect_tx(bar_a_full + 8 * slot, x_slot_bytes);
-            tma_load_3d(x_ring + slot * x_slot_bytes, map, bar_a_full + 8 * slot, 0, k0 >> 6);
+          if (elect_one()) {
+            if (kPair) {
+              // each CTA loads its half of the token rows; all bytes are counted on the leader's barrier
+              if (is_lead) mbar_arrive_expect_tx(bar_a_full + 8 * slot, 2 * x_slot_bytes);
+              tma_load_3d_pair(x_ring + slot * x_slot_bytes, map, map_to_rank(bar_a_full + 8 * slot, 0), (int)rank * MTL, k0 >> 6);
+            } else {
+              mbar_arrive_expect_tx(bar_a_full + 8 * slot, x_slot_bytes);
+              tma_load_3d(x_ring + slot * x_slot_bytes, map, bar_a_full + 8 * slot, 0, k0 >> 6);
+            }
           }
+          __syncwarp();
         }
       }
       // (in a pair the leader's barriers count the copies of both CTAs, and the peer stays until the cluster
       // barrier at the end of the kernel, which the leader reaches after this drain)
-      if (ab.set() && is_lead) {
+      if (lane == 0 && ab.set() && is_lead) {
         for (int back = 1; back <= NS && back <= gc; ++back) {
           const int u = gc - back;
           for (int it = 0; it < kDrainPolls; ++it)

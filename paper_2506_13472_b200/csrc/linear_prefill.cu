@@ -327,78 +327,56 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
         }
       }
     } else if (!kDense && warp == 0) {
-      // ---------------- weight-tile producer
-      if (lane == 0) {
-        const int NWT = NW / kPfTeams, qbytes = quant_tile_bytes(kBits);
-        uint32_t idx4 = 0, lap4 = 0;
-        unsigned long long fills4 = 0;
-        int j = 0;
-        bool live = true;
-        int u = u_begin, wk, g0, g1;
-        while (live && !ab.set() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
-          // (the second CTA of a pair on an odd last tile streams that tile again; its results are dropped)
-          int col_pair;
-          const int prob = pf_problem(p, wk, col_pair);
-          const int my_tile = min(2 * col_pair + (int)rank, p.n_tiles[prob] - 1);
-          const uint8_t *tile_base = p.blob[prob] + (long long)my_tile * p.tile_stride;
-          for (int g = g0; g < g1 && live; ++g, ++j) {
-            const bool f16 = g < p.g_fp16;
-            const uint8_t *src = tile_base + (f16 ? (long long)g * kFp16TileBytes
-                                                  : (long long)p.g_fp16 * kFp16TileBytes + (long long)(g - p.g_fp16) * qbytes);
-            const int nsub = f16 ? 4 : 1;
-            const uint32_t bytes = f16 ? kFp16SubBytes : qbytes;
-            const int team = j & (kPfTeams - 1);
-            uint32_t idx = (idx4 >> (8 * team)) & 0xffu;
-            for (int sub = 0; sub < nsub; ++sub) {
-              const int slot = team * NWT + (int)idx;
-              if (!ab.wait(bar_w_empty + 8 * slot, ((lap4 >> team) & 1u) ^ 1u)) {
-                live = false;
-                break;
-              }
-              mbar_arrive_expect_tx(bar_w_full + 8 * slot, bytes);
-              bulk_copy_g2s(w_ring + slot * kWSlotBytes, src + (long long)sub * kFp16SubBytes, bytes, bar_w_full + 8 * slot);
-              fills4 += 1ull << (16 * team);
-              if (++idx == (uint32_t)NWT) {
-                idx = 0;
-                lap4 ^= 1u << team;
-              }
-            }
-            idx4 = (idx4 & ~(0xffu << (8 * team))) | (idx << (8 * team));
+      // ---------------- weight-tile producers
+      if (lane < kPfTeams) {
+        const int qbytes = quant_tile_bytes(kBits), team = lane;
+        int u = u_begin, wk, j0 = 0, g = -kPfTeams, g_end = 0;
+        const uint8_t *base = nullptr;
+        feed_teams<kPfTeams, false>(ab, team, NW / kPfTeams, w_ring, bar_w_full, bar_w_empty, [&](WeightCopies &c) {
+          g += kPfTeams;                             // the team's next group, in this piece or a later one
+          while (g >= g_end) {
+            int g0;
+            if (!pf_next_piece(u, u_end, G, wk, g0, g_end)) return false;
+            // (the second CTA of a pair on an odd last tile streams that tile again; its results are dropped)
+            int col_pair;
+            const int prob = pf_problem(p, wk, col_pair);
+            const int my_tile = min(2 * col_pair + (int)rank, p.n_tiles[prob] - 1);
+            base = p.blob[prob] + (long long)my_tile * p.tile_stride;
+            g = g0 + ((team - j0) & (kPfTeams - 1));
+            j0 += g_end - g0;
           }
-        }
-        if (ab.set()) {  // let copies already in flight land before the CTA goes away
-          for (int team = 0; team < kPfTeams; ++team) {
-            const int f = (int)((fills4 >> (16 * team)) & 0xffffu);
-            for (int back = 1; back <= NWT && back <= f; ++back) {
-              const int k = f - back;
-              for (int it = 0; it < kDrainPolls; ++it)
-                if (mbar_try_wait(bar_w_full + 8 * (team * NWT + k % NWT), (k / NWT) & 1)) break;
-            }
-          }
-        }
+          const bool f16 = g < p.g_fp16;
+          c.src = base + (f16 ? (long long)g * kFp16TileBytes : (long long)p.g_fp16 * kFp16TileBytes + (long long)(g - p.g_fp16) * qbytes);
+          c.bytes = f16 ? kFp16SubBytes : qbytes;
+          c.left = f16 ? 3 : 0;
+          return true;
+        });
       }
     } else if (!kDense && warp == 1) {
-      // ---------------- activation producer: this CTA's half of the token rows of every group
-      if (lane == 0) {
+      // ---------------- activation producer: this CTA's half of the token rows of every group (the whole warp, converged)
+      {
         grid_dep_wait();                                       // x may be the previous kernel's output
         int gc = 0;
         Ring rs{0, 0};
         bool live = true;
         int u = u_begin, wk, g0, g1;
-        while (live && !ab.set() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
+        while (live && !ab.set_all() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
           const int tok0 = (wk % p.n_tok_blocks) * NT + (int)rank * rows;
           for (int g = g0; g < g1; ++g, ++gc, rs.advance(kPfStages)) {
             const int slot = rs.idx;
-            if (!ab.wait(bar_s_empty + 8 * slot, rs.lap ^ 1u)) {
+            if (!ab.wait_all(bar_s_empty + 8 * slot, rs.lap ^ 1u)) {
               live = false;
               break;
             }
             // all bytes are counted on the leader's barrier
-            if (is_lead) mbar_arrive_expect_tx(bar_a_full + 8 * slot, 2 * x_slot_bytes);
-            tma_load_3d_pair(x_ring + slot * x_slot_bytes, &p.xmap, map_to_rank(bar_a_full + 8 * slot, lead), tok0, 2 * g);
+            if (elect_one()) {
+              if (is_lead) mbar_arrive_expect_tx(bar_a_full + 8 * slot, 2 * x_slot_bytes);
+              tma_load_3d_pair(x_ring + slot * x_slot_bytes, &p.xmap, map_to_rank(bar_a_full + 8 * slot, lead), tok0, 2 * g);
+            }
+            __syncwarp();
           }
         }
-        if (ab.set() && is_lead) {
+        if (lane == 0 && ab.set() && is_lead) {
           for (int back = 1; back <= kPfStages && back <= gc; ++back) {
             const int k = gc - back;
             for (int it = 0; it < kDrainPolls; ++it)
