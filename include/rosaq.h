@@ -64,7 +64,8 @@ typedef struct rosaq_plan rosaq_plan;         /* a list of rotations / linears t
 typedef struct {
   int32_t d;           /* total dimension */
   int32_t n_blocks;    /* d % n_blocks == 0 */
-  const void *q;       /* DEVICE [n_blocks][d/n_blocks][d/n_blocks] */
+  const void *q;       /* DEVICE [n_blocks][d/n_blocks][d/n_blocks]; 16-byte aligned for rosaq_rotation_create,
+                        * on any element for rosaq_quantize */
   int32_t q_dtype;     /* ROSAQ_F32 for rosaq_quantize, ROSAQ_F16 for rosaq_rotation_create */
   const int32_t *perm; /* DEVICE [d] or NULL; must be a permutation of 0..d-1 */
 } rosaq_rot;

@@ -281,7 +281,8 @@ rotate_tile_kernel(const RotateArgs a, const TiledOperand t) {
     const int i = (threadIdx.x & 31) * 4 + e + c0;
     pc[e] = i >= a.dh ? -1 : (perm ? perm[i] : i);
   }
-  const bool a_vec = perm == nullptr && a.dh % 8 == 0, b_vec = a.d_out % 8 == 0;
+  // (W is 16-byte aligned; R may lie on any element)
+  const bool a_vec = perm == nullptr && a.dh % 8 == 0 && reinterpret_cast<uintptr_t>(a.q) % (4 * sizeof(TQ)) == 0, b_vec = a.d_out % 8 == 0;
   auto fetch_a = [&](int k, int, Raw4<TQ> &raw) {
     if (k < a.dh && a_vec && pc[3] >= 0) {
       raw.load4(R + (long long)k * a.dh + pc[0]);

@@ -47,3 +47,22 @@ def test_quantize_tile_edges_bit_exact(heads, dh, d_out, perm, half, scaled, bit
         assert ctx.last_status() == rb.ROSAQ_OK
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("heads,half,off", [(1, False, 1), (1, False, 2), (1, True, 1), (1, True, 3), (2, False, 3), (2, True, 2)])
+def test_rotation_on_any_element(heads, half, off):
+    """R at an address that is no multiple of four elements (a view into a larger buffer)."""
+    dh, d_out = 256 // heads, 136
+    rng = synth.rng_for(82, "offset", heads, half)
+    Rb = np.stack([synth.orthogonal_qr(dh, rng) for _ in range(heads)]).astype(np.float16 if half else np.float32)
+    W = synth.weights(256, d_out, seed=82, key="offset", outlier_frac=0.01)
+    q = dev(np.concatenate([np.zeros(off, Rb.dtype), Rb.ravel()]))[off:].view(heads, dh, dh)
+    assert q.data_ptr() % (8 if half else 16)
+    qd = H.oracle_quantized(W, Rb.astype(np.float32) if heads > 1 else Rb[0].astype(np.float32), None, 4, 128)
+    ctx = rb.Context(0)
+    try:
+        w = ctx.quantize(dev(W), q if heads > 1 else q[0], None, bits=4, k_salient=128)
+        H.assert_export_matches(H.export_to_numpy(w.export()), qd)
+        assert ctx.last_status() == rb.ROSAQ_OK
+    finally:
+        ctx.close()
