@@ -187,9 +187,12 @@ __device__ __forceinline__ void quant_tile(const float *tile, float2 *ends, cons
     }
     return;
   }
-  float lo = col[0], hi = col[0];
+  // The scan of a whole column starts with its first value and skips NaNs after it; a part that starts further down starts
+  // with the empty range, so that a NaN there is skipped as well.
+  const float inf = __int_as_float(0x7f800000);
+  float lo = part == 0 ? col[0] : inf, hi = part == 0 ? col[0] : -inf;
 #pragma unroll 16
-  for (int k = 1; k < kRows; ++k) {
+  for (int k = 0; k < kRows; ++k) {
     const float w = col[k * kTilePitch];
     lo = w < lo ? w : lo;
     hi = w > hi ? w : hi;

@@ -66,3 +66,24 @@ def test_rotation_on_any_element(heads, half, off):
         assert ctx.last_status() == rb.ROSAQ_OK
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("bits", [3, 4])
+def test_nan_inside_a_group(bits):
+    """NaNs behind the first row of a group are no extremes: scale, zero-point and the other rows' codes as in one scan down
+    the column, wherever the threads of a column start.  (A NaN has no code; the kernel stores 0.)"""
+    d, d_out = 384, 140
+    W = synth.weights(d, d_out, seed=83, key="nan", outlier_frac=0.01)
+    for n, row in enumerate((1, 31, 32, 33, 64, 65, 95, 96, 127)):
+        W[128 + row, n] = np.nan
+        W[256 + row, 130 + n] = np.nan
+    W[128 + 32:128 + 64, 20] = np.nan
+    W[256 + 1:384, 21] = np.nan
+    qd = orc.quantize(W.astype(np.float32), bits, 128, 128)
+    codes = np.where(np.isnan(W[128:].astype(np.float32)), 0, qd["codes"]).astype(np.uint8)
+    qd["qw"], qd["cols"] = orc.pack(codes, bits), np.arange(d_out)
+    ctx = rb.Context(0)
+    try:
+        H.assert_export_matches(H.export_to_numpy(ctx.quantize(dev(W), None, bits=bits, k_salient=128).export()), qd)
+    finally:
+        ctx.close()
