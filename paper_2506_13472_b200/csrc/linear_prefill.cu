@@ -792,11 +792,20 @@ bool prefill_supported(const TiledOperand &t, const int32_t *col_map) {
          (t.bits == 3 || t.bits == 4);
 }
 
-// How a launch is cut, and about how long it takes (us).  The figures are a fit to 7B and 13B shapes and smaller ones at
-// 65 ... 1900 tokens: a launch costs about 5.5 us + 0.016 per token of a tile, an exchange in a cluster of more than four
-// CTAs 0.012 per token more, the exchange through L2 7; a group takes a pair 0.3 us + 0.0008 per token, and more the more
-// pairs run (they share the L2 and the power limit).
+// How a launch is cut, and about how long it takes (us) in a chain of launches.  A fit to the launches that linear_tc_estimate is
+// fitted to, each cut measured by itself (clusters 4 % rms, equal shares 6 %): a launch and `token` us per token of a tile;
+// `exchange` between the pairs of a cluster; a group of a pair 0.0021 us per token, and more the more pairs run (they share the L2
+// and the power limit); `full` when more than half of the SMs are taken, so that the next launch has to wait for
+// this one to end.  Equal shares: the exchange through L2, more of it the more pairs hold a tile (13824 -> 128 at 160
+// tokens, 74 holders: 33 us; four pairs in a cluster 17; the per-call kernel 11.6).
 PrefillCut prefill_choose(rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts) {
+  struct Cluster { double launch, token, exchange[kPfMaxSplits + 1], group, group_token, full, crowd; };
+  static constexpr Cluster kClusterQuant{3.493, 0.0166, {0, 0, 0.813, 1.16, 1.994}, 0.0236, 0.0022, 1.972, 0.2853};
+  static constexpr Cluster kClusterDense{2.515, 0.0161, {0, 0, 1.683, 2.241, 2.838}, 0.0478, 0.0021, 0.615, 0.2883};
+  struct Shares { double launch, token, group, group_token, holder, tile; };
+  static constexpr Shares kSharesQuant{9.427, 0.0192, -0.0607, 0.0034, 0.2175, 2.462};
+  static constexpr Shares kSharesDense{4.217, 0.028, 0.2805, 0.0021, 0.2613, 2.633};
+  const bool dense = ts[0]->g_quant == 0;
   const int G = groups_per_tile(*ts[0]);
   long long col_pairs = 0;
   for (int i = 0; i < n; ++i) col_pairs += (ts[i]->n_tiles + 1) / 2;
@@ -804,16 +813,19 @@ PrefillCut prefill_choose(rosaq_ctx *ctx, int M, int n, const TiledOperand *cons
   const int blocks = (M + kPfMaxTokens - 1) / kPfMaxTokens;
   best.NT = ((M + blocks - 1) / blocks + 31) / 32 * 32;
   best.n_tok_blocks = (M + best.NT - 1) / best.NT;
-  const double NT = best.NT, tiles = (double)col_pairs * best.n_tok_blocks;
-  const double dense = ts[0]->g_quant == 0 ? 2.0 : 0.0;
-  auto group_us = [&](double pairs) { return 0.3 + 0.0008 * NT + (0.0011 + 0.0000133 * NT) * pairs; };
-  const double pairs = prefill_clusters(ctx, 1), units = tiles * G;
-  best.S = 0;
-  best.us = 12.5 + 0.026 * NT + dense + units / (pairs > 0 ? pairs : 1) * group_us(std::min(pairs, units));
+  const double NT = best.NT, tiles = (double)col_pairs * best.n_tok_blocks, half = ctx->sm_count / 4;
+  {
+    const Shares &f = dense ? kSharesDense : kSharesQuant;
+    const double units = tiles * G, pairs = std::max(1.0, std::min((double)prefill_clusters(ctx, 1), units));
+    best.S = 0;
+    best.us = f.launch + f.token * NT + units / pairs * (f.group + f.group_token * NT) + f.holder * std::max(0.0, pairs / tiles - 2) + f.tile * tiles / pairs;
+  }
+  const Cluster &f = dense ? kClusterDense : kClusterQuant;
   for (int S = 1; S <= kPfMaxSplits && S <= G; ++S) {
     const int res = prefill_clusters(ctx, S);
     if (res < 1 || tiles > res) continue;                    // (a second round of clusters costs more than equal shares)
-    const double us = 5.5 + 0.016 * NT + (S > 2 ? 0.012 * NT : 0.0) + dense + (double)((G + S - 1) / S) * group_us(tiles * S);
+    const double over = std::max(0.0, tiles * S / half - 1);
+    const double us = f.launch + f.token * NT + f.exchange[S] + (over > 0 ? f.full : 0.0) + (double)((G + S - 1) / S) * (f.group + f.group_token * NT) * (1 + f.crowd * over);
     if (us < best.us) best.us = us, best.S = S;
   }
   return best;

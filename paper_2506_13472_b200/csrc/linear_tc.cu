@@ -874,19 +874,29 @@ int launch_permute_rows(__half *y, int M, long long ldy, int d, const int32_t *c
   return ROSAQ_OK;
 }
 
-// About how long launch_linear_tc_multi takes (us) for more than 128 tokens: 0.9 us per group of a CTA's share (fp16 1.3), two
-// CTAs per SM; a last round that is not full is shorter, its CTAs having an SM to themselves.
+// About how long launch_linear_tc_multi takes (us) for more than 128 tokens, in a chain of launches.  A fit (6 % rms) to 1900
+// launches of 256 ... 13824 channels and columns, 129 ... 2048 tokens, one to four weights, dense and head-wise rotations:
+//   * a launch, and `token` us per token of a tile more;
+//   * a group 0.46 us while the CTAs have an SM each, 0.73 when two share one (from 60 CTAs on clusters begin to: they do not spread
+//     evenly), which also keeps the next launch of the chain out until this one ends (`shared`);
+//   * past the first round of two CTAs per SM, each further one at about 1.3 of the first.
 double linear_tc_estimate(const rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts) {
+  struct Fit { double launch, token, shared, unsplit, group, group_shared, group_token, round, part0, part1, rounds; };
+  static constexpr Fit kQuant{1.459, 0.0312, 2.211, 1.331, 0.461, 0.272, 0.0024, 5.696, 0.6876, 0.7121, 1.3162};
+  static constexpr Fit kDense{1.270, 0.0314, 2.028, 1.270, 0.7716, 0.1495, 0.002, 7.585, 1.630, -0.728, 1.5636};
   const TiledOperand &t = *ts[0];
+  const Fit &f = t.g_quant == 0 ? kDense : kQuant;
   long long tiles = 0;
   for (int i = 0; i < n; ++i) tiles += ts[i]->n_tiles;
-  tiles *= (M + 127) / 128;
-  const int G = groups_per_tile(t);
-  const int S = linear_tc_splits(ctx, tiles, G, 6);
-  const double rounds = (double)tiles * S / (2.0 * ctx->sm_count), whole = (double)(long long)rounds, part = rounds - whole;
-  const double full = rounds <= 1.0 ? 1.0 : whole + (part > 0 ? 0.65 + 0.4 * part : 0.0);
-  const bool dense = t.g_quant == 0;
-  return (dense ? 7.0 : 5.5) + full * ((G + S - 1) / S) * (dense ? 1.3 : 0.9);
+  const int m_tiles = (M + 127) / 128, G = groups_per_tile(t);
+  tiles *= m_tiles;
+  const int S = linear_tc_splits(ctx, tiles, G, 6), groups = (G + S - 1) / S;
+  const double tokens = ((M + m_tiles - 1) / m_tiles + 15) / 16 * 16, ctas = (double)tiles * S, sms = ctx->sm_count;
+  const double x = S > 1 ? std::min(1.0, std::max(0.0, (ctas - 0.4 * sms) / (0.57 * sms))) : (ctas > sms ? 1.0 : 0.0);   // share of the SMs with two CTAs
+  const double rounds = std::max(1.0, ctas / (2 * sms)), whole = (double)(long long)rounds, part = rounds - whole;
+  const double k = 1 + f.rounds * (whole - 1) + (part > 0 ? f.part0 + f.part1 * part : 0.0);
+  return f.launch + f.token * tokens + x * (S > 1 ? f.shared : f.shared - f.unsplit) +
+         groups * (f.group + x * (f.group_shared + f.group_token * (tokens - 128))) * k + f.round * (rounds - 1);
 }
 
 static int launch_linear_sk(const rosaq_ctx *ctx, const __half *x, long long ldx, const TiledOperand &t, const SkParams &q,

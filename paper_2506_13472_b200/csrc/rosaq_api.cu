@@ -146,12 +146,15 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
     return st == ROSAQ_OK ? launch_permute_rows(ys[0], M, ldys[0], ts[0]->d_out, col_map, s) : st;
   }
   // More than 128 tokens may run on 256-column tiles shared by pairs of CTAs, one dequantisation per 256 tokens; the
-  // estimates of the two kernels decide.  Per-call kernel / pairs, measured (us): 4096 -> 4096 at 200 tokens 13.4 / 15.8, at
-  // 768 33.6 / 31.3; 4096 -> 3 x 4096 at 200 30.5 / 27.0, at 1900 180 / 172; 4096 -> 2 x 11008 at 200 53.7 / 46.0, at 1900
-  // 338 / 288; 11008 -> 4096 at 200 25.3 / 28.3, at 768 92.8 / 61.2; 5120 x 5120 rotation at 200 21.3 / 18.8, at 1900 157 / 89.
+  // estimates of the two kernels decide.  Over 1900 shapes the pick is 0.2 % slower than the faster of the two on
+  // average, by more than 10 % on 7; the margin keeps small launches, where the estimates err most, on the per-call
+  // kernel.  Per-call kernel / pairs, measured (us): 13824 -> 128 at 160 tokens 11.7 / 17.1, 4096 -> 4096 at 200 13.0 / 16.3, at 768
+  // 28.7 / 28.7, 4096 -> 11008 at 1900 160 / 138, 4096 -> 3 x 4096 at 200 27.0 / 25.9, 5120 x 5120 rotation at 200 18.8 / 17.1, at
+  // 1900 130 / 84.
+  constexpr double kMarginUs = 0.4;
   if (prefill_supported(*ts[0], col_map) && (ctx->impl == 5 || (ctx->impl == 0 && M > 128))) {
     const PrefillCut cut = prefill_choose(ctx, M, n, ts);
-    if (ctx->impl == 5 || cut.us < 0.97 * linear_tc_estimate(ctx, M, n, ts)) return launch_linear_prefill(ctx, x, M, ldx, n, ts, ys, ldys, cut, s);
+    if (ctx->impl == 5 || cut.us < linear_tc_estimate(ctx, M, n, ts) - kMarginUs) return launch_linear_prefill(ctx, x, M, ldx, n, ts, ys, ldys, cut, s);
   }
   return launch_linear_tc_multi(ctx, x, M, ldx, n, ts, col_map, ys, ldys, s);
 }

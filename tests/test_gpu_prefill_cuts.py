@@ -36,7 +36,8 @@ def same(a, b):
     (33, 1152, [6000], 4),              # narrow token tile, one pair per tile
     (300, 384, [512, 200, 136], 4),     # three weights, two token blocks
     (520, 1024, [11008, 1000], 3),      # equal shares
-    (260, 2048, [10496], 4),            # equal shares, many holders of a tile
+    (260, 2048, [10496], 4),            # equal shares, two holders of most tiles
+    (300, 24576, [136], 4),             # equal shares, 37 holders of each tile
 ])
 def test_prefill_cuts(ctx, M, d_in, widths, bits):
     Ws = [synth.weights(d_in, n, seed=91, key=f"cut{n}", outlier_frac=0.01) for n in widths]
@@ -102,4 +103,20 @@ def test_rotations_at_prefill_sizes(ctx, M, d, heads):
             finally:
                 ctx.set_linear_impl(0)
         rot.free()
+    assert ctx.last_status() == rb.ROSAQ_OK
+
+
+def test_few_tiles_of_a_long_k_stay_on_the_per_call_kernel(ctx):
+    """Where a launch has one or two tiles of many groups the exchange of the pair tiles costs more than the launch on the
+    per-call kernel (11.7 us against 17 to 43 at 160 tokens); the same kernel gives the same bits as implementation 3."""
+    for d_in, widths in ((13824, [128]), (11008, [384]), (13824, [128, 128, 128, 128])):
+        rng = synth.rng_for(93, "longk", d_in)
+        ws = [ctx.quantize(dev(synth.weights(d_in, n, seed=93, key=f"longk{i}", outlier_frac=0.01)), None, bits=4, k_salient=128)
+              for i, n in enumerate(widths)]
+        for M in (129, 160, 300):
+            x = dev(rng.standard_normal((M, d_in)).astype(np.float16))
+            ctx.set_linear_impl(3)
+            ref = [y.clone() for y in ctx.linear_multi(x, ws)]
+            ctx.set_linear_impl(0)
+            assert all(same(y, r) for y, r in zip(ctx.linear_multi(x, ws), ref))
     assert ctx.last_status() == rb.ROSAQ_OK
