@@ -270,11 +270,12 @@ __global__ void __launch_bounds__(kFmaThreads, 2)
 rotate_tile_kernel(const RotateArgs a, const TiledOperand t) {
   extern __shared__ __align__(16) float smem[];
   const FmaThread ft;
-  const int nt = blockIdx.x, n0 = a.n_base + nt * kBN;
-  // rows of the tile: output channels of group blockIdx.y, or (kSpill) source columns of one head block
+  // (kSpill: the row tiles, one and more per head block, in the grid's x: there may be more than 65535)
+  const int nt = kSpill ? blockIdx.y : blockIdx.x, row = kSpill ? blockIdx.x : blockIdx.y, n0 = a.n_base + nt * kBN;
+  // rows of the tile: output channels of group `row`, or (kSpill) source columns of one head block
   const int per_block = (a.dh + kBM - 1) / kBM;
-  const int h = kSpill ? (int)blockIdx.y / per_block : (a.perm ? 0 : (int)blockIdx.y * kBM / a.dh);
-  const int c0 = kSpill ? ((int)blockIdx.y % per_block) * kBM : (int)blockIdx.y * kBM - h * a.dh;   // first column inside the block
+  const int h = kSpill ? row / per_block : (a.perm ? 0 : row * kBM / a.dh);
+  const int c0 = kSpill ? (row % per_block) * kBM : row * kBM - h * a.dh;   // first column inside the block
   const TQ *R = static_cast<const TQ *>(a.q) + (long long)h * a.dh * a.dh;
   const __half *W = a.W + (long long)h * a.dh * a.d_out;
   const int32_t *perm = kSpill ? nullptr : a.perm;
@@ -315,7 +316,7 @@ rotate_tile_kernel(const RotateArgs a, const TiledOperand t) {
   if (!kSpill) {
     store_tile_smem(smem, ft, acc);                                  // (the K loop ends with a barrier)
     __syncthreads();
-    quant_tile<kBits, 1>(smem, nullptr, t, nt, blockIdx.y);
+    quant_tile<kBits, 1>(smem, nullptr, t, nt, row);
   } else {
 #pragma unroll
     for (int ia = 0; ia < 8; ++ia) {
@@ -399,7 +400,7 @@ static int rotate_quantize_typed(const RotateArgs &args, int n_blocks, const Til
     for (int nt0 = 0; nt0 < t.n_tiles; nt0 += tiles_max) {
       const int nts = std::min(tiles_max, t.n_tiles - nt0);
       a.n_base = nt0 * kTileN;
-      spilling<<<dim3(nts, row_tiles), kFmaThreads, kFmaSmemBytes, s>>>(a, t);
+      spilling<<<dim3(row_tiles, nts), kFmaThreads, kFmaSmemBytes, s>>>(a, t);
       quant<<<dim3(nts, groups), kQuantThreads, kQuantSmemBytes, s>>>(a.spill, nullptr, nullptr, nt0, a.spill_cols, t);
     }
   }

@@ -87,3 +87,20 @@ def test_nan_inside_a_group(bits):
         H.assert_export_matches(H.export_to_numpy(ctx.quantize(dev(W), None, bits=bits, k_salient=128).export()), qd)
     finally:
         ctx.close()
+
+
+def test_more_head_blocks_than_a_grid_dimension_holds():
+    """70016 head blocks of one channel: R is a diagonal of signs, so W' is W with the signs, in a column order."""
+    d, d_out = 70016, 8
+    rng = synth.rng_for(84, "blocks", d)
+    sign = rng.choice(np.asarray([-1.0, 1.0], np.float32), d)
+    p = rng.permutation(d).astype(np.int32)
+    W = synth.weights(d, d_out, seed=84, key="blocks", outlier_frac=0.01)
+    qd = orc.quantize((W.astype(np.float32) * sign[:, None])[p], 4, 128, 128)
+    qd["qw"], qd["cols"] = orc.pack(qd["codes"], 4), np.arange(d_out)
+    ctx = rb.Context(0)
+    try:
+        w = ctx.quantize(dev(W), dev(sign.reshape(d, 1, 1)), dev(p), bits=4, k_salient=128)
+        H.assert_export_matches(H.export_to_numpy(w.export()), qd)
+    finally:
+        ctx.close()
