@@ -203,7 +203,7 @@ __device__ __forceinline__ void feed_teams(const Abort &ab, int team, int NWT, u
       continue;
     }
     // (a poll here is a few dozen nanoseconds where the other waits block for up to a microsecond)
-    if (++idle > kPollsPerWait * ab.limit) {
+    if (++idle / kPollsPerWait > ab.limit) {              // (any limit: the product could overflow)
       if (team == 0 && !ab.set()) ab.raise();
       break;
     }

@@ -122,7 +122,7 @@ __device__ __forceinline__ bool wait_counter(const Abort &ab, const unsigned *ct
 // a count in shared memory that one warp raises and another waits for
 __device__ __forceinline__ void st_flag(uint32_t addr, int v) { asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 __device__ __forceinline__ bool wait_flag(const Abort &ab, uint32_t addr, int target) {
-  for (long long it = 0; it < kPollsPerWait * ab.limit; ++it) {
+  for (long long it = 0; it / kPollsPerWait < ab.limit; ++it) {
     int v;
     asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     if (v >= target) return true;

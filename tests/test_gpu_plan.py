@@ -202,3 +202,32 @@ def test_7b_layer_plan_all_columns(ctx, bits, pairs):
         assert torch.equal(v.view(torch.int16), first[k].view(torch.int16)), k
     plan.free()
     ctx.set_plan_pairs(False)
+
+
+@pytest.mark.parametrize("limit", [2 ** 59, 2 ** 63 - 1])
+def test_waits_take_any_limit(ctx, limit):
+    """The polls that count several to one wait do not multiply the limit: the largest one gives the results of the default."""
+    W = synth.weights(512, 640, 23, "limit", outlier_frac=0.01)
+    rot, w = ctx.rotation_create(dev(H.config_tiny()["R16"])), ctx.quantize(dev(W), None, bits=4, k_salient=128)
+    x = dev(synth.rng_for(23, "limit").standard_normal((64, 512)).astype(np.float16))
+    xr, y = empty(64, 512), empty(64, 640)
+
+    def results():
+        plan = ctx.plan_create(64, [(x, None, rot, xr), (None, 0, w, y)])
+        plan.run()
+        assert ctx.last_status() == rb.ROSAQ_OK
+        ctx.set_linear_impl(5)
+        try:
+            pair = ctx.linear(x, w)
+        finally:
+            ctx.set_linear_impl(0)
+        assert ctx.last_status() == rb.ROSAQ_OK
+        return y.clone(), pair
+
+    want = results()
+    old = ctx.set_wait_limit(limit)
+    try:
+        got = results()
+    finally:
+        ctx.set_wait_limit(old)
+    assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(got, want))
