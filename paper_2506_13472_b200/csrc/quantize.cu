@@ -438,7 +438,7 @@ int launch_rotate_quantize(const void *q, int q_is_f32, int n_blocks, const int3
 // width (4096 tokens x 512 channels: 634 us with all tiles of both triangles and a CTA each, 67 so; x 2048: 1003 and 418).
 template <typename T>
 __global__ void __launch_bounds__(kFmaThreads, 2)
-gram_fma_kernel(const T *__restrict__ X, long long ldx, int dh, float *__restrict__ C, int n_tokens, int Z) {
+gram_fma_kernel(const T *X, long long ldx, int dh, float *C, int n_tokens, int Z) {   // (X: not read-only while the kernel before may still write it)
   extern __shared__ __align__(16) float tile[];
   const FmaThread ft;
   int bi = 0;

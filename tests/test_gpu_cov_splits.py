@@ -43,3 +43,40 @@ def test_calib_cov_splits(dtype, n_tokens, d, n_blocks):
     got = runs[0].astype(np.float64)
     assert np.all(np.abs(got - Cref) <= H.cov_tolerance(Cref, n_tokens) + 1e-30)
     assert np.array_equal(got, np.swapaxes(got, -1, -2))
+
+
+def test_calib_cov_reads_what_the_launch_before_wrote():
+    """The fp32 kernel is chained to the launch before it, which may still be writing its input when it starts: rotation and
+    Gram matrix of narrow blocks from a captured chain, the same bits as with a synchronization in between."""
+    M, d, nb = 600, 256, 8
+    ctx = rb.Context(0)
+    try:
+        rng = synth.rng_for(48, "chain")
+        rot = ctx.rotation_create(torch.from_numpy(synth.orthogonal_qr(d, rng).astype(np.float16)).cuda(),
+                                  torch.from_numpy(rng.permutation(d).astype(np.int32)).cuda())
+        xs = [torch.from_numpy(rng.standard_normal((M, d)).astype(np.float16)).cuda() for _ in range(4)]
+        xr, Cg = torch.empty((M, d), dtype=torch.float16, device="cuda"), torch.zeros((nb, d // nb, d // nb), device="cuda")
+        want = []
+        for x in xs:
+            ctx.rotate(x, rot, out=xr)
+            torch.cuda.synchronize()
+            ctx.calib_cov(xr, Cg, nb)
+            want.append(Cg.clone())
+        x, out = xs[0].clone(), [torch.empty_like(Cg) for _ in xs]
+        side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side):
+            for src, o in zip(xs, out):
+                x.copy_(src)
+                ctx.rotate(x, rot, out=xr)
+                ctx.calib_cov(xr, Cg, nb)
+                o.copy_(Cg)
+        for _ in range(3):
+            xr.fill_(float("nan"))
+            Cg.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert all(torch.equal(o, w) for o, w in zip(out, want))
+        assert ctx.last_status() == rb.ROSAQ_OK
+    finally:
+        ctx.close()
