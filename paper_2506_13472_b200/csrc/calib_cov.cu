@@ -179,7 +179,6 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
   const int Z = p.splits, z = blockIdx.z;
   const int n_stages_all = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
   const int s_begin = (int)((long long)n_stages_all * z / Z), n_stages_total = (int)((long long)n_stages_all * (z + 1) / Z) - s_begin;
-  cov_grid_dep_launch();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kCovStages; ++i) {
@@ -225,6 +224,7 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
         }
         if (++idx == kCovStages) idx = 0, lap ^= 1u;
       }
+      cov_grid_dep_launch();
       if (ab.set()) {  // let loads already in flight land before the CTA goes away
         for (int back = 1; back <= kCovStages && back <= issued; ++back) {
           const int u = issued - back;
@@ -435,7 +435,6 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   const int Z = p.splits, z = blockIdx.z;
   const int n_stages_all = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
   const int s_begin = (int)((long long)n_stages_all * z / Z), n_stages_total = (int)((long long)n_stages_all * (z + 1) / Z) - s_begin;
-  cov_grid_dep_launch();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kPairStages; ++i) {
@@ -485,6 +484,7 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         }
         if (++idx == kPairStages) idx = 0, lap ^= 1u;
       }
+      cov_grid_dep_launch();
       // On a timeout the leader lets the loads of both CTAs land (they are all counted on its barriers)
       // before the final cluster barrier releases the pair; phases whose expectation it never posted
       // cannot complete and are bounded by the drain limit.

@@ -6,6 +6,8 @@
 
 namespace rosaq {
 
+// Lets the next kernel of the stream start.  To be called when little is left to do: the bounded waits of that kernel run from its
+// start, and the time of a Gram matrix grows with its tokens without a bound.
 __device__ __forceinline__ void cov_grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void cov_grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void cov_cluster_sync() {

@@ -448,7 +448,6 @@ gram_fma_kernel(const T *X, long long ldx, int dh, float *C, int n_tokens, int Z
   // split z of the tokens (a cluster shares the tile), cut at multiples of the K step
   const int z = blockIdx.z, steps = (n_tokens + kBK - 1) / kBK;
   const int t0 = (int)((long long)steps * z / Z) * kBK, K = min(n_tokens, (int)((long long)steps * (z + 1) / Z) * kBK) - t0;
-  cov_grid_dep_launch();
   cov_grid_dep_wait();
   X += (long long)t0 * ldx + (long long)blockIdx.y * dh;
   C += (long long)blockIdx.y * dh * dh;
@@ -460,6 +459,7 @@ gram_fma_kernel(const T *X, long long ldx, int dh, float *C, int n_tokens, int Z
   fma_tile<T, T, false>(
       tile, K, ft, [&](int k, int c, Raw4<T> &raw) { fetch(k, i0 + c, raw); },
       [&](int k, int c, Raw4<T> &raw) { fetch(k, n0 + c, raw); }, [](int) { return 0.f; }, acc);
+  cov_grid_dep_launch();
   store_tile_smem(tile, ft, acc);
   __syncthreads();
   const int r_begin = kBM * z / Z, r_end = kBM * (z + 1) / Z;        // rows of the tile that this CTA finishes

@@ -80,3 +80,33 @@ def test_calib_cov_reads_what_the_launch_before_wrote():
         assert ctx.last_status() == rb.ROSAQ_OK
     finally:
         ctx.close()
+
+
+def test_a_long_calib_cov_does_not_use_up_the_waits_of_the_launch_behind_it():
+    """Eight CTAs that take 10 ms leave the other SMs to the launch behind them, whose waits last a few hundred microseconds:
+    it must not start counting before the Gram matrix is nearly complete."""
+    ctx = rb.Context(0)
+    try:
+        X = torch.ones((1 << 20, 64), device="cuda")
+        Cg = torch.zeros((64, 64), device="cuda")
+        W = synth.weights(1024, 512, seed=49, key="behind", outlier_frac=0.01)
+        w = ctx.quantize(torch.from_numpy(W).cuda(), None, bits=4, k_salient=128)
+        x = torch.randn((64, 1024), device="cuda").half()
+        y = torch.empty((64, 512), dtype=torch.float16, device="cuda")
+        want = ctx.linear(x, w).clone()
+        plan = ctx.plan_create(64, [(x, None, w, y)])
+        ctx.calib_cov(X[:64], Cg)
+        old = ctx.set_wait_limit(300)
+        try:
+            for run in (lambda: ctx.linear(x, w, out=y), plan.run):
+                Cg.zero_()
+                y.zero_()
+                torch.cuda.synchronize()
+                ctx.calib_cov(X, Cg)
+                run()
+                assert ctx.last_status() == rb.ROSAQ_OK
+                assert torch.all(Cg == 1 << 20) and (y - want).norm() <= 2e-4 * want.norm()
+        finally:
+            ctx.set_wait_limit(old)
+    finally:
+        ctx.close()
