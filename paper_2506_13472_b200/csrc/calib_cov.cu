@@ -41,6 +41,8 @@ constexpr int kBoxBytes = 64 * kCovTokens * 2;          // one TMA box: 64 chann
 constexpr int kOperandBytes = 2 * kBoxBytes;            // 128 channels (operand A)
 constexpr int kStageBytes = 6 * kBoxBytes;              // A (2 boxes) and up to 256 channels of B (4 boxes)
 constexpr uint32_t kCovTmemCols = 256;
+constexpr int kCovTailStages = 32;                       // the next launch may start when no more than these are left (10 - 20 us); unsplit tiles
+                                                         // fill the chip: nothing to gain before they end
 constexpr int kCovDrainPolls = 1 << 16;                 // for work in flight when a CTA gives up (not the context's limit)
 
 struct CovParams {
@@ -149,6 +151,7 @@ __device__ __forceinline__ void cov_stage_row(uint32_t lane_addr, float *row, in
   }
 }
 
+template <bool kSplit>
 __global__ void __launch_bounds__(kCovThreads, 1)
 cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap map2,
               const __grid_constant__ CUtensorMap map4, const CovParams p) {
@@ -176,7 +179,7 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
   const int b_boxes = p.bn / 64;
   // on a diagonal tile operand A is the slice of B that holds row block bi
   const uint32_t a_in_b = diag ? (uint32_t)((bi % ratio) * kOperandBytes) : 0u;
-  const int Z = p.splits, z = blockIdx.z;
+  const int Z = kSplit ? p.splits : 1, z = kSplit ? (int)blockIdx.z : 0;
   const int n_stages_all = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
   const int s_begin = (int)((long long)n_stages_all * z / Z), n_stages_total = (int)((long long)n_stages_all * (z + 1) / Z) - s_begin;
 
@@ -207,6 +210,7 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
       int issued = 0, idx = 0;
       uint32_t lap = 0;
       for (int s = 0; s < n_stages_total && !ab.set(); ++s, ++issued) {
+        if (kSplit && s == max(0, n_stages_total - kCovTailStages)) cov_grid_dep_launch();
         if (!ab.wait(bar_empty + 8 * idx, lap ^ 1u)) break;
         const uint32_t dst = base + idx * kStageBytes;
         const int tok = (s_begin + s) * kCovTokens;
@@ -224,7 +228,6 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
         }
         if (++idx == kCovStages) idx = 0, lap ^= 1u;
       }
-      cov_grid_dep_launch();
       if (ab.set()) {  // let loads already in flight land before the CTA goes away
         for (int back = 1; back <= kCovStages && back <= issued; ++back) {
           const int u = issued - back;
@@ -407,6 +410,7 @@ __device__ __forceinline__ void tc_mma4_ss_pair(uint32_t d_tmem, uint64_t a, uin
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+template <bool kSplit>
 __global__ void __launch_bounds__(kCovThreads, 1)
 cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap map2,
                    const CovParams p) {
@@ -420,7 +424,7 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   const uint32_t bar_d = smem_u32(&bars[2 * kPairStages]);           // accumulators final (multicast commit)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // a cluster of 2 Z CTAs: ranks 2 z, 2 z + 1 are the pair with split z of the tokens
-  const uint32_t rank = blockIdx.x & 1u, lead = 2u * blockIdx.z;
+  const uint32_t rank = blockIdx.x & 1u, lead = kSplit ? 2u * blockIdx.z : 0u;
   const CovAbort ab{reinterpret_cast<volatile int *>(&misc[1]), p.status, p.wait_limit};
 
   // 256 x 256 tile (bi >= bj) of the lower triangle from the pair index bi (bi + 1) / 2 + bj
@@ -432,7 +436,7 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   const bool diag = bi == bj;
   const int i0 = bi * 256 + (int)rank * kCovTile, j0 = bj * 256;
   const int col_a = h * p.dh + i0, col_b = h * p.dh + j0 + (int)rank * kCovTile;
-  const int Z = p.splits, z = blockIdx.z;
+  const int Z = kSplit ? p.splits : 1, z = kSplit ? (int)blockIdx.z : 0;
   const int n_stages_all = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
   const int s_begin = (int)((long long)n_stages_all * z / Z), n_stages_total = (int)((long long)n_stages_all * (z + 1) / Z) - s_begin;
 
@@ -466,6 +470,7 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
       int issued = 0, idx = 0;
       uint32_t lap = 0;
       for (int s = 0; s < n_stages_total && !ab.set(); ++s, ++issued) {
+        if (kSplit && s == max(0, n_stages_total - kCovTailStages)) cov_grid_dep_launch();
         if (!ab.wait(bar_empty + 8 * idx, lap ^ 1u)) break;
         const uint32_t dst = base + idx * kPairStageBytes;
         const int tok = (s_begin + s) * kCovTokens;
@@ -484,7 +489,6 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         }
         if (++idx == kPairStages) idx = 0, lap ^= 1u;
       }
-      cov_grid_dep_launch();
       // On a timeout the leader lets the loads of both CTAs land (they are all counted on its barriers)
       // before the final cluster barrier releases the pair; phases whose expectation it never posted
       // cannot complete and are bounded by the drain limit.
@@ -674,17 +678,24 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
   p.status = ctx->d_status;
   p.wait_limit = ctx->wait_limit;
   const size_t smem = 1024 + (size_t)kCovStages * kStageBytes;   // the 128 x (bn + 1) fp32 staging tile fits inside
+  const size_t smem2 = 1024 + (size_t)kPairStages * kPairStageBytes;
   static bool attr_done_all[64] = {};                    // function attributes are per device
   if (ctx->device < 0 || ctx->device >= 64) return ROSAQ_ERR_INVALID_ARG;
-  bool &attr_done = attr_done_all[ctx->device];
-  static std::mutex attr_mutex;                          // contexts of several host threads share this cache
-  std::lock_guard<std::mutex> attr_lock(attr_mutex);
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(cov_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return ROSAQ_ERR_CUDA;
+  {
+    static std::mutex attr_mutex;                        // contexts of several host threads share this cache
+    std::lock_guard<std::mutex> attr_lock(attr_mutex);
+    bool &attr_done = attr_done_all[ctx->device];
+    if (!attr_done) {
+      constexpr auto kAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+      if (cudaFuncSetAttribute(cov_tc_kernel<false>, kAttr, (int)smem) != cudaSuccess ||
+          cudaFuncSetAttribute(cov_tc_kernel<true>, kAttr, (int)smem) != cudaSuccess ||
+          cudaFuncSetAttribute(cov_tc_pair_kernel<false>, kAttr, (int)smem2) != cudaSuccess ||
+          cudaFuncSetAttribute(cov_tc_pair_kernel<true>, kAttr, (int)smem2) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ROSAQ_ERR_CUDA;
+      }
+      attr_done = true;
     }
-    attr_done = true;
   }
   const int n_row_blocks = (dh + kCovTile - 1) / kCovTile, ratio = p.bn / kCovTile;
   int tiles = 0;
@@ -692,6 +703,7 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
   // Single CTAs with 128 x 256 tiles, or pairs with 256 x 256 tiles (half the loads per product).  A stage of 64 tokens
   // costs either the same time, so what counts is the number of stages in a row: with the tokens split as far as SMs,
   // cluster size and tokens (four stages each) allow, pairs are taken unless they leave the chip emptier (512 ... 896 channels).
+  // One kernel each for split and whole tiles: with the splits as a variable whole tiles were 3 ... 6 % slower (1500 x 3072 40.6 us, 38.7 so).
   const int nb2 = (dh + 255) / 256, pair_tiles = nb2 * (nb2 + 1) / 2;
   const long long stages = (n_tokens + kCovTokens - 1) / kCovTokens;
   // (a cluster lives inside one GPC and these CTAs fill an SM: about 7/8 of the SMs can hold clusters of four, 3/4 of eight;
@@ -702,25 +714,17 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
       const int slots = c == 2 ? ctx->sm_count : (c == 4 ? ctx->sm_count * 7 / 8 : ctx->sm_count * 3 / 4);
       if (c > ctas_per_split && cov_splits(ctas, slots, stages / 4, c / ctas_per_split) == c / ctas_per_split) z = c / ctas_per_split;
     }
-    return z;
+    // (the exchange of single CTAs costs what eleven stages do: 40 heads at 600 tokens 8.4 us unsplit and 9.6 in two, at 1000 10.0 and
+    // 10.7; 4 x 256 channels at 700 12.6 and 14.9; 2048 channels at 1000 as unsplit pairs 20.1, as single CTAs in two 21.1)
+    return ctas_per_split == 1 && stages - stages / z < 12 ? 1 : z;
   };
   const int z1 = splits((long long)tiles * n_blocks, 1), z2 = splits(2ll * pair_tiles * n_blocks, 2);
   if (dh >= 512 && z2 >= z1) {
-    const size_t smem2 = 1024 + (size_t)kPairStages * kPairStageBytes;
-    static bool attr2_done_all[64] = {};
-    bool &attr2_done = attr2_done_all[ctx->device];
-    if (!attr2_done) {
-      if (cudaFuncSetAttribute(cov_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ROSAQ_ERR_CUDA;
-      }
-      attr2_done = true;
-    }
     p.splits = z2;
-    return cov_launch(cov_tc_pair_kernel, dim3(2 * pair_tiles, n_blocks, z2), kCovThreads, smem2, 2, z2, s, xmap, map2, p);
+    return cov_launch(z2 > 1 ? cov_tc_pair_kernel<true> : cov_tc_pair_kernel<false>, dim3(2 * pair_tiles, n_blocks, z2), kCovThreads, smem2, 2, z2, s, xmap, map2, p);
   }
   p.splits = z1;
-  return cov_launch(cov_tc_kernel, dim3(tiles, n_blocks, z1), kCovThreads, smem, 1, z1, s, xmap, map2, map4, p);
+  return cov_launch(z1 > 1 ? cov_tc_kernel<true> : cov_tc_kernel<false>, dim3(tiles, n_blocks, z1), kCovThreads, smem, 1, z1, s, xmap, map2, map4, p);
 }
 
 }  // namespace rosaq
