@@ -469,20 +469,35 @@ gram_fma_kernel(const T *X, long long ldx, int dh, float *C, int n_tokens, int Z
     __syncthreads();
   }
   const int c4 = (threadIdx.x & 31) * 4, r_first = threadIdx.x >> 5;
-  auto add4 = [](float *dst, float4 v) {
-    const float4 o = *reinterpret_cast<const float4 *>(dst);
-    *reinterpret_cast<float4 *>(dst) = make_float4(__fadd_rn(o.x, v.x), __fadd_rn(o.y, v.y), __fadd_rn(o.z, v.z), __fadd_rn(o.w, v.w));
+  // C[row0 + r][col .. + 3] += value(r) for r = r0, r0 + step, ... < end: eight loads in flight, because a round trip to L2 costs
+  // half a microsecond and a row at a time is 64 of them (64 tokens x 256 channels: 23.9 us, 17.0 so; 20 x 640 19.8 and 12.6)
+  auto add_rows = [&](int row0, int col, int r0, int step, int end, auto value) {
+    float *dst = C + (long long)row0 * dh + col;
+    for (; r0 < end; r0 += 8 * step) {
+      float4 old[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (r0 + e * step < end) old[e] = *reinterpret_cast<const float4 *>(dst + (long long)(r0 + e * step) * dh);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int r = r0 + e * step;
+        if (r >= end) break;
+        const float4 v = value(r);
+        *reinterpret_cast<float4 *>(dst + (long long)r * dh) = make_float4(__fadd_rn(old[e].x, v.x), __fadd_rn(old[e].y, v.y),
+                                                                           __fadd_rn(old[e].z, v.z), __fadd_rn(old[e].w, v.w));
+      }
+    }
   };
   if (n0 + c4 < dh)
-    for (int r = r_begin + r_first; r < r_end && i0 + r < dh; r += 4)
-      add4(C + (long long)(i0 + r) * dh + n0 + c4, *reinterpret_cast<const float4 *>(tile + r * kTilePitch + c4));
+    add_rows(i0, n0 + c4, r_begin + r_first, 4, min(r_end, dh - i0),
+             [&](int r) { return *reinterpret_cast<const float4 *>(tile + r * kTilePitch + c4); });
   // mirror: the share's rows, four at a time, x all columns
   const int n_quads = (r_end - r_begin) / 4, m4 = r_begin + 4 * (threadIdx.x % n_quads);
   if (bi != bj && i0 + m4 < dh)
-    for (int r = threadIdx.x / n_quads; r < kBN && n0 + r < dh; r += kFmaThreads / n_quads) {
+    add_rows(n0, i0 + m4, threadIdx.x / n_quads, kFmaThreads / n_quads, min(kBN, dh - n0), [&](int r) {
       const float *tc = tile + m4 * kTilePitch + r;
-      add4(C + (long long)(n0 + r) * dh + i0 + m4, make_float4(tc[0], tc[kTilePitch], tc[2 * kTilePitch], tc[3 * kTilePitch]));
-    }
+      return make_float4(tc[0], tc[kTilePitch], tc[2 * kTilePitch], tc[3 * kTilePitch]);
+    });
   if (Z > 1) cov_cluster_sync();                                     // nobody reads this CTA's tile any more
 }
 
