@@ -69,11 +69,23 @@ int pool_alloc(rosaq_ctx *ctx, void **p, size_t bytes, cudaStream_t s) {
   return cuda_status(cudaMallocFromPoolAsync(p, bytes, ctx->pool->handle, s));
 }
 
-// work in flight on any stream may still read the memory: like cudaFree on plain memory, wait for the device first
-void pool_free(void *p) {
-  if (!p) return;
-  (void)cudaDeviceSynchronize();
-  (void)cudaFree(p);
+// Waits until nothing on the device can read an operand any more.  cudaFree of ordinary memory does; so does
+// cudaDeviceSynchronize, but that is not allowed while any stream is being captured (it would invalidate the capture), where
+// cudaFree is in the relaxed mode.  False: not waited.
+bool device_idle() {
+  void *p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, 1);
+  if (e == cudaSuccess) return cudaFree(p) == cudaSuccess;
+  (void)cudaGetLastError();
+  return e == cudaErrorMemoryAllocation && cudaDeviceSynchronize() == cudaSuccess;
+}
+
+// cudaFree of pooled memory does not wait for anything by itself.  Memory that cannot be waited for is not given back before
+// its pool goes.
+void pool_free(void *p, void *q = nullptr) {
+  if ((!p && !q) || !device_idle()) return;
+  if (p) (void)cudaFree(p);
+  if (q) (void)cudaFree(q);
 }
 
 int alloc_blob(rosaq_ctx *ctx, TiledOperand *t, cudaStream_t s) {
@@ -505,8 +517,7 @@ int rosaq_rotation_create(rosaq_ctx *ctx, const rosaq_rot *rot, rosaq_rotation *
   if (st == ROSAQ_OK) st = launch_rotation_tiles(static_cast<const __half *>(rot->q), rot->d, rot->n_blocks, r->t, s);
   if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(s));
   if (st != ROSAQ_OK) {
-    pool_free(r->t.blob);
-    pool_free(r->col_map);
+    pool_free(r->t.blob, r->col_map);
     pool_release(r->pool);
     delete r;
     return st;
@@ -519,8 +530,7 @@ int rosaq_rotation_free(rosaq_rotation *r) {
   if (!r) return ROSAQ_ERR_INVALID_ARG;
   DeviceGuard guard(r->device);
   if (guard.ok) {
-    pool_free(r->t.blob);
-    pool_free(r->col_map);
+    pool_free(r->t.blob, r->col_map);
     pool_release(r->pool);
     (void)cudaGetLastError();
   }
