@@ -21,6 +21,9 @@
  *   - Device-side waits are bounded; if one expires the kernel records
  *     ROSAQ_ERR_TIMEOUT in the context's device status word (read it with
  *     rosaq_last_status) and returns, leaving the CUDA context usable.
+ *   - A weight or rotation that another device's context made is accepted by rosaq_rotate, rosaq_linear,
+ *     rosaq_linear_multi, rosaq_linear_static and rosaq_weight_export where that device can be reached
+ *     (cudaDeviceCanAccessPeer), else ROSAQ_ERR_CUDA; its memory is read over the link on every call.
  *   - Handles (rosaq_ctx, rosaq_weight, rosaq_rotation) are owned by the library
  *     and released with the matching *_destroy / *_free.  They are not
  *     thread-safe; use one context per host thread and device.
@@ -152,7 +155,8 @@ int rosaq_calib_cov(rosaq_ctx *ctx, const void *X, int x_dtype, int64_t n_tokens
  *   z = clamp(-rint(lo/s), 0, 2^bits-1), stored as +0 when lo >= 0,
  *   code = clamp(rint(w/s) + z, 0, 2^bits-1), all IEEE fp32, ties to even.
  * Allocates the result (*out, release with rosaq_weight_free) from the context's memory pool, which keeps up to 64 MB
- * of freed memory for reuse and is released with the context; a rotation with a column permutation takes scratch from
+ * of freed memory for reuse (out of the reach of other allocators meanwhile) and is released with the context and the last
+ * operand in it; head blocks that are no multiple of 128 channels, or that come with a column permutation, take scratch from
  * it too (at most 16 MB, or one 128-column strip of W' in fp32).  Synchronizes `stream`.
  * d_in % 128 == 0 required; d_out >= 1 (padded internally to a multiple of 128).
  */

@@ -58,6 +58,9 @@ extern "C" int rosaq_linear_static(rosaq_ctx *ctx, const void *x, int M, int64_t
   if (!rosaq::aligned16(x) || !rosaq::aligned16(y) || (ldx % 8) != 0 || (ldy % 8) != 0) return ROSAQ_ERR_ALIGNMENT;
   if (r && r->d != w->t.d_in) return ROSAQ_ERR_INVALID_ARG;
   if (r && sizeof(__half) * (size_t)M * (size_t)r->d > kStaticScratchBytes) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
+  int st = rosaq::operand_reach(ctx, w->device, w->pool);
+  if (st == ROSAQ_OK && r) st = rosaq::operand_reach(ctx, r->device, r->pool);
+  if (st != ROSAQ_OK) return st;
   rosaq::DeviceGuard guard(ctx->device);
   if (!guard.ok) return ROSAQ_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -65,7 +68,7 @@ extern "C" int rosaq_linear_static(rosaq_ctx *ctx, const void *x, int M, int64_t
   long long ld = ldx;
   if (r) {
     void *scratch = nullptr;
-    int st = scratch_for_device(ctx->device, &scratch);
+    st = scratch_for_device(ctx->device, &scratch);
     if (st != ROSAQ_OK) return st;
     // every element of the [M][d] intermediate is written by the rotation before the GEMM stage reads
     // it (rows past M are zero-filled by the activation copy itself), so nothing has to be cleared

@@ -421,7 +421,8 @@ int rosaq_weight_export(rosaq_ctx *ctx, const rosaq_weight *w, uint32_t *qw, voi
   if (!ctx || !w) return ROSAQ_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return ROSAQ_ERR_CUDA;
-  return launch_export(w->t, qw, static_cast<__half *>(scales_f16), static_cast<__half *>(zeros_f16),
+  const int st = operand_reach(ctx, w->device, w->pool);
+  return st != ROSAQ_OK ? st : launch_export(w->t, qw, static_cast<__half *>(scales_f16), static_cast<__half *>(zeros_f16),
                        static_cast<__half *>(salient_f16), static_cast<cudaStream_t>(stream));
 }
 
@@ -549,6 +550,7 @@ int rosaq_rotate(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
   if (!ctx || !r) return ROSAQ_ERR_INVALID_ARG;
   int st = check_act(x, M, ldx, r->d);
   if (st == ROSAQ_OK) st = check_act(x_rot, M, ldxr, r->d);
+  if (st == ROSAQ_OK) st = operand_reach(ctx, r->device, r->pool);
   if (st != ROSAQ_OK) return st;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return ROSAQ_ERR_CUDA;
@@ -567,6 +569,9 @@ int rosaq_linear(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
   if (st == ROSAQ_OK) st = check_act(y, M, ldy, w->t.d_out);
   if (st != ROSAQ_OK) return st;
   if (r && r->d != w->t.d_in) return ROSAQ_ERR_INVALID_ARG;
+  st = operand_reach(ctx, w->device, w->pool);
+  if (st == ROSAQ_OK && r) st = operand_reach(ctx, r->device, r->pool);
+  if (st != ROSAQ_OK) return st;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return ROSAQ_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -607,6 +612,9 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
   }
   if (st != ROSAQ_OK) return st;
   if (r && r->d != w[0]->t.d_in) return ROSAQ_ERR_INVALID_ARG;
+  for (int i = 0; i < n && st == ROSAQ_OK; ++i) st = operand_reach(ctx, w[i]->device, w[i]->pool);
+  if (st == ROSAQ_OK && r) st = operand_reach(ctx, r->device, r->pool);
+  if (st != ROSAQ_OK) return st;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return ROSAQ_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -245,6 +245,7 @@ namespace rosaq {
 struct MemPool {
   cudaMemPool_t handle = nullptr;
   std::atomic<int> users{1};          // the context and the operands that live in it
+  std::atomic<uint64_t> open_to{0};   // other devices that may read it, a bit each
 };
 }  // namespace rosaq
 
@@ -309,6 +310,24 @@ struct DeviceGuard {
     if (prev >= 0) (void)cudaSetDevice(prev);
   }
 };
+
+// The calls on single linears and rotations take operands of another device's context, as far as the devices reach each other.
+// Memory of cudaMalloc would follow cudaDeviceEnablePeerAccess; a pool has to be opened to the device itself.
+inline int operand_reach(const rosaq_ctx *ctx, int device, MemPool *pool) {
+  if (device == ctx->device) return ROSAQ_OK;
+  const uint64_t bit = 1ull << (ctx->device & 63);
+  if (pool->open_to.load() & bit) return ROSAQ_OK;
+  cudaMemAccessDesc to{};
+  to.location.type = cudaMemLocationTypeDevice;
+  to.location.id = ctx->device;
+  to.flags = cudaMemAccessFlagsProtReadWrite;
+  if (cudaMemPoolSetAccess(pool->handle, &to, 1) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return ROSAQ_ERR_CUDA;
+  }
+  pool->open_to.fetch_or(bit);
+  return ROSAQ_OK;
+}
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
