@@ -121,7 +121,7 @@ int ensure_workspace(rosaq_ctx *ctx, size_t bytes, cudaStream_t s) {
 }
 
 constexpr int kBlockTokens = 128;
-constexpr int kScatterTokens = 16;
+constexpr int kScatterTokens = 22, kScatterElements = 28000;
 
 int run_ops(rosaq_ctx *ctx, int M, int n, const PlanOp *ops, cudaStream_t s);
 
@@ -151,9 +151,10 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
   if (ctx->impl == 6 && n == 1 && M > 64 && M <= kBlockTokens * kPlanMaxOps)
     return run_token_blocks(ctx, x, M, ldx, *ts[0], col_map, ys[0], ldys[0], s);
   // A permuted output (head-wise rotation) is a scatter of 2-byte elements; in column order and then moved inside each row
-  // it is faster from 32 tokens on, the second launch included: d = 5120, 16 tokens 5.9 us scattered and 6.5 so, 32: 7.6
-  // and 6.8, 64: 12.5 and 7.5, 512: 38.8 and 12.6, 1900: 97.9 and 31.6.
-  if (ctx->impl == 0 && n == 1 && col_map && M > kScatterTokens && ts[0]->d_out <= kPermuteMaxColumns) {
+  // it is faster, the second launch included, once there are enough of them.  us, scattered / moved: d = 512 at 40 tokens 4.9 / 5.2,
+  // at 56 5.7 / 5.5; 1024 at 24 4.6 / 4.9, at 36 5.5 / 5.25; 2048 at 20 5.0 / 5.15, at 24 5.2 / 5.1; 5120 at 17 5.7 / 6.15, at 24 6.3 / 6.0, at
+  // 64 11.2 / 7.3, at 512 38.8 / 12.6.
+  if (ctx->impl == 0 && n == 1 && col_map && M > kScatterTokens && (long long)M * ts[0]->d_out > kScatterElements && ts[0]->d_out <= kPermuteMaxColumns) {
     const int st = run_gemm(ctx, x, M, ldx, n, ts, nullptr, ys, ldys, s);
     return st == ROSAQ_OK ? launch_permute_rows(ys[0], M, ldys[0], ts[0]->d_out, col_map, s) : st;
   }

@@ -120,3 +120,19 @@ def test_few_tiles_of_a_long_k_stay_on_the_per_call_kernel(ctx):
             ctx.set_linear_impl(0)
             assert all(same(y, r) for y, r in zip(ctx.linear_multi(x, ws), ref))
     assert ctx.last_status() == rb.ROSAQ_OK
+
+
+@pytest.mark.parametrize("d", [512, 1536])
+def test_column_order_scattered_or_moved(ctx, d):
+    """Either side of the sizes where the column order is no longer written by the epilogue but by a second launch: the same
+    sums, so the same bits as the scattering kernel (implementation 3)."""
+    rng = synth.rng_for(94, "order", d)
+    q = np.stack([synth.orthogonal_qr(128, rng) for _ in range(d // 128)]).astype(np.float16)
+    rot = ctx.rotation_create(dev(q), dev(rng.permutation(d).astype(np.int32)))
+    for M in (16, 17, 22, 23, 54, 55, 64, 100, 128):
+        x = dev(rng.standard_normal((M, d)).astype(np.float16))
+        ctx.set_linear_impl(3)
+        ref = ctx.rotate(x, rot).clone()
+        ctx.set_linear_impl(0)
+        assert same(ctx.rotate(x, rot), ref), M
+    assert ctx.last_status() == rb.ROSAQ_OK
