@@ -95,15 +95,27 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *ptr) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
   return v;
 }
-__device__ __forceinline__ PlanSeg load_seg(const PlanSeg *s) {
+__device__ __forceinline__ PlanSeg make_seg(const uint4 &a, const uint4 &b, const uint4 &c) {
   PlanSeg r;
-  const int4 *q = reinterpret_cast<const int4 *>(s);
-  int4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
   r.prob = a.x, r.tile = a.y, r.g_begin = a.z, r.g_end = a.w;
   r.n_contrib = b.x, r.contrib_idx = b.y, r.slot0 = b.z, r.counter = b.w;
   r.closer_idx = c.x, r.n_closers = c.y, r.tok_begin = c.z, r.tok_end = c.w;
   return r;
 }
+// Every role walks over the CTA's pieces, and a round trip to L2 per piece and role is what a launch over small layers spends most
+// of its time on: the first kPlSegs pieces of a CTA lie in shared memory (3 at 512 channels, 12 at 5120).  us per launch, ten operations of
+// a layer, pieces read from global memory / from shared memory: 1024 channels at 100 tokens 34.0 / 31.1, at 64 25.7 / 25.4;
+// 7B at 64 58.1 / 55.6, at 100 71.6 / 68.0.
+constexpr int kPlSegs = 24;
+struct Pieces {
+  const PlanSeg *global;      // of this CTA
+  uint32_t smem;
+  __device__ __forceinline__ PlanSeg operator[](int i) const {
+    if (i < kPlSegs) return make_seg(lds128(smem + i * 48), lds128(smem + i * 48 + 16), lds128(smem + i * 48 + 32));
+    const uint4 *q = reinterpret_cast<const uint4 *>(global + i);
+    return make_seg(__ldg(q), __ldg(q + 1), __ldg(q + 2));
+  }
+};
 // waits until *ctr >= target; false when the wait gave up
 __device__ __forceinline__ bool wait_counter(const Abort &ab, const unsigned *ctr, unsigned target, unsigned pause = 0) {
   for (long long it = 0; it < ab.limit; ++it) {
@@ -248,6 +260,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const uint32_t bar_d_empty = bar_d_full + 16;                // accumulator drained
   const uint32_t bar_drain = bar_d_empty + 16;
   const uint32_t misc = bar_drain + 16;                         // [0] TMEM base, [1] abort flag, [2] last CTA out, [3] dependencies met
+  const uint32_t seg_smem = misc + 16;
   uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
   volatile uint32_t *misc_ptr = reinterpret_cast<volatile uint32_t *>(gen + (misc - base));
 
@@ -255,7 +268,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const uint32_t rank = kPair ? (blockIdx.x & 1u) : 0u;        // position in the pair; 0 = leader
   const bool is_lead = rank == 0;
   const int cta = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;   // entry of the schedule
-  const int s_begin = p.seg_begin[cta], s_end = p.seg_begin[cta + 1];
+  const int s_first = p.seg_begin[cta], n_segs = p.seg_begin[cta + 1] - s_first;
+  const Pieces pieces{p.segs + s_first, seg_smem};
   const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit};
   const int tile_mul = kPair ? 2 : 1;                          // this CTA's column tile of a piece: tile_mul * tile + rank
 
@@ -283,6 +297,10 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (threadIdx.x >= 128 && (int)threadIdx.x - 128 < 3 * min(n_segs, kPlSegs)) {
+    const int i = (int)threadIdx.x - 128;
+    *reinterpret_cast<uint4 *>(gen + (seg_smem - base) + 16 * i) = __ldg(reinterpret_cast<const uint4 *>(pieces.global) + i);
+  }
   if (warp == 2) {
     if (kPair) tmem_alloc_pair<kPlTmemCols>(misc);             // both CTAs of the pair, same warp index
     else tmem_alloc<kPlTmemCols>(misc);
@@ -302,15 +320,13 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     // ---------------- weight-tile producers: stream every piece of every phase, wait for ring slots only
     if (lane < kPlTeams) {
       const int team = lane;
-      int si = s_begin, j0 = 0, g = -kPlTeams, g_end = 0, g_fp16 = 0;
+      int si = 0, j0 = 0, g = -kPlTeams, g_end = 0, g_fp16 = 0;
       const uint8_t *base = nullptr;
-      PlanSeg ahead = load_seg(p.segs + (s_begin < s_end ? s_begin : 0));
       feed_teams<kPlTeams, true>(ab, team, p.NW >> 2, w_ring, bar_w_full, bar_w_empty, [&](WeightCopies &c) {
         g += kPlTeams;                                         // the team's next group, in this piece or a later one
         while (g >= g_end) {
-          if (si == s_end) return false;
-          const PlanSeg s = ahead;
-          if (++si < s_end) ahead = load_seg(p.segs + si);
+          if (si == n_segs) return false;
+          const PlanSeg s = pieces[si++];
           const PlProblem &P = p.prob[s.prob];
           // (the second CTA of a pair on an odd last tile streams that tile again; its results are dropped)
           int my_tile = tile_mul * s.tile + (int)rank;
@@ -336,8 +352,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
       Ring rs{0, 0};
       int last_prob = -1;
       bool live = true;
-      for (int si = s_begin; si < s_end && live && !ab.set_all(); ++si) {
-        const PlanSeg s = load_seg(p.segs + si);
+      for (int si = 0; si < n_segs && live && !ab.set_all(); ++si) {
+        const PlanSeg s = pieces[si];
         const PlProblem &P = p.prob[s.prob];
         if (s.prob != last_prob) {
           last_prob = s.prob;
@@ -391,8 +407,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
       int nseg = 0;
       bool live = true, issued = false;
       Ring rs{0, 0};
-      for (int si = s_begin; si < s_end && live; ++si, ++nseg) {
-        const PlanSeg s = load_seg(p.segs + si);
+      for (int si = 0; si < n_segs && live; ++si, ++nseg) {
+        const PlanSeg s = pieces[si];
         const int buf = nseg & 1;
         if (!ab.wait_all(bar_d_empty + 8 * buf, ((nseg >> 1) & 1) ^ 1u)) break;   // the piece before last has been drained
         tc_fence_after();
@@ -433,8 +449,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     if (lane == 0) {
       grid_dep_wait();
       int last_prob = -1, n_deps = 0;
-      for (int si = s_begin; si < s_end && !ab.set(); ++si) {
-        const int prob = load_seg(p.segs + si).prob;
+      for (int si = 0; si < n_segs && !ab.set(); ++si) {
+        const int prob = pieces[si].prob;
         if (prob == last_prob) continue;
         last_prob = prob;
         const PlProblem &P = p.prob[prob];
@@ -457,8 +473,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     Ring rw{0, 0};
     bool ok = true;
     int j0 = 0;                                      // position of the piece's first group in the CTA's stream
-    for (int si = s_begin; si < s_end && ok; ++si) {
-      const PlanSeg s = load_seg(p.segs + si);
+    for (int si = 0; si < n_segs && ok; ++si) {
+      const PlanSeg s = pieces[si];
       const int g_fp16 = p.prob[s.prob].g_fp16;
       for (int g = s.g_begin + ((team - j0) & (kPlTeams - 1)); g < s.g_end && ok; g += kPlTeams) {
         const bool f16 = g < g_fp16;
@@ -503,8 +519,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     const bool wide = (half_tok & 15) == 0;                    // sixteen tokens per batch, else eight
     int nseg = 0;
     grid_dep_wait();
-    for (int si = s_begin; si < s_end; ++si, ++nseg) {
-      const PlanSeg s = load_seg(p.segs + si);
+    for (int si = 0; si < n_segs; ++si, ++nseg) {
+      const PlanSeg s = pieces[si];
       const PlProblem &P = p.prob[s.prob];
       const int buf = nseg & 1;
       bool have_d = ab.wait(bar_d_full + 8 * buf, (nseg >> 1) & 1);
@@ -675,13 +691,13 @@ bool plan_encode_x(CUtensorMap *map, const __half *x, int M, long long ldx, int 
 
 // ring depth and shared memory for MTL token rows per CTA
 int plan_nw(int MTL, int ns) {
-  const int budget = kPlSmemBytes - 1024 - ns * MTL * 256 - 512;
+  const int budget = kPlSmemBytes - 1024 - ns * MTL * 256 - 512 - kPlSegs * (int)sizeof(PlanSeg);
   const int nw = (budget / kWSlotBytes) & ~3;          // four sub-rings of equal depth, one per team
   return nw > 20 ? 20 : nw;
 }
 
 size_t plan_smem_bytes(int MTL, int NW, int ns) {
-  return 1024 + (size_t)ns * MTL * 256 + (size_t)NW * kWSlotBytes + 8 * (2 * NW + 2 * kPlMaxStages + 6) + 16;
+  return 1024 + (size_t)ns * MTL * 256 + (size_t)NW * kWSlotBytes + 8 * (2 * NW + 2 * kPlMaxStages + 6) + 16 + kPlSegs * sizeof(PlanSeg);
 }
 
 template <typename K>

@@ -231,3 +231,23 @@ def test_waits_take_any_limit(ctx, limit):
     finally:
         ctx.set_wait_limit(old)
     assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("M,d_out,n_ops", [(16, 40960, 12), (100, 24576, 12), (5, 2048, 3)])
+def test_plan_with_many_pieces_per_cta(ctx, M, d_out, n_ops):
+    """Lists whose CTAs hold more pieces than their shared memory keeps (26 and 16 of one group each on 148 SMs), and fewer than
+    one: against the same operations as separate calls, twice."""
+    w = ctx.quantize(dev(synth.weights(128, d_out, 29, f"pieces{d_out}", outlier_frac=0.01)), None, bits=4, k_salient=128)
+    rng = synth.rng_for(29, "pieces", M)
+    xs = [dev(rng.standard_normal((M, 128)).astype(np.float16)) for _ in range(n_ops)]
+    ys = [empty(M, d_out) for _ in xs]
+    plan = ctx.plan_create(M, [(x, None, w, y) for x, y in zip(xs, ys)])
+    for _ in range(2):
+        for y in ys:
+            y.fill_(float("nan"))
+        plan.run()
+        assert ctx.last_status() == rb.ROSAQ_OK
+        for x, y in zip(xs, ys):
+            sep = ctx.linear(x, w).double()
+            assert (y.double() - sep).norm() <= 2e-4 * sep.norm()
+    plan.free()
