@@ -304,13 +304,15 @@ int small_tiles(int n, const TiledOperand *const *ts) {
 // Whether this kernel is the faster one, from its room: x' of M tokens and the rings of a CTA must leave space for a second CTA
 // where the launch has more slices than SMs (5120 -> 5120 at six / eight tokens: 8.8 / 11.5 us here, 9.3 us on the tcgen05
 // kernel), and for a third where it has many rounds of them (4096 -> 32000: four tokens 22.5 and 26.6 us, eight 28.0 and 26.6 us);
-// and few CTAs must not each copy a long x' (11008 -> 1024 INT3: six tokens 10.2 and 10.0 us, eight 10.8 and 10.1 us).
+// and where the slices leave half of the SMs idle, where the tcgen05 kernel splits K, a CTA must not have a long K to itself
+// (here / there: 8192 -> 512 at three, four and eight tokens 6.7 / 6.5, 6.9 / 6.5, 7.7 / 6.5; 11008 -> 512 at two and six 8.1 / 7.8, 9.2 /
+// 7.9, INT3 at two and five 8.9 / 8.1, 9.8 / 8.1).  Over 936 shapes the pick is 0.6 % slower than the faster one on average.
 bool linear_small_supported(const rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts) {
   const int G = groups_per_tile(*ts[0]);
   if (M > kSmallTokens || n < 1 || n > kSmMaxProblems || G <= 0) return false;
   const int bytes = small_bytes(M, *ts[0], 2), slices = 4 * small_tiles(n, ts), rounds = (slices + ctx->sm_count - 1) / ctx->sm_count;
   const int resident = rounds > 5 ? kSmCtas : std::min(rounds, 2);
-  if (4 * slices <= ctx->sm_count && M * G > 600) return false;
+  if (2 * slices <= ctx->sm_count && M * G > (ts[0]->g_quant > 0 && ts[0]->bits == 3 ? 180 : 260)) return false;
   return bytes <= kSmMaxSmem && resident * (bytes + kSmSharedCta) <= kSmSharedSm;
 }
 

@@ -38,6 +38,10 @@ def same(a, b):
     (2, 1024, [16384], 4),              # more slices than SMs: three CTAs of a launch on an SM
     (8, 5120, [5120], 4),               # x' leaves no room for the second CTA: the tcgen05 kernel
     (9, 512, [512], 4),                 # past its tokens
+    (3, 11008, [72], 4),                # few slices, the longest K of INT4 that stays ...
+    (4, 11008, [72], 4),                # ... the tcgen05 kernel
+    (2, 11008, [200], 3),               # the same for INT3
+    (3, 11008, [200], 3),
 ])
 def test_linear(ctx, M, d_in, widths, bits):
     Ws = [synth.weights(d_in, n, seed=17, key=f"small{n}", outlier_frac=0.01) for n in widths]
