@@ -91,7 +91,8 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
       "l"(map), "r"(bar), "r"(0), "r"(tok), "r"(blk)
       : "memory");
 }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
+// (to be called by one lane: unlike the commits of the linear kernels it elects none)
+__device__ __forceinline__ void tc_commit_lane(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -251,10 +252,10 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
         const uint64_t a = make_mn_desc(diag ? b_addr + a_in_b : b_addr - kOperandBytes);
         tc_mma4_ss(tmem, a, b, idesc, accumulate);
         accumulate = 1;
-        tc_commit(bar_empty + 8 * idx);
+        tc_commit_lane(bar_empty + 8 * idx);
         if (++idx == kCovStages) idx = 0, lap ^= 1u;
       }
-      tc_commit(bar_d);
+      tc_commit_lane(bar_d);
       if (ab.set()) {  // MMAs already issued must retire before the tensor memory is given back
         for (int it = 0; it < kCovDrainPolls; ++it)
           if (mbar_try_wait(bar_d, 0)) break;
@@ -392,7 +393,7 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t smem_addr, uint32_t ran
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint32_t lead) {
+__device__ __forceinline__ void tc_commit_pair_lane(uint32_t bar, uint32_t lead) {
   asm volatile(
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
       "h"((unsigned short)(3u << lead))
@@ -515,10 +516,10 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         const uint64_t a = diag ? b : make_mn_desc(b_addr - kOperandBytes);
         tc_mma4_ss_pair(tmem, a, b, idesc, accumulate);
         accumulate = 1;
-        tc_commit_pair(bar_empty + 8 * idx, lead);
+        tc_commit_pair_lane(bar_empty + 8 * idx, lead);
         if (++idx == kPairStages) idx = 0, lap ^= 1u;
       }
-      tc_commit_pair(bar_d, lead);
+      tc_commit_pair_lane(bar_d, lead);
       if (ab.set()) {  // MMAs already issued must retire before the tensor memory is given back
         for (int it = 0; it < kCovDrainPolls; ++it)
           if (mbar_try_wait(bar_d, 0)) break;
