@@ -80,7 +80,8 @@ typedef struct {
  * through which the CTAs of one rosaq_linear launch exchange partial output tiles
  * (64 KB per CTA of a two-CTAs-per-SM grid, 19 MB on a 148-SM device, plus 4 KB of
  * counters) and, lazily at the first call that needs it, a workspace for the rotated
- * activations.  A context serves one stream at a time: calls on different streams
+ * activations.  A workspace that a later call outgrows stays allocated until the context is destroyed (at most twice
+ * the largest one in all), so that launches captured before keep working.  A context serves one stream at a time: calls on different streams
  * that overlap in time need a context each.  Synchronous. */
 int rosaq_create(rosaq_ctx **out, int device);
 int rosaq_destroy(rosaq_ctx *ctx);
@@ -219,7 +220,7 @@ int rosaq_rotate(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
  * (code - zero) * scale rounded to fp16; fp32 accumulation; y rounded once to fp16.
  *   r == NULL : x is already rotated (only the GEMM stage runs)
  *   r != NULL : x . R goes through the context workspace (grown on demand: this call
- *               may then allocate and synchronize once), then the GEMM stage runs
+ *               may then allocate once), then the GEMM stage runs
  * Only the first d_out columns of each y row are written.  ldx, ldy multiples of 8.
  * Any M >= 1.  The kernel is chosen by size: up to 128 tokens the weight-streaming kernels; larger batches run, where an
  * estimate says that it pays, on tiles of 256 columns x up to 256 tokens shared by two CTAs on adjacent SMs

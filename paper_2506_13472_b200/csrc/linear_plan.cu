@@ -1019,21 +1019,8 @@ int plan_prepare(rosaq_ctx *ctx, int M, int n, const PlanOp *ops, PlanLaunch *ou
   const int MTL = MT / tile_div;                       // token rows a CTA keeps in shared memory
   const int slot_floats = MT * kTileN;
   const size_t need = (size_t)tile_div * std::max(s->n_slots, 1) * slot_floats * sizeof(float);
-  if (ctx->pl_partial_bytes < need) {
-    // the old buffer may still be in use by work queued on some stream
-    if (cudaDeviceSynchronize() != cudaSuccess) {
-      (void)cudaGetLastError();
-      return ROSAQ_ERR_CUDA;
-    }
-    if (ctx->pl_partials) (void)cudaFree(ctx->pl_partials);
-    ctx->pl_partials = nullptr;
-    ctx->pl_partial_bytes = 0;
-    if (cudaMalloc(reinterpret_cast<void **>(&ctx->pl_partials), need) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return ROSAQ_ERR_ALLOC;
-    }
-    ctx->pl_partial_bytes = need;
-  }
+  st = grow_workspace(ctx, reinterpret_cast<void **>(&ctx->pl_partials), &ctx->pl_partial_bytes, need);
+  if (st != ROSAQ_OK) return st;
   PlParams *q = new (std::nothrow) PlParams();
   if (!q) return ROSAQ_ERR_ALLOC;
   for (int i = 0; i < n; ++i) {

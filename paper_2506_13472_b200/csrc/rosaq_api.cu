@@ -104,20 +104,8 @@ int check_quant_args(int d_in, int d_out, int bits, int group, int k_salient) {
   return ROSAQ_OK;
 }
 
-int ensure_workspace(rosaq_ctx *ctx, size_t bytes, cudaStream_t s) {
-  if (ctx->ws_bytes >= bytes) return ROSAQ_OK;
-  // the old buffer may still be in use by work queued on some stream
-  int st = cuda_status(cudaDeviceSynchronize());
-  if (st != ROSAQ_OK) return st;
-  (void)s;
-  if (ctx->ws) (void)cudaFree(ctx->ws);
-  ctx->ws = nullptr;
-  ctx->ws_bytes = 0;
-  size_t want = bytes < (size_t)(4 << 20) ? (size_t)(4 << 20) : bytes;
-  st = cuda_status(cudaMalloc(&ctx->ws, want));
-  if (st != ROSAQ_OK) return st;
-  ctx->ws_bytes = want;
-  return ROSAQ_OK;
+int ensure_workspace(rosaq_ctx *ctx, size_t bytes) {
+  return grow_workspace(ctx, &ctx->ws, &ctx->ws_bytes, std::max(bytes, (size_t)(4 << 20)));
 }
 
 constexpr int kBlockTokens = 128;
@@ -237,6 +225,7 @@ int rosaq_create(rosaq_ctx **out, int device) {
   ctx->sm_count = prop.multiProcessorCount;
   ctx->ws = nullptr;
   ctx->ws_bytes = 0;
+  ctx->n_retired = 0;
   ctx->wait_limit = 1ll << 20;
   ctx->impl = 0;
   ctx->sk_partials = nullptr;
@@ -292,6 +281,7 @@ int rosaq_destroy(rosaq_ctx *ctx) {
   if (guard.ok) {
     (void)cudaDeviceSynchronize();
     if (ctx->ws) (void)cudaFree(ctx->ws);
+    for (int i = 0; i < ctx->n_retired; ++i) (void)cudaFree(ctx->retired[i]);
     if (ctx->d_status) (void)cudaFree(ctx->d_status);
     if (ctx->sk_partials) (void)cudaFree(ctx->sk_partials);
     if (ctx->sk_arrive) (void)cudaFree(ctx->sk_arrive);
@@ -579,7 +569,7 @@ int rosaq_linear(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
   const __half *xin = static_cast<const __half *>(x);
   long long ld = ldx;
   if (r) {
-    st = ensure_workspace(ctx, sizeof(__half) * (size_t)M * r->d, s);
+    st = ensure_workspace(ctx, sizeof(__half) * (size_t)M * r->d);
     if (st != ROSAQ_OK) return st;
   }
   if (use_plan(ctx, M, r != nullptr)) {
@@ -622,7 +612,7 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
   const __half *xin = static_cast<const __half *>(x);
   long long ld = ldx;
   if (r) {
-    st = ensure_workspace(ctx, sizeof(__half) * (size_t)M * r->d, s);
+    st = ensure_workspace(ctx, sizeof(__half) * (size_t)M * r->d);
     if (st != ROSAQ_OK) return st;
   }
   if (use_plan(ctx, M, r != nullptr)) {

@@ -249,6 +249,10 @@ struct MemPool {
 };
 }  // namespace rosaq
 
+namespace rosaq {
+constexpr int kMaxRetired = 96;
+}
+
 struct rosaq_ctx {
   int device;
   int sm_count;
@@ -256,6 +260,8 @@ struct rosaq_ctx {
   void *ws;            // rotated-activation workspace
   size_t ws_bytes;
   rosaq::MemPool *pool;   // memory of the weights and rotations
+  void *retired[rosaq::kMaxRetired];   // workspaces that were outgrown: captured launches may still use them
+  int n_retired;
   long long wait_limit;
   int impl;            // 0 tensor-core, 1 CUDA-core, 2 tensor-core with CTA pairs, 3 tensor-core without stream-K,
                        // 4 persistent launch for every call, 5 prefill tiles for every weight
@@ -326,6 +332,30 @@ inline int operand_reach(const rosaq_ctx *ctx, int device, MemPool *pool) {
     return ROSAQ_ERR_CUDA;
   }
   pool->open_to.fetch_or(bit);
+  return ROSAQ_OK;
+}
+
+// Makes a workspace of the context at least `need` bytes large.  The one that it replaces stays allocated as long as the context:
+// launches in flight use it, and so does every later replay of a captured one.  (Growing by half at least bounds what is kept
+// to twice the present size.)
+inline int grow_workspace(rosaq_ctx *ctx, void **ws, size_t *bytes, size_t need) {
+  if (*bytes >= need) return ROSAQ_OK;
+  if (ctx->n_retired == kMaxRetired) return ROSAQ_ERR_ALLOC;
+  size_t want = need > *bytes + *bytes / 2 ? need : *bytes + *bytes / 2;
+  void *p = nullptr;
+  cudaError_t e = cudaMalloc(&p, want);
+  if (e == cudaErrorMemoryAllocation && want > need) {
+    (void)cudaGetLastError();
+    want = need;
+    e = cudaMalloc(&p, want);
+  }
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? ROSAQ_ERR_ALLOC : ROSAQ_ERR_CUDA;
+  }
+  if (*ws) ctx->retired[ctx->n_retired++] = *ws;
+  *ws = p;
+  *bytes = want;
   return ROSAQ_OK;
 }
 

@@ -73,3 +73,43 @@ def test_free_waits_for_launches_that_read_the_operand(ctx):
         torch.cuda.synchronize()
         assert all(torch.equal(y, want[k % 2]) for y in ys)
     assert ctx.last_status() == rb.ROSAQ_OK
+
+
+def test_captured_launches_outlive_the_workspace_they_used(ctx):
+    """A workspace grows when a later call or plan needs more.  Launches captured before -- a linear whose rotated activations
+    lie in it, pair tiles and a plan whose partial tiles do -- replay on the one they were captured with."""
+    d = 1024
+    rot = ctx.rotation_create((torch.randn((d, d), device="cuda") / d ** 0.5).half())
+    w, wide = weight(ctx, "ws", d, d), weight(ctx, "wsw", d, 11008)
+    x, xp = torch.randn((64, d), device="cuda").half(), torch.randn((520, d), device="cuda").half()
+    y, yp, xr, yl = (torch.empty(s, dtype=torch.float16, device="cuda") for s in ((64, d), (520, 11008), (64, d), (64, d)))
+    plan = ctx.plan_create(64, [(x, None, rot, xr), (None, 0, w, yl)])
+
+    def launches():
+        ctx.linear(x, w, rot, out=y)
+        ctx.linear(xp, wide, out=yp)
+        plan.run()
+
+    launches()
+    want = [t.clone() for t in (y, yp, yl)]
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side):
+        launches()
+    big = torch.randn((6000, d), device="cuda").half()
+    for m in (2100, 3000, 6000):                                     # 4.3, 6.1, 12.3 MB of rotated activations
+        ctx.linear(big[:m], w, rot)
+    # twelve operations one after the other, each with partial tiles in every CTA: more of them than the context starts with
+    # (768 of 64 KB on 148 SMs)
+    xl = torch.randn((128, d), device="cuda").half()
+    outs = [torch.empty((128, d), dtype=torch.float16, device="cuda") for _ in range(12)]
+    ctx.plan_create(128, [(xl if k == 0 else None, None if k == 0 else k - 1, w, o) for k, o in enumerate(outs)]).run()
+    filler = [torch.full((1 << 22,), float("nan"), device="cuda") for _ in range(8)]
+    for _ in range(2):
+        for t in (y, yp, yl):
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip((y, yp, yl), want))
+    assert ctx.last_status() == rb.ROSAQ_OK
+    del filler
