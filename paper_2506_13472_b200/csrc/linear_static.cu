@@ -43,12 +43,6 @@ int scratch_for_device(int device, void **out) {
   return ROSAQ_OK;
 }
 
-int run_stage(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, const rosaq::TiledOperand &t,
-              const int32_t *col_map, __half *y, long long ldy, cudaStream_t s) {
-  if (ctx->impl == 1) return rosaq::launch_linear_simt(ctx, x, M, ldx, t, col_map, y, ldy, s);
-  return rosaq::launch_linear_tc(ctx, x, M, ldx, t, col_map, y, ldy, s);
-}
-
 }  // namespace
 
 extern "C" int rosaq_linear_static(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_rotation *r,
@@ -72,10 +66,10 @@ extern "C" int rosaq_linear_static(rosaq_ctx *ctx, const void *x, int M, int64_t
     if (st != ROSAQ_OK) return st;
     // every element of the [M][d] intermediate is written by the rotation before the GEMM stage reads
     // it (rows past M are zero-filled by the activation copy itself), so nothing has to be cleared
-    st = run_stage(ctx, xin, M, ldx, r->t, r->col_map, static_cast<__half *>(scratch), r->d, s);
+    st = rosaq::run_stage(ctx, xin, M, ldx, r->t, r->col_map, static_cast<__half *>(scratch), r->d, s);
     if (st != ROSAQ_OK) return st;
     xin = static_cast<const __half *>(scratch);
     ld = r->d;
   }
-  return run_stage(ctx, xin, M, ld, w->t, nullptr, static_cast<__half *>(y), ldy, s);
+  return rosaq::run_stage(ctx, xin, M, ld, w->t, nullptr, static_cast<__half *>(y), ldy, s);
 }

@@ -943,14 +943,6 @@ static int launch_linear_sk(const rosaq_ctx *ctx, const __half *x, long long ldx
   return ROSAQ_OK;
 }
 
-int launch_linear_tc(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t,
-                     const int32_t *col_map, __half *y, long long ldy, cudaStream_t s) {
-  const TiledOperand *ts[1] = {&t};
-  __half *ys[1] = {y};
-  long long ldys[1] = {ldy};
-  return launch_linear_tc_multi(ctx, x, M, ldx, 1, ts, col_map, ys, ldys, s);
-}
-
 // n weights of identical geometry applied to the same activations in one launch
 int launch_linear_tc_multi(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n,
                            const TiledOperand *const *ts, const int32_t *col_map, __half *const *ys,

@@ -136,8 +136,6 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
     return st;
   }
   if (ctx->impl == 0 && linear_small_supported(ctx, M, n, ts)) return launch_linear_small(ctx, x, M, ldx, n, ts, col_map, ys, ldys, s);
-  if (ctx->impl == 6 && n == 1 && M > 64 && M <= kBlockTokens * kPlanMaxOps)
-    return run_token_blocks(ctx, x, M, ldx, *ts[0], col_map, ys[0], ldys[0], s);
   // A permuted output (head-wise rotation) is a scatter of 2-byte elements; in column order and then moved inside each row
   // it is faster, the second launch included, once there are enough of them.  us, scattered / moved: d = 512 at 40 tokens 4.9 / 5.2,
   // at 56 5.7 / 5.5; 1024 at 24 4.6 / 4.9, at 36 5.5 / 5.25; 2048 at 20 5.0 / 5.15, at 24 5.2 / 5.1; 5120 at 17 5.7 / 6.15, at 24 6.3 / 6.0, at
@@ -160,11 +158,6 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
   return launch_linear_tc_multi(ctx, x, M, ldx, n, ts, col_map, ys, ldys, s);
 }
 
-int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t, const int32_t *col_map,
-             __half *y, long long ldy, cudaStream_t s) {
-  const TiledOperand *ts[1] = {&t};
-  return run_gemm(ctx, x, M, ldx, 1, ts, col_map, &y, &ldy, s);
-}
 
 // The persistent launch (rosaq_plan) pays off when a list is long: it saves a launch, a pipeline fill and a
 // drain per operation, but a list of one or two operations exposes its own fixed costs (the exchange of
@@ -187,6 +180,21 @@ int run_ops(rosaq_ctx *ctx, int M, int n, const PlanOp *ops, cudaStream_t s) {
 }
 
 }  // namespace
+
+namespace rosaq {
+int run_stage(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t, const int32_t *col_map,
+              __half *y, long long ldy, cudaStream_t s) {
+  const TiledOperand *ts[1] = {&t};
+  return run_gemm(ctx, x, M, ldx, 1, ts, col_map, &y, &ldy, s);
+}
+}  // namespace rosaq
+
+// the same for the calls that may allocate: implementation 6 plans a launch
+static int run_call(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t, const int32_t *col_map,
+                    __half *y, long long ldy, cudaStream_t s) {
+  if (ctx->impl == 6 && M > 64 && M <= kBlockTokens * kPlanMaxOps) return run_token_blocks(ctx, x, M, ldx, t, col_map, y, ldy, s);
+  return run_stage(ctx, x, M, ldx, t, col_map, y, ldy, s);
+}
 
 extern "C" {
 
@@ -549,7 +557,7 @@ int rosaq_rotate(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
     const PlanOp op{static_cast<const __half *>(x), ldx, -1, &r->t, r->col_map, static_cast<__half *>(x_rot), ldxr};
     return run_ops(ctx, M, 1, &op, static_cast<cudaStream_t>(stream));
   }
-  return run_gemm(ctx, static_cast<const __half *>(x), M, ldx, r->t, r->col_map, static_cast<__half *>(x_rot), ldxr,
+  return run_call(ctx, static_cast<const __half *>(x), M, ldx, r->t, r->col_map, static_cast<__half *>(x_rot), ldxr,
                   static_cast<cudaStream_t>(stream));
 }
 
@@ -581,12 +589,12 @@ int rosaq_linear(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
     return run_ops(ctx, M, n + 1, ops, s);
   }
   if (r) {
-    st = run_gemm(ctx, xin, M, ldx, r->t, r->col_map, static_cast<__half *>(ctx->ws), r->d, s);
+    st = run_call(ctx, xin, M, ldx, r->t, r->col_map, static_cast<__half *>(ctx->ws), r->d, s);
     if (st != ROSAQ_OK) return st;
     xin = static_cast<const __half *>(ctx->ws);
     ld = r->d;
   }
-  return run_gemm(ctx, xin, M, ld, w->t, nullptr, static_cast<__half *>(y), ldy, s);
+  return run_call(ctx, xin, M, ld, w->t, nullptr, static_cast<__half *>(y), ldy, s);
 }
 
 int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_rotation *r, int n,
@@ -623,7 +631,7 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
     return run_ops(ctx, M, k, ops, s);
   }
   if (r) {
-    st = run_gemm(ctx, xin, M, ldx, r->t, r->col_map, static_cast<__half *>(ctx->ws), r->d, s);
+    st = run_call(ctx, xin, M, ldx, r->t, r->col_map, static_cast<__half *>(ctx->ws), r->d, s);
     if (st != ROSAQ_OK) return st;
     xin = static_cast<const __half *>(ctx->ws);
     ld = r->d;
@@ -632,6 +640,7 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
   __half *ys[4];
   long long ldys[4];
   for (int i = 0; i < n; ++i) ts[i] = &w[i]->t, ys[i] = static_cast<__half *>(y[i]), ldys[i] = ldy[i];
+  if (n == 1) return run_call(ctx, xin, M, ld, *ts[0], nullptr, ys[0], ldys[0], s);
   return run_gemm(ctx, xin, M, ld, n, ts, nullptr, ys, ldys, s);
 }
 

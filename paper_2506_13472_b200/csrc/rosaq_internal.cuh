@@ -375,10 +375,11 @@ int launch_cov_fma(int sm_count, const void *X, int x_dtype, long long n_tokens,
                    cudaStream_t s);
 int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tokens, int d, long long ldx,
                int n_blocks, float *C, cudaStream_t s);
+// one rotation or GEMM stage on the kernel that its size asks for (rosaq_api.cu); allocates nothing
+int run_stage(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t, const int32_t *col_map, __half *y,
+              long long ldy, cudaStream_t s);
 int launch_linear_simt(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t,
                        const int32_t *col_map, __half *y, long long ldy, cudaStream_t s);
-int launch_linear_tc(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &t,
-                     const int32_t *col_map, __half *y, long long ldy, cudaStream_t s);
 int launch_linear_tc_multi(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n,
                            const TiledOperand *const *ts, const int32_t *col_map, __half *const *ys,
                            const long long *ldys, cudaStream_t s);

@@ -77,3 +77,18 @@ def test_static_variant_rejects_what_does_not_fit_its_array():
         assert ctx.last_status() == rb.ROSAQ_OK
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("M", [1, 5, 17, 64, 150, 300])
+def test_static_variant_gives_the_bits_of_rosaq_linear(M):
+    """The same kernels, whatever the token count picks."""
+    ctx = rb.Context(0)
+    try:
+        c = H.config_headwise()
+        w = ctx.quantize(dev(c["W"]), dev(c["Rb32"]), dev(c["perm"]), bits=4, k_salient=128)
+        rot = ctx.rotation_create(dev(c["Rb16"]), dev(c["perm"]))
+        x = dev(synth.HeadwiseActivationLaw(c["heads"], c["head_dim"], 3, "hw").sample(M, "static-d", np.float16))
+        assert torch.equal(ctx.linear_static(x, w, rot).view(torch.int16), ctx.linear(x, w, rot).view(torch.int16))
+        assert ctx.last_status() == rb.ROSAQ_OK
+    finally:
+        ctx.close()
