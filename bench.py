@@ -752,7 +752,7 @@ def run_ours(args):
         e1.record()
         torch.cuda.synchronize()
         ms_k = max_over_ranks(e0.elapsed_time(e1)) / args.steps
-        # ... and, because K steps of 66 us are over before a clock sample is taken, the same replay for at
+        # ... and, because K steps of 60 us are over before a clock sample is taken, the same replay for at
         # least a second in five segments: the median segment is the reported figure
         ms_per_step, steps_timed, ms_total = time_replays(graph, n_layers)
     ms_per_step = max_over_ranks(ms_per_step)

@@ -250,8 +250,8 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
  * (Eq. 2; Eq. 6 for block-diagonal R) and every GEMM stage x' . W^ (Eq. 3) of, say, a decoder layer.
  * All CTAs of the grid stream the operands of the whole list back to back; an operation whose input is
  * another operation's output starts when that output is complete.  It pays off for long lists (the ten
- * operations of a 7B decoder layer: 66 us against 100 us as seven calls); for one or two operations the
- * single calls are faster (rotation + 4096 -> 4096 linear: 30 us as a plan, 21 us as rosaq_linear).
+ * operations of a 7B decoder layer: 51 us in a burst, 60 us under the power cap, against 84 us as seven calls); for one or
+ * two operations the single calls are faster (rotation + 4096 -> 4096 linear: 26.5 us as a plan, 18.5 us as rosaq_linear).
  *   op.r / op.w  exactly one is non-NULL: the operation is y = x . R, or y = x . W^ (x already rotated)
  *   op.x, ldx    DEVICE [M][ldx] fp16 input; ignored when x_from >= 0
  *   op.x_from    -1, or the index (smaller than this operation's) of the operation whose y is this one's
@@ -262,8 +262,8 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
  * included), is rejected with ROSAQ_ERR_INVALID_ARG (column ranges of one wider buffer with the same row
  * stride do not overlap; views with different row strides must not share any address range).  All quantized weights of a list
  * have the same bit width.  1 <= M <= 128 and 1 <= n_ops <= 12, otherwise ROSAQ_ERR_UNSUPPORTED_SHAPE.
- * From 65 tokens on the launch keeps accumulators of 128 tokens (a 7B decoder layer: 97 us at 128 tokens,
- * 65 us at 64).
+ * From 65 tokens on the launch keeps accumulators of 128 tokens (a 7B decoder layer under the power cap: 85 us at 128
+ * tokens, 60 us at 64).
  * Each y is the sum rosaq_linear computes, added in an order that depends on how the list is divided
  * among the CTAs: results agree with the separate calls to fp32 summation order (a few 1e-5 relative) and
  * are the same bits on every run of the same plan.
@@ -324,7 +324,7 @@ int rosaq_plan_schedule(int n_ops, const int32_t *n_tiles, const int32_t *groups
                         int32_t *pieces, int max_pieces);
 
 /*
- * Same result as rosaq_linear, for callers that cannot allocate device memory.  (The paper has
+ * Same result as rosaq_linear, bit for bit (implementations 4 and 6 apart), for callers that cannot allocate device memory.  (The paper has
  * no counterpart; this entry point exists for deployment reasons only.)
  *
  * rosaq_linear keeps the rotated activations x . R in a context workspace that it grows with

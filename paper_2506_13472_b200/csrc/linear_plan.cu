@@ -37,6 +37,7 @@
 //   * and one converged warp that issues the MMAs (14 ... 33 cycles each), one accumulator per piece:              53.3 / 45.5
 //   * the counters of a problem's input polled by a warp of its own, ahead of the activation copies (52.4 / 44.3), and the
 //     launch chained to the one before it (its set-up and first weight copies under that one's tail):               52.5 / 43.9
+//   * the pieces of a CTA in shared memory:                                                                       51.4 / 42.8
 // Six operand buffers instead of four: 53.3 / 46.6 (the room comes off the weight ring).
 // Warp 0 = weight-tile producers (bulk copies, L2 evict-first; one sub-ring of slots and one lane per team), 1 =
 // activation producer (TMA), 2 = MMA issuer and owner of the tensor memory, 4..19 = four dequantisation teams (group j goes

@@ -3,9 +3,8 @@
 //
 // Why another kernel.  With a few hundred tokens the stage is bound by the tensor pipe, not by the weight
 // stream, and what counts is how many tokens share one dequantisation of a weight tile and how often an
-// operand byte is fetched from L2: a tcgen05.mma of 128 x N x 16 runs at full rate from N = 128 on (64
-// cycles, 128 for N = 256; 55 for N = 64 is 58 %), a weight tile dequantised for 128 tokens costs as many
-// instructions as one dequantised for 256, and a CTA that multiplies 128 columns with 256 tokens on its own
+// operand byte is fetched from L2: a weight tile dequantised for 128 tokens costs as many instructions (317 cycles of an SM)
+// as one dequantised for 256, next to 512 and 1024 cycles of MMAs, and a CTA that multiplies 128 columns with 256 tokens on its own
 // pulls 64 KB of activations per 128-channel group.  Here two CTAs of a cluster (adjacent SMs) share a
 // tile of 256 columns x NT <= 256 tokens as a cta_group::2 pair: rank r dequantises column tile 2 c + r into its own
 // tensor memory (the A operand, 128 lanes each) and loads half of the token rows (its half of the B

@@ -163,8 +163,8 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
 // drain per operation, but a list of one or two operations exposes its own fixed costs (the exchange of
 // shared tiles goes through L2 instead of a cluster's shared memory, and the phase after a rotation starts
 // only when the rotation's last tile is written).  Measured at 64 tokens, 4096 -> 4096 INT4: a GEMM stage
-// alone 15.9 us against 9.7 us on the per-call kernel; rotation + linear 30.5 us against 20.7 us as two
-// launches; the ten operations of a 7B decoder layer 66 us against 100 us as seven launches.  So the single
+// alone 13.6 us against 8.4 us on the per-call kernel; rotation + linear 26.5 us against 18.5 us as two
+// launches; the ten operations of a 7B decoder layer 51 us (60 under the power cap) against 84 us as seven calls.  So the single
 // calls stay on the per-call kernels; implementation 4 routes them through the persistent launch.
 bool use_plan(const rosaq_ctx *ctx, int M, bool with_rotation) {
   (void)with_rotation;

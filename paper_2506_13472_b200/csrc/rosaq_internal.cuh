@@ -178,16 +178,15 @@ constexpr int kPlanMaxCtas = 512;
 constexpr int kPlMaxCounters = 4096;                // column tiles shared between CTAs in one launch
 constexpr int kPlSyncFinished = 0, kPlSyncDone = 4, kPlSyncArrive = 16;   // word offsets in the sync buffer
 constexpr int kPlSyncWords = kPlSyncArrive + kPlMaxCounters;
-// Relative cost of the work items when a phase is cut into equal shares.  Both kinds of group cost the
-// tensor pipe eight MMAs (about 700 cycles in place); an fp16 group also moves 32 KB, which takes an SM's
-// share of the HBM bandwidth about 1400 cycles when every SM streams fp16 tiles, less when some run
-// quantized groups next to it.  Measured on the 7B decoder layer: 12 : 7 (64.7 us per step; 10 : 7 65.4,
-// 14 : 7 64.9, 10 : 5 65.6; 10 : 3 ... 10 : 10 all within 10 %).  Every tile a CTA starts costs a little for switching accumulators; a tile copy whose
-// output is scattered keeps the epilogue warps busy for about as long as seven quantized groups keep
-// the MMA threads.
+// Relative cost of the work items when a phase is cut into equal shares.  Either kind of group costs its dequantisation and eight
+// MMAs; an fp16 group also moves 32 KB, which takes an SM's share of the HBM bandwidth about 1400 cycles when every SM
+// streams fp16 tiles, less when some run quantized groups next to it.  Ten operations of a layer, us at fp16 : quantized = 8 : 7 / 10 : 7 /
+// 12 : 7 / 14 : 7 / 16 : 7: 7B at 64 tokens 58.4 / 58.2 / 57.9 / 57.7 / 57.3, 13B 86.5 / 86.0 / 85.1 / 87.9 / 89.2, 7B at 100 76.3 / 76.2 / 76.0 / 76.4 /
+// 76.6 (12 : 5 and tile costs of 0 and 3 within 2 %).  Every tile a CTA starts costs a little for switching accumulators; a tile copy
+// whose output is scattered keeps the epilogue warps busy for about as long as seven quantized groups keep the others.
 constexpr int kPlanCostFp16 = 12, kPlanCostQuant = 7, kPlanCostTile = 1, kPlanCostScatterTile = 48;
 // Pairs of CTAs: a quantized group costs each SM half the MMAs, but the measured layer step is again
-// shortest near 10 : 7 (76 us; 85 us at 12 : 4, 90 us at 15 : 4) -- a pair is not bound by its bytes either.
+// shortest near 10 : 7 (76 us; 85 us at 12 : 4, 90 us at 15 : 4; 67 us for single CTAs then) -- a pair is not bound by its bytes either.
 constexpr int kPlanPairCostFp16 = 10, kPlanPairCostQuant = 7, kPlanPairCostTile = 1, kPlanPairCostScatterTile = 64;
 
 // One piece of work of a CTA: groups [g_begin, g_end) of column tile `tile` of problem `prob`.
