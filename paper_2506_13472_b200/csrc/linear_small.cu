@@ -13,7 +13,7 @@
 //     W^, B = 16 channels x 8 tokens;
 //   * launches are chained with programmatic stream serialization: the rings of a launch fill under the tail of the one before;
 //     x' and y are touched after griddepcontrol.wait.
-// What bounds it: at 4096 -> 2 x 11008 the issue slots (377 instructions per unit of 2176 bytes, 0.58 issued per cycle and
+// What bounds it: at 4096 -> 2 x 11008 the issue slots (362 instructions per unit of 2176 bytes, 0.57 issued per cycle and
 // scheduler), at the smaller ones the last round of CTAs and the time to start.  Measured in a graph of distinct weights (us,
 // INT4, one token; tcgen05 kernel / this one): 512 -> 512 3.3 / 1.6, 4096 -> 4096 7.7 / 4.4, 4096 -> 3 x 4096 13.9 / 9.2,
 // 4096 -> 2 x 11008 19.9 / 14.3 (3.2 TB/s), 11008 -> 4096 13.1 / 9.2, rotations: dense 4096 9.9 / 6.8 (4.9 TB/s), head-wise
