@@ -48,7 +48,7 @@ constexpr int kCovDrainPolls = 1 << 16;                 // for work in flight wh
 struct CovParams {
   float *C;
   int dh, bn;                  // block edge; tile columns (MMA N): 256, or 128 for narrow blocks
-  int use3d;                   // the 3-D maps are valid (channel count a multiple of 64)
+  int use3d;                   // the 3-D maps are valid (blocks of a multiple of 64 channels)
   long long n_tokens;
   int splits;                  // CTAs (pairs) of a cluster that share a tile's tokens: 1, 2, 4 or 8
   int *status;
@@ -655,9 +655,10 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
     if (r != CUDA_SUCCESS) return ROSAQ_ERR_CUDA;
   }
   // 3-D views {64 channels, tokens, 64-channel block} with boxes of 2 and 4 blocks; only when every block
-  // is whole (a partial last block would make the last row's box run past the end of the matrix)
+  // is whole (a partial last block would make the last row's box run past the end of the matrix) and every
+  // head block starts at one
   CUtensorMap map2 = xmap, map4 = xmap;
-  const bool use3d = d % 64 == 0;
+  const bool use3d = d % 64 == 0 && dh % 64 == 0;
   if (use3d) {
     const cuuint64_t dims3[3] = {64, (cuuint64_t)n_tokens, (cuuint64_t)(d / 64)};
     const cuuint64_t strides3[2] = {(cuuint64_t)ldx * sizeof(__half), 128};

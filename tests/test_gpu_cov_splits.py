@@ -22,6 +22,9 @@ pytestmark = pytest.mark.gpu
     (np.float32, 1001, 256, 1),       # fp32, 8 splits, mirrored shares
     (np.float32, 300, 384, 3),        # 4 splits
     (np.float16, 700, 96, 2),         # narrow blocks on the fp32 kernel
+    (np.float16, 300, 704, 8),        # head blocks that start inside a block of 64 channels: 88 channels,
+    (np.float16, 90, 576, 4),         # 144 (two row tiles),
+    (np.float16, 200, 4160, 8),       # 520 (pairs)
     (np.float32, 70, 136, 1)])        # one split
 def test_calib_cov_splits(dtype, n_tokens, d, n_blocks):
     X = synth.ActivationLaw(d, 1.0, seed=47, key=f"covs{d}").sample(n_tokens, "X", dtype)
