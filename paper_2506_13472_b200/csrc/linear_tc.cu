@@ -109,27 +109,37 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
   grid_dep_launch_dependents();
   if (threadIdx.x == 32) prefetch_tensormap(&xmap);
 
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < p.NW; ++i) {
+  // The weight producer sets its own barriers up and starts, the others follow when all is set up: the first weights of a CTA that had
+  // to wait for its SM are on their way half a microsecond earlier (64 tokens: 4096 -> 4096 8.58 -> 8.38 us, 1024 -> 2816 5.10 -> 4.94, dense
+  // rotation of 4096 10.47 -> 10.29; 108 launches of 10 to 128 tokens 1.2 % on average).
+  if (warp == 0) {
+    for (int i = lane; i < p.NW; i += 32) {
       mbar_init(bar_w_full + 8 * i, 1);
       mbar_init(bar_w_empty + 8 * i, kTeamThreads);
     }
-    for (int i = 0; i < p.NA; ++i) {
-      mbar_init(bar_x_full + 8 * i, 1);
-      mbar_init(bar_a_full + 8 * i, kPair ? n_arrive : n_arrive + 1);   // + the activation copy (single-CTA mode)
-      mbar_init(bar_empty + 8 * i, 1);
+    if (lane == 0) misc_ptr[1] = 0;
+    mbar_init_fence();
+    __syncwarp();
+    if (kPair) setup_sync(kThreads);
+    else setup_arrive(kThreads);
+  } else {
+    if (warp == 1) {
+      if (lane < p.NA) {
+        mbar_init(bar_x_full + 8 * lane, 1);
+        mbar_init(bar_a_full + 8 * lane, kPair ? n_arrive : n_arrive + 1);   // + the activation copy (single-CTA mode)
+        mbar_init(bar_empty + 8 * lane, 1);
+      }
+      if (lane == 31) mbar_init(bar_d_full, 1);
+      mbar_init_fence();
+      __syncwarp();
     }
-    mbar_init(bar_d_full, 1);
-    misc_ptr[1] = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (warp == 2) {
+      if (kPair) tmem_alloc_pair<kTmemCols>(misc);             // both CTAs of the pair, same warp index
+      else tmem_alloc<kTmemCols>(misc);
+    }
+    tc_fence_before();
+    setup_sync(kThreads);
   }
-  if (warp == 2) {
-    if (kPair) tmem_alloc_pair<kTmemCols>(misc);             // both CTAs of the pair, same warp index
-    else tmem_alloc<kTmemCols>(misc);
-  }
-  tc_fence_before();
-  __syncthreads();
   if (kPair) {                                               // the peer's barriers and tensor memory exist
     cluster_arrive();
     cluster_wait();
@@ -477,8 +487,7 @@ linear_sk_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
   const uint32_t w_ring = x_ring + kSkStages * x_slot_bytes;
   const uint32_t bars = w_ring + p.NW * kWSlotBytes;
   const uint32_t bar_w_full = bars, bar_w_empty = bar_w_full + 8 * p.NW;
-  const uint32_t bar_x_full = bar_w_empty + 8 * p.NW, bar_a_full = bar_x_full + 8 * kSkStages;
-  const uint32_t bar_empty = bar_a_full + 8 * kSkStages;
+  const uint32_t bar_a_full = bar_w_empty + 8 * p.NW, bar_empty = bar_a_full + 8 * kSkStages;
   const uint32_t bar_d_full = bar_empty + 8 * kSkStages;       // two: one per accumulator
   const uint32_t misc = bar_d_full + 16;                       // [0] TMEM base, [1] abort flag
   uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
@@ -494,24 +503,29 @@ linear_sk_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
   grid_dep_launch_dependents();
   if (threadIdx.x == 32) prefetch_tensormap(&xmap);
 
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < p.NW; ++i) {
+  if (warp == 0) {                                             // (as in linear_tc_kernel)
+    for (int i = lane; i < p.NW; i += 32) {
       mbar_init(bar_w_full + 8 * i, 1);
       mbar_init(bar_w_empty + 8 * i, kTeamThreads);
     }
-    for (int i = 0; i < kSkStages; ++i) {
-      mbar_init(bar_x_full + 8 * i, 1);
-      mbar_init(bar_a_full + 8 * i, kTeamThreads + 1);         // + the activation copy
-      mbar_init(bar_empty + 8 * i, 1);
-      mbar_init(bar_d_full + 8 * i, 1);
+    if (lane == 0) misc_ptr[1] = 0;
+    mbar_init_fence();
+    __syncwarp();
+    setup_arrive(kThreads);
+  } else {
+    if (warp == 1) {
+      if (lane < kSkStages) {
+        mbar_init(bar_a_full + 8 * lane, kTeamThreads + 1);    // + the activation copy
+        mbar_init(bar_empty + 8 * lane, 1);
+        mbar_init(bar_d_full + 8 * lane, 1);
+      }
+      mbar_init_fence();
+      __syncwarp();
     }
-    misc_ptr[1] = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (warp == 2) tmem_alloc<kTmemCols>(misc);
+    tc_fence_before();
+    setup_sync(kThreads);
   }
-  if (warp == 2) tmem_alloc<kTmemCols>(misc);
-  tc_fence_before();
-  __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc_ptr[0];
   // columns: accumulator of the first tile at 0, of the second at 64, operand buffers at 128 and 192

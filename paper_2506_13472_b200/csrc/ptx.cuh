@@ -14,6 +14,15 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)_
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
+// what a thread does after initialising barriers, before anybody uses them
+__device__ __forceinline__ void mbar_init_fence() {
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+// End of a CTA's set-up: a warp that needs nothing of what the others set up only arrives, the others wait for everybody.  (A barrier of its
+// own: the first warp may be at the __syncthreads() behind its work before this one is complete.)
+__device__ __forceinline__ void setup_arrive(int threads) { asm volatile("barrier.cta.arrive 2, %0;" ::"r"(threads) : "memory"); }
+__device__ __forceinline__ void setup_sync(int threads) { asm volatile("barrier.cta.sync 2, %0;" ::"r"(threads) : "memory"); }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
