@@ -995,7 +995,7 @@ int launch_linear_tc_multi(const rosaq_ctx *ctx, const __half *x, int M, long lo
   p.bits = t.bits;
   p.block_groups = t.block_groups;
   p.M = M;
-  const int m_tiles = (M + 127) / 128;
+  const int m_tiles = ctx->impl != 2 && scatter_tiles(ctx, M, t, col_map) ? (M + kScatterTile - 1) / kScatterTile : (M + 127) / 128;
   const int per_tile = (M + m_tiles - 1) / m_tiles;
   p.MT = ((per_tile + 15) / 16) * 16;
   p.col_map = col_map;

@@ -136,11 +136,12 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
     return st;
   }
   if (ctx->impl == 0 && linear_small_supported(ctx, M, n, ts)) return launch_linear_small(ctx, x, M, ldx, n, ts, col_map, ys, ldys, s);
-  // A permuted output (head-wise rotation) is a scatter of 2-byte elements; in column order and then moved inside each row
-  // it is faster, the second launch included, once there are enough of them.  us, scattered / moved: d = 512 at 40 tokens 4.9 / 5.2,
-  // at 56 5.7 / 5.5; 1024 at 24 4.6 / 4.9, at 36 5.5 / 5.25; 2048 at 20 5.0 / 5.15, at 24 5.2 / 5.1; 5120 at 17 5.7 / 6.15, at 24 6.3 / 6.0, at
-  // 64 11.2 / 7.3, at 512 38.8 / 12.6.
-  if (ctx->impl == 0 && n == 1 && col_map && M > kScatterTokens && (long long)M * ts[0]->d_out > kScatterElements && ts[0]->d_out <= kPermuteMaxColumns) {
+  // A permuted output is scattered while scatter_tiles() spreads it over the SMs; beyond that it is written in column order and then
+  // moved inside each row, which is faster, the second launch included, once there are enough elements.  us, scattered by one CTA
+  // per head / moved: d = 512 at 40 tokens 4.9 / 5.2, at 56 5.7 / 5.5; 2048 at 20 5.0 / 5.15, at 24 5.2 / 5.1; 5120 at 24 6.3 / 6.0, at 64 11.2 / 7.3, at 512
+  // 38.8 / 12.6.
+  if (ctx->impl == 0 && n == 1 && col_map && !scatter_tiles(ctx, M, *ts[0], col_map) && M > kScatterTokens && (long long)M * ts[0]->d_out > kScatterElements &&
+      ts[0]->d_out <= kPermuteMaxColumns) {
     const int st = run_gemm(ctx, x, M, ldx, n, ts, nullptr, ys, ldys, s);
     return st == ROSAQ_OK ? launch_permute_rows(ys[0], M, ldys[0], ts[0]->d_out, col_map, s) : st;
   }

@@ -384,6 +384,16 @@ int launch_linear_tc_multi(const rosaq_ctx *ctx, const __half *x, int M, long lo
                            const long long *ldys, cudaStream_t s);
 double linear_tc_estimate(const rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts);
 constexpr int kPermuteMaxColumns = 24576;            // a row in 48 KB of shared memory
+// A permuted output (head-wise rotation) is a scatter of 2-byte elements, which a CTA issues at one element in two to three cycles
+// whatever its share of the batch: with one or two groups per tile (little else to do) the batch is cut into tiles of sixteen tokens
+// while the SMs have one of them each, two if the heads are few.  us, this / written in column order and then moved (permute_rows_kernel):
+// 512 channels at 64 tokens 3.5 / 5.0, at 512 5.3 / 7.8; 1024 at 128 4.6 / 7.0, at 512 6.1 / 8.2; 2048 at 32 4.2 / 4.7, at 128 6.1 / 6.9; 4096 at 64 6.4 / 6.8;
+// past the line: 1024 at 640 9.9 / 7.2, 1536 at 320 7.1 / 6.7, 4096 at 96 7.0 / 6.7, 5120 at 64 7.1 / 6.9, at 128 11.9 / 8.2.
+constexpr int kScatterTile = 16;
+inline bool scatter_tiles(const rosaq_ctx *ctx, int M, const TiledOperand &t, const int32_t *col_map) {
+  const bool few = t.n_tiles <= 8;
+  return col_map && groups_per_tile(t) <= 2 && (few || M <= 128) && (long long)t.n_tiles * ((M + kScatterTile - 1) / kScatterTile) <= (few ? 2 : 1) * ctx->sm_count;
+}
 int launch_permute_rows(__half *y, int M, long long ldy, int d, const int32_t *col_map, cudaStream_t s);
 
 constexpr int kSmallTokens = 8;                      // most tokens of launch_linear_small

@@ -136,3 +136,23 @@ def test_column_order_scattered_or_moved(ctx, d):
         ctx.set_linear_impl(0)
         assert same(ctx.rotate(x, rot), ref), M
     assert ctx.last_status() == rb.ROSAQ_OK
+
+
+@pytest.mark.parametrize("d,M", [(512, 9), (512, 33), (512, 1184), (512, 1185), (1152, 128), (1152, 129), (4096, 64), (4096, 65), (5120, 48), (128, 40)])
+def test_column_order_in_tiles_of_sixteen_tokens(ctx, d, M):
+    """Up to one CTA per SM (of sixteen tokens and one head; two per SM where the heads are few) and behind it, ragged last tiles: the columns
+    of the rotation without an order, moved; the rows behind the batch and the columns behind the last one stay untouched."""
+    rng = synth.rng_for(95, "tiles", d, M)
+    q = dev((rng.standard_normal((d // 128, 128, 128)) / 128 ** 0.5).astype(np.float16))
+    perm = rng.permutation(d).astype(np.int32)
+    x = dev(rng.standard_normal((M, d)).astype(np.float16))
+    ctx.set_linear_impl(3)
+    want = ctx.rotate(x, ctx.rotation_create(q))[:, torch.from_numpy(perm).cuda().long()]
+    ctx.set_linear_impl(0)
+    buf = torch.full((M + 1, d + 8), 7.0, dtype=torch.float16, device="cuda")
+    rot = ctx.rotation_create(q, dev(perm))
+    for _ in range(2):
+        ctx.rotate(x, rot, out=buf[:M, :d])
+    assert same(buf[:M, :d].contiguous(), want.contiguous())
+    assert torch.all(buf[M:] == 7.0) and torch.all(buf[:, d:] == 7.0)
+    assert ctx.last_status() == rb.ROSAQ_OK
