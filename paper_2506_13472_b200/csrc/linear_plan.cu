@@ -14,19 +14,20 @@
 //     column tile that a CTA holds), so the MMA warp starts the next piece while four epilogue warps
 //     drain the previous one;
 //   * a column tile whose groups are spread over several CTAs is summed through a workspace in L2: every
-//     holder stores its fp32 partial tile and counts itself in; the holders for which this tile is the
-//     last piece of their range ("closers") wait for the count, then each adds the partial tiles of a
-//     share of the token rows, in ascending K order whatever the timing, and writes those rows of y.
+//     holder stores its fp32 partial tile; the holders for which this tile is the
+//     last piece of their range ("closers") each add the partial tiles of a
+//     share of the token rows, in ascending K order whatever the timing, and write those rows of y.
 //     Closers come to the tile at the end of their range, the other holders at the beginning of theirs,
-//     so nobody waits long;
+//     so nobody waits long.  The values announce themselves: an empty slot holds kEmpty, a pattern no partial sum has, and the
+//     reader polls the values until they are others, then empties the slot again (store, fence, count, poll, load took four
+//     trips to L2 where this takes one and a half);
 //   * a problem that reads another problem's output waits (activation producer only) until every tile of
 //     that output has been written, counted in a per-problem counter.
 // The launch is cooperative (one CTA per SM), so the whole grid is resident and every wait is on work
 // that some resident CTA performs without waiting for anything later in the list.
 // Every wait is bounded: when a limit expires the CTA records ROSAQ_ERR_TIMEOUT in the context's status
 // word, stops issuing work, lets its copies and MMAs in flight finish, frees its tensor memory and
-// returns.  The last CTA to leave clears the counters, so the next launch starts from zero whatever
-// happened.
+// returns.  A launch finds its counters at zero and its slots empty whatever happened before (sync_set, and the wipe in the epilogue).
 //
 // One CTA owns an SM.  Per 128-channel group at 64 tokens the tensor pipe needs 8 x 33 cycles, the group's bytes 375 at the HBM
 // rate, the four schedulers about 430 (1700 warp instructions); what paced a CTA before were its single-lane roles.  Measured
@@ -38,6 +39,8 @@
 //   * the counters of a problem's input polled by a warp of its own, ahead of the activation copies (52.4 / 44.3), and the
 //     launch chained to the one before it (its set-up and first weight copies under that one's tail):               52.5 / 43.9
 //   * the pieces of a CTA in shared memory:                                                                       51.4 / 42.8
+//   * partial tiles that announce themselves, counters that need no clearing (1024 channels at 20 tokens 23.8 -> 14.6):      51.4 / 39.3
+// Under the power cap (64 tokens and more in a loop) a launch takes what its energy takes: 58 us, with and without the last step.
 // Six operand buffers instead of four: 53.3 / 46.6 (the room comes off the weight ring).
 // Warp 0 = weight-tile producers (bulk copies, L2 evict-first; one sub-ring of slots and one lane per team), 1 =
 // activation producer (TMA), 2 = MMA issuer and owner of the tensor memory, 4..19 = four dequantisation teams (group j goes
@@ -84,13 +87,19 @@ struct alignas(64) PlParams {
   const PlanSeg *segs;
   const int *seg_begin;       // [CTAs + 1]
   float *partials;            // [slot][token][128 columns]
-  unsigned *sync;             // kPlSyncFinished, kPlSyncDone + problem, kPlSyncArrive + counter
+  unsigned *sync;             // kPlSyncFinished, then two sets of kPlSyncSet words: done counters, wiped counter
   int *status;
   long long wait_limit;
-  int n_counters, M, MT, NW, slot_floats;
+  int M, MT, NW, slot_floats;
 };
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// epi_bar with a verdict that all 256 threads share: they leave together or stay together for the barriers behind it
+__device__ __forceinline__ bool epi_all(bool v) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred p, 1, 256, q;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "r"((uint32_t)v) : "memory");
+  return r != 0;
+}
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *ptr) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
@@ -146,15 +155,61 @@ __device__ __forceinline__ bool wait_flag(const Abort &ab, uint32_t addr, int ta
   return false;
 }
 
+// The counters of a launch: launches take the two sets in turn (all CTAs together add kPlanMaxCtas to the finished count as they leave,
+// so it tells them apart while one is running), and clear the other one, which nobody uses then.  Nothing is left to be cleared at the
+// end, where a CTA would wait for its count among the others: 1 us per launch.  Behind griddepcontrol.wait only.
+__device__ __forceinline__ unsigned *sync_set(unsigned *sync) {
+  return sync + kPlSyncSets + (ld_acquire_u32(sync + kPlSyncFinished) / (unsigned)kPlanMaxCtas & 1u) * kPlSyncSet;
+}
+__device__ __forceinline__ unsigned *other_set(unsigned *sync, unsigned *set) { return set == sync + kPlSyncSets ? set + kPlSyncSet : set - kPlSyncSet; }
+
 template <int CH>
 __device__ __forceinline__ void tmem_ld_chunk(uint32_t taddr, uint32_t *v) {
   if (CH == 16) tmem_ld16(taddr, v);
   else tmem_ld8(taddr, v);
 }
 
-// Finishes tokens [c_begin, c_end) of one output column from the accumulator in tensor memory: adds, when
-// `keep`, the partial tiles 1 .. S-1 of the workspace in that order (this CTA's groups come first), rounds
-// once and writes the rows inside [t0, t1).  CH loads from the workspace are in flight per thread.
+// ---- partial tiles in the workspace: [token / 4][128 columns][4 tokens] fp32, kEmpty where nothing has been stored since the last reader.
+// Only the quads of tokens that the tile's piece writes are stored and read.
+constexpr int kQuadFloats = 4 * kTileN;
+__device__ __forceinline__ void st_quad(float *p, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ uint32_t not_empty(uint32_t v) { return min(v, kEmpty - 1); }   // (a NaN stays one)
+// N quads of this thread, null pointers read as zeros, by a converged warp: polled until all of them have arrived, then emptied for the
+// next launch.  False: gave up.
+template <int N>
+__device__ __forceinline__ bool take_quads(const Abort &ab, float *const (&src)[N], float (&v)[N][4]) {
+  for (long long it = 0;; ++it) {
+    uint32_t top = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      uint32_t w[4] = {0, 0, 0, 0};
+      if (src[k])
+        asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(src[k]) : "memory");
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[k][e] = __uint_as_float(w[e]);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) top = max(top, __float_as_uint(v[k][e]));
+    if (__all_sync(0xffffffffu, top != kEmpty)) break;         // (kEmpty is the largest pattern)
+    if (it >= ab.limit) {
+      if ((threadIdx.x & 31) == 0) ab.raise();
+      __syncwarp();
+      return false;
+    }
+    if ((it & 15) == 15 && ab.set_all()) return false;
+    __nanosleep(32);
+  }
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+    if (src[k]) st_quad(src[k], kEmpty, kEmpty, kEmpty, kEmpty);
+  return true;
+}
+
 // Tokens [c0, c0 + CH) of one column of the accumulator.
 template <int CH>
 __device__ __forceinline__ void epi_load_acc(uint32_t d_addr, int c0, float *acc) {
@@ -165,38 +220,33 @@ __device__ __forceinline__ void epi_load_acc(uint32_t d_addr, int c0, float *acc
   for (int e = 0; e < CH; ++e) acc[e] = __uint_as_float(v[e]);
 }
 
+// Finishes tokens [c_begin, c_end) of one output column from the accumulator in tensor memory: adds, when
+// `keep`, the partial tiles 1 .. S-1 of the workspace in that order (this CTA's groups come first), rounds
+// once and writes the rows inside [t0, t1).  Two holders' quads of CH tokens are in flight per thread.  False: gave up.
 template <int CH>
-__device__ __forceinline__ void epi_finish(uint32_t d_addr, int c_begin, int c_end, bool keep, int S, const float *src0,
-                                           long long slot_floats, int M, bool n_ok, int t0, int t1, __half *y_col,
-                                           long long ldy) {
+__device__ __forceinline__ bool epi_finish(const Abort &ab, uint32_t d_addr, int c_begin, int c_end, bool keep, int S, float *src0,
+                                           long long slot_floats, bool n_ok, int t0, int t1, __half *y_col, long long ldy) {
   for (int c0 = c_begin; c0 < c_end; c0 += CH) {
     if (c0 >= t1 || c0 + CH <= t0) continue;
     float acc[CH];
     epi_load_acc<CH>(d_addr, c0, acc);
     if (keep) {
-      // two holders' tiles per round trip to L2 (a round trip costs 1.4 us and more while the weight stream
-      // runs, and the readers of this tile wait for it), added in holder order
       for (int i = 1; i < S; i += 2) {
-        const float *src = src0 + (long long)i * slot_floats + c0 * kTileN;
-        const bool two = i + 1 < S;
-        const float *src2 = two ? src + slot_floats : src;
-        float w[CH], w2[CH];
-        if (c0 + CH <= M) {
+        float *src[CH / 2];
+        float w[CH / 2][4];
 #pragma unroll
-          for (int e = 0; e < CH; ++e) w[e] = __ldcg(src + e * kTileN);
-#pragma unroll
-          for (int e = 0; e < CH; ++e) w2[e] = __ldcg(src2 + e * kTileN);
-        } else {
-#pragma unroll
-          for (int e = 0; e < CH; ++e) w[e] = c0 + e < M ? __ldcg(src + e * kTileN) : 0.f;
-#pragma unroll
-          for (int e = 0; e < CH; ++e) w2[e] = c0 + e < M ? __ldcg(src2 + e * kTileN) : 0.f;
+        for (int k = 0; k < CH / 4; ++k) {
+          const bool mine = c0 + 4 * k < t1 && c0 + 4 * k + 4 > t0;
+          float *at = src0 + (long long)i * slot_floats + (c0 / 4 + k) * kQuadFloats;
+          src[k] = mine ? at : nullptr;
+          src[CH / 4 + k] = mine && i + 1 < S ? at + slot_floats : nullptr;
         }
+        if (!take_quads(ab, src, w)) return false;
 #pragma unroll
-        for (int e = 0; e < CH; ++e) acc[e] = __fadd_rn(acc[e], w[e]);
-        if (two) {
+        for (int e = 0; e < CH; ++e) acc[e] = __fadd_rn(acc[e], w[e / 4][e % 4]);
+        if (i + 1 < S) {
 #pragma unroll
-          for (int e = 0; e < CH; ++e) acc[e] = __fadd_rn(acc[e], w2[e]);
+          for (int e = 0; e < CH; ++e) acc[e] = __fadd_rn(acc[e], w[CH / 4 + e / 4][e % 4]);
         }
       }
     }
@@ -212,23 +262,21 @@ __device__ __forceinline__ void epi_finish(uint32_t d_addr, int c_begin, int c_e
       }
     }
   }
+  return true;
 }
 
-// Stores tokens [c_begin, c_end) of one column of the accumulator to a partial tile [token][128 columns].
+// Stores the quads of tokens [t0, t1) inside [c_begin, c_end) of one column of the accumulator to a partial tile.
 template <int CH>
-__device__ __forceinline__ void epi_store_partial(uint32_t d_addr, int c_begin, int c_end, int M, float *dst) {
-  for (int c0 = c_begin; c0 < c_end && c0 < M; c0 += CH) {
-    float acc[CH];
-    epi_load_acc<CH>(d_addr, c0, acc);
-    float *dp = dst + c0 * kTileN;
-    if (c0 + CH <= M) {
+__device__ __forceinline__ void epi_store_partial(uint32_t d_addr, int c_begin, int c_end, int t0, int t1, float *dst) {
+  for (int c0 = c_begin; c0 < c_end; c0 += CH) {
+    if (c0 >= t1 || c0 + CH <= t0) continue;
+    uint32_t v[CH];
+    tmem_ld_chunk<CH>(d_addr + c0, v);
+    tc_wait_ld();
 #pragma unroll
-      for (int e = 0; e < CH; ++e) dp[e * kTileN] = acc[e];
-    } else {
-#pragma unroll
-      for (int e = 0; e < CH; ++e)
-        if (c0 + e < M) dp[e * kTileN] = acc[e];
-    }
+    for (int k = 0; k < CH / 4; ++k)
+      if (c0 + 4 * k < t1 && c0 + 4 * k + 4 > t0)
+        st_quad(dst + (c0 / 4 + k) * kQuadFloats, not_empty(v[4 * k]), not_empty(v[4 * k + 1]), not_empty(v[4 * k + 2]), not_empty(v[4 * k + 3]));
   }
 }
 
@@ -260,7 +308,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
   const uint32_t bar_d_full = bar_s_empty + 8 * kPlMaxStages;  // accumulator complete (two accumulators)
   const uint32_t bar_d_empty = bar_d_full + 16;                // accumulator drained
   const uint32_t bar_drain = bar_d_empty + 16;
-  const uint32_t misc = bar_drain + 16;                         // [0] TMEM base, [1] abort flag, [2] last CTA out, [3] dependencies met
+  const uint32_t misc = bar_drain + 16;                         // [0] TMEM base, [1] abort flag, [3] dependencies met
   const uint32_t seg_smem = misc + 16;
   uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
   volatile uint32_t *misc_ptr = reinterpret_cast<volatile uint32_t *>(gen + (misc - base));
@@ -293,7 +341,6 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     }
     mbar_init(bar_drain, 1);
     misc_ptr[1] = 0;
-    misc_ptr[2] = 0;
     misc_ptr[3] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -449,6 +496,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     // the activation producer (a counter in L2 is seen two to four microseconds after it was complete)
     if (lane == 0) {
       grid_dep_wait();
+      const unsigned *done = sync_set(p.sync);
       int last_prob = -1, n_deps = 0;
       for (int si = 0; si < n_segs && !ab.set(); ++si) {
         const int prob = pieces[si].prob;
@@ -456,7 +504,7 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         last_prob = prob;
         const PlProblem &P = p.prob[prob];
         if (P.dep < 0) continue;
-        if (!wait_counter(ab, p.sync + kPlSyncDone + P.dep, P.dep_target, 200)) break;
+        if (!wait_counter(ab, done + P.dep, P.dep_target, 200)) break;
         st_flag(misc + 12, ++n_deps);
       }
     }
@@ -520,13 +568,33 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     const bool wide = (half_tok & 15) == 0;                    // sixteen tokens per batch, else eight
     int nseg = 0;
     grid_dep_wait();
+    unsigned *const done = sync_set(p.sync);
+    if (blockIdx.x == 0 && threadIdx.x - kPlFirstEpiWarp * 32 < (unsigned)kPlSyncSet)   // the set of the launch before: zero for the one behind
+      other_set(p.sync, done)[threadIdx.x - kPlFirstEpiWarp * 32] = 0;
+    if (!epi_all(*reinterpret_cast<volatile const int *>(p.status) == 0)) {
+      // A launch has given up since the status was last read and may have left partial tiles behind: every CTA empties the slots that it
+      // is going to fill, and nobody reads before all have.
+      for (int si = 0; si < n_segs; ++si) {
+        const PlanSeg s = pieces[si];
+        if (s.n_contrib == 1) continue;
+        float *slot = p.partials + ((long long)tile_mul * (s.slot0 + s.contrib_idx) + rank) * p.slot_floats;
+        for (int i = ((int)threadIdx.x - kPlFirstEpiWarp * 32) * 4; i < p.slot_floats; i += kPlEpiThreads * 4) st_quad(slot + i, kEmpty, kEmpty, kEmpty, kEmpty);
+      }
+      epi_bar();
+      if (lead) {
+        __threadfence();
+        atomicAdd(done + kPlSyncWiped, 1u);
+        wait_counter(ab, done + kPlSyncWiped, gridDim.x);
+      }
+      epi_bar();
+    }
     for (int si = 0; si < n_segs; ++si, ++nseg) {
       const PlanSeg s = pieces[si];
       const PlProblem &P = p.prob[s.prob];
       const int buf = nseg & 1;
-      bool have_d = ab.wait(bar_d_full + 8 * buf, (nseg >> 1) & 1);
-      have_d = __all_sync(0xffffffffu, have_d && !ab.set());
-      if (!have_d) break;
+      const bool have_d = ab.wait(bar_d_full + 8 * buf, (nseg >> 1) & 1);
+      if (!epi_all(have_d && !ab.set())) break;
+      bool gave_up = false;                                    // (goes on to the barriers of this piece, then everybody leaves)
       tc_fence_after();
       const uint32_t d_addr = lane_addr + (uint32_t)buf * kTok;
       const int n_glob = (tile_mul * s.tile + (int)rank) * kTileN + n;
@@ -539,20 +607,15 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
       // the only closer of a shared tile (it holds the tile's first groups) keeps its accumulator and adds
       // the other holders' partial tiles to it
       const bool keep = !sole && s.n_closers == 1 && s.closer_idx == 0;
-      // (the two CTAs of a pair exchange their own tiles: slots and counters are interleaved by rank)
-      unsigned *ctr = p.sync + kPlSyncArrive + tile_mul * s.counter + rank;
+      // (the two CTAs of a pair exchange their own tiles: slots are interleaved by rank)
       const long long slot_step = (long long)tile_mul * p.slot_floats;            // from one holder's slot to the next
-      const float *src0 = p.partials + ((long long)tile_mul * s.slot0 + rank) * p.slot_floats + n;
-      if (keep) {
-        if (lead) wait_counter(ab, ctr, (unsigned)(S - 1));
-        epi_bar();
-        if (ab.set()) break;
-      }
+      float *const src0 = p.partials + ((long long)tile_mul * s.slot0 + rank) * p.slot_floats + 4 * n;
+      // token rows this piece writes (the schedule counts them in 64ths of the capacity)
+      const int t0 = s.tok_begin * (kTok / kPlTokens), t1 = min(s.tok_end * (kTok / kPlTokens), P.m);
       if (sole || keep) {
-        // token rows this piece writes (the schedule counts them in 64ths of the capacity)
-        const int t0 = s.tok_begin * (kTok / kPlTokens), t1 = min(s.tok_end * (kTok / kPlTokens), P.m);
-        if (wide) epi_finish<16>(d_addr, c_begin, c_end, keep, S, src0, slot_step, P.m, n_ok, t0, t1, y_out + out_col, ldy);
-        else epi_finish<8>(d_addr, c_begin, c_end, keep, S, src0, slot_step, P.m, n_ok, t0, t1, y_out + out_col, ldy);
+        const bool done_ok = wide ? epi_finish<16>(ab, d_addr, c_begin, c_end, keep, S, src0, slot_step, n_ok, t0, t1, y_out + out_col, ldy)
+                                  : epi_finish<8>(ab, d_addr, c_begin, c_end, keep, S, src0, slot_step, n_ok, t0, t1, y_out + out_col, ldy);
+        if (!done_ok) gave_up = true;
         tc_fence_before();
         __syncwarp();                                          // one arrival per warp, where the issuer waits
         if (lane == 0) {
@@ -561,19 +624,18 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         }
         if (P.signal) {
           epi_bar();                                           // all stores of the CTA are issued ...
-          if (lead) {
+          if (lead && !ab.set()) {
             __threadfence();                                   // ... and ordered before the count (cumulative fence)
-            atomicAdd(p.sync + kPlSyncDone + s.prob, 1u);
+            atomicAdd(done + s.prob, 1u);
           }
         }
         continue;
       }
-      // store the partial tile [token][column] (a warp writes 128 contiguous bytes per token), give the
-      // accumulator back, count this CTA in
+      // store the partial tile, give the accumulator back
       {
-        float *dst = p.partials + ((long long)tile_mul * (s.slot0 + s.contrib_idx) + rank) * p.slot_floats + n;
-        if (wide) epi_store_partial<16>(d_addr, c_begin, c_end, P.m, dst);
-        else epi_store_partial<8>(d_addr, c_begin, c_end, P.m, dst);
+        float *dst = src0 + (long long)s.contrib_idx * slot_step;
+        if (wide) epi_store_partial<16>(d_addr, c_begin, c_end, t0, t1, dst);
+        else epi_store_partial<8>(d_addr, c_begin, c_end, t0, t1, dst);
       }
       tc_fence_before();
       __syncwarp();
@@ -581,52 +643,43 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         if (kPair) mbar_arrive_cluster(map_to_rank(bar_d_empty + 8 * buf, 0));
         else mbar_arrive(bar_d_empty + 8 * buf);
       }
-      epi_bar();
-      if (lead) {
-        __threadfence();
-        atomicAdd(ctr, 1u);
-      }
       if (s.closer_idx < 0) continue;
-      // one of several closers: when every holder has stored its partial tile, add them for token rows
-      // closer_idx, closer_idx + n_closers, ... in ascending K order and write those rows of y
-      if (lead) wait_counter(ab, ctr, (unsigned)S);
-      epi_bar();
-      if (ab.set()) break;
+      // one of several closers: adds the partial tiles of its share of the quads in ascending K order and writes those rows of y.  (Leaving
+      // its own out of the workspace and adding it from tensor memory saves a third of the traffic, but not time: 1024 channels at 20 tokens
+      // 14.5 us so, 15.6 then.)
       {
-        // (the two warps of a quadrant take alternate batches of eight rows; 32 loads are in flight per
-        // thread and round; a holder index past S adds +0, which changes nothing)
-        const int nc = s.n_closers;
-        const int t0 = s.tok_begin * (kTok / kPlTokens), t1 = min(s.tok_end * (kTok / kPlTokens), P.m);
-        for (int r0 = s.closer_idx + ((warp - kPlFirstEpiWarp) >> 2) * 8 * nc; r0 < t1; r0 += 16 * nc) {
-          float acc[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u] = 0.f;
-          for (int i = 0; i < S; i += 4) {
+        // (the two warps of a quadrant take alternate quads; eight are in flight per thread; a holder index past S adds +0, which
+        // changes nothing)
+        const int q0 = t0 >> 2, nq = ((t1 + 3) >> 2) - q0, nc = s.n_closers;
+        const int q_end = q0 + nq * (s.closer_idx + 1) / nc;
+        for (int q = q0 + nq * s.closer_idx / nc + ((warp - kPlFirstEpiWarp) >> 2); q < q_end && !gave_up; q += 2) {
+          float acc[4] = {0.f, 0.f, 0.f, 0.f};
+          for (int i = 0; i < S; i += 8) {
+            float *src[8];
             float w[8][4];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const int r = r0 + u * nc;
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                w[u][k] = (r < t1 && i + k < S) ? __ldcg(src0 + (long long)(i + k) * slot_step + r * kTileN) : 0.f;
+            for (int k = 0; k < 8; ++k) src[k] = i + k < S ? src0 + (long long)(i + k) * slot_step + q * kQuadFloats : nullptr;
+            if (!take_quads(ab, src, w)) {
+              gave_up = true;
+              break;
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
+            for (int k = 0; k < 8; ++k)
 #pragma unroll
-              for (int k = 0; k < 4; ++k) acc[u] = __fadd_rn(acc[u], w[u][k]);
+              for (int e = 0; e < 4; ++e) acc[e] = __fadd_rn(acc[e], w[k][e]);
           }
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int r = r0 + u * nc;
-            if (n_ok && r >= t0 && r < t1) y_out[(long long)r * ldy + out_col] = __float2half_rn(acc[u]);
+          for (int e = 0; e < 4; ++e) {
+            const int row = 4 * q + e;
+            if (n_ok && !gave_up && row >= t0 && row < t1) y_out[(long long)row * ldy + out_col] = __float2half_rn(acc[e]);
           }
         }
       }
       if (P.signal) {
         epi_bar();
-        if (lead) {
+        if (lead && !ab.set()) {
           __threadfence();
-          atomicAdd(p.sync + kPlSyncDone + s.prob, 1u);
+          atomicAdd(done + s.prob, 1u);
         }
       }
     }
@@ -643,19 +696,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
     if (kPair) tmem_dealloc_pair<kPlTmemCols>(tmem);
     else tmem_dealloc<kPlTmemCols>(tmem);
   }
-  // the last CTA to leave puts every counter back to zero for the next launch
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned old = atomicAdd(p.sync + kPlSyncFinished, 1u);
-    __threadfence();
-    misc_ptr[2] = old == gridDim.x - 1 ? 1u : 0u;
-  }
-  __syncthreads();
-  if (misc_ptr[2]) {
-    for (int i = threadIdx.x; i < p.n_counters; i += kPlThreads) p.sync[kPlSyncArrive + i] = 0;
-    if (threadIdx.x < kPlanMaxOps) p.sync[kPlSyncDone + threadIdx.x] = 0;
-    if (threadIdx.x == 0) p.sync[kPlSyncFinished] = 0;
-  }
+  // (512 in all per launch, none before this CTA is through with the counters)
+  if (threadIdx.x == 0) atomicAdd(p.sync + kPlSyncFinished, blockIdx.x == 0 ? (unsigned)(kPlanMaxCtas + 1) - gridDim.x : 1u);
 }
 
 // ---------------------------------------------------------------------------------- host side
@@ -946,7 +988,6 @@ static int plan_get_schedule(rosaq_ctx *ctx, const std::vector<PlanGeom> &geom, 
   s->geom = geom;
   for (int i = 0; i < 3; ++i) s->cost[i] = cost[i];
   int st = plan_build_schedule(geom, P, cost, s);
-  if (st == ROSAQ_OK && s->n_counters > kPlMaxCounters) st = ROSAQ_ERR_UNSUPPORTED_SHAPE;
   if (st == ROSAQ_OK) {
     const size_t seg_bytes = std::max<size_t>(s->segs.size(), 1) * sizeof(PlanSeg), beg_bytes = (size_t)(P + 1) * sizeof(int);
     if (cudaMalloc(reinterpret_cast<void **>(&s->d_segs), seg_bytes) != cudaSuccess ||
@@ -1015,12 +1056,11 @@ int plan_prepare(rosaq_ctx *ctx, int M, int n, const PlanOp *ops, PlanLaunch *ou
   const PlanSchedule *s = nullptr;
   int st = plan_get_schedule(ctx, geom, plan_units(ctx, pair), cost, &s);
   if (st != ROSAQ_OK) return st;
-  if (tile_div * s->n_counters > kPlMaxCounters) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
   const int MT = pair ? ((M + 31) / 32) * 32 : ((M + 15) / 16) * 16;
   const int MTL = MT / tile_div;                       // token rows a CTA keeps in shared memory
   const int slot_floats = MT * kTileN;
   const size_t need = (size_t)tile_div * std::max(s->n_slots, 1) * slot_floats * sizeof(float);
-  st = grow_workspace(ctx, reinterpret_cast<void **>(&ctx->pl_partials), &ctx->pl_partial_bytes, need);
+  st = grow_exchange(ctx, need);
   if (st != ROSAQ_OK) return st;
   PlParams *q = new (std::nothrow) PlParams();
   if (!q) return ROSAQ_ERR_ALLOC;
@@ -1052,11 +1092,10 @@ int plan_prepare(rosaq_ctx *ctx, int M, int n, const PlanOp *ops, PlanLaunch *ou
     if (ops[i].dep >= 0) q->prob[ops[i].dep].signal = 1;
   q->segs = s->d_segs;
   q->seg_begin = s->d_seg_begin;
-  q->partials = ctx->pl_partials;
+  q->partials = ctx->pl_exchange;
   q->sync = ctx->pl_sync;
   q->status = ctx->d_status;
   q->wait_limit = ctx->wait_limit;
-  q->n_counters = tile_div * s->n_counters;
   q->M = M;
   q->MT = MT;
   q->NW = plan_nw(MTL, pair ? kPlPairStages : kPlStages);
@@ -1078,8 +1117,8 @@ void plan_release(PlanLaunch *l) {
 int plan_launch(rosaq_ctx *ctx, const PlanLaunch &l, cudaStream_t s) {
   PlParams *q = static_cast<PlParams *>(l.params);
   if (!q) return ROSAQ_ERR_INVALID_ARG;
-  if (ctx->pl_partial_bytes < l.partial_bytes) return ROSAQ_ERR_INVALID_ARG;
-  q->partials = ctx->pl_partials;                      // the workspace may have grown since the plan was made
+  if (ctx->pl_exchange_bytes < l.partial_bytes) return ROSAQ_ERR_INVALID_ARG;
+  q->partials = ctx->pl_exchange;                      // the workspace may have grown since the plan was made
   q->wait_limit = ctx->wait_limit;
   const size_t smem = plan_smem_bytes(l.pair ? q->MT / 2 : q->MT, q->NW, l.pair ? kPlPairStages : kPlStages);
   if (l.pair) return l.bits == 3 ? plan_launch_kernel(linear_plan_kernel<3, 1>, l, *q, smem, s)

@@ -889,10 +889,9 @@ int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx,
   if (units < 1 || units > (1ll << 30)) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
   p.units = (int)units;
   const int n_pairs = p.S > 0 ? (int)tiles * p.S : (int)std::min<long long>(units, max_pairs);
-  // two slots of 2 x NT x 128 floats per pair, in the workspace of the persistent launch (launches of one
-  // context do not overlap on the GPU)
-  if (p.S == 0 && ctx->pl_partial_bytes < (size_t)n_pairs * 4 * p.NT * kTileN * sizeof(float)) return ROSAQ_ERR_ALLOC;
-  p.partials = ctx->pl_partials;
+  // two slots of 2 x NT x 128 floats per pair, (launches of one context do not overlap on the GPU)
+  if (p.S == 0 && ctx->pf_partial_bytes < (size_t)n_pairs * 4 * p.NT * kTileN * sizeof(float)) return ROSAQ_ERR_ALLOC;
+  p.partials = ctx->pf_partials;
   p.flags = ctx->pf_flags;
   p.status = ctx->d_status;
   p.wait_limit = ctx->wait_limit;

@@ -245,8 +245,8 @@ int rosaq_create(rosaq_ctx **out, int device) {
   ctx->pl_mode = 1;   // pairs of CTAs are built and tested but measured slower so far: off unless asked for
   ctx->pl_cost_set = 0;
   ctx->pl_cost[0] = kPlanCostFp16, ctx->pl_cost[1] = kPlanCostQuant, ctx->pl_cost[2] = kPlanCostTile;
-  ctx->pl_partials = nullptr;
-  ctx->pl_partial_bytes = 0;
+  ctx->pl_exchange = ctx->pf_partials = nullptr;
+  ctx->pl_exchange_bytes = ctx->pf_partial_bytes = 0;
   ctx->pl_sync = nullptr;
   for (int i = 0; i < 4; ++i) ctx->pf_clusters[i] = 0;
   ctx->pf_flags = nullptr;
@@ -263,16 +263,17 @@ int rosaq_create(rosaq_ctx **out, int device) {
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pf_flags), (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pf_flags, 0, (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
-  // the partial tiles of a launch whose CTAs all share tiles at both ends of two phases (grown if a plan needs more)
-  if (st == ROSAQ_OK) {
-    const size_t bytes = (size_t)4 * ctx->sk_ctas * rosaq::kSkPartialBytes;
-    st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pl_partials), bytes));
-    if (st == ROSAQ_OK) ctx->pl_partial_bytes = bytes;
-  }
+  // the partial tiles of a launch whose CTAs all share tiles at both ends of two phases (grown if a plan needs more), and of one on the
+  // prefill tiles
+  const size_t tile_bytes = (size_t)4 * ctx->sk_ctas * rosaq::kSkPartialBytes;
+  if (st == ROSAQ_OK) st = rosaq::grow_exchange(ctx, tile_bytes);
+  if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pf_partials), tile_bytes));
+  if (st == ROSAQ_OK) ctx->pf_partial_bytes = tile_bytes;
   if (st != ROSAQ_OK) {
     if (ctx->pl_sync) (void)cudaFree(ctx->pl_sync);
     if (ctx->pf_flags) (void)cudaFree(ctx->pf_flags);
-    if (ctx->pl_partials) (void)cudaFree(ctx->pl_partials);
+    if (ctx->pl_exchange) (void)cudaFree(ctx->pl_exchange);
+    if (ctx->pf_partials) (void)cudaFree(ctx->pf_partials);
     if (ctx->d_status) (void)cudaFree(ctx->d_status);
     if (ctx->sk_partials) (void)cudaFree(ctx->sk_partials);
     if (ctx->sk_arrive) (void)cudaFree(ctx->sk_arrive);
@@ -296,7 +297,8 @@ int rosaq_destroy(rosaq_ctx *ctx) {
     if (ctx->sk_arrive) (void)cudaFree(ctx->sk_arrive);
     if (ctx->pl_sync) (void)cudaFree(ctx->pl_sync);
     if (ctx->pf_flags) (void)cudaFree(ctx->pf_flags);
-    if (ctx->pl_partials) (void)cudaFree(ctx->pl_partials);
+    if (ctx->pl_exchange) (void)cudaFree(ctx->pl_exchange);
+    if (ctx->pf_partials) (void)cudaFree(ctx->pf_partials);
     plan_free_schedules(ctx);
     pool_release(ctx->pool);
     (void)cudaGetLastError();
@@ -318,7 +320,11 @@ int rosaq_last_status(rosaq_ctx *ctx, void *stream) {
   if (host != 0) {
     st = cuda_status(cudaMemset(ctx->d_status, 0, sizeof(int)));
     if (st != ROSAQ_OK) return st;
-    // a launch that gave up may have left arrival counters of the stream-K exchange behind
+    // a launch that gave up may have left arrival counters of the stream-K exchange behind, and partial tiles
+    st = cuda_status(cudaMemset(ctx->pl_exchange, 0xff, ctx->pl_exchange_bytes));
+    for (int i = 0; i < ctx->n_retired && st == ROSAQ_OK; ++i)
+      if (ctx->retired_exchange[i]) st = cuda_status(cudaMemset(ctx->retired[i], 0xff, ctx->retired_exchange[i]));
+    if (st != ROSAQ_OK) return st;
     st = cuda_status(cudaMemset(ctx->sk_arrive, 0, rosaq::kSkCounterInts * sizeof(int)));
     if (st != ROSAQ_OK) return st;
     st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));

@@ -175,9 +175,9 @@ constexpr size_t kSkPartialBytes = 128 * 64 * sizeof(float);   // one partial ti
 // ---- the persistent multi-problem launch (linear_plan.cu) --------------------------------
 constexpr int kPlanMaxOps = 12;                     // problems in one launch
 constexpr int kPlanMaxCtas = 512;
-constexpr int kPlMaxCounters = 4096;                // column tiles shared between CTAs in one launch
-constexpr int kPlSyncFinished = 0, kPlSyncDone = 4, kPlSyncArrive = 16;   // word offsets in the sync buffer
-constexpr int kPlSyncWords = kPlSyncArrive + kPlMaxCounters;
+// words of the sync buffer: the finished count; two sets of a done counter per problem and the count of CTAs that have wiped their slots
+constexpr int kPlSyncFinished = 0, kPlSyncSets = 32, kPlSyncSet = 32, kPlSyncWiped = kPlanMaxOps, kPlSyncWords = kPlSyncSets + 2 * kPlSyncSet;
+constexpr uint32_t kEmpty = 0xffffffffu;            // an exchanged word that has not been stored; bytes of 0xff
 // Relative cost of the work items when a phase is cut into equal shares.  Either kind of group costs its dequantisation and eight
 // MMAs; an fp16 group also moves 32 KB, which takes an SM's share of the HBM bandwidth about 1400 cycles when every SM
 // streams fp16 tiles, less when some run quantized groups next to it.  Ten operations of a layer, us at fp16 : quantized = 8 : 7 / 10 : 7 /
@@ -260,6 +260,7 @@ struct rosaq_ctx {
   size_t ws_bytes;
   rosaq::MemPool *pool;   // memory of the weights and rotations
   void *retired[rosaq::kMaxRetired];   // workspaces that were outgrown: captured launches may still use them
+  size_t retired_exchange[rosaq::kMaxRetired];   // bytes of those that are kEmpty between launches, else 0
   int n_retired;
   long long wait_limit;
   int impl;            // 0 tensor-core, 1 CUDA-core, 2 tensor-core with CTA pairs, 3 tensor-core without stream-K,
@@ -273,11 +274,13 @@ struct rosaq_ctx {
   int pl_mode;                                   // 0: pairs of CTAs where the operands allow, 1: single CTAs only
   int pl_cost[3];                                // cost of an fp16 group, a quantized group, a tile's epilogue ...
   int pl_cost_set;                               // ... when set through rosaq_set_plan_costs, else the defaults
-  float *pl_partials;                            // partial tiles exchanged between CTAs; grown on demand
-  size_t pl_partial_bytes;
-  unsigned *pl_sync;                             // counters, zero between launches
+  float *pl_exchange;                            // partial tiles exchanged between CTAs, kEmpty between launches; grown on demand
+  size_t pl_exchange_bytes;
+  unsigned *pl_sync;                             // counters
   std::vector<rosaq::PlanSchedule *> pl_schedules;   // one per geometry seen, owned
-  // prefill tiles (pairs of CTAs; the partial tiles of a launch live in pl_partials)
+  // prefill tiles (pairs of CTAs)
+  float *pf_partials;                            // partial tiles of a launch cut into equal shares
+  size_t pf_partial_bytes;
   int pf_clusters[4];                            // clusters of 1 .. 4 pairs the device keeps resident at once (0 until first asked for)
   unsigned *pf_flags;                            // [pair][2][rank]: readers that have yet to fetch a partial tile; zero between launches
 };
@@ -352,10 +355,32 @@ inline int grow_workspace(rosaq_ctx *ctx, void **ws, size_t *bytes, size_t need)
     (void)cudaGetLastError();
     return e == cudaErrorMemoryAllocation ? ROSAQ_ERR_ALLOC : ROSAQ_ERR_CUDA;
   }
-  if (*ws) ctx->retired[ctx->n_retired++] = *ws;
+  if (*ws) {
+    ctx->retired_exchange[ctx->n_retired] = 0;
+    ctx->retired[ctx->n_retired++] = *ws;
+  }
   *ws = p;
   *bytes = want;
   return ROSAQ_OK;
+}
+
+// the workspace of exchanged partial tiles, all of it empty
+inline int grow_exchange(rosaq_ctx *ctx, size_t need) {
+  if (ctx->pl_exchange_bytes >= need) return ROSAQ_OK;
+  float *const old = ctx->pl_exchange;
+  const size_t old_bytes = ctx->pl_exchange_bytes;
+  const int st = grow_workspace(ctx, reinterpret_cast<void **>(&ctx->pl_exchange), &ctx->pl_exchange_bytes, need);
+  if (st != ROSAQ_OK) return st;
+  if (old) ctx->retired_exchange[ctx->n_retired - 1] = old_bytes;
+  cudaStream_t s;                // (one of its own: the legacy stream may not be used next to a capture)
+  if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess) {
+    const bool ok = cudaMemsetAsync(ctx->pl_exchange, 0xff, ctx->pl_exchange_bytes, s) == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
+    (void)cudaStreamDestroy(s);
+    if (ok) return ROSAQ_OK;
+  }
+  (void)cudaGetLastError();
+  ctx->pl_exchange_bytes = 0;   // (not to be used as it is: the next call grows it again)
+  return ROSAQ_ERR_CUDA;
 }
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }

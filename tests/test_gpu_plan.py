@@ -251,3 +251,33 @@ def test_plan_with_many_pieces_per_cta(ctx, M, d_out, n_ops):
             sep = ctx.linear(x, w).double()
             assert (y.double() - sep).norm() <= 2e-4 * sep.norm()
     plan.free()
+
+
+@pytest.mark.parametrize("M,d,d_out", [(16, 512, 640), (64, 1024, 3000), (100, 640, 2816)])
+def test_plan_behind_one_that_gave_up(ctx, M, d, d_out):
+    """A launch that gives up may leave partial tiles in the workspace and counts behind.  The next one computes the right bits whether the
+    status was read in between (the host empties the workspace) or not (the launch does)."""
+    rng = synth.rng_for(31, "gaveup", M, d)
+    rot = ctx.rotation_create(dev((rng.standard_normal((d, d)) / d ** 0.5).astype(np.float16)))
+    w = ctx.quantize(dev(synth.weights(d, d_out, 31, "gaveup", outlier_frac=0.01)), None, bits=4, k_salient=128)
+    x = dev(rng.standard_normal((M, d)).astype(np.float16))
+    xr, y = empty(M, d), empty(M, d_out)
+    plan = ctx.plan_create(M, [(x, None, rot, xr), (None, 0, w, y)])
+    plan.run()
+    assert ctx.last_status() == rb.ROSAQ_OK
+    want = y.clone()
+    for read in (False, True, False):
+        old = ctx.set_wait_limit(1)
+        try:
+            for _ in range(3):
+                plan.run()
+        finally:
+            ctx.set_wait_limit(old)
+        if read:
+            assert ctx.last_status() in (rb.ROSAQ_OK, rb.ROSAQ_ERR_TIMEOUT)
+        for _ in range(3):
+            y.fill_(float("nan"))
+            plan.run()
+            assert torch.equal(y.view(torch.int16), want.view(torch.int16))
+        assert ctx.last_status() in (rb.ROSAQ_OK, rb.ROSAQ_ERR_TIMEOUT)
+    plan.free()
