@@ -176,8 +176,8 @@ __device__ __forceinline__ void st_quad(float *p, uint32_t a, uint32_t b, uint32
   asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 __device__ __forceinline__ uint32_t not_empty(uint32_t v) { return min(v, kEmpty - 1); }   // (a NaN stays one)
-// N quads of this thread, null pointers read as zeros, by a converged warp: polled until all of them have arrived, then emptied for the
-// next launch.  False: gave up.
+// N quads of this thread, null pointers read as zeros, by a converged warp: polled until all of them have arrived.  False: gave up.  The
+// reader empties them for the next launch when it has nothing more urgent to store (an SM stores some 25 bytes per cycle).
 template <int N>
 __device__ __forceinline__ bool take_quads(const Abort &ab, float *const (&src)[N], float (&v)[N][4]) {
   for (long long it = 0;; ++it) {
@@ -204,11 +204,9 @@ __device__ __forceinline__ bool take_quads(const Abort &ab, float *const (&src)[
     if ((it & 15) == 15 && ab.set_all()) return false;
     __nanosleep(32);
   }
-#pragma unroll
-  for (int k = 0; k < N; ++k)
-    if (src[k]) st_quad(src[k], kEmpty, kEmpty, kEmpty, kEmpty);
   return true;
 }
+__device__ __forceinline__ void empty_quad(float *p) { st_quad(p, kEmpty, kEmpty, kEmpty, kEmpty); }
 
 // Tokens [c0, c0 + CH) of one column of the accumulator.
 template <int CH>
@@ -629,6 +627,11 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
             atomicAdd(done + s.prob, 1u);
           }
         }
+        if (keep) {
+          const int qa = max(c_begin, t0) >> 2, qb = (min(c_end, t1) + 3) >> 2;
+          for (int i = 1; i < S; ++i)
+            for (int q = qa; q < qb; ++q) empty_quad(src0 + (long long)i * slot_step + q * kQuadFloats);
+        }
         continue;
       }
       // store the partial tile, give the accumulator back
@@ -647,12 +650,12 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
       // one of several closers: adds the partial tiles of its share of the quads in ascending K order and writes those rows of y.  (Leaving
       // its own out of the workspace and adding it from tensor memory saves a third of the traffic, but not time: 1024 channels at 20 tokens
       // 14.5 us so, 15.6 then.)
+      // (the two warps of a quadrant take alternate quads; eight are in flight per thread; a holder index past S adds +0, which
+      // changes nothing)
+      const int q0 = t0 >> 2, nq = ((t1 + 3) >> 2) - q0, nc = s.n_closers;
+      const int q_begin = q0 + nq * s.closer_idx / nc + ((warp - kPlFirstEpiWarp) >> 2), q_end = q0 + nq * (s.closer_idx + 1) / nc;
       {
-        // (the two warps of a quadrant take alternate quads; eight are in flight per thread; a holder index past S adds +0, which
-        // changes nothing)
-        const int q0 = t0 >> 2, nq = ((t1 + 3) >> 2) - q0, nc = s.n_closers;
-        const int q_end = q0 + nq * (s.closer_idx + 1) / nc;
-        for (int q = q0 + nq * s.closer_idx / nc + ((warp - kPlFirstEpiWarp) >> 2); q < q_end && !gave_up; q += 2) {
+        for (int q = q_begin; q < q_end && !gave_up; q += 2) {
           float acc[4] = {0.f, 0.f, 0.f, 0.f};
           for (int i = 0; i < S; i += 8) {
             float *src[8];
@@ -682,6 +685,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
           atomicAdd(done + s.prob, 1u);
         }
       }
+      for (int q = q_begin; q < q_end; q += 2)
+        for (int i = 0; i < S; ++i) empty_quad(src0 + (long long)i * slot_step + q * kQuadFloats);
     }
   }
 
