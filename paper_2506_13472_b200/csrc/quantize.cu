@@ -17,19 +17,22 @@ namespace rosaq {
 // The fp32 chain.  out[i][n] = sum_k A[k][i] * B[k][n] as one fused multiply-add per term, k ascending, a single
 // fp32 accumulator per output started at +0: the canonical order of W' = R^T W (and, with A = B = X, the Gram
 // matrix of fp32 calibration activations).  A CTA of 128 threads computes a 128 x 128 tile, 8 x 16 outputs per
-// thread, K stepped by 8 through two shared-memory buffers.  Zero padding is harmless: fma(0, 0, acc) = acc.
+// thread, K stepped by kBK through two shared-memory buffers.  Zero padding is harmless: fma(0, 0, acc) = acc.
 //
 // Bound: the fp32 pipe (one multiply-add per lane and cycle, 128 lanes per SM) -- as long as the operands keep up.
 // A 16-byte shared-memory load occupies the SM's load path for four cycles whatever it broadcasts, so an 8 x 8 thread
 // tile (four loads per 64 multiply-adds) is bound by its loads; an 8 x 16 one (six per 128) is not.  Scalar
 // multiply-adds then lose a quarter of their issue cycles to register-port stalls (3.27 ms in the example below);
-// fma.rn.f32x2, two independent IEEE multiply-adds on register pairs, does not and leaves issue slots free.
+// fma.rn.f32x2, two independent IEEE multiply-adds on register pairs, does not and leaves issue slots free.  (On registers alone
+// two warps per scheduler reach 2.2 cycles per paired multiply-add, 63 TFLOP/s; one warp 2.2 to 3.0, by their order.)
+// Steps of sixteen: 2.52 ms, of eight 2.65, of thirty-two 3.35 (the operands in flight no longer fit the registers).  The Gram kernel, whose
+// operands are both fp32, gains from them where an SM has one CTA (4096 tokens x 512 channels 64.4 -> 59.9 us), and loses where two hide
+// each other's barriers (x 2048: 382 -> 391).
 // Measured at 4096 -> 4096 INT4, dense R, the rotation and the quantization: 3.41 ms (41 TFLOP/s; 8 x 8 scalar per
-// thread, one buffer, W' through global memory) before, 2.59 ms (53 TFLOP/s) after.
+// thread, one buffer, W' through global memory) at first, 2.65 ms with the pairs, 2.52 ms (54 TFLOP/s) now.
 // =====================================================================================
-constexpr int kBM = 128, kBN = 128, kBK = 8;
+constexpr int kBM = 128, kBN = 128;
 constexpr int kFmaThreads = 128;
-constexpr int kFmaBufFloats = kBK * (kBM + kBN);
 constexpr int kTilePitch = 132;                                  // floats; the finished tile reuses the buffers
 constexpr int kFmaSmemBytes = 128 * kTilePitch * 4;
 
@@ -91,19 +94,21 @@ struct Raw4<__half> {
 // The K loop.  fetch_a(k, c, raw) / fetch_b(k, c, raw) deliver A[k][c .. c + 3] / B[k][c .. c + 3] (tile columns; 0 outside
 // the operand, also for k >= K); with kScaled row k of B is multiplied by fetch_s(k), one rounding per product.
 // acc[ia][2 q + e] is row(ia), columns 32 q + tx * 4 + 2 e, + 1.
-template <typename TA, typename TB, bool kScaled, typename FA, typename FB, typename FS>
+template <int kBK, typename TA, typename TB, bool kScaled, typename FA, typename FB, typename FS>
 __device__ __forceinline__ void fma_tile(float *smem, int K, const FmaThread &ft, FA fetch_a, FB fetch_b, FS fetch_s, unsigned long long acc[8][8]) {
 #pragma unroll
   for (int ia = 0; ia < 8; ++ia)
 #pragma unroll
     for (int ib = 0; ib < 8; ++ib) acc[ia][ib] = 0ull;
-  const int lr = threadIdx.x >> 5, lc = (threadIdx.x & 31) * 4;      // loader: rows lr and lr + 4 of the K step, four columns
-  Raw4<TA> ra[2];
-  Raw4<TB> rb[2];
-  float rs[2];
+  constexpr int kFmaBufFloats = kBK * (kBM + kBN), kRows = kBK / 4;
+  static_assert(2 * kFmaBufFloats * 4 <= kFmaSmemBytes, "two buffers");
+  const int lr = threadIdx.x >> 5, lc = (threadIdx.x & 31) * 4;      // loader: rows lr, lr + 4, ... of the K step, four columns
+  Raw4<TA> ra[kRows];
+  Raw4<TB> rb[kRows];
+  float rs[kRows];
   auto fetch = [&](int k0) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < kRows; ++h) {
       fetch_a(k0 + lr + 4 * h, lc, ra[h]);
       fetch_b(k0 + lr + 4 * h, lc, rb[h]);
       if (kScaled) rs[h] = fetch_s(k0 + lr + 4 * h);
@@ -111,7 +116,7 @@ __device__ __forceinline__ void fma_tile(float *smem, int K, const FmaThread &ft
   };
   auto put = [&](float *buf) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < kRows; ++h) {
       *reinterpret_cast<float4 *>(buf + (lr + 4 * h) * kBM + lc) = ra[h].expand();
       float4 b = rb[h].expand();
       if (kScaled) b = make_float4(__fmul_rn(rs[h], b.x), __fmul_rn(rs[h], b.y), __fmul_rn(rs[h], b.z), __fmul_rn(rs[h], b.w));
@@ -265,7 +270,7 @@ struct RotateArgs {
 // W' = R^T W for one 128 x 128 tile, then either quantized and packed from shared memory (kSpill = false: the tile is
 // a whole group, so W' never reaches global memory), or, when the rows of a group come from different head blocks (a
 // block-diagonal R with a column order), stored to a slab of W' that quant_tile_kernel reads.
-template <typename TQ, int kBits, bool kSpill, bool kScaled>
+template <typename TQ, int kBits, bool kSpill, bool kScaled, int kBK>
 __global__ void __launch_bounds__(kFmaThreads, 2)
 rotate_tile_kernel(const RotateArgs a, const TiledOperand t) {
   extern __shared__ __align__(16) float smem[];
@@ -312,7 +317,7 @@ rotate_tile_kernel(const RotateArgs a, const TiledOperand t) {
   };
   const float *ds = kScaled ? a.in_scale + (long long)h * a.dh : nullptr;
   unsigned long long acc[8][8];
-  fma_tile<TQ, __half, kScaled>(smem, a.dh, ft, fetch_a, fetch_b, [&](int k) { return k < a.dh ? ds[k] : 0.f; }, acc);
+  fma_tile<kBK, TQ, __half, kScaled>(smem, a.dh, ft, fetch_a, fetch_b, [&](int k) { return k < a.dh ? ds[k] : 0.f; }, acc);
   if (!kSpill) {
     store_tile_smem(smem, ft, acc);                                  // (the K loop ends with a barrier)
     __syncthreads();
@@ -387,7 +392,10 @@ static bool allow_smem(K kern, int bytes) {
 template <typename TQ, int kBits, bool kScaled>
 static int rotate_quantize_typed(const RotateArgs &args, int n_blocks, const TiledOperand &t, cudaStream_t s) {
   RotateArgs a = args;
-  const auto fused = rotate_tile_kernel<TQ, kBits, false, kScaled>, spilling = rotate_tile_kernel<TQ, kBits, true, kScaled>;
+  // (steps of sixteen for a dense R; head blocks of 128 channels are eight such steps, most of them start and end: 2048 channels 70.4 us
+  // with steps of eight, 75.8 with sixteen)
+  const auto fused = n_blocks == 1 ? rotate_tile_kernel<TQ, kBits, false, kScaled, 16> : rotate_tile_kernel<TQ, kBits, false, kScaled, 8>;
+  const auto spilling = rotate_tile_kernel<TQ, kBits, true, kScaled, 8>;
   const auto quant = quant_tile_kernel<kBits>;
   if (!allow_smem(fused, kFmaSmemBytes) || !allow_smem(spilling, kFmaSmemBytes) || !allow_smem(quant, kQuantSmemBytes)) return ROSAQ_ERR_CUDA;
   const int groups = groups_per_tile(t);
@@ -436,7 +444,7 @@ int launch_rotate_quantize(const void *q, int q_is_f32, int n_blocks, const int3
 // tokens in the same order, so the mirrored bits are those a tile of its own would produce).  With few tiles a cluster of up
 // to eight CTAs shares the tokens of a tile and adds the partial tiles in order: a tile costs 128 cycles per token whatever the
 // width (4096 tokens x 512 channels: 634 us with all tiles of both triangles and a CTA each, 67 so; x 2048: 1003 and 418).
-template <typename T>
+template <typename T, int kBK>
 __global__ void __launch_bounds__(kFmaThreads, 2)
 gram_fma_kernel(const T *X, long long ldx, int dh, float *C, int n_tokens, int Z) {   // (X: not read-only while the kernel before may still write it)
   extern __shared__ __align__(16) float tile[];
@@ -456,7 +464,7 @@ gram_fma_kernel(const T *X, long long ldx, int dh, float *C, int n_tokens, int Z
     else raw.zero();
   };
   unsigned long long acc[8][8];
-  fma_tile<T, T, false>(
+  fma_tile<kBK, T, T, false>(
       tile, K, ft, [&](int k, int c, Raw4<T> &raw) { fetch(k, i0 + c, raw); },
       [&](int k, int c, Raw4<T> &raw) { fetch(k, n0 + c, raw); }, [](int) { return 0.f; }, acc);
   cov_grid_dep_launch();
@@ -505,16 +513,22 @@ int launch_cov_fma(int sm_count, const void *X, int x_dtype, long long n_tokens,
                    cudaStream_t s) {
   const int dh = d / n_blocks, nb = (dh + kBM - 1) / kBM;
   const dim3 grid(nb * (nb + 1) / 2, n_blocks);
-  if (!allow_smem(gram_fma_kernel<float>, kFmaSmemBytes) || !allow_smem(gram_fma_kernel<__half>, kFmaSmemBytes)) return ROSAQ_ERR_CUDA;
+  if (!allow_smem(gram_fma_kernel<float, 8>, kFmaSmemBytes) || !allow_smem(gram_fma_kernel<float, 16>, kFmaSmemBytes) ||
+      !allow_smem(gram_fma_kernel<__half, 16>, kFmaSmemBytes))
+    return ROSAQ_ERR_CUDA;
   for (long long t0 = 0; t0 < n_tokens; t0 += 1ll << 30) {           // (the kernel counts tokens in 32 bits)
     const int n = (int)std::min(n_tokens - t0, 1ll << 30);
     // (two CTAs fit an SM; a split keeps at least 64 tokens)
     const int Z = cov_splits((long long)grid.x * grid.y, 2 * sm_count, n / 64, 8);
     const dim3 g(grid.x, grid.y, Z);
-    const int st = x_dtype == ROSAQ_F32 ? cov_launch(gram_fma_kernel<float>, g, kFmaThreads, kFmaSmemBytes, 1, Z, s,
-                                                     static_cast<const float *>(X) + t0 * ldx, ldx, dh, C, n, Z)
-                                        : cov_launch(gram_fma_kernel<__half>, g, kFmaThreads, kFmaSmemBytes, 1, Z, s,
-                                                     static_cast<const __half *>(X) + t0 * ldx, ldx, dh, C, n, Z);
+    auto launch = [&](auto kern, const auto *x) {
+      return cov_launch(kern, g, kFmaThreads, kFmaSmemBytes, 1, Z, s, x + t0 * ldx, ldx, dh, C, n, Z);
+    };
+    // (clusters of eight double up on some SMs from about fifteen of them on: 14 blocks of 128 channels 41.6 -> 39.3 us, 16 of them 62.1 -> 65.3)
+    const bool one_per_sm = (long long)g.x * g.y * g.z <= sm_count * 4 / 5;
+    const int st = x_dtype != ROSAQ_F32 ? launch(gram_fma_kernel<__half, 16>, static_cast<const __half *>(X))
+                   : one_per_sm         ? launch(gram_fma_kernel<float, 16>, static_cast<const float *>(X))
+                                        : launch(gram_fma_kernel<float, 8>, static_cast<const float *>(X));
     if (st != ROSAQ_OK) return st;
   }
   return ROSAQ_OK;

@@ -113,3 +113,22 @@ def test_a_long_calib_cov_does_not_use_up_the_waits_of_the_launch_behind_it():
             ctx.set_wait_limit(old)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n_tokens,n_blocks", [(509, 14), (509, 15), (7, 1), (17, 2)])
+def test_calib_cov_either_step_of_the_fp32_kernel(n_tokens, n_blocks):
+    """The fp32 kernel steps through sixteen tokens at a time where an SM has one CTA (up to 118 of them on 148 SMs), else through eight:
+    both sides of the line, tokens that fill no whole step, one step, less than one."""
+    d = 128 * n_blocks
+    X = synth.ActivationLaw(d, 1.0, seed=49, key=f"covk{d}").sample(n_tokens, "X", np.float32)
+    ctx = rb.Context(0)
+    try:
+        Cg = torch.zeros((n_blocks, 128, 128), dtype=torch.float32, device="cuda")
+        ctx.calib_cov(torch.from_numpy(X).cuda(), Cg, n_blocks)
+        assert ctx.last_status() == rb.ROSAQ_OK
+    finally:
+        ctx.close()
+    Cref = orc.cov(X, n_blocks).reshape(n_blocks, 128, 128)
+    got = Cg.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - Cref) <= H.cov_tolerance(Cref, n_tokens) + 1e-30)
+    assert np.array_equal(got, np.swapaxes(got, -1, -2))
