@@ -170,20 +170,53 @@ __device__ __forceinline__ void unit_int3(uint32_t stage, uint32_t scales, const
   }
 }
 
-template <int kBits, int STAGES>
-__global__ void __launch_bounds__(kSmThreads, kSmCtas)
-linear_small_kernel(const __grid_constant__ SmParams p) {
-  extern __shared__ __align__(128) uint8_t smem[];
+// A rotation and the linears that read it in one launch: the first CTAs are the slices of the rotation, the others copy its output
+// as it appears.  (The hardware starts CTAs in order, so those that are waited for are never behind the ones that wait.)  The
+// buffer between them announces its values itself: it is all ones, which no rounded value is, where nothing has been written yet.
+struct SmPair {
+  SmParams rot, lin;
+  int n_rot;                 // CTAs of the rotation
+  __half *between;           // two buffers of kSmBetween values, for launches in turn; a launch empties the other one
+  unsigned *left;            // kSmLaunch times the launches so far, and the CTAs of this one that have left
+  int *status;
+  long long wait_limit;
+};
+constexpr unsigned kSmLaunch = 1u << 16;
+enum SmRole { kSmAlone, kSmProducer, kSmConsumer };
+
+__device__ __forceinline__ unsigned sm_turn(const SmPair *pair) {   // (behind griddepcontrol.wait)
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(pair->left) : "memory");
+  return (v / kSmLaunch) & 1u;
+}
+// All CTAs of a launch together add kSmLaunch, so the count tells a launch that is running from the one before.
+__device__ __forceinline__ void sm_leave(const SmPair *pair) {
+  if (threadIdx.x == 0) atomicAdd(pair->left, blockIdx.x == 0 ? kSmLaunch + 1 - gridDim.x : 1u);
+}
+// some half of v is 0xffff
+__device__ __forceinline__ uint32_t sm_missing(uint32_t v) {
+  const uint32_t t = ~v;
+  return (t - 0x00010001u) & ~t & 0x80008000u;
+}
+
+template <int kBits, int STAGES, SmRole kRole>
+__device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, int block, const SmPair *pair) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   grid_dep_launch_dependents();
 
   const int u_fp16 = p.u_fp16, n_units = p.n_units, M = p.M;
-  int prob = 0, tile = blockIdx.x >> 2;
-  const int col = (blockIdx.x & 3) * kSmSlice;
+  int prob = 0, tile = block >> 2;
+  const int col = (block & 3) * kSmSlice;
   while (prob + 1 < p.n_prob && tile >= p.tile_start[prob + 1]) ++prob;
   tile -= p.tile_start[prob];
-  if (tile * kTileN + col >= p.d_out[prob]) return;              // past the last column of a ragged last tile
+  if (tile * kTileN + col >= p.d_out[prob]) {                    // past the last column of a ragged last tile
+    if (kRole != kSmAlone) {
+      grid_dep_wait();                                           // (the launch before may still be counting)
+      sm_leave(pair);
+    }
+    return;
+  }
 
   const int x_row = (u_fp16 * 32 + (n_units - u_fp16) * kGroup) * 2;
   const uint32_t x_smem = smem_u32(smem), ring = x_smem + M * x_row + warp * (STAGES * kSmStage), ring_end = ring + STAGES * kSmStage;
@@ -212,6 +245,51 @@ linear_small_kernel(const __grid_constant__ SmParams p) {
   for (int s = 0; s < STAGES; ++s, f += kSmWarps) fetch(ring + s * kSmStage, f);
 
   grid_dep_wait();                                               // x may be the previous kernel's output, y its input
+  __half *between = nullptr;
+  if (kRole != kSmAlone) {
+    const unsigned turn = sm_turn(pair);
+    between = pair->between + turn * kSmBetween;
+    if (kRole == kSmProducer) {
+      uint4 *other = reinterpret_cast<uint4 *>(pair->between + (turn ^ 1u) * kSmBetween);
+      for (int i = block * kSmThreads + threadIdx.x; i < kSmBetween / 8; i += pair->n_rot * kSmThreads) other[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+  }
+  if (kRole == kSmConsumer) {
+    int ok = 1;
+    const int n_full = x_row >> 4, n_all = M * n_full;
+    for (int i0 = threadIdx.x; i0 < n_all && ok; i0 += 4 * kSmThreads) {   // four chunks in flight
+      uint4 v[4];
+      for (long long it = 0;; ++it) {
+        uint32_t missing = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int i = min(i0 + k * kSmThreads, n_all - 1);
+          asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(v[k].x), "=r"(v[k].y), "=r"(v[k].z), "=r"(v[k].w)
+                       : "l"(between + 8 * i)
+                       : "memory");
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) missing |= sm_missing(v[k].x) | sm_missing(v[k].y) | sm_missing(v[k].z) | sm_missing(v[k].w);
+        if (!missing) break;
+        if (it >= pair->wait_limit) {
+          ok = 0;
+          break;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int i = i0 + k * kSmThreads, r = i / n_full;
+        if (i < n_all) *reinterpret_cast<uint4 *>(smem + r * x_row + x_pos(r, i - r * n_full)) = v[k];
+      }
+    }
+    if (!__syncthreads_and(ok)) {
+      if (threadIdx.x == 0) atomicExch(pair->status, (int)ROSAQ_ERR_TIMEOUT);
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      sm_leave(pair);
+      return;
+    }
+  } else
   {
     // block-diagonal operand: a tile multiplies its own channels
     const __half *xs = p.x + (p.block_groups > 0 ? (tile / p.block_groups) * p.block_groups * kGroup : 0) + threadIdx.x * 8;
@@ -221,8 +299,8 @@ linear_small_kernel(const __grid_constant__ SmParams p) {
       for (int c = threadIdx.x; c < n_full; c += kSmThreads, dst += kSmThreads * 16) cp_async16(dst, xs + (c - (int)threadIdx.x) * 8);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
   }
-  __syncthreads();
 
   // (rows past M repeat the last one, their products are dropped)
   const int x_tok = min(g, M - 1);
@@ -271,11 +349,34 @@ linear_small_kernel(const __grid_constant__ SmParams p) {
     float v = 0.f;
 #pragma unroll
     for (int w = 0; w < kSmWarps; ++w) v += part[w * part_stride + warp * kSmSlice + lane];
-    p.y[prob][warp * p.ldy[prob] + (p.col_map ? p.col_map[nn] : nn)] = __float2half_rn(v);
+    const long long at = warp * p.ldy[prob] + (p.col_map ? p.col_map[nn] : nn);
+    if (kRole == kSmProducer) asm volatile("st.relaxed.gpu.global.u16 [%0], %1;" ::"l"(between + at), "h"(__half_as_ushort(__float2half_rn(v))) : "memory");
+    else p.y[prob][at] = __float2half_rn(v);
   }
+  if (kRole != kSmAlone) sm_leave(pair);
+}
+
+template <int kBits, int STAGES>
+__global__ void __launch_bounds__(kSmThreads, kSmCtas)
+linear_small_kernel(const __grid_constant__ SmParams p) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  small_slice<kBits, STAGES, kSmAlone>(smem, p, blockIdx.x, nullptr);
+}
+
+template <int kBits, int STAGES>
+__global__ void __launch_bounds__(kSmThreads, kSmCtas)
+rotate_linear_small_kernel(const __grid_constant__ SmPair p) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  if ((int)blockIdx.x < p.n_rot) small_slice<4, STAGES, kSmProducer>(smem, p.rot, blockIdx.x, &p);
+  else small_slice<kBits, 2, kSmConsumer>(smem, p.lin, blockIdx.x - p.n_rot, &p);
 }
 
 typedef void (*SmallKernel)(SmParams);
+typedef void (*SmallPairKernel)(SmPair);
+SmallPairKernel small_pair_pick(bool int3, int stages) {
+  if (int3) return stages == 8 ? rotate_linear_small_kernel<3, 8> : stages == 4 ? rotate_linear_small_kernel<3, 4> : rotate_linear_small_kernel<3, 2>;
+  return stages == 8 ? rotate_linear_small_kernel<4, 8> : stages == 4 ? rotate_linear_small_kernel<4, 4> : rotate_linear_small_kernel<4, 2>;
+}
 SmallKernel small_pick(bool int3, int stages) {
   if (int3) return linear_small_kernel<3, 2>;
   return stages == 8 ? linear_small_kernel<4, 8> : stages == 4 ? linear_small_kernel<4, 4> : linear_small_kernel<4, 2>;
@@ -286,6 +387,11 @@ bool small_attrs() {
   for (SmallKernel kern : {small_pick(true, 2), small_pick(false, 2), small_pick(false, 4), small_pick(false, 8)})
     ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess &&
          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmMaxSmem) == cudaSuccess;
+  for (int i = 0; i < 6; ++i) {
+    const SmallPairKernel kern = small_pair_pick(i & 1, 2 << (i >> 1));
+    ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess &&
+         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmMaxSmem) == cudaSuccess;
+  }
   if (!ok) (void)cudaGetLastError();
   return ok;
 }
@@ -316,12 +422,11 @@ bool linear_small_supported(const rosaq_ctx *ctx, int M, int n, const TiledOpera
   return bytes <= kSmMaxSmem && resident * (bytes + kSmSharedCta) <= kSmSharedSm;
 }
 
-// n weights of identical geometry applied to the same activations in one launch
-int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const TiledOperand *const *ts,
-                        const int32_t *col_map, __half *const *ys, const long long *ldys, cudaStream_t s) {
+static int small_params(const __half *x, int M, long long ldx, int n, const TiledOperand *const *ts, const int32_t *col_map, __half *const *ys,
+                        const long long *ldys, SmParams *out) {
   if (n < 1 || n > kSmMaxProblems || M < 1 || M > kSmallTokens) return ROSAQ_ERR_INVALID_ARG;
   const TiledOperand &t = *ts[0];
-  SmParams p{};
+  SmParams &p = *out;
   p.n_prob = n;
   int tiles = 0;
   for (int i = 0; i < n; ++i) {
@@ -339,17 +444,49 @@ int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long 
   p.u_fp16 = 4 * t.g_fp16, p.n_units = p.u_fp16 + t.g_quant, p.block_groups = t.block_groups;
   p.M = M;
   p.col_map = col_map;
-  if (p.n_units <= 0 || small_bytes(M, t, 2) > kSmMaxSmem) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
+  return p.n_units <= 0 || small_bytes(M, t, 2) > kSmMaxSmem ? ROSAQ_ERR_UNSUPPORTED_SHAPE : ROSAQ_OK;
+}
+
+static int small_prepare(const rosaq_ctx *ctx) {
+  static bool done[kSmMaxDevices] = {};                          // function attributes are per device
+  static std::mutex mu;
   if (ctx->device < 0 || ctx->device >= kSmMaxDevices) return ROSAQ_ERR_INVALID_ARG;
-  {
-    static bool done[kSmMaxDevices] = {};                        // function attributes are per device
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!done[ctx->device]) {
-      if (!small_attrs()) return ROSAQ_ERR_CUDA;
-      done[ctx->device] = true;
-    }
+  std::lock_guard<std::mutex> lock(mu);
+  if (!done[ctx->device]) {
+    if (!small_attrs()) return ROSAQ_ERR_CUDA;
+    done[ctx->device] = true;
   }
+  return ROSAQ_OK;
+}
+
+template <typename K, typename P>
+static int small_launch(K kern, const P &p, int ctas, int smem, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kSmThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kern, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return ROSAQ_ERR_CUDA;
+  }
+  return ROSAQ_OK;
+}
+
+// n weights of identical geometry applied to the same activations in one launch
+int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const TiledOperand *const *ts,
+                        const int32_t *col_map, __half *const *ys, const long long *ldys, cudaStream_t s) {
+  const TiledOperand &t = *ts[0];
+  SmParams p{};
+  int st = small_params(x, M, ldx, n, ts, col_map, ys, ldys, &p);
+  if (st == ROSAQ_OK) st = small_prepare(ctx);
+  if (st != ROSAQ_OK) return st;
+  const int tiles = p.tile_start[n];
   // Residency: no more CTAs per SM than the slices of this launch fill, because the CTAs of chained launches otherwise pile up
   // on some SMs while others idle (4096 -> 4096, one token, room for one / two / three CTAs: 4.4 / 6.2 / 7.5 us; 4096 -> 2 x
   // 11008 20.9 / 16.0 / 14.3 us).  Stages: two suffice for quantized groups (4096 -> 4096 4.4, with four 4.7 us); an all-fp16
@@ -359,22 +496,53 @@ int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long 
   int stages = 2;
   if (t.g_quant == 0)
     while (stages < 8 && small_bytes(M, t, 2 * stages) <= room) stages *= 2;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(4 * tiles);
-  cfg.blockDim = dim3(kSmThreads);
   // (more than a (ctas + 1)-th of an SM's shared memory)
-  cfg.dynamicSmemBytes = std::max(small_bytes(M, t, stages), ctas < kSmCtas ? (kSmSharedSm / (ctas + 1) - kSmSharedCta) / 128 * 128 + 128 : 0);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, small_pick(t.g_quant > 0 && t.bits == 3, stages), p) != cudaSuccess) {
+  const int smem = std::max(small_bytes(M, t, stages), ctas < kSmCtas ? (kSmSharedSm / (ctas + 1) - kSmSharedCta) / 128 * 128 + 128 : 0);
+  return small_launch(small_pick(t.g_quant > 0 && t.bits == 3, stages), p, 4 * tiles, smem, s);
+}
+
+// The rotation r of x and the n linears that read it in one launch: calls that are bound by the host's two launches (2.3 us each).  That is
+// so while all slices find an SM of their own; then the launch takes the device about what the two take (us in a graph, two launches /
+// one: 512 -> 512 at one, four and eight tokens 3.4 / 3.8, 4.0 / 4.2, 4.8 / 4.8; 1024 -> 3 x 1024 4.3 / 4.5, 4.8 / 5.1, 5.7 / 5.6; 2048 -> 2048 5.4 / 5.9, 6.4 / 6.4,
+// 7.1 / 7.8; call by call 9.1 / 6.1 at 512 -> 512), and 4096 -> 4096 would take 13.8 instead of 9.4.  A launch that is being captured costs the host
+// nothing later, so captured calls stay two, and so do column orders, whose scatter the readers' polls disturb (1024 -> 3 x 1024 4.6 / 9.3).
+// The results are the same bits.
+bool rotate_linear_small_supported(const rosaq_ctx *ctx, int M, const TiledOperand &r, const int32_t *col_map, int n, const TiledOperand *const *ts,
+                                   cudaStream_t s) {
+  const TiledOperand *rs[1] = {&r};
+  if (col_map || (long long)M * r.d_out > kSmBetween || 4 * (r.n_tiles + small_tiles(n, ts)) > ctx->sm_count || !linear_small_supported(ctx, M, 1, rs) ||
+      !linear_small_supported(ctx, M, n, ts))
+    return false;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
     (void)cudaGetLastError();
-    return ROSAQ_ERR_CUDA;
+    return false;
   }
-  return ROSAQ_OK;
+  return capture == cudaStreamCaptureStatusNone;
+}
+
+int launch_rotate_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &r, int n,
+                               const TiledOperand *const *ts, __half *const *ys, const long long *ldys, cudaStream_t s) {
+  const TiledOperand &t = *ts[0];
+  const TiledOperand *rs[1] = {&r};
+  const long long ldxr = r.d_out;
+  SmPair p{};
+  p.between = ctx->sm_between;
+  int st = small_params(x, M, ldx, 1, rs, nullptr, &p.between, &ldxr, &p.rot);
+  if (st == ROSAQ_OK) st = small_params(p.between, M, ldxr, n, ts, nullptr, ys, ldys, &p.lin);
+  if (st == ROSAQ_OK) st = small_prepare(ctx);
+  if (st != ROSAQ_OK) return st;
+  p.n_rot = 4 * r.n_tiles;
+  p.left = ctx->sm_left;
+  p.status = ctx->d_status;
+  p.wait_limit = ctx->wait_limit;
+  const int grid = p.n_rot + 4 * p.lin.tile_start[n], ctas = std::max(1, std::min(kSmCtas, (grid + ctx->sm_count - 1) / ctx->sm_count));
+  const int room = std::min(kSmMaxSmem, kSmSharedSm / ctas - kSmSharedCta);
+  int stages = 2;
+  while (stages < 8 && small_bytes(M, r, 2 * stages) <= room) stages *= 2;
+  const int need = std::max(small_bytes(M, r, stages), small_bytes(M, t, 2));
+  const int smem = std::max(need, ctas < kSmCtas ? (kSmSharedSm / (ctas + 1) - kSmSharedCta) / 128 * 128 + 128 : 0);
+  return small_launch(small_pair_pick(t.g_quant > 0 && t.bits == 3, stages), p, grid, smem, s);
 }
 
 }  // namespace rosaq

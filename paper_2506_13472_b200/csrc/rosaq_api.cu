@@ -248,6 +248,7 @@ int rosaq_create(rosaq_ctx **out, int device) {
   ctx->pl_exchange = ctx->pf_partials = nullptr;
   ctx->pl_exchange_bytes = ctx->pf_partial_bytes = 0;
   ctx->pl_sync = nullptr;
+  ctx->sm_between = nullptr;
   for (int i = 0; i < 4; ++i) ctx->pf_clusters[i] = 0;
   ctx->pf_flags = nullptr;
   ctx->pool = nullptr;
@@ -259,6 +260,13 @@ int rosaq_create(rosaq_ctx **out, int device) {
     st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->sk_partials), (size_t)ctx->sk_ctas * 2 * rosaq::kSkPartialBytes));
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->sk_arrive), rosaq::kSkCounterInts * sizeof(int)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->sk_arrive, 0, rosaq::kSkCounterInts * sizeof(int)));
+  constexpr size_t kBetweenBytes = 2 * rosaq::kSmBetween * sizeof(__half);
+  if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->sm_between), kBetweenBytes + sizeof(unsigned)));
+  if (st == ROSAQ_OK) {
+    ctx->sm_left = reinterpret_cast<unsigned *>(ctx->sm_between + 2 * rosaq::kSmBetween);
+    st = cuda_status(cudaMemset(ctx->sm_between, 0xff, kBetweenBytes));
+  }
+  if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->sm_left, 0, sizeof(unsigned)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pl_sync), rosaq::kPlSyncWords * sizeof(unsigned)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pf_flags), (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
@@ -269,8 +277,10 @@ int rosaq_create(rosaq_ctx **out, int device) {
   if (st == ROSAQ_OK) st = rosaq::grow_exchange(ctx, tile_bytes);
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pf_partials), tile_bytes));
   if (st == ROSAQ_OK) ctx->pf_partial_bytes = tile_bytes;
+  if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(cudaStreamLegacy));   // (the memsets above)
   if (st != ROSAQ_OK) {
     if (ctx->pl_sync) (void)cudaFree(ctx->pl_sync);
+    if (ctx->sm_between) (void)cudaFree(ctx->sm_between);
     if (ctx->pf_flags) (void)cudaFree(ctx->pf_flags);
     if (ctx->pl_exchange) (void)cudaFree(ctx->pl_exchange);
     if (ctx->pf_partials) (void)cudaFree(ctx->pf_partials);
@@ -296,6 +306,7 @@ int rosaq_destroy(rosaq_ctx *ctx) {
     if (ctx->sk_partials) (void)cudaFree(ctx->sk_partials);
     if (ctx->sk_arrive) (void)cudaFree(ctx->sk_arrive);
     if (ctx->pl_sync) (void)cudaFree(ctx->pl_sync);
+    if (ctx->sm_between) (void)cudaFree(ctx->sm_between);
     if (ctx->pf_flags) (void)cudaFree(ctx->pf_flags);
     if (ctx->pl_exchange) (void)cudaFree(ctx->pl_exchange);
     if (ctx->pf_partials) (void)cudaFree(ctx->pf_partials);
@@ -330,6 +341,7 @@ int rosaq_last_status(rosaq_ctx *ctx, void *stream) {
     st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));
     if (st != ROSAQ_OK) return st;
     st = cuda_status(cudaMemset(ctx->pf_flags, 0, (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
+    if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(cudaStreamLegacy));   // (the caller's streams may not wait for it)
     if (st != ROSAQ_OK) return st;
   }
   return host;
@@ -595,13 +607,18 @@ int rosaq_linear(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
     ops[n] = PlanOp{xin, ldx, r ? 0 : -1, &w->t, nullptr, static_cast<__half *>(y), ldy};
     return run_ops(ctx, M, n + 1, ops, s);
   }
+  const TiledOperand *ts[1] = {&w->t};
+  __half *const ys[1] = {static_cast<__half *>(y)};
+  const long long ldys[1] = {ldy};
+  if (r && ctx->impl == 0 && rotate_linear_small_supported(ctx, M, r->t, r->col_map, 1, ts, s))
+    return launch_rotate_linear_small(ctx, xin, M, ldx, r->t, 1, ts, ys, ldys, s);
   if (r) {
     st = run_call(ctx, xin, M, ldx, r->t, r->col_map, static_cast<__half *>(ctx->ws), r->d, s);
     if (st != ROSAQ_OK) return st;
     xin = static_cast<const __half *>(ctx->ws);
     ld = r->d;
   }
-  return run_call(ctx, xin, M, ld, w->t, nullptr, static_cast<__half *>(y), ldy, s);
+  return run_call(ctx, xin, M, ld, w->t, nullptr, ys[0], ldy, s);
 }
 
 int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_rotation *r, int n,
@@ -637,16 +654,18 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
     for (int i = 0; i < n; ++i) ops[k++] = PlanOp{xin, ldx, r ? 0 : -1, &w[i]->t, nullptr, static_cast<__half *>(y[i]), ldy[i]};
     return run_ops(ctx, M, k, ops, s);
   }
+  const TiledOperand *ts[4];
+  __half *ys[4];
+  long long ldys[4];
+  for (int i = 0; i < n; ++i) ts[i] = &w[i]->t, ys[i] = static_cast<__half *>(y[i]), ldys[i] = ldy[i];
+  if (r && ctx->impl == 0 && rotate_linear_small_supported(ctx, M, r->t, r->col_map, n, ts, s))
+    return launch_rotate_linear_small(ctx, xin, M, ldx, r->t, n, ts, ys, ldys, s);
   if (r) {
     st = run_call(ctx, xin, M, ldx, r->t, r->col_map, static_cast<__half *>(ctx->ws), r->d, s);
     if (st != ROSAQ_OK) return st;
     xin = static_cast<const __half *>(ctx->ws);
     ld = r->d;
   }
-  const TiledOperand *ts[4];
-  __half *ys[4];
-  long long ldys[4];
-  for (int i = 0; i < n; ++i) ts[i] = &w[i]->t, ys[i] = static_cast<__half *>(y[i]), ldys[i] = ldy[i];
   if (n == 1) return run_call(ctx, xin, M, ld, *ts[0], nullptr, ys[0], ldys[0], s);
   return run_gemm(ctx, xin, M, ld, n, ts, nullptr, ys, ldys, s);
 }

@@ -98,3 +98,43 @@ def test_rotation(ctx, M, d, head):
     w = ctx.quantize(dev(synth.weights(d, 384, seed=19, key="chain", outlier_frac=0.01)), None, bits=4, k_salient=128)
     assert same(ctx.linear(x, w, rotation=r), ctx.linear(got, w))
     assert ctx.last_status() == rb.ROSAQ_OK
+
+
+@pytest.mark.parametrize("kind,d,widths,bits", [
+    ("dense", 128, [128], 4),              # eight CTAs
+    ("dense", 512, [200], 4),              # a slice with eight columns, one past the last
+    ("heads", 384, [72, 384, 1000], 3),
+    ("dense", 2048, [2688], 3),            # 148 CTAs, the most on 148 SMs; one tile more below
+    ("dense", 2048, [2696], 4),
+])
+def test_rotation_and_linears_in_one_launch(ctx, kind, d, widths, bits):
+    """A small rotated call is one launch (unless it is captured): the bits of the rotation and the linears called one by one, with
+    other calls in between, with values that are no numbers, and behind a call that gave up."""
+    rng = synth.rng_for(21, "onelaunch", d)
+    if kind == "dense":
+        r = ctx.rotation_create(dev((rng.standard_normal((d, d)) / d ** 0.5).astype(np.float16)))
+    else:
+        r = ctx.rotation_create(dev((rng.standard_normal((d // 128, 128, 128)) / 128 ** 0.5).astype(np.float16)))
+    ws = [ctx.quantize(dev(synth.weights(d, n, 21, f"onelaunch{i}", outlier_frac=0.01)), None, bits=bits, k_salient=128) for i, n in enumerate(widths)]
+    for M in (1, 3, 8, 2, 8):
+        x = dev(rng.standard_normal((M, d)).astype(np.float16))
+        if M == 2:
+            x[0, 5], x[1, 7] = float("inf"), float("nan")
+        xr = ctx.rotate(x, r)
+        want = ctx.linear_multi(xr, ws)
+        if M == 3:
+            old = ctx.set_wait_limit(1)
+            ctx.linear_multi(x, ws, r)
+            ctx.set_wait_limit(old)
+            assert ctx.last_status() in (rb.ROSAQ_OK, rb.ROSAQ_ERR_TIMEOUT)
+        for _ in range(3):
+            assert all(same(y, v) for y, v in zip(ctx.linear_multi(x, ws, r), want))
+            assert same(ctx.linear(x, ws[0], r), want[0])
+        y, graph, side = torch.empty_like(want[0]), torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side):
+            ctx.linear(x, ws[0], r, out=y)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert same(y, want[0]) and same(ctx.linear(x, ws[0], r), want[0])
+    assert ctx.last_status() == rb.ROSAQ_OK
