@@ -35,11 +35,11 @@ namespace {
 
 constexpr int kCovTile = 128;      // output tile rows (MMA M)
 constexpr int kCovTokens = 64;     // tokens per pipeline stage
-constexpr int kCovStages = 4;
+constexpr int kCovMaxStages = 12;
 constexpr int kCovThreads = 192;
 constexpr int kBoxBytes = 64 * kCovTokens * 2;          // one TMA box: 64 channels x 64 tokens fp16
 constexpr int kOperandBytes = 2 * kBoxBytes;            // 128 channels (operand A)
-constexpr int kStageBytes = 6 * kBoxBytes;              // A (2 boxes) and up to 256 channels of B (4 boxes)
+constexpr int kCovRingBytes = 24 * kBoxBytes;           // stages of A (2 boxes; none on a diagonal tile) and 128 or 256 channels of B (2 or 4 boxes)
 constexpr uint32_t kCovTmemCols = 256;
 constexpr int kCovTailStages = 32;                       // the next launch may start when no more than these are left (10 - 20 us); unsplit tiles
                                                          // fill the chip: nothing to gain before they end
@@ -157,12 +157,12 @@ __global__ void __launch_bounds__(kCovThreads, 1)
 cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap map2,
               const __grid_constant__ CUtensorMap map4, const CovParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ uint64_t bars[2 * kCovStages + 1];
+  __shared__ uint64_t bars[2 * kCovMaxStages + 1];
   __shared__ uint32_t misc[2];                       // [0] TMEM base, [1] abort flag
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t bar_full = smem_u32(&bars[0]), bar_empty = smem_u32(&bars[kCovStages]);
-  const uint32_t bar_d = smem_u32(&bars[2 * kCovStages]);
+  const uint32_t bar_full = smem_u32(&bars[0]), bar_empty = smem_u32(&bars[kCovMaxStages]);
+  const uint32_t bar_d = smem_u32(&bars[2 * kCovMaxStages]);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CovAbort ab{reinterpret_cast<volatile int *>(&misc[1]), p.status, p.wait_limit};
 
@@ -180,17 +180,23 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
   const int b_boxes = p.bn / 64;
   // on a diagonal tile operand A is the slice of B that holds row block bi
   const uint32_t a_in_b = diag ? (uint32_t)((bi % ratio) * kOperandBytes) : 0u;
+  // A stage takes the room of the boxes that it has: 12 of them for blocks of up to 128 channels, whose only operand is 16 KB; with four, as
+  // off-diagonal tiles have, 64 KB in flight per SM paced 32 blocks of 128 channels (4096 tokens 14.5 us, now 12.9; 16384 33.6 and 28.8).
+  const int boxes = (diag ? 0 : 2) + b_boxes, n_ring = 24 / boxes;
+  const uint32_t stage_bytes = (uint32_t)boxes * kBoxBytes, b_at = diag ? 0u : (uint32_t)kOperandBytes;
   const int Z = kSplit ? p.splits : 1, z = kSplit ? (int)blockIdx.z : 0;
   const int n_stages_all = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
   const int s_begin = (int)((long long)n_stages_all * z / Z), n_stages_total = (int)((long long)n_stages_all * (z + 1) / Z) - s_begin;
 
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kCovStages; ++i) {
-      mbar_init(bar_full + 8 * i, 1);
-      mbar_init(bar_empty + 8 * i, 1);
+  if (warp == 0) {
+    if (lane < kCovMaxStages) {
+      mbar_init(bar_full + 8 * lane, 1);
+      mbar_init(bar_empty + 8 * lane, 1);
+    } else if (lane == 31) {
+      mbar_init(bar_d, 1);
+      misc[1] = 0;
+      asm volatile("prefetch.tensormap [%0];" ::"l"(p.use3d ? (b_boxes == 4 ? &map4 : &map2) : &xmap) : "memory");
     }
-    mbar_init(bar_d, 1);
-    misc[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -213,27 +219,27 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
       for (int s = 0; s < n_stages_total && !ab.set(); ++s, ++issued) {
         if (kSplit && s == max(0, n_stages_total - kCovTailStages)) cov_grid_dep_launch();
         if (!ab.wait(bar_empty + 8 * idx, lap ^ 1u)) break;
-        const uint32_t dst = base + idx * kStageBytes;
+        const uint32_t dst = base + idx * stage_bytes;
         const int tok = (s_begin + s) * kCovTokens;
-        mbar_arrive_expect_tx(bar_full + 8 * idx, (uint32_t)((diag ? 0 : 2) + b_boxes) * kBoxBytes);
+        mbar_arrive_expect_tx(bar_full + 8 * idx, stage_bytes);
         if (p.use3d) {
           if (!diag) tma_load_3d(dst, &map2, bar_full + 8 * idx, tok, col_a >> 6);
-          tma_load_3d(dst + kOperandBytes, b_boxes == 4 ? &map4 : &map2, bar_full + 8 * idx, tok, col_b >> 6);
+          tma_load_3d(dst + b_at, b_boxes == 4 ? &map4 : &map2, bar_full + 8 * idx, tok, col_b >> 6);
         } else {
           if (!diag) {
             tma_load_2d(dst, &xmap, bar_full + 8 * idx, col_a, tok);
             tma_load_2d(dst + kBoxBytes, &xmap, bar_full + 8 * idx, col_a + 64, tok);
           }
           for (int b = 0; b < b_boxes; ++b)
-            tma_load_2d(dst + kOperandBytes + b * kBoxBytes, &xmap, bar_full + 8 * idx, col_b + 64 * b, tok);
+            tma_load_2d(dst + b_at + b * kBoxBytes, &xmap, bar_full + 8 * idx, col_b + 64 * b, tok);
         }
-        if (++idx == kCovStages) idx = 0, lap ^= 1u;
+        if (++idx == n_ring) idx = 0, lap ^= 1u;
       }
       if (ab.set()) {  // let loads already in flight land before the CTA goes away
-        for (int back = 1; back <= kCovStages && back <= issued; ++back) {
+        for (int back = 1; back <= n_ring && back <= issued; ++back) {
           const int u = issued - back;
           for (int it = 0; it < kCovDrainPolls; ++it)
-            if (mbar_try_wait(bar_full + 8 * (u % kCovStages), (u / kCovStages) & 1)) break;
+            if (mbar_try_wait(bar_full + 8 * (u % n_ring), (u / n_ring) & 1)) break;
         }
       }
     }
@@ -247,13 +253,13 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
       for (int s = 0; s < n_stages_total; ++s) {
         if (!ab.wait(bar_full + 8 * idx, lap)) break;
         tc_fence_after();
-        const uint32_t b_addr = base + idx * kStageBytes + kOperandBytes;
+        const uint32_t b_addr = base + idx * stage_bytes + b_at;
         const uint64_t b = make_mn_desc(b_addr);
         const uint64_t a = make_mn_desc(diag ? b_addr + a_in_b : b_addr - kOperandBytes);
         tc_mma4_ss(tmem, a, b, idesc, accumulate);
         accumulate = 1;
         tc_commit_lane(bar_empty + 8 * idx);
-        if (++idx == kCovStages) idx = 0, lap ^= 1u;
+        if (++idx == n_ring) idx = 0, lap ^= 1u;
       }
       tc_commit_lane(bar_d);
       if (ab.set()) {  // MMAs already issued must retire before the tensor memory is given back
@@ -265,52 +271,52 @@ cov_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
     // ---------------- epilogue: TMEM -> shared (transposable staging) -> C += tile, C^T += tile^T
     const int quad = warp & 3;                        // warps 2..5 cover the four lane quadrants
     const int row = quad * 32 + lane;                 // tile row i = TMEM lane
+    cov_grid_dep_wait();                              // C may still be in use by the previous kernel
+    const int tid = threadIdx.x - 64;                 // 0..127
+    float *Cb = p.C + (long long)h * p.dh * p.dh;
+    const int i0 = bi * kCovTile, j0 = bj * p.bn;
+    const int r_begin = kCovTile * z / Z, r_end = kCovTile * (z + 1) / Z;   // rows of the tile that this CTA finishes
+    const int n_rows = min(r_end, p.dh - i0), n_cols = min(p.bn, p.dh - j0);   // both multiples of 8
+    // The update of C is latency-bound (read-modify-write through L2), so each thread keeps eight
+    // independent 16-byte loads in flight, the first of them under the main loop.  Direct part: C[i0 + r][j0 + 4 q .. + 3] += tile[r][4 q .. + 3].
+    const int quads = p.bn >> 2, sets = 128 / quads;  // 64 x 2 or 32 x 4 (column quads x interleaved row sets)
+    const int q = tid % quads, r_first = r_begin + tid / quads;
+    float *const dst = Cb + (long long)i0 * p.dh + j0 + 4 * q;
+    float4 old[8];
+    auto load_old = [&](int r0) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int r = r0 + sets * e;
+        old[e] = r < n_rows && 4 * q < n_cols ? __ldcg(reinterpret_cast<const float4 *>(dst + (long long)r * p.dh)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
+    load_old(r_first);
     bool have = ab.wait(bar_d, 0);
     have = __all_sync(0xffffffffu, have && !ab.set());
     float *stage = reinterpret_cast<float *>(gen);    // [128][bn + 1] fp32, reuses the operand ring
     const int pitch = p.bn + 1;
-    cov_grid_dep_wait();                              // C may still be in use by the previous kernel
     if (have) {
       tc_fence_after();
       cov_stage_row(tmem + ((uint32_t)(quad * 32) << 16), stage + row * pitch, p.bn);
     }
     cov_epi_bar();
-    const int r_begin = kCovTile * z / Z, r_end = kCovTile * (z + 1) / Z;   // rows of the tile that this CTA finishes
     if (Z > 1) {
       cov_cluster_sync();                             // every partial tile is staged
       if (!ab.set()) cov_sum_rows(smem_u32(stage), stage, pitch, p.bn, r_begin, r_end, Z, 1, 0u, (int)threadIdx.x - 64, 128);
       cov_epi_bar();
     }
     if (!ab.set()) {
-      const int tid = threadIdx.x - 64;               // 0..127
-      float *Cb = p.C + (long long)h * p.dh * p.dh;
-      const int i0 = bi * kCovTile, j0 = bj * p.bn;
-      // C[i0 + r][j0 + c] += tile[r][c]: a warp touches 32 consecutive floats of one row of C
-      // The update of C is latency-bound (read-modify-write through L2), so each thread keeps eight
-      // independent 16-byte loads in flight.  Direct part: C[i0 + r][j0 + 4 q .. + 3] += tile[r][4 q .. + 3].
-      const int n_rows = min(r_end, p.dh - i0), n_cols = min(p.bn, p.dh - j0);   // both multiples of 8
-      {
-        const int quads = p.bn >> 2, sets = 128 / quads;   // 64 x 2 or 32 x 4 (column quads x interleaved row sets)
-        const int q = tid % quads, r_first = tid / quads;
-        if (4 * q < n_cols) {
-          float *dst = Cb + (long long)i0 * p.dh + j0 + 4 * q;
-          for (int r0 = r_begin + r_first; r0 < n_rows; r0 += 8 * sets) {
-            float4 old[8];
+      if (4 * q < n_cols) {
+        for (int r0 = r_first; r0 < n_rows; r0 += 8 * sets) {
+          if (r0 != r_first) load_old(r0);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int r = r0 + sets * e;
-              old[e] = r < n_rows ? __ldcg(reinterpret_cast<const float4 *>(dst + (long long)r * p.dh))
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int r = r0 + sets * e;
-              if (r < n_rows) {
-                const float *t = stage + r * pitch + 4 * q;
-                *reinterpret_cast<float4 *>(dst + (long long)r * p.dh) =
-                    make_float4(__fadd_rn(old[e].x, t[0]), __fadd_rn(old[e].y, t[1]), __fadd_rn(old[e].z, t[2]),
-                                __fadd_rn(old[e].w, t[3]));
-              }
+          for (int e = 0; e < 8; ++e) {
+            const int r = r0 + sets * e;
+            if (r < n_rows) {
+              const float *t = stage + r * pitch + 4 * q;
+              *reinterpret_cast<float4 *>(dst + (long long)r * p.dh) =
+                  make_float4(__fadd_rn(old[e].x, t[0]), __fadd_rn(old[e].y, t[1]), __fadd_rn(old[e].z, t[2]),
+                              __fadd_rn(old[e].w, t[3]));
             }
           }
         }
@@ -679,7 +685,7 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
   p.n_tokens = n_tokens;
   p.status = ctx->d_status;
   p.wait_limit = ctx->wait_limit;
-  const size_t smem = 1024 + (size_t)kCovStages * kStageBytes;   // the 128 x (bn + 1) fp32 staging tile fits inside
+  const size_t smem = 1024 + (size_t)kCovRingBytes;      // the 128 x (bn + 1) fp32 staging tile fits inside
   const size_t smem2 = 1024 + (size_t)kPairStages * kPairStageBytes;
   static bool attr_done_all[64] = {};                    // function attributes are per device
   if (ctx->device < 0 || ctx->device >= 64) return ROSAQ_ERR_INVALID_ARG;
