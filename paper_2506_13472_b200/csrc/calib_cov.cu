@@ -623,6 +623,212 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   }
 }
 
+// =====================================================================================
+// The paired kernel for more tiles than the device holds pairs: every pair takes tiles in turn, with two accumulators, so that the
+// update of C (a read-modify-write of two megabytes per pair and tile, all pairs at once) runs under the next tile's main loop.
+// The ring is busy then, so the epilogue goes from tensor memory to C without staging: a thread has a row of the tile, its own
+// columns are 16 bytes at a time of one row of C, and the same values transposed are, lane by lane, 128 consecutive bytes.
+// 5120 channels, 210 tiles on 74 pairs, us: 600 tokens 89.7 -> 75, 4000 144 -> 128, 16384 347 -> 324 alone, 429 -> 423 in a loop under the power cap, where
+// the tensor work costs what it costs; 4096 channels at 6000 122 -> 111.  (Rows of C 32 bytes at a time: with 16 the launch reads C twice, 431 us.)
+// =====================================================================================
+// eight floats = one sector per lane; p on 32 bytes
+__device__ __forceinline__ void cov_ld8(const float *p, float *v) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void cov_st8(float *p, const float *v) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]),
+               "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+struct CovTile {
+  int h, i0, j0;             // block, first row (of this CTA) and column inside it
+  bool diag;
+};
+__device__ __forceinline__ CovTile cov_tile(int t, int tiles, uint32_t rank) {
+  const int h = t / tiles, k = t - h * tiles;
+  int bi = 0;
+  while ((bi + 1) * (bi + 2) / 2 <= k) ++bi;
+  const int bj = k - bi * (bi + 1) / 2;
+  return CovTile{h, bi * 256 + (int)rank * kCovTile, bj * 256, bi == bj};
+}
+
+__global__ void __launch_bounds__(kCovThreads, 1)
+cov_tc_tiles_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap map2, const CovParams p, int tiles, int n_tiles) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  __shared__ uint64_t bars[2 * kPairStages + 4];
+  __shared__ uint32_t misc[2];                       // [0] TMEM base, [1] abort flag
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t bar_tma = smem_u32(&bars[0]), bar_empty = smem_u32(&bars[kPairStages]);   // as in cov_tc_pair_kernel
+  const uint32_t bar_d = smem_u32(&bars[2 * kPairStages]);           // accumulators final (multicast commit)
+  const uint32_t bar_free = smem_u32(&bars[2 * kPairStages + 2]);    // leader's copy: accumulators read by the epilogues of both CTAs
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = blockIdx.x & 1u;
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const CovAbort ab{reinterpret_cast<volatile int *>(&misc[1]), p.status, p.wait_limit};
+  const int n_stages = (int)((p.n_tokens + kCovTokens - 1) / kCovTokens);
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kPairStages; ++i) {
+      mbar_init(bar_tma + 8 * i, 1);
+      mbar_init(bar_empty + 8 * i, 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar_d + 8 * i, 1);
+      mbar_init(bar_free + 8 * i, 8);                // the epilogue warps of both CTAs
+    }
+    misc[1] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&misc[0])), "n"(2 * kCovTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cov_cluster_sync();                                // the peer's barriers and tensor memory exist
+  tc_fence_after();
+  const uint32_t tmem = misc[0];
+
+  if (warp == 0) {
+    if (lane == 0) {
+      cov_grid_dep_wait();                           // X may be the previous kernel's output
+      const uint32_t lead_tma = map_to_rank(bar_tma, 0);
+      int issued = 0, idx = 0;
+      uint32_t lap = 0;
+      bool live = true;
+      for (int t = pair; t < n_tiles && live; t += n_pairs) {
+        const CovTile ct = cov_tile(t, tiles, rank);
+        const int col_a = ct.h * p.dh + ct.i0, col_b = ct.h * p.dh + ct.j0 + (int)rank * kCovTile;
+        const uint32_t stage_bytes = ct.diag ? kOperandBytes : kPairStageBytes;
+        for (int s = 0; s < n_stages; ++s, ++issued) {
+          if (ab.set() || !ab.wait(bar_empty + 8 * idx, lap ^ 1u)) {
+            live = false;
+            break;
+          }
+          const uint32_t dst = base + idx * kPairStageBytes, lb = lead_tma + 8 * idx;
+          const int tok = s * kCovTokens;
+          if (rank == 0) mbar_arrive_expect_tx(bar_tma + 8 * idx, 2 * stage_bytes);   // both CTAs' bytes
+          if (p.use3d) {
+            if (!ct.diag) tma_load_3d_pair(dst, &map2, lb, tok, col_a >> 6);
+            tma_load_3d_pair(dst + kOperandBytes, &map2, lb, tok, col_b >> 6);
+          } else {
+            if (!ct.diag) {
+              tma_load_2d_pair(dst, &xmap, lb, col_a, tok);
+              tma_load_2d_pair(dst + kBoxBytes, &xmap, lb, col_a + 64, tok);
+            }
+            tma_load_2d_pair(dst + kOperandBytes, &xmap, lb, col_b, tok);
+            tma_load_2d_pair(dst + kOperandBytes + kBoxBytes, &xmap, lb, col_b + 64, tok);
+          }
+          if (++idx == kPairStages) idx = 0, lap ^= 1u;
+        }
+      }
+      if (ab.set() && rank == 0) {                   // (see cov_tc_pair_kernel)
+        for (int back = 1; back <= kPairStages && back <= issued; ++back) {
+          const int u = issued - back;
+          for (int it = 0; it < kCovDrainPolls; ++it)
+            if (mbar_try_wait(bar_tma + 8 * (u % kPairStages), (u / kPairStages) & 1)) break;
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {
+      const uint32_t idesc = (1u << 4) | (1u << 15) | (1u << 16) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      int idx = 0, n = 0;
+      uint32_t lap = 0;
+      bool live = true;
+      for (int t = pair; t < n_tiles && live; t += n_pairs, ++n) {
+        const bool diag = cov_tile(t, tiles, 0).diag;
+        const int buf = n & 1;
+        if (!ab.wait(bar_free + 8 * buf, ((uint32_t)(n >> 1) & 1u) ^ 1u)) break;   // the tile before last has been read
+        tc_fence_after();
+        uint32_t accumulate = 0;
+        for (int s = 0; s < n_stages; ++s) {
+          if (!ab.wait(bar_tma + 8 * idx, lap)) {
+            live = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t b_addr = base + idx * kPairStageBytes + kOperandBytes;
+          const uint64_t b = make_mn_desc(b_addr), a = diag ? b : make_mn_desc(b_addr - kOperandBytes);
+          tc_mma4_ss_pair(tmem + buf * kCovTmemCols, a, b, idesc, accumulate);
+          accumulate = 1;
+          tc_commit_pair_lane(bar_empty + 8 * idx, 0);
+          if (++idx == kPairStages) idx = 0, lap ^= 1u;
+        }
+        if (live) tc_commit_pair_lane(bar_d + 8 * buf, 0);
+      }
+      if (ab.set()) {  // MMAs already issued must retire before the tensor memory is given back
+        const uint32_t bar = bar_d + 8 * (n & 1);    // (its phase of this tile has not been committed)
+        tc_commit_pair_lane(bar, 0);
+        for (int it = 0; it < kCovDrainPolls; ++it)
+          if (mbar_try_wait(bar, (uint32_t)(n >> 1) & 1u)) break;
+      }
+    }
+  } else {
+    const int quad = warp & 3, row = quad * 32 + lane;
+    cov_grid_dep_wait();                             // C may still be in use by the previous kernel
+    int n = 0;
+    for (int t = pair; t < n_tiles; t += n_pairs, ++n) {
+      const CovTile ct = cov_tile(t, tiles, rank);
+      const int buf = n & 1;
+      const bool got = ab.wait(bar_d + 8 * buf, (uint32_t)(n >> 1) & 1u);
+      if (!__all_sync(0xffffffffu, got && !ab.set())) break;
+      tc_fence_after();
+      const int gi = ct.i0 + row, n_cols = min(256, p.dh - ct.j0);
+      const bool live = gi < p.dh;
+      float *const Cb = p.C + (long long)ct.h * p.dh * p.dh;
+      float *direct = Cb + (long long)gi * p.dh + ct.j0;
+      float *mirror = Cb + (long long)ct.j0 * p.dh + gi;
+      for (int c0 = 0; c0 < n_cols; c0 += 32, direct += 32, mirror += 32ll * p.dh) {
+        uint32_t v[32];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                       : "=r"(v[8 * q]), "=r"(v[8 * q + 1]), "=r"(v[8 * q + 2]), "=r"(v[8 * q + 3]), "=r"(v[8 * q + 4]), "=r"(v[8 * q + 5]),
+                         "=r"(v[8 * q + 6]), "=r"(v[8 * q + 7])
+                       : "r"(tmem + ((uint32_t)(quad * 32) << 16) + buf * kCovTmemCols + c0 + 8 * q)
+                       : "memory");
+        float od[32], om[32];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (live && c0 + 8 * k < n_cols) cov_ld8(direct + 8 * k, od + 8 * k);
+        if (!ct.diag) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e)
+            if (live && c0 + e < n_cols) om[e] = __ldcg(mirror + (long long)e * p.dh);
+        }
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int e = 0; e < 32; ++e) od[e] = __fadd_rn(od[e], __uint_as_float(v[e]));
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (live && c0 + 8 * k < n_cols) cov_st8(direct + 8 * k, od + 8 * k);
+        if (!ct.diag) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e)
+            if (live && c0 + e < n_cols) mirror[(long long)e * p.dh] = __fadd_rn(om[e], __uint_as_float(v[e]));
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(map_to_rank(bar_free + 8 * buf, 0)) : "memory");
+    }
+  }
+
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  cov_cluster_sync();                                // neither CTA leaves while the pair's MMAs may touch it
+  if (warp == 1) {
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(2 * kCovTmemCols) : "memory");
+  }
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -698,7 +904,8 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
       if (cudaFuncSetAttribute(cov_tc_kernel<false>, kAttr, (int)smem) != cudaSuccess ||
           cudaFuncSetAttribute(cov_tc_kernel<true>, kAttr, (int)smem) != cudaSuccess ||
           cudaFuncSetAttribute(cov_tc_pair_kernel<false>, kAttr, (int)smem2) != cudaSuccess ||
-          cudaFuncSetAttribute(cov_tc_pair_kernel<true>, kAttr, (int)smem2) != cudaSuccess) {
+          cudaFuncSetAttribute(cov_tc_pair_kernel<true>, kAttr, (int)smem2) != cudaSuccess ||
+          cudaFuncSetAttribute(cov_tc_tiles_kernel, kAttr, (int)smem2) != cudaSuccess) {
         (void)cudaGetLastError();
         return ROSAQ_ERR_CUDA;
       }
@@ -729,6 +936,8 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
   const int z1 = splits((long long)tiles * n_blocks, 1), z2 = splits(2ll * pair_tiles * n_blocks, 2);
   if (dh >= 512 && z2 >= z1) {
     p.splits = z2;
+    const int n_tiles = pair_tiles * n_blocks, pairs = ctx->sm_count / 2;
+    if (n_tiles > pairs && reinterpret_cast<uintptr_t>(C) % 32 == 0) return cov_launch(cov_tc_tiles_kernel, dim3(2 * pairs, 1, 1), kCovThreads, smem2, 2, 1, s, xmap, map2, p, pair_tiles, n_tiles);
     return cov_launch(z2 > 1 ? cov_tc_pair_kernel<true> : cov_tc_pair_kernel<false>, dim3(2 * pair_tiles, n_blocks, z2), kCovThreads, smem2, 2, z2, s, xmap, map2, p);
   }
   p.splits = z1;

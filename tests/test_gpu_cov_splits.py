@@ -132,3 +132,31 @@ def test_calib_cov_either_step_of_the_fp32_kernel(n_tokens, n_blocks):
     got = Cg.cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - Cref) <= H.cov_tolerance(Cref, n_tokens) + 1e-30)
     assert np.array_equal(got, np.swapaxes(got, -1, -2))
+
+
+@pytest.mark.parametrize("n_tokens,d,n_blocks", [(130, 3000, 1), (64, 3072, 1), (200, 4608, 2), (1, 4104, 1)])
+def test_calib_cov_more_tiles_than_pairs(n_tokens, d, n_blocks):
+    """78 to 153 tiles for the 74 pairs of 148 SMs: pairs that take a second and a third tile while the first is added to C.  A C that does
+    not lie on 32 bytes takes the kernel with a pair per tile, whose bits it has to give; tokens and channels that fill no whole tile."""
+    dh = d // n_blocks
+    X = (torch.randn((n_tokens, d), generator=torch.Generator().manual_seed(51)) * torch.linspace(2, 0.1, d)).half().cuda()
+    ctx = rb.Context(0)
+    try:
+        got = []
+        for off in (0, 4):
+            C = torch.empty(n_blocks * dh * dh + 8, device="cuda")[off:off + n_blocks * dh * dh].view(n_blocks, dh, dh)
+            assert C.data_ptr() % 32 == 4 * off
+            C.fill_(0.5)
+            ctx.calib_cov(X, C, n_blocks)
+            ctx.calib_cov(X[:n_tokens // 2 + 1], C, n_blocks)
+            got.append(C)
+        assert ctx.last_status() == rb.ROSAQ_OK
+    finally:
+        ctx.close()
+    assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[0].transpose(1, 2))
+    Xd = X.double().view(n_tokens, n_blocks, dh).transpose(0, 1)
+    Xh = Xd[:, :n_tokens // 2 + 1]
+    want = Xd.transpose(1, 2) @ Xd + Xh.transpose(1, 2) @ Xh
+    diag = want.diagonal(dim1=1, dim2=2)
+    bound = (n_tokens / 16 + 12) * 2.0 ** -23 * (diag[:, :, None] * diag[:, None, :]).sqrt() + 1e-6   # (0.5 and two sums rounded)
+    assert torch.all((got[0].double() - 0.5 - want).abs() <= bound)
