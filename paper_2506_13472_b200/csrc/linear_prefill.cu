@@ -67,6 +67,7 @@ static_assert(128 * kPfRegsRoles + kPfTeams * kTeamThreads * kPfRegsDequant + kP
 constexpr int kPfMaxNW = 16;                        // weight slots (a multiple of the teams)
 constexpr int kPfMaxSmemBytes = 227 * 1024;
 constexpr int kPfMaxProblems = 4;
+constexpr int kPfMaxPairs = 96;                     // of a launch cut into equal shares
 constexpr int kPfMaxSplits = 4;                     // pairs in a cluster (eight CTAs: the portable limit)
 constexpr int kDenseBits = 16;                      // an operand without quantized groups
 constexpr int kPdEpiWarp = 4, kPdThreads = kPdEpiWarp * 32 + kPfEpiThreads;   // 384
@@ -74,7 +75,7 @@ constexpr int kPdMaxStages = 8;                     // stages of 64 channels
 constexpr int kPdABytes = kFp16TileBytes / 2;       // 64 channels x 128 columns
 
 struct alignas(64) PfParams {
-  CUtensorMap xmap;
+  CUtensorMap xmap, xmap_last;                      // boxes of NT / 2 tokens, of NT_last / 2
   CUtensorMap wmap[kPfMaxProblems];                 // all-fp16 operands: the blob as rows of 128 bytes
   int n_prob;
   int pair_start[kPfMaxProblems + 1];
@@ -86,6 +87,7 @@ struct alignas(64) PfParams {
   int g_fp16, groups, block_groups;
   int n_tok_blocks, M;
   int NT;                     // tokens per tile (a multiple of 32); a CTA keeps NT / 2 rows of x in shared memory
+  int NT_last;                // of the tiles of the last token block, which may hold fewer
   int NW;                     // weight slots; all-fp16 operands: stages
   int units;                  // (column pairs x token blocks) x groups
   int S;
@@ -93,18 +95,12 @@ struct alignas(64) PfParams {
   unsigned *flags;            // [pair][2][rank]: readers that still have to fetch from the slot
   int *status;
   long long wait_limit;
+  int bounds[kPfMaxPairs + 1];   // S = 0: pair i holds the units [bounds[i], bounds[i + 1])
 };
 
-__device__ __forceinline__ int pf_range_begin(int pair, int n_pairs, int units) {
-  return (int)(((long long)pair * units) / n_pairs);
-}
-// the pair whose range holds unit u
-__device__ __forceinline__ int pf_owner(int u, int n_pairs, int units) {
-  int q = (int)(((long long)u * n_pairs) / units);
-  while (q + 1 < n_pairs && pf_range_begin(q + 1, n_pairs, units) <= u) ++q;
-  while (q > 0 && pf_range_begin(q, n_pairs, units) > u) --q;
-  return q;
-}
+// whether work item wk is a tile of the last token block, and its tokens
+__device__ __forceinline__ bool pf_last_block(const PfParams &p, int wk) { return (wk + 1) % p.n_tok_blocks == 0; }
+__device__ __forceinline__ int pf_tokens(const PfParams &p, int wk) { return pf_last_block(p, wk) ? p.NT_last : p.NT; }
 // next piece of the range [u, end): groups [g0, g1) of work item wk; false when the range is used up
 __device__ __forceinline__ bool pf_next_piece(int &u, int end, int G, int &wk, int &g0, int &g1) {
   if (u >= end) return false;
@@ -252,7 +248,7 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
     const int wk0 = (pair / S) * G;
     u_begin = wk0 + G * split / S, u_end = wk0 + G * (split + 1) / S;
   } else {
-    u_begin = pf_range_begin(pair, n_pairs, p.units), u_end = pf_range_begin(pair + 1, n_pairs, p.units);
+    u_begin = p.bounds[pair], u_end = p.bounds[pair + 1];
   }
   const Abort ab{reinterpret_cast<volatile int *>(misc_ptr + 1), p.status, p.wait_limit};
   grid_dep_launch_dependents();
@@ -301,7 +297,9 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
           const int prob = pf_problem(p, wk, col_pair);
           const int my_tile = min(2 * col_pair + (int)rank, p.n_tiles[prob] - 1);
           const int a_row0 = (int)((long long)my_tile * p.tile_stride >> 7);     // rows of 128 bytes
-          const int tok0 = (wk % p.n_tok_blocks) * NT + (int)rank * rows;
+          const int n_tok = pf_tokens(p, wk), tok0 = (wk % p.n_tok_blocks) * NT + (int)rank * (n_tok >> 1);
+          const CUtensorMap *const xmap = n_tok == NT ? &p.xmap : &p.xmap_last;
+          const uint32_t bytes = 2 * (kPdABytes + (uint32_t)(n_tok >> 1) * 128u);
           // block-diagonal operand: the pair of column tiles multiplies the channels of its own diagonal block
           const int g_block0 = p.block_groups > 0 ? (2 * col_pair / p.block_groups) * p.block_groups : 0;
           for (int h = 2 * g0; h < 2 * g1; ++h, ++issued, rs.advance(NW)) {
@@ -309,10 +307,10 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
               live = false;
               break;
             }
-            if (is_lead) mbar_arrive_expect_tx(bar_w_full + 8 * rs.idx, 2 * d_stage_bytes);
+            if (is_lead) mbar_arrive_expect_tx(bar_w_full + 8 * rs.idx, bytes);
             const uint32_t bar = map_to_rank(bar_w_full + 8 * rs.idx, lead), dst = base + rs.idx * d_stage_bytes;
             tma_load_2d_pair(dst, &p.wmap[prob], bar, 0, a_row0 + h * (kPdABytes / 128));
-            tma_load_3d_pair(dst + kPdABytes, &p.xmap, bar, tok0, 2 * g_block0 + h);
+            tma_load_3d_pair(dst + kPdABytes, xmap, bar, tok0, 2 * g_block0 + h);
           }
         }
         // (the leader's barriers count the copies of both CTAs, and the peer stays until the cluster barrier
@@ -360,7 +358,8 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
         bool live = true;
         int u = u_begin, wk, g0, g1;
         while (live && !ab.set_all() && pf_next_piece(u, u_end, G, wk, g0, g1)) {
-          const int tok0 = (wk % p.n_tok_blocks) * NT + (int)rank * rows;
+          const int n_tok = pf_tokens(p, wk), tok0 = (wk % p.n_tok_blocks) * NT + (int)rank * (n_tok >> 1);
+          const CUtensorMap *const xmap = n_tok == NT ? &p.xmap : &p.xmap_last;
           for (int g = g0; g < g1; ++g, ++gc, rs.advance(kPfStages)) {
             const int slot = rs.idx;
             if (!ab.wait_all(bar_s_empty + 8 * slot, rs.lap ^ 1u)) {
@@ -369,8 +368,8 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
             }
             // all bytes are counted on the leader's barrier
             if (elect_one()) {
-              if (is_lead) mbar_arrive_expect_tx(bar_a_full + 8 * slot, 2 * x_slot_bytes);
-              tma_load_3d_pair(x_ring + slot * x_slot_bytes, &p.xmap, map_to_rank(bar_a_full + 8 * slot, lead), tok0, 2 * g);
+              if (is_lead) mbar_arrive_expect_tx(bar_a_full + 8 * slot, (uint32_t)n_tok * 256u);
+              tma_load_3d_pair(x_ring + slot * x_slot_bytes, xmap, map_to_rank(bar_a_full + 8 * slot, lead), tok0, 2 * g);
             }
             __syncwarp();
           }
@@ -386,9 +385,8 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
     } else if (warp == 2) {
       // ---------------- MMA issuer (leader): per group one wait, eight MMAs of 256 x NT x 16, one commit (dense: half a group)
       if (is_lead) {
-        const uint32_t idesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | (16u << 24);
         const uint64_t desc0 = make_b_desc(kDense ? base + kPdABytes : x_ring), adesc0 = make_a_desc(base);
-        const uint32_t slot16 = (kDense ? d_stage_bytes : x_slot_bytes) >> 4, half16 = (uint32_t)(rows * 128) >> 4;
+        const uint32_t slot16 = (kDense ? d_stage_bytes : x_slot_bytes) >> 4;
         Ring rs{0, 0};
         int n_done = 0;
         bool live = true, issued = false;
@@ -398,26 +396,30 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
           if (!ab.wait_all(bar_d_empty + 8 * buf, (uint32_t)((n_done / kAcc) & 1) ^ 1u)) break;   // the last piece in it has been drained
           tc_fence_after();
           const uint32_t d_tmem = tmem + buf * kPfMaxTokens;
-          uint32_t accumulate = 0;
           const int n = (g1 - g0) * (kDense ? 2 : 1);
-          for (int i = 0; i < n; ++i, rs.advance(kDense ? NW : kPfStages)) {
-            const int st = rs.idx;
-            if (!ab.wait_all((kDense ? bar_w_full : bar_a_full) + 8 * st, rs.lap)) {
-              live = false;
-              break;
+          // (n_tok comes straight from the parameters in either call, so the descriptors stay in uniform registers: selected, each MMA moved
+          // them there, and launches of equal blocks were 2 to 5 % slower)
+          auto run = [&](const int n_tok) {
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(n_tok >> 3) << 17) | (16u << 24), half16 = (uint32_t)n_tok * 4u;   // (n_tok / 2 rows of 128 bytes)
+            uint32_t accumulate = 0;
+            for (int i = 0; i < n; ++i, rs.advance(kDense ? NW : kPfStages)) {
+              const int st = rs.idx;
+              if (!ab.wait_all((kDense ? bar_w_full : bar_a_full) + 8 * st, rs.lap)) return false;
+              tc_fence_after();
+              const uint64_t b0 = desc0 + (uint64_t)(st * slot16);
+              if (kDense) {
+                tc_mma4_ss_pair(d_tmem, adesc0 + (uint64_t)(st * slot16), b0, idesc, accumulate);
+                tc_commit_mc(bar_w_empty + 8 * st, pair_mask);   // frees the stage in both CTAs
+              } else {
+                tc_mma8_ts_pair(d_tmem, tmem + a_col0 + st * 64, b0, b0 + (uint64_t)half16, idesc, accumulate);
+                tc_commit_mc(bar_s_empty + 8 * st, pair_mask);
+              }
+              accumulate = 1;
+              issued = true;
             }
-            tc_fence_after();
-            const uint64_t b0 = desc0 + (uint64_t)(st * slot16);
-            if (kDense) {
-              tc_mma4_ss_pair(d_tmem, adesc0 + (uint64_t)(st * slot16), b0, idesc, accumulate);
-              tc_commit_mc(bar_w_empty + 8 * st, pair_mask);   // frees the stage in both CTAs
-            } else {
-              tc_mma8_ts_pair(d_tmem, tmem + a_col0 + st * 64, b0, b0 + (uint64_t)half16, idesc, accumulate);
-              tc_commit_mc(bar_s_empty + 8 * st, pair_mask);
-            }
-            accumulate = 1;
-            issued = true;
-          }
+            return true;
+          };
+          live = pf_last_block(p, wk) ? run(p.NT_last) : run(p.NT);
           if (!live) break;
           tc_commit_mc(bar_d_full + 8 * buf, pair_mask);
         }
@@ -525,8 +527,11 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
       const int tok0 = (wk % p.n_tok_blocks) * NT;
       const int n_blk = (min(NT, p.M - tok0) + 15) >> 4;       // blocks of sixteen tokens in this tile
       // the pairs `first` .. `last` hold the tile's groups, ascending K
-      const int first = S > 0 || g0 == 0 ? pair : pf_owner(wk * G, n_pairs, p.units);
-      const int last = S > 0 || g1 == G ? pair : pf_owner(wk * G + G - 1, n_pairs, p.units);
+      int first = pair, last = pair;
+      if (S == 0) {
+        while (p.bounds[first] > wk * G) --first;
+        while (p.bounds[last + 1] < (wk + 1) * G) ++last;
+      }
       const int closers = last - first;                        // all holders but the last share the tile's token rows
       if (closers == 0) {
         // the whole tile is here: round it into registers, give the accumulator back, then store
@@ -812,10 +817,12 @@ PrefillCut prefill_choose(rosaq_ctx *ctx, int M, int n, const TiledOperand *cons
   const int blocks = (M + kPfMaxTokens - 1) / kPfMaxTokens;
   best.NT = ((M + blocks - 1) / blocks + 31) / 32 * 32;
   best.n_tok_blocks = (M + best.NT - 1) / best.NT;
+  best.NT_last = (M - (best.n_tok_blocks - 1) * best.NT + 31) / 32 * 32;
   const double NT = best.NT, tiles = (double)col_pairs * best.n_tok_blocks, half = ctx->sm_count / 4;
+  const double whole = (double)col_pairs * (best.n_tok_blocks - 1 + best.NT_last / NT);   // tiles of NT tokens that are as much work
   {
     const Shares &f = dense ? kSharesDense : kSharesQuant;
-    const double units = tiles * G, pairs = std::max(1.0, std::min((double)prefill_clusters(ctx, 1), units));
+    const double units = whole * G, pairs = std::max(1.0, std::min((double)prefill_clusters(ctx, 1), units));
     best.S = 0;
     best.us = f.launch + f.token * NT + units / pairs * (f.group + f.group_token * NT) + f.holder * std::max(0.0, pairs / tiles - 2) + f.tile * tiles / pairs;
   }
@@ -859,6 +866,7 @@ int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx,
   p.block_groups = t.block_groups;
   p.M = M;
   p.NT = cut.NT;
+  p.NT_last = cut.NT_last;
   p.n_tok_blocks = cut.n_tok_blocks;
   p.S = cut.S;
   const bool dense = t.g_quant == 0;
@@ -878,6 +886,12 @@ int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return ROSAQ_ERR_CUDA;
+  const cuuint32_t box_last[3] = {64, (cuuint32_t)(p.NT_last / 2), box[2]};
+  p.xmap_last = p.xmap;
+  if (p.NT_last != p.NT &&
+      encode(&p.xmap_last, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half *>(x), dims, strides, box_last, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return ROSAQ_ERR_CUDA;
   for (int i = 0; i < n && dense; ++i) {
     const cuuint64_t wdims[2] = {64, (cuuint64_t)(ts[i]->bytes / 128)}, wstrides[1] = {128};
     const cuuint32_t wbox[2] = {64, kPdABytes / 128}, west[2] = {1, 1};
@@ -888,7 +902,23 @@ int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx,
   const long long tiles = (long long)col_pairs * p.n_tok_blocks, units = tiles * p.groups;
   if (units < 1 || units > (1ll << 30)) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
   p.units = (int)units;
-  const int n_pairs = p.S > 0 ? (int)tiles * p.S : (int)std::min<long long>(units, max_pairs);
+  const int n_pairs = p.S > 0 ? (int)tiles * p.S : (int)std::min<long long>(units, std::min(max_pairs, kPfMaxPairs));
+  // The cut into equal shares: pair i begins at the first unit that i n-ths of the cost lie before.  A unit of the last token block
+  // costs less when that block holds fewer tokens: 1900 are seven blocks of 256 and one of 108, which takes 128.  A unit costs what its tokens
+  // do and about 100 tokens more.  us, all blocks of NT / this, in a loop: 4096 -> 3 x 4096 at 600 tokens 68.1 / 61.1, at 1570 145.8 / 139.9, at 1900 169.4 / 162.4;
+  // 4096 -> 2 x 11008 at 900 153.5 / 145.1, at 1900 290.4 / 280.4; dense rotation of 5120 at 1900 104.0 / 99.0.  (No range may be empty, so each has
+  // to be worth a unit.)
+  if (p.S == 0) {
+    const int fixed = dense ? 4 : 3;                         // of a group, in 32 tokens
+    long long cost = p.NT / 32 + fixed, cost_last = p.NT_last / 32 + fixed;
+    const long long G = p.groups, nb = p.n_tok_blocks;
+    if (col_pairs * G * ((nb - 1) * cost + cost_last) < n_pairs * cost) cost = cost_last = 1;
+    const long long head = (nb - 1) * G * cost, per_col = head + G * cost_last;
+    for (int i = 0; i <= n_pairs; ++i) {
+      const long long c = i * (col_pairs * per_col) / n_pairs, col = c / per_col, rest = c - col * per_col;
+      p.bounds[i] = (int)(col * G * nb + (rest <= head ? (rest + cost - 1) / cost : (nb - 1) * G + (rest - head + cost_last - 1) / cost_last));
+    }
+  }
   // two slots of 2 x NT x 128 floats per pair, (launches of one context do not overlap on the GPU)
   if (p.S == 0 && ctx->pf_partial_bytes < (size_t)n_pairs * 4 * p.NT * kTileN * sizeof(float)) return ROSAQ_ERR_ALLOC;
   p.partials = ctx->pf_partials;

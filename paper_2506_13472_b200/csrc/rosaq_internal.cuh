@@ -437,6 +437,7 @@ int launch_rotate_linear_small(const rosaq_ctx *ctx, const __half *x, int M, lon
 bool prefill_supported(const TiledOperand &t, const int32_t *col_map);
 struct PrefillCut {
   int NT = 0, n_tok_blocks = 0;   // tokens per tile
+  int NT_last = 0;                // of those of the last token block
   int S = 0;                      // > 0: a cluster of S pairs per tile; 0: equal shares of the whole launch
   double us = 0;                  // estimate
 };

@@ -156,3 +156,29 @@ def test_column_order_in_tiles_of_sixteen_tokens(ctx, d, M):
     assert same(buf[:M, :d].contiguous(), want.contiguous())
     assert torch.all(buf[M:] == 7.0) and torch.all(buf[:, d:] == 7.0)
     assert ctx.last_status() == rb.ROSAQ_OK
+
+
+@pytest.mark.parametrize("M", [257, 600, 1570, 1793])
+def test_last_token_block_of_its_own_size(ctx, M):
+    """Token blocks of 160 and 128, 224 and 160, 256 and 64, 256 and 32: equal shares of uneven units (64 to 128 tiles of 512 channels) and, for
+    the head-wise rotation, clusters."""
+    d, n = 512, 4096
+    rng = synth.rng_for(97, "last", M)
+    x = dev(rng.standard_normal((M, d)).astype(np.float16))
+    w = ctx.quantize(dev(synth.weights(d, n, seed=97, key="last", outlier_frac=0.01)), None, bits=4, k_salient=128)
+    xw = dev(rng.standard_normal((M, n)).astype(np.float16))
+    dense = ctx.rotation_create(dev((rng.standard_normal((n, n)) / n ** 0.5).astype(np.float16)))
+    heads = ctx.rotation_create(dev((rng.standard_normal((n // 128, 128, 128)) / 128 ** 0.5).astype(np.float16)))
+    for call, args in ((ctx.linear, (x, w)), (ctx.rotate, (xw, dense)), (ctx.rotate, (xw, heads))):
+        ctx.set_linear_impl(3)
+        ref = call(*args).clone()
+        ctx.set_linear_impl(5)
+        buf = torch.full((M + 1, n + 8), 7.0, dtype=torch.float16, device="cuda")
+        runs = []
+        for _ in range(2):
+            call(*args, out=buf[:M, :n])
+            runs.append(buf[:M, :n].clone())
+        ctx.set_linear_impl(0)
+        assert same(runs[0], runs[1]) and torch.all(buf[M:] == 7.0) and torch.all(buf[:, n:] == 7.0)
+        assert H.rel_fro(runs[0].cpu().numpy(), ref.cpu().numpy()) <= 2e-4
+    assert ctx.last_status() == rb.ROSAQ_OK
