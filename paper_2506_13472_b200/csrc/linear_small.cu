@@ -3,7 +3,7 @@
 // Why another kernel.  At a few tokens a launch of the tcgen05 kernel is bound by its latencies, not by the weight stream: every
 // group is a chain through tensor memory (dequantise, store, barrier, eight MMAs, commit),
 // and the splits of K meet in a cluster exchange of several microseconds before the next launch can begin.  Here
-//   * a CTA owns a slice of 32 output columns and ALL of K, so nothing is exchanged between CTAs: its eight warps take the
+//   * a CTA owns a slice of 32 output columns and ALL of K, so nothing is exchanged between CTAs: its eight or sixteen warps take the
 //     units of K in turn (a unit = a quantized group, or 32 channels of an fp16 group: 2 KB of a slice either way) and the
 //     partial sums are added once, in shared memory, in warp order (the sums do not depend on timing);
 //   * a warp streams its units on its own, with 16-byte asynchronous copies into a ring of its own: no barrier is shared with
@@ -16,8 +16,8 @@
 // What bounds it: at 4096 -> 2 x 11008 the issue slots (362 instructions per unit of 2176 bytes, 0.57 issued per cycle and
 // scheduler), at the smaller ones the last round of CTAs and the time to start.  Measured in a graph of distinct weights (us,
 // INT4, one token; tcgen05 kernel / this one): 512 -> 512 3.3 / 1.6, 4096 -> 4096 7.7 / 4.4, 4096 -> 3 x 4096 13.9 / 9.2,
-// 4096 -> 2 x 11008 19.9 / 14.3 (3.2 TB/s), 11008 -> 4096 13.1 / 9.2, rotations: dense 4096 9.9 / 6.8 (4.9 TB/s), head-wise
-// 4096 4.1 / 1.95; eight tokens: 7.8 / 5.3, 14.1 / 12.9, 20.1 / 19.8, 13.3 / 11.5, 10.0 / 7.4, 4.7 / 3.0.
+// 4096 -> 2 x 11008 19.9 / 14.3 (3.2 TB/s), 11008 -> 4096 13.1 / 8.6, rotations: dense 4096 9.9 / 6.8 (4.9 TB/s), head-wise
+// 4096 4.1 / 1.95; eight tokens: 7.8 / 5.3, 14.1 / 12.9, 20.1 / 19.8, 13.3 / 11.6, 10.0 / 7.4, 4.7 / 3.0.
 //
 // Which channel sits in which k position of an MMA is free as long as both operands agree, so a thread feeds it the codes of
 // the 16-byte chunk it loads: thread t of a quad takes channels 32 t .. 32 t + 31 of a quantized group (INT4: chunk t, INT3:
@@ -37,6 +37,7 @@ constexpr int kSmRow = kSmSlice * 16 + 32;                       // bytes from o
 constexpr int kSmStage = 4 * kSmRow + kSmSlice * 4;              // 2304: rows, then scales and zero-points
 constexpr int kSmWarps = 8;                                      // a multiple of 4: all fp16 units of a warp are the same quarter of a group
 constexpr int kSmThreads = kSmWarps * 32;
+constexpr int kSmWarpsLong = 16;                                 // of a CTA that has an SM and many units to itself
 constexpr int kSmCtas = 3;                                       // resident CTAs per SM at most (80 registers)
 constexpr int kSmSharedSm = 228 * 1024, kSmSharedCta = 1024;     // shared memory of an SM, and what the system takes of it per CTA
 constexpr int kSmMaxProblems = 4;
@@ -199,8 +200,10 @@ __device__ __forceinline__ uint32_t sm_missing(uint32_t v) {
   return (t - 0x00010001u) & ~t & 0x80008000u;
 }
 
-template <int kBits, int STAGES, SmRole kRole>
+template <int kBits, int STAGES, int kWarps, SmRole kRole>
 __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, int block, const SmPair *pair) {
+  constexpr int kThreads = kWarps * 32;
+  static_assert(kWarps % 4 == 0 && kWarps >= kSmallTokens, "all fp16 units of a warp are the same quarter of a group; a token per warp");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   grid_dep_launch_dependents();
@@ -221,7 +224,7 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
   const int x_row = (u_fp16 * 32 + (n_units - u_fp16) * kGroup) * 2;
   const uint32_t x_smem = smem_u32(smem), ring = x_smem + M * x_row + warp * (STAGES * kSmStage), ring_end = ring + STAGES * kSmStage;
 
-  // ---- this warp's units are warp, warp + kSmWarps, ...; the weights do not depend on the launches before
+  // ---- this warp's units are warp, warp + kWarps, ...; the weights do not depend on the launches before
   constexpr int rows = kBits == 4 ? 4 : 3, quant_bytes = rows * kTileN * 16 + kScaleBytes;
   const uint8_t *const base16 = p.blob[prob] + (long long)tile * p.tile_stride + col * 16 + lane * 16;
   const uint8_t *const baseq = base16 + (long long)u_fp16 * kFp16SubBytes;
@@ -242,7 +245,7 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
   };
   int f = warp;
 #pragma unroll
-  for (int s = 0; s < STAGES; ++s, f += kSmWarps) fetch(ring + s * kSmStage, f);
+  for (int s = 0; s < STAGES; ++s, f += kWarps) fetch(ring + s * kSmStage, f);
 
   grid_dep_wait();                                               // x may be the previous kernel's output, y its input
   __half *between = nullptr;
@@ -251,19 +254,19 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
     between = pair->between + turn * kSmBetween;
     if (kRole == kSmProducer) {
       uint4 *other = reinterpret_cast<uint4 *>(pair->between + (turn ^ 1u) * kSmBetween);
-      for (int i = block * kSmThreads + threadIdx.x; i < kSmBetween / 8; i += pair->n_rot * kSmThreads) other[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+      for (int i = block * kThreads + threadIdx.x; i < kSmBetween / 8; i += pair->n_rot * kThreads) other[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
     }
   }
   if (kRole == kSmConsumer) {
     int ok = 1;
     const int n_full = x_row >> 4, n_all = M * n_full;
-    for (int i0 = threadIdx.x; i0 < n_all && ok; i0 += 4 * kSmThreads) {   // four chunks in flight
+    for (int i0 = threadIdx.x; i0 < n_all && ok; i0 += 4 * kThreads) {   // four chunks in flight
       uint4 v[4];
       for (long long it = 0;; ++it) {
         uint32_t missing = 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const int i = min(i0 + k * kSmThreads, n_all - 1);
+          const int i = min(i0 + k * kThreads, n_all - 1);
           asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
                        : "=r"(v[k].x), "=r"(v[k].y), "=r"(v[k].z), "=r"(v[k].w)
                        : "l"(between + 8 * i)
@@ -279,7 +282,7 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int i = i0 + k * kSmThreads, r = i / n_full;
+        const int i = i0 + k * kThreads, r = i / n_full;
         if (i < n_all) *reinterpret_cast<uint4 *>(smem + r * x_row + x_pos(r, i - r * n_full)) = v[k];
       }
     }
@@ -296,7 +299,7 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
     const int n_full = x_row >> 4;
     for (int r = 0; r < M; ++r, xs += p.ldx) {
       uint32_t dst = x_smem + r * x_row + x_pos(r, threadIdx.x);
-      for (int c = threadIdx.x; c < n_full; c += kSmThreads, dst += kSmThreads * 16) cp_async16(dst, xs + (c - (int)threadIdx.x) * 8);
+      for (int c = threadIdx.x; c < n_full; c += kThreads, dst += kThreads * 16) cp_async16(dst, xs + (c - (int)threadIdx.x) * 8);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -314,17 +317,17 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
   auto next = [&] {
     __syncwarp();                                                // every lane has read the stage
     fetch(st, f);
-    f += kSmWarps;
+    f += kWarps;
     st += kSmStage;
     if (st == ring_end) st = ring;
   };
-  for (; u < u_fp16; u += kSmWarps) {
+  for (; u < u_fp16; u += kWarps) {
     cp_async_wait<STAGES - 1>();
     __syncwarp();
     unit_fp16(st + t * kSmRow + g * 16, lds128(x16 + (u >> 2) * (kGroup * 2)), acc);
     next();
   }
-  for (; u < n_units; u += kSmWarps) {
+  for (; u < n_units; u += kWarps) {
     cp_async_wait<STAGES - 1>();
     __syncwarp();
     const uint32_t x_unit = (u - u_fp16) * (kGroup * 2), scales = st + 4 * kSmRow + g * 4;
@@ -345,10 +348,10 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
     }
   __syncthreads();
   const int nn = tile * kTileN + col + lane;
-  if (warp < M && nn < p.d_out[prob]) {                          // (kSmallTokens = kSmWarps: a token per warp)
+  if (warp < M && nn < p.d_out[prob]) {                          // (a token per warp)
     float v = 0.f;
 #pragma unroll
-    for (int w = 0; w < kSmWarps; ++w) v += part[w * part_stride + warp * kSmSlice + lane];
+    for (int w = 0; w < kWarps; ++w) v += part[w * part_stride + warp * kSmSlice + lane];
     const long long at = warp * p.ldy[prob] + (p.col_map ? p.col_map[nn] : nn);
     if (kRole == kSmProducer) asm volatile("st.relaxed.gpu.global.u16 [%0], %1;" ::"l"(between + at), "h"(__half_as_ushort(__float2half_rn(v))) : "memory");
     else p.y[prob][at] = __float2half_rn(v);
@@ -356,19 +359,19 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
   if (kRole != kSmAlone) sm_leave(pair);
 }
 
-template <int kBits, int STAGES>
-__global__ void __launch_bounds__(kSmThreads, kSmCtas)
+template <int kBits, int STAGES, int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, kWarps == kSmWarps ? kSmCtas : 1)
 linear_small_kernel(const __grid_constant__ SmParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
-  small_slice<kBits, STAGES, kSmAlone>(smem, p, blockIdx.x, nullptr);
+  small_slice<kBits, STAGES, kWarps, kSmAlone>(smem, p, blockIdx.x, nullptr);
 }
 
 template <int kBits, int STAGES>
 __global__ void __launch_bounds__(kSmThreads, kSmCtas)
 rotate_linear_small_kernel(const __grid_constant__ SmPair p) {
   extern __shared__ __align__(128) uint8_t smem[];
-  if ((int)blockIdx.x < p.n_rot) small_slice<4, STAGES, kSmProducer>(smem, p.rot, blockIdx.x, &p);
-  else small_slice<kBits, 2, kSmConsumer>(smem, p.lin, blockIdx.x - p.n_rot, &p);
+  if ((int)blockIdx.x < p.n_rot) small_slice<4, STAGES, kSmWarps, kSmProducer>(smem, p.rot, blockIdx.x, &p);
+  else small_slice<kBits, 2, kSmWarps, kSmConsumer>(smem, p.lin, blockIdx.x - p.n_rot, &p);
 }
 
 typedef void (*SmallKernel)(SmParams);
@@ -377,14 +380,16 @@ SmallPairKernel small_pair_pick(bool int3, int stages) {
   if (int3) return stages == 8 ? rotate_linear_small_kernel<3, 8> : stages == 4 ? rotate_linear_small_kernel<3, 4> : rotate_linear_small_kernel<3, 2>;
   return stages == 8 ? rotate_linear_small_kernel<4, 8> : stages == 4 ? rotate_linear_small_kernel<4, 4> : rotate_linear_small_kernel<4, 2>;
 }
-SmallKernel small_pick(bool int3, int stages) {
-  if (int3) return linear_small_kernel<3, 2>;
-  return stages == 8 ? linear_small_kernel<4, 8> : stages == 4 ? linear_small_kernel<4, 4> : linear_small_kernel<4, 2>;
+SmallKernel small_pick(bool int3, int stages, int warps) {
+  if (warps == kSmWarpsLong) return int3 ? linear_small_kernel<3, 2, kSmWarpsLong> : linear_small_kernel<4, 2, kSmWarpsLong>;
+  if (int3) return linear_small_kernel<3, 2, kSmWarps>;
+  return stages == 8 ? linear_small_kernel<4, 8, kSmWarps> : stages == 4 ? linear_small_kernel<4, 4, kSmWarps> : linear_small_kernel<4, 2, kSmWarps>;
 }
 
 bool small_attrs() {
   bool ok = true;
-  for (SmallKernel kern : {small_pick(true, 2), small_pick(false, 2), small_pick(false, 4), small_pick(false, 8)})
+  for (SmallKernel kern : {small_pick(true, 2, kSmWarps), small_pick(false, 2, kSmWarps), small_pick(false, 4, kSmWarps), small_pick(false, 8, kSmWarps),
+                           small_pick(true, 2, kSmWarpsLong), small_pick(false, 2, kSmWarpsLong)})
     ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess &&
          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmMaxSmem) == cudaSuccess;
   for (int i = 0; i < 6; ++i) {
@@ -396,8 +401,19 @@ bool small_attrs() {
   return ok;
 }
 
-int small_bytes(int M, const TiledOperand &t, int stages) {
-  return M * groups_per_tile(t) * kGroup * 2 + kSmWarps * stages * kSmStage;
+int small_bytes(int M, const TiledOperand &t, int stages, int warps = kSmWarps) {
+  return M * groups_per_tile(t) * kGroup * 2 + warps * stages * kSmStage;
+}
+// A CTA that has an SM to itself issues 0.3 instructions per cycle and scheduler with two warps on each: a round of its warps (a unit each)
+// takes 1300 cycles of which 724 are issue, with four warps 1800 of 1450.  Sixteen warps where that saves rounds: six rounds of eight and
+// more (an INT3 unit is a longer chain: from five and a half).  us, eight / sixteen warps, one token: 11008 -> 4096 9.27 / 8.63 (INT3 9.75 /
+// 8.75), 8192 -> 1024 6.8 / 6.1, 13824 -> 2048 10.2 / 9.3, 5504 -> 2048 5.35 / 5.10; up to the line 4096 -> 4096 4.78 / 5.05 (INT3 4.95 / 4.99),
+// 512 -> 512 at eight tokens 2.37 / 2.62; twenty-four warps at 11008 -> 4096 9.09.  With two CTAs on an SM there are sixteen warps already.
+int small_warps(const rosaq_ctx *ctx, int M, const TiledOperand &t, int tiles) {
+  const int units = 4 * t.g_fp16 + t.g_quant;
+  return 4 * tiles <= ctx->sm_count && t.g_quant > 0 && units > (t.bits == 3 ? 35 : 40) && small_bytes(M, t, 2, kSmWarpsLong) <= kSmMaxSmem
+             ? kSmWarpsLong
+             : kSmWarps;
 }
 int small_tiles(int n, const TiledOperand *const *ts) {
   int tiles = 0;
@@ -411,14 +427,16 @@ int small_tiles(int n, const TiledOperand *const *ts) {
 // where the launch has more slices than SMs (5120 -> 5120 at six / eight tokens: 8.8 / 11.5 us here, 9.3 us on the tcgen05
 // kernel), and for a third where it has many rounds of them (4096 -> 32000: four tokens 22.5 and 26.6 us, eight 28.0 and 26.6 us);
 // and where the slices leave half of the SMs idle, where the tcgen05 kernel splits K, a CTA must not have a long K to itself
-// (here / there: 8192 -> 512 at three, four and eight tokens 6.7 / 6.5, 6.9 / 6.5, 7.7 / 6.5; 11008 -> 512 at two and six 8.1 / 7.8, 9.2 /
-// 7.9, INT3 at two and five 8.9 / 8.1, 9.8 / 8.1).  Over 936 shapes the pick is 0.6 % slower than the faster one on average.
+// (here, sixteen warps / there: 8192 -> 512 at four and eight tokens 6.3 / 6.4, 7.2 / 6.4, 8192 -> 1024 6.7 / 7.3, 7.55 / 7.3; 11008 -> 512 at
+// three and six 7.8 / 7.75, 8.6 / 7.8; 13824 -> 2048 at two to five 9.6-10.5 / 11.9, at six, where the rings of sixteen warps have no room,
+// 12.1 / 11.8; INT3 11008 -> 512 at three 8.1 / 8.0, 13824 -> 2048 at four 10.6 / 12.6).
 bool linear_small_supported(const rosaq_ctx *ctx, int M, int n, const TiledOperand *const *ts) {
   const int G = groups_per_tile(*ts[0]);
   if (M > kSmallTokens || n < 1 || n > kSmMaxProblems || G <= 0) return false;
   const int bytes = small_bytes(M, *ts[0], 2), slices = 4 * small_tiles(n, ts), rounds = (slices + ctx->sm_count - 1) / ctx->sm_count;
   const int resident = rounds > 5 ? kSmCtas : std::min(rounds, 2);
-  if (2 * slices <= ctx->sm_count && M * G > (ts[0]->g_quant > 0 && ts[0]->bits == 3 ? 180 : 260)) return false;
+  const bool int3 = ts[0]->g_quant > 0 && ts[0]->bits == 3, wide = small_warps(ctx, M, *ts[0], slices / 4) == kSmWarpsLong;
+  if (2 * slices <= ctx->sm_count && M * G > std::max(int3 ? 180 : 260, wide ? (int3 ? 150 : 180) + 6 * slices : 0)) return false;
   return bytes <= kSmMaxSmem && resident * (bytes + kSmSharedCta) <= kSmSharedSm;
 }
 
@@ -460,10 +478,10 @@ static int small_prepare(const rosaq_ctx *ctx) {
 }
 
 template <typename K, typename P>
-static int small_launch(K kern, const P &p, int ctas, int smem, cudaStream_t s) {
+static int small_launch(K kern, const P &p, int ctas, int threads, int smem, cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(kSmThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -496,9 +514,10 @@ int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long 
   int stages = 2;
   if (t.g_quant == 0)
     while (stages < 8 && small_bytes(M, t, 2 * stages) <= room) stages *= 2;
+  const int warps = small_warps(ctx, M, t, tiles);
   // (more than a (ctas + 1)-th of an SM's shared memory)
-  const int smem = std::max(small_bytes(M, t, stages), ctas < kSmCtas ? (kSmSharedSm / (ctas + 1) - kSmSharedCta) / 128 * 128 + 128 : 0);
-  return small_launch(small_pick(t.g_quant > 0 && t.bits == 3, stages), p, 4 * tiles, smem, s);
+  const int smem = std::max(small_bytes(M, t, stages, warps), ctas < kSmCtas ? (kSmSharedSm / (ctas + 1) - kSmSharedCta) / 128 * 128 + 128 : 0);
+  return small_launch(small_pick(t.g_quant > 0 && t.bits == 3, stages, warps), p, 4 * tiles, warps * 32, smem, s);
 }
 
 // The rotation r of x and the n linears that read it in one launch: calls that are bound by the host's two launches (2.3 us each).  That is
@@ -506,12 +525,12 @@ int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long 
 // one: 512 -> 512 at one, four and eight tokens 3.4 / 3.8, 4.0 / 4.2, 4.8 / 4.8; 1024 -> 3 x 1024 4.3 / 4.5, 4.8 / 5.1, 5.7 / 5.6; 2048 -> 2048 5.4 / 5.9, 6.4 / 6.4,
 // 7.1 / 7.8; call by call 9.1 / 6.1 at 512 -> 512), and 4096 -> 4096 would take 13.8 instead of 9.4.  A launch that is being captured costs the host
 // nothing later, so captured calls stay two, and so do column orders, whose scatter the readers' polls disturb (1024 -> 3 x 1024 4.6 / 9.3).
-// The results are the same bits.
+// The results are the same bits (linears whose sums sixteen warps share are not taken).
 bool rotate_linear_small_supported(const rosaq_ctx *ctx, int M, const TiledOperand &r, const int32_t *col_map, int n, const TiledOperand *const *ts,
                                    cudaStream_t s) {
   const TiledOperand *rs[1] = {&r};
   if (col_map || (long long)M * r.d_out > kSmBetween || 4 * (r.n_tiles + small_tiles(n, ts)) > ctx->sm_count || !linear_small_supported(ctx, M, 1, rs) ||
-      !linear_small_supported(ctx, M, n, ts))
+      !linear_small_supported(ctx, M, n, ts) || small_warps(ctx, M, *ts[0], small_tiles(n, ts)) != kSmWarps)
     return false;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
@@ -542,7 +561,7 @@ int launch_rotate_linear_small(const rosaq_ctx *ctx, const __half *x, int M, lon
   while (stages < 8 && small_bytes(M, r, 2 * stages) <= room) stages *= 2;
   const int need = std::max(small_bytes(M, r, stages), small_bytes(M, t, 2));
   const int smem = std::max(need, ctas < kSmCtas ? (kSmSharedSm / (ctas + 1) - kSmSharedCta) / 128 * 128 + 128 : 0);
-  return small_launch(small_pair_pick(t.g_quant > 0 && t.bits == 3, stages), p, grid, smem, s);
+  return small_launch(small_pair_pick(t.g_quant > 0 && t.bits == 3, stages), p, grid, kSmThreads, smem, s);
 }
 
 }  // namespace rosaq

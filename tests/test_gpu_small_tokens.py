@@ -138,3 +138,25 @@ def test_rotation_and_linears_in_one_launch(ctx, kind, d, widths, bits):
         torch.cuda.synchronize()
         assert same(y, want[0]) and same(ctx.linear(x, ws[0], r), want[0])
     assert ctx.last_status() == rb.ROSAQ_OK
+
+
+@pytest.mark.parametrize("M,d_in,widths,bits", [
+    (1, 4736, [4736], 4),               # 40 units: eight warps, the most slices with an SM each ...
+    (1, 4864, [4600, 136], 4),          # ... 41: sixteen, the last round nearly empty; a ragged tile, two weights
+    (1, 4864, [4744], 4),               # one tile more
+    (2, 4096, [328], 3),                # 35 and
+    (7, 4224, [328], 3),                # 36 units of INT3
+    (5, 13824, [2048], 4),              # x' of the most tokens next to the rings of sixteen warps,
+    (8, 11008, [4096], 3),              # of one token more than that: eight
+    (8, 6144, [4096], 4),
+])
+def test_long_k_on_sixteen_warps(ctx, M, d_in, widths, bits):
+    """The line between eight and sixteen warps per slice, and a rotated call on either side of it, which is one launch on the near one:
+    the bits of two calls."""
+    test_linear(ctx, M, d_in, widths, bits)
+    rng = synth.rng_for(23, "sixteen", d_in)
+    r = ctx.rotation_create(dev((rng.standard_normal((d_in // 128, 128, 128)) / 128 ** 0.5).astype(np.float16)))
+    w = ctx.quantize(dev(synth.weights(d_in, 72, 23, "sixteen", outlier_frac=0.01)), None, bits=bits, k_salient=128)
+    x = dev(rng.standard_normal((2, d_in)).astype(np.float16))
+    assert same(ctx.linear(x, w, rotation=r), ctx.linear(ctx.rotate(x, r), w))
+    assert ctx.last_status() == rb.ROSAQ_OK
