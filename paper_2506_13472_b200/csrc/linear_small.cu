@@ -172,28 +172,20 @@ __device__ __forceinline__ void unit_int3(uint32_t stage, uint32_t scales, const
 }
 
 // A rotation and the linears that read it in one launch: the first CTAs are the slices of the rotation, the others copy its output
-// as it appears.  (The hardware starts CTAs in order, so those that are waited for are never behind the ones that wait.)  The
-// buffer between them announces its values itself: it is all ones, which no rounded value is, where nothing has been written yet.
-struct SmPair {
-  SmParams rot, lin;
+// as it appears.  The buffer between them announces its values itself: it is all ones, which no rounded value is, where nothing has been
+// written yet.  The CTAs that wait need no order of starting: the launch has no more CTAs than the device has SMs, so each of them gets its
+// room as soon as other launches leave it, whether the waiting ones hold theirs or not (a cooperative launch, which would say the same to the
+// runtime, takes 6.2 us where this takes 4.3: 512 -> 512 at one token).
+// (Aligned for its size: a launch takes the host 6.7 us with 408 or 416 bytes of parameters, 7.05 with 400, 424 or 440.)
+struct alignas(32) SmPair {
+  SmParams rot, lin;         // (lin.x: the values between)
   int n_rot;                 // CTAs of the rotation
-  __half *between;           // two buffers of kSmBetween values, for launches in turn; a launch empties the other one
-  unsigned *left;            // kSmLaunch times the launches so far, and the CTAs of this one that have left
+  __half *other;             // the buffer of the launch before and of the one behind, kSmBetween values: emptied here
   int *status;
   long long wait_limit;
 };
-constexpr unsigned kSmLaunch = 1u << 16;
 enum SmRole { kSmAlone, kSmProducer, kSmConsumer };
 
-__device__ __forceinline__ unsigned sm_turn(const SmPair *pair) {   // (behind griddepcontrol.wait)
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(pair->left) : "memory");
-  return (v / kSmLaunch) & 1u;
-}
-// All CTAs of a launch together add kSmLaunch, so the count tells a launch that is running from the one before.
-__device__ __forceinline__ void sm_leave(const SmPair *pair) {
-  if (threadIdx.x == 0) atomicAdd(pair->left, blockIdx.x == 0 ? kSmLaunch + 1 - gridDim.x : 1u);
-}
 // some half of v is 0xffff
 __device__ __forceinline__ uint32_t sm_missing(uint32_t v) {
   const uint32_t t = ~v;
@@ -213,13 +205,7 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
   const int col = (block & 3) * kSmSlice;
   while (prob + 1 < p.n_prob && tile >= p.tile_start[prob + 1]) ++prob;
   tile -= p.tile_start[prob];
-  if (tile * kTileN + col >= p.d_out[prob]) {                    // past the last column of a ragged last tile
-    if (kRole != kSmAlone) {
-      grid_dep_wait();                                           // (the launch before may still be counting)
-      sm_leave(pair);
-    }
-    return;
-  }
+  if (tile * kTileN + col >= p.d_out[prob]) return;              // past the last column of a ragged last tile
 
   const int x_row = (u_fp16 * 32 + (n_units - u_fp16) * kGroup) * 2;
   const uint32_t x_smem = smem_u32(smem), ring = x_smem + M * x_row + warp * (STAGES * kSmStage), ring_end = ring + STAGES * kSmStage;
@@ -248,14 +234,18 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
   for (int s = 0; s < STAGES; ++s, f += kWarps) fetch(ring + s * kSmStage, f);
 
   grid_dep_wait();                                               // x may be the previous kernel's output, y its input
-  __half *between = nullptr;
-  if (kRole != kSmAlone) {
-    const unsigned turn = sm_turn(pair);
-    between = pair->between + turn * kSmBetween;
-    if (kRole == kSmProducer) {
-      uint4 *other = reinterpret_cast<uint4 *>(pair->between + (turn ^ 1u) * kSmBetween);
-      for (int i = block * kThreads + threadIdx.x; i < kSmBetween / 8; i += pair->n_rot * kThreads) other[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  if (kRole != kSmConsumer) {
+    // block-diagonal operand: a tile multiplies its own channels
+    const __half *xs = p.x + (p.block_groups > 0 ? (tile / p.block_groups) * p.block_groups * kGroup : 0) + threadIdx.x * 8;
+    const int n_full = x_row >> 4;
+    for (int r = 0; r < M; ++r, xs += p.ldx) {
+      uint32_t dst = x_smem + r * x_row + x_pos(r, threadIdx.x);
+      for (int c = threadIdx.x; c < n_full; c += kThreads, dst += kThreads * 16) cp_async16(dst, xs + (c - (int)threadIdx.x) * 8);
     }
+  }
+  if (kRole == kSmProducer) {                                    // (under the copies of x)
+    uint4 *other = reinterpret_cast<uint4 *>(pair->other);
+    for (int i = block * kThreads + threadIdx.x; i < kSmBetween / 8; i += pair->n_rot * kThreads) other[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
   }
   if (kRole == kSmConsumer) {
     int ok = 1;
@@ -269,7 +259,7 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
           const int i = min(i0 + k * kThreads, n_all - 1);
           asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
                        : "=r"(v[k].x), "=r"(v[k].y), "=r"(v[k].z), "=r"(v[k].w)
-                       : "l"(between + 8 * i)
+                       : "l"(p.x + 8 * i)
                        : "memory");
         }
 #pragma unroll
@@ -289,18 +279,9 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
     if (!__syncthreads_and(ok)) {
       if (threadIdx.x == 0) atomicExch(pair->status, (int)ROSAQ_ERR_TIMEOUT);
       asm volatile("cp.async.wait_all;" ::: "memory");
-      sm_leave(pair);
       return;
     }
-  } else
-  {
-    // block-diagonal operand: a tile multiplies its own channels
-    const __half *xs = p.x + (p.block_groups > 0 ? (tile / p.block_groups) * p.block_groups * kGroup : 0) + threadIdx.x * 8;
-    const int n_full = x_row >> 4;
-    for (int r = 0; r < M; ++r, xs += p.ldx) {
-      uint32_t dst = x_smem + r * x_row + x_pos(r, threadIdx.x);
-      for (int c = threadIdx.x; c < n_full; c += kThreads, dst += kThreads * 16) cp_async16(dst, xs + (c - (int)threadIdx.x) * 8);
-    }
+  } else {
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
   }
@@ -352,11 +333,10 @@ __device__ __forceinline__ void small_slice(uint8_t *smem, const SmParams &p, in
     float v = 0.f;
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) v += part[w * part_stride + warp * kSmSlice + lane];
-    const long long at = warp * p.ldy[prob] + (p.col_map ? p.col_map[nn] : nn);
-    if (kRole == kSmProducer) asm volatile("st.relaxed.gpu.global.u16 [%0], %1;" ::"l"(between + at), "h"(__half_as_ushort(__float2half_rn(v))) : "memory");
-    else p.y[prob][at] = __float2half_rn(v);
+    __half *const at = p.y[prob] + warp * p.ldy[prob] + (p.col_map ? p.col_map[nn] : nn);
+    if (kRole == kSmProducer) asm volatile("st.relaxed.gpu.global.u16 [%0], %1;" ::"l"(at), "h"(__half_as_ushort(__float2half_rn(v))) : "memory");
+    else *at = __float2half_rn(v);
   }
-  if (kRole != kSmAlone) sm_leave(pair);
 }
 
 template <int kBits, int STAGES, int kWarps>
@@ -375,6 +355,7 @@ rotate_linear_small_kernel(const __grid_constant__ SmPair p) {
 }
 
 typedef void (*SmallKernel)(SmParams);
+static_assert(sizeof(SmPair) == 416, "see there");
 typedef void (*SmallPairKernel)(SmPair);
 SmallPairKernel small_pair_pick(bool int3, int stages) {
   if (int3) return stages == 8 ? rotate_linear_small_kernel<3, 8> : stages == 4 ? rotate_linear_small_kernel<3, 4> : rotate_linear_small_kernel<3, 2>;
@@ -520,12 +501,16 @@ int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long 
   return small_launch(small_pick(t.g_quant > 0 && t.bits == 3, stages, warps), p, 4 * tiles, warps * 32, smem, s);
 }
 
-// The rotation r of x and the n linears that read it in one launch: calls that are bound by the host's two launches (2.3 us each).  That is
-// so while all slices find an SM of their own; then the launch takes the device about what the two take (us in a graph, two launches /
-// one: 512 -> 512 at one, four and eight tokens 3.4 / 3.8, 4.0 / 4.2, 4.8 / 4.8; 1024 -> 3 x 1024 4.3 / 4.5, 4.8 / 5.1, 5.7 / 5.6; 2048 -> 2048 5.4 / 5.9, 6.4 / 6.4,
-// 7.1 / 7.8; call by call 9.1 / 6.1 at 512 -> 512), and 4096 -> 4096 would take 13.8 instead of 9.4.  A launch that is being captured costs the host
-// nothing later, so captured calls stay two, and so do column orders, whose scatter the readers' polls disturb (1024 -> 3 x 1024 4.6 / 9.3).
-// The results are the same bits (linears whose sums sixteen warps share are not taken).
+// The rotation r of x and the n linears that read it in one launch, while every slice finds an SM of its own (4096 -> 4096 would take 13.8
+// us instead of 9.4) and the values between are few: each reader copies all of them, and from 16384 on that takes longer than a second launch.
+// us, two launches / one, behind a long kernel (a full queue: the device is the bound) and call by call (the host is):
+//   512 -> 512    one token 4.35 / 3.9, 7.7 / 5.3     eight 5.7 / 4.8, 7.7 / 5.3
+//   1024 -> 1024  one 4.95 / 4.35, 7.7 / 5.3          eight 6.4 / 5.5, 7.7 / 5.6
+//   2048 -> 2048  one 6.3 / 5.9, 7.6 / 6.0            eight 7.7 / 7.6, 7.7 / 7.7
+// past the line 2304 -> 1024 at eight 8.4 / 8.7, 3072 -> 1600 at six 8.8 / 9.35; 4096 -> 512 at four, on it, 11.4 / 11.6 (head-wise 6.8 / 7.1, call
+// by call 7.7 / 7.2).
+// A launch that is being captured costs the host nothing later, so captured calls stay two, and so do column orders, whose scatter the
+// readers' polls disturb (1024 -> 3 x 1024 4.6 / 9.3).  The results are the same bits (linears whose sums sixteen warps share are not taken).
 bool rotate_linear_small_supported(const rosaq_ctx *ctx, int M, const TiledOperand &r, const int32_t *col_map, int n, const TiledOperand *const *ts,
                                    cudaStream_t s) {
   const TiledOperand *rs[1] = {&r};
@@ -540,19 +525,20 @@ bool rotate_linear_small_supported(const rosaq_ctx *ctx, int M, const TiledOpera
   return capture == cudaStreamCaptureStatusNone;
 }
 
-int launch_rotate_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &r, int n,
+int launch_rotate_linear_small(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &r, int n,
                                const TiledOperand *const *ts, __half *const *ys, const long long *ldys, cudaStream_t s) {
   const TiledOperand &t = *ts[0];
   const TiledOperand *rs[1] = {&r};
   const long long ldxr = r.d_out;
   SmPair p{};
-  p.between = ctx->sm_between;
-  int st = small_params(x, M, ldx, 1, rs, nullptr, &p.between, &ldxr, &p.rot);
-  if (st == ROSAQ_OK) st = small_params(p.between, M, ldxr, n, ts, nullptr, ys, ldys, &p.lin);
+  // (launches of one context run in the order in which they are issued, one at a time; none of these is captured, to be run again later)
+  __half *between = ctx->sm_between + (ctx->sm_turn ? kSmBetween : 0);
+  p.other = ctx->sm_between + (ctx->sm_turn ? 0 : kSmBetween);
+  int st = small_params(x, M, ldx, 1, rs, nullptr, &between, &ldxr, &p.rot);
+  if (st == ROSAQ_OK) st = small_params(between, M, ldxr, n, ts, nullptr, ys, ldys, &p.lin);
   if (st == ROSAQ_OK) st = small_prepare(ctx);
   if (st != ROSAQ_OK) return st;
   p.n_rot = 4 * r.n_tiles;
-  p.left = ctx->sm_left;
   p.status = ctx->d_status;
   p.wait_limit = ctx->wait_limit;
   const int grid = p.n_rot + 4 * p.lin.tile_start[n], ctas = std::max(1, std::min(kSmCtas, (grid + ctx->sm_count - 1) / ctx->sm_count));
@@ -561,7 +547,9 @@ int launch_rotate_linear_small(const rosaq_ctx *ctx, const __half *x, int M, lon
   while (stages < 8 && small_bytes(M, r, 2 * stages) <= room) stages *= 2;
   const int need = std::max(small_bytes(M, r, stages), small_bytes(M, t, 2));
   const int smem = std::max(need, ctas < kSmCtas ? (kSmSharedSm / (ctas + 1) - kSmSharedCta) / 128 * 128 + 128 : 0);
-  return small_launch(small_pair_pick(t.g_quant > 0 && t.bits == 3, stages), p, grid, kSmThreads, smem, s);
+  st = small_launch(small_pair_pick(t.g_quant > 0 && t.bits == 3, stages), p, grid, kSmThreads, smem, s);
+  if (st == ROSAQ_OK) ctx->sm_turn ^= 1;
+  return st;
 }
 
 }  // namespace rosaq

@@ -249,6 +249,7 @@ int rosaq_create(rosaq_ctx **out, int device) {
   ctx->pl_exchange_bytes = ctx->pf_partial_bytes = 0;
   ctx->pl_sync = nullptr;
   ctx->sm_between = nullptr;
+  ctx->sm_turn = 0;
   for (int i = 0; i < 4; ++i) ctx->pf_clusters[i] = 0;
   ctx->pf_flags = nullptr;
   ctx->pool = nullptr;
@@ -261,12 +262,8 @@ int rosaq_create(rosaq_ctx **out, int device) {
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->sk_arrive), rosaq::kSkCounterInts * sizeof(int)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->sk_arrive, 0, rosaq::kSkCounterInts * sizeof(int)));
   constexpr size_t kBetweenBytes = 2 * rosaq::kSmBetween * sizeof(__half);
-  if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->sm_between), kBetweenBytes + sizeof(unsigned)));
-  if (st == ROSAQ_OK) {
-    ctx->sm_left = reinterpret_cast<unsigned *>(ctx->sm_between + 2 * rosaq::kSmBetween);
-    st = cuda_status(cudaMemset(ctx->sm_between, 0xff, kBetweenBytes));
-  }
-  if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->sm_left, 0, sizeof(unsigned)));
+  if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->sm_between), kBetweenBytes));
+  if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->sm_between, 0xff, kBetweenBytes));
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pl_sync), rosaq::kPlSyncWords * sizeof(unsigned)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));
   if (st == ROSAQ_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&ctx->pf_flags), (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));

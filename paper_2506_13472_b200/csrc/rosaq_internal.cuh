@@ -170,7 +170,7 @@ namespace rosaq {
 constexpr int kPfFlagsPerSm = 2;                    // prefill tiles: two partial-tile slots per CTA
 constexpr int kSkMaxCtas = 320;                     // stream-K grid limit (two CTAs per SM)
 constexpr int kSkCounterInts = 1024;                // arrival counters (one per column tile of a launch)
-constexpr int kSmBetween = 8 * 4096;                // values between a rotation and its linears in one launch
+constexpr int kSmBetween = 8 * 2048;                // most values between a rotation and its linears in one launch
 constexpr size_t kSkPartialBytes = 128 * 64 * sizeof(float);   // one partial tile: 128 columns x 64 tokens
 
 // ---- the persistent multi-problem launch (linear_plan.cu) --------------------------------
@@ -269,8 +269,8 @@ struct rosaq_ctx {
   float *sk_partials;  // stream-K: fp32 partial tiles, [sk_ctas][2][64 tokens][128 columns]
   int *sk_arrive;      // stream-K: per-tile arrival counters, zero between launches
   int sk_ctas;         // CTAs the partial-tile workspace was sized for
-  __half *sm_between;  // a rotation and its linears in one launch: two buffers of kSmBetween values, and the count of CTAs that have left
-  unsigned *sm_left;
+  __half *sm_between;  // a rotation and its linears in one launch: two buffers of kSmBetween values, for launches in turn
+  int sm_turn;         // the buffer that the next one uses; the other is not empty
   // persistent multi-problem launch
   int pl_ctas;                                   // CTAs of its grid, one per SM (0 until first asked for)
   int pl_pairs;                                  // clusters of two CTAs the device keeps resident at once
@@ -431,7 +431,7 @@ int launch_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long 
 
 bool rotate_linear_small_supported(const rosaq_ctx *ctx, int M, const TiledOperand &r, const int32_t *col_map, int n, const TiledOperand *const *ts,
                                    cudaStream_t s);
-int launch_rotate_linear_small(const rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &r, int n,
+int launch_rotate_linear_small(rosaq_ctx *ctx, const __half *x, int M, long long ldx, const TiledOperand &r, int n,
                                const TiledOperand *const *ts, __half *const *ys, const long long *ldys, cudaStream_t s);
 
 bool prefill_supported(const TiledOperand &t, const int32_t *col_map);

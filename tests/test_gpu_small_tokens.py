@@ -106,6 +106,7 @@ def test_rotation(ctx, M, d, head):
     ("heads", 384, [72, 384, 1000], 3),
     ("dense", 2048, [2688], 3),            # 148 CTAs, the most on 148 SMs; one tile more below
     ("dense", 2048, [2696], 4),
+    ("heads", 2304, [136], 4),             # seven tokens are the most with one launch
 ])
 def test_rotation_and_linears_in_one_launch(ctx, kind, d, widths, bits):
     """A small rotated call is one launch (unless it is captured): the bits of the rotation and the linears called one by one, with
