@@ -326,18 +326,15 @@ int rosaq_last_status(rosaq_ctx *ctx, void *stream) {
   st = cuda_status(cudaMemcpy(&host, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost));
   if (st != ROSAQ_OK) return st;
   if (host != 0) {
-    st = cuda_status(cudaMemset(ctx->d_status, 0, sizeof(int)));
-    if (st != ROSAQ_OK) return st;
-    // a launch that gave up may have left arrival counters of the stream-K exchange behind, and partial tiles
+    // A launch that gave up may have left partial tiles behind, and arrival counters of the stream-K exchange.  The status word is cleared
+    // when they are gone: a set one is what makes the next launch empty its slots.
     st = cuda_status(cudaMemset(ctx->pl_exchange, 0xff, ctx->pl_exchange_bytes));
     for (int i = 0; i < ctx->n_retired && st == ROSAQ_OK; ++i)
       if (ctx->retired_exchange[i]) st = cuda_status(cudaMemset(ctx->retired[i], 0xff, ctx->retired_exchange[i]));
-    if (st != ROSAQ_OK) return st;
-    st = cuda_status(cudaMemset(ctx->sk_arrive, 0, rosaq::kSkCounterInts * sizeof(int)));
-    if (st != ROSAQ_OK) return st;
-    st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));
-    if (st != ROSAQ_OK) return st;
-    st = cuda_status(cudaMemset(ctx->pf_flags, 0, (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
+    if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->sk_arrive, 0, rosaq::kSkCounterInts * sizeof(int)));
+    if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pl_sync, 0, rosaq::kPlSyncWords * sizeof(unsigned)));
+    if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->pf_flags, 0, (size_t)rosaq::kPfFlagsPerSm * ctx->sm_count * sizeof(unsigned)));
+    if (st == ROSAQ_OK) st = cuda_status(cudaMemset(ctx->d_status, 0, sizeof(int)));
     if (st == ROSAQ_OK) st = cuda_status(cudaStreamSynchronize(cudaStreamLegacy));   // (the caller's streams may not wait for it)
     if (st != ROSAQ_OK) return st;
   }
