@@ -497,10 +497,11 @@ cov_tc_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         if (++idx == kPairStages) idx = 0, lap ^= 1u;
       }
       // On a timeout the leader lets the loads of both CTAs land (they are all counted on its barriers)
-      // before the final cluster barrier releases the pair; phases whose expectation it never posted
-      // cannot complete and are bounded by the drain limit.
+      // before the final cluster barrier releases the pair.  The peer may have asked for stages that the leader never posted: the
+      // last one waited for here is the first of those, which cannot complete, so the wait lasts for the drain limit (65 ms),
+      // long past the microseconds that the peer's loads take.
       if (ab.set() && rank == 0) {
-        for (int back = 1; back <= kPairStages && back <= issued; ++back) {
+        for (int back = min(kPairStages, issued); back >= 0; --back) {
           const int u = issued - back;
           for (int it = 0; it < kCovDrainPolls; ++it)
             if (mbar_try_wait(bar_tma + 8 * (u % kPairStages), (u / kPairStages) & 1)) break;
@@ -727,7 +728,7 @@ cov_tc_tiles_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
         }
       }
       if (ab.set() && rank == 0) {                   // (see cov_tc_pair_kernel)
-        for (int back = 1; back <= kPairStages && back <= issued; ++back) {
+        for (int back = min(kPairStages, issued); back >= 0; --back) {
           const int u = issued - back;
           for (int it = 0; it < kCovDrainPolls; ++it)
             if (mbar_try_wait(bar_tma + 8 * (u % kPairStages), (u / kPairStages) & 1)) break;

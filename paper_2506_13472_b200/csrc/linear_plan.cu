@@ -434,9 +434,10 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
         }
       }
       // (in a pair the leader's barriers count the copies of both CTAs, and the peer stays until the cluster
-      // barrier at the end of the kernel, which the leader reaches after this drain)
+      // barrier at the end of the kernel, which the leader reaches after this drain: the last stage that it waits for, for as long as
+      // the limit goes, is one that it has not posted, but the peer may have asked for)
       if (lane == 0 && ab.set() && is_lead) {
-        for (int back = 1; back <= NS && back <= gc; ++back) {
+        for (int back = min(NS, gc); back >= (kPair ? 0 : 1); --back) {
           const int u = gc - back;
           for (int it = 0; it < kDrainPolls; ++it)
             if (mbar_try_wait(bar_a_full + 8 * (u % NS), (u / NS) & 1)) break;

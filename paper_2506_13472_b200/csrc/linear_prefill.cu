@@ -314,9 +314,10 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
           }
         }
         // (the leader's barriers count the copies of both CTAs, and the peer stays until the cluster barrier
-        // at the end of the kernel, which the leader reaches after this drain)
+        // at the end of the kernel, which the leader reaches after this drain: the last stage that it waits for, for as long as the
+        // limit goes, is one that it has not posted, but the peer may have asked for)
         if (ab.set() && is_lead) {
-          for (int back = 1; back <= NW && back <= issued; ++back) {
+          for (int back = min(NW, issued); back >= 0; --back) {
             const int k = issued - back;
             for (int it = 0; it < kDrainPolls; ++it)
               if (mbar_try_wait(bar_w_full + 8 * (k % NW), (k / NW) & 1)) break;
@@ -375,7 +376,7 @@ linear_prefill_kernel(const __grid_constant__ PfParams p) {
           }
         }
         if (lane == 0 && ab.set() && is_lead) {
-          for (int back = 1; back <= kPfStages && back <= gc; ++back) {
+          for (int back = min(kPfStages, gc); back >= 0; --back) {     // (as above)
             const int k = gc - back;
             for (int it = 0; it < kDrainPolls; ++it)
               if (mbar_try_wait(bar_a_full + 8 * (k % kPfStages), (k / kPfStages) & 1)) break;

@@ -204,10 +204,11 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         }
       }
       // (in a pair the leader's barriers count the loads of both CTAs, and the peer stays until the
-      // cluster barrier at the end of the kernel, which the leader reaches after this drain)
+      // cluster barrier at the end of the kernel, which the leader reaches after this drain: the last stage that it waits for, for as
+      // long as the limit goes, is one that it has not posted, but the peer may have asked for)
       if (ab.set() && is_lead) {
         const uint32_t bar_copy = kPair ? bar_x_full : bar_a_full;
-        for (int back = 1; back <= p.NA && back <= gc; ++back) {
+        for (int back = min(p.NA, gc); back >= (kPair ? 0 : 1); --back) {
           const int u = gc - back;
           for (int it = 0; it < kDrainPolls; ++it)
             if (mbar_try_wait(bar_copy + 8 * (u % p.NA), (u / p.NA) & 1)) break;

@@ -160,3 +160,30 @@ def test_calib_cov_more_tiles_than_pairs(n_tokens, d, n_blocks):
     diag = want.diagonal(dim1=1, dim2=2)
     bound = (n_tokens / 16 + 12) * 2.0 ** -23 * (diag[:, :, None] * diag[:, None, :]).sqrt() + 1e-6   # (0.5 and two sums rounded)
     assert torch.all((got[0].double() - 0.5 - want).abs() <= bound)
+
+
+@pytest.mark.parametrize("d", [768, 2048])
+def test_calib_cov_behind_one_that_gave_up(d):
+    """A Gram matrix that gives up (its epilogue waits for hundreds of microseconds, with a limit of one poll), on single CTAs and on pairs,
+    where one CTA may give up long before the other.  The status says so, both leave, and the next call gives the bits of the first."""
+    X = (torch.randn((32768, d), generator=torch.Generator().manual_seed(53)) * 0.5).half().cuda()
+    ctx = rb.Context(0)
+    try:
+        def gram(x):
+            C = torch.zeros((d, d), device="cuda")
+            ctx.calib_cov(x, C)
+            return C
+
+        want = gram(X[:1000])
+        assert ctx.last_status() == rb.ROSAQ_OK
+        for _ in range(3):
+            old = ctx.set_wait_limit(1)
+            try:
+                gram(X)
+            finally:
+                ctx.set_wait_limit(old)
+            assert ctx.last_status() == rb.ROSAQ_ERR_TIMEOUT
+            assert torch.equal(gram(X[:1000]), want)
+            assert ctx.last_status() == rb.ROSAQ_OK
+    finally:
+        ctx.close()
