@@ -399,10 +399,10 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t smem_addr, uint32_t ran
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void tc_commit_pair_lane(uint32_t bar, uint32_t lead) {
+__device__ __forceinline__ void tc_commit_pair_lane(uint32_t bar, uint32_t lead, uint32_t ranks = 3u) {
   asm volatile(
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"((unsigned short)(3u << lead))
+      "h"((unsigned short)(ranks << lead))
       : "memory");
 }
 __device__ __forceinline__ void tc_mma4_ss_pair(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
@@ -659,12 +659,13 @@ __device__ __forceinline__ CovTile cov_tile(int t, int tiles, uint32_t rank) {
 __global__ void __launch_bounds__(kCovThreads, 1)
 cov_tc_tiles_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap map2, const CovParams p, int tiles, int n_tiles) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ uint64_t bars[2 * kPairStages + 4];
+  __shared__ uint64_t bars[2 * kPairStages + 5];
   __shared__ uint32_t misc[2];                       // [0] TMEM base, [1] abort flag
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t bar_tma = smem_u32(&bars[0]), bar_empty = smem_u32(&bars[kPairStages]);   // as in cov_tc_pair_kernel
   const uint32_t bar_d = smem_u32(&bars[2 * kPairStages]);           // accumulators final (multicast commit)
   const uint32_t bar_free = smem_u32(&bars[2 * kPairStages + 2]);    // leader's copy: accumulators read by the epilogues of both CTAs
+  const uint32_t bar_drain = smem_u32(&bars[2 * kPairStages + 4]);   // leader's copy: MMAs of a launch that gives up
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = blockIdx.x & 1u;
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
@@ -680,6 +681,7 @@ cov_tc_tiles_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
       mbar_init(bar_d + 8 * i, 1);
       mbar_init(bar_free + 8 * i, 8);                // the epilogue warps of both CTAs
     }
+    mbar_init(bar_drain, 1);
     misc[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -762,11 +764,12 @@ cov_tc_tiles_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_const
         }
         if (live) tc_commit_pair_lane(bar_d + 8 * buf, 0);
       }
-      if (ab.set()) {  // MMAs already issued must retire before the tensor memory is given back
-        const uint32_t bar = bar_d + 8 * (n & 1);    // (its phase of this tile has not been committed)
-        tc_commit_pair_lane(bar, 0);
+      if (ab.set()) {
+        // MMAs already issued must retire before the tensor memory is given back.  (On a barrier that only the leader waits for: the
+        // peer's epilogue, which may not have given up yet, must not take this for the end of a tile and add half of one to C.)
+        tc_commit_pair_lane(bar_drain, 0, 1u);
         for (int it = 0; it < kCovDrainPolls; ++it)
-          if (mbar_try_wait(bar, (uint32_t)(n >> 1) & 1u)) break;
+          if (mbar_try_wait(bar_drain, 0)) break;
       }
     }
   } else {

@@ -162,10 +162,10 @@ def test_calib_cov_more_tiles_than_pairs(n_tokens, d, n_blocks):
     assert torch.all((got[0].double() - 0.5 - want).abs() <= bound)
 
 
-@pytest.mark.parametrize("d", [768, 2048])
+@pytest.mark.parametrize("d", [768, 2048, 3328])
 def test_calib_cov_behind_one_that_gave_up(d):
-    """A Gram matrix that gives up (its epilogue waits for hundreds of microseconds, with a limit of one poll), on single CTAs and on pairs,
-    where one CTA may give up long before the other.  The status says so, both leave, and the next call gives the bits of the first."""
+    """A Gram matrix that gives up (its epilogue waits for hundreds of microseconds, with a limit of one poll), on single CTAs, on a
+    pair per tile and on pairs that take tiles in turn, where one CTA may give up long before the other.  The status says so, both leave, and the next call gives the bits of the first."""
     X = (torch.randn((32768, d), generator=torch.Generator().manual_seed(53)) * 0.5).half().cuda()
     ctx = rb.Context(0)
     try:
