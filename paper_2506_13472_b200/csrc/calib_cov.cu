@@ -941,7 +941,11 @@ int launch_cov(const rosaq_ctx *ctx, const void *X, int x_dtype, long long n_tok
   if (dh >= 512 && z2 >= z1) {
     p.splits = z2;
     const int n_tiles = pair_tiles * n_blocks, pairs = ctx->sm_count / 2;
-    if (n_tiles > pairs && reinterpret_cast<uintptr_t>(C) % 32 == 0) return cov_launch(cov_tc_tiles_kernel, dim3(2 * pairs, 1, 1), kCovThreads, smem2, 2, 1, s, xmap, map2, p, pair_tiles, n_tiles);
+    // (Tiles in turn: where few tokens leave a second round of a few tiles, that round is a tile's epilogue behind another, longer without the
+    // staging than a pair's own.  78 tiles, us, a pair per tile / in turn: 2880 channels at 64 tokens 23.1 / 25.9, 450 26.5 / 28.6, 1000 31.7 / 32.3, 2000 41.6 /
+    // 39.9; 3072 at 200 28.1 / 29.8, 1000 35.9 / 35.7.  90 tiles at 64 and 450 tokens 29.0 / 29.9, 33.6 / 32.8; 91 at 64 32.7 / 29.2.)
+    if (n_tiles > pairs && (5 * n_tiles > 6 * pairs || stages >= 16) && reinterpret_cast<uintptr_t>(C) % 32 == 0)
+      return cov_launch(cov_tc_tiles_kernel, dim3(2 * pairs, 1, 1), kCovThreads, smem2, 2, 1, s, xmap, map2, p, pair_tiles, n_tiles);
     return cov_launch(z2 > 1 ? cov_tc_pair_kernel<true> : cov_tc_pair_kernel<false>, dim3(2 * pair_tiles, n_blocks, z2), kCovThreads, smem2, 2, z2, s, xmap, map2, p);
   }
   p.splits = z1;

@@ -134,9 +134,10 @@ def test_calib_cov_either_step_of_the_fp32_kernel(n_tokens, n_blocks):
     assert np.array_equal(got, np.swapaxes(got, -1, -2))
 
 
-@pytest.mark.parametrize("n_tokens,d,n_blocks", [(130, 3000, 1), (64, 3072, 1), (200, 4608, 2), (1, 4104, 1)])
+@pytest.mark.parametrize("n_tokens,d,n_blocks", [(130, 3000, 1), (64, 3072, 1), (200, 4608, 2), (1, 4104, 1), (1919, 3000, 1), (1921, 3000, 1)])
 def test_calib_cov_more_tiles_than_pairs(n_tokens, d, n_blocks):
-    """78 to 153 tiles for the 74 pairs of 148 SMs: pairs that take a second and a third tile while the first is added to C.  A C that does
+    """78 to 153 tiles for the 74 pairs of 148 SMs: pairs that take a second and a third tile while the first is added to C (78 tiles: from 961
+    tokens, both calls of the last case, on).  A C that does
     not lie on 32 bytes takes the kernel with a pair per tile, whose bits it has to give; tokens and channels that fill no whole tile."""
     dh = d // n_blocks
     X = (torch.randn((n_tokens, d), generator=torch.Generator().manual_seed(51)) * torch.linspace(2, 0.1, d)).half().cuda()
