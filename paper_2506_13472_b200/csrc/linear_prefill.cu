@@ -22,7 +22,7 @@
 //     (two cluster barriers, 2-3 us).  Used while all clusters are resident at once.
 //   * S = 0, equal shares: the list of (tile, 128-channel group) units, token blocks of one column pair
 //     next to each other so that the second one finds the packed weights in L2, is cut into one contiguous range
-//     of equal length per pair (a 13B projection at 512 tokens is 108 tiles for 74 pairs: whole tiles
+//     of about equal cost per pair (a 13B projection at 512 tokens is 108 tiles for 74 pairs: whole tiles
 //     would take two rounds, equal ranges take 1.46).  The first piece of a range can be the end of a tile; its partial tile
 //     (fp32) goes to a workspace and a flag is raised.  The last piece can be a tile without its last groups: the pairs that
 //     hold it so ("closers") each finish a share of its token rows: they store the other rows of their own partial tile, wait
@@ -904,20 +904,27 @@ int launch_linear_prefill(rosaq_ctx *ctx, const __half *x, int M, long long ldx,
   if (units < 1 || units > (1ll << 30)) return ROSAQ_ERR_UNSUPPORTED_SHAPE;
   p.units = (int)units;
   const int n_pairs = p.S > 0 ? (int)tiles * p.S : (int)std::min<long long>(units, std::min(max_pairs, kPfMaxPairs));
-  // The cut into equal shares: pair i begins at the first unit that i n-ths of the cost lie before.  A unit of the last token block
+  // The cut into equal shares: pair i begins at the unit nearest to i n-ths of the cost.  A unit of the last token block
   // costs less when that block holds fewer tokens: 1900 are seven blocks of 256 and one of 108, which takes 128.  A unit costs what its tokens
   // do and about 100 tokens more.  us, all blocks of NT / this, in a loop: 4096 -> 3 x 4096 at 600 tokens 68.1 / 61.1, at 1570 145.8 / 139.9, at 1900 169.4 / 162.4;
   // 4096 -> 2 x 11008 at 900 153.5 / 145.1, at 1900 290.4 / 280.4; dense rotation of 5120 at 1900 104.0 / 99.0.  (No range may be empty, so each has
   // to be worth a unit.)
+  // A range does not end with the first group or two of a tile (`snap`, for as little as a tenth of a range): the
+  // epilogue still stores the tile before it then, and the exchange of this one begins only behind that.  us, with such ends / without: 1280 -> 10672 at 1782 tokens 63 / 53, 1408 -> 9000 at 1300 48 / 40, 1408 -> 3 x 6024 at
+  // 569 44 / 37, INT3 4480 -> 3 x 4600 at 439 55 / 48; 330 launches of 200 to 2048 tokens 0.8 % on average.
   if (p.S == 0) {
     const int fixed = dense ? 4 : 3;                         // of a group, in 32 tokens
     long long cost = p.NT / 32 + fixed, cost_last = p.NT_last / 32 + fixed;
     const long long G = p.groups, nb = p.n_tok_blocks;
     if (col_pairs * G * ((nb - 1) * cost + cost_last) < n_pairs * cost) cost = cost_last = 1;
     const long long head = (nb - 1) * G * cost, per_col = head + G * cost_last;
+    const long long snap = std::min(3ll, std::max(1ll, units / (10 * n_pairs)));
     for (int i = 0; i <= n_pairs; ++i) {
       const long long c = i * (col_pairs * per_col) / n_pairs, col = c / per_col, rest = c - col * per_col;
-      p.bounds[i] = (int)(col * G * nb + (rest <= head ? (rest + cost - 1) / cost : (nb - 1) * G + (rest - head + cost_last - 1) / cost_last));
+      long long at = col * G * nb + (rest <= head ? (2 * rest + cost) / (2 * cost) : (nb - 1) * G + (2 * (rest - head) + cost_last) / (2 * cost_last));
+      const long long tail = at % G;
+      if (i > 0 && i < n_pairs && tail <= snap && 2 * snap < G && at - tail > p.bounds[i - 1]) at -= tail;
+      p.bounds[i] = (int)at;
     }
   }
   // two slots of 2 x NT x 128 floats per pair, (launches of one context do not overlap on the GPU)

@@ -182,3 +182,20 @@ def test_last_token_block_of_its_own_size(ctx, M):
         assert same(runs[0], runs[1]) and torch.all(buf[M:] == 7.0) and torch.all(buf[:, n:] == 7.0)
         assert H.rel_fro(runs[0].cpu().numpy(), ref.cpu().numpy()) <= 2e-4
     assert ctx.last_status() == rb.ROSAQ_OK
+
+
+@pytest.mark.parametrize("d_in,n,M", [(1408, 9000, 1300), (1280, 10672, 300), (896, 3000, 520), (384, 4768, 1782), (256, 6840, 1127)])
+def test_equal_shares_without_short_ends(ctx, d_in, n, M):
+    """Shares that would end with the first groups of a tile end with the tile before it, where a tile has three groups and more (here 11, 10,
+    7, 3 and 2; shares of 7 to 29 groups)."""
+    rng = synth.rng_for(98, "ends", d_in, M)
+    x = dev(rng.standard_normal((M, d_in)).astype(np.float16))
+    w = ctx.quantize(dev(synth.weights(d_in, n, seed=98, key="ends", outlier_frac=0.01)), None, bits=4, k_salient=128)
+    ctx.set_linear_impl(3)
+    ref = ctx.linear(x, w).clone()
+    ctx.set_linear_impl(5)
+    runs = [ctx.linear(x, w).clone() for _ in range(2)]
+    ctx.set_linear_impl(0)
+    assert ctx.last_status() == rb.ROSAQ_OK
+    assert same(runs[0], runs[1])
+    assert (runs[0].double() - ref.double()).norm() <= 2e-4 * ref.double().norm()
