@@ -76,10 +76,10 @@ typedef struct {
 /* ---- context ---------------------------------------------------------------- */
 
 /* Creates a context on CUDA device `device` (must be compute capability 10.x, else
- * ROSAQ_ERR_UNSUPPORTED_ARCH).  Allocates a small device status word, the workspace
- * through which the CTAs of one rosaq_linear launch exchange partial output tiles
- * (64 KB per CTA of a two-CTAs-per-SM grid, 19 MB on a 148-SM device, plus 4 KB of
- * counters) and, lazily at the first call that needs it, a workspace for the rotated
+ * ROSAQ_ERR_UNSUPPORTED_ARCH).  Allocates a small device status word, the workspaces
+ * through which the CTAs of one launch exchange partial output tiles (97 MB on a 148-SM device: 64 KB per CTA of a
+ * two-CTAs-per-SM grid for single linears, twice that for plans and for the large-batch tiles each), counters and 64 KB
+ * between a rotation and its linears, and, lazily at the first call that needs it, a workspace for the rotated
  * activations.  A workspace that a later call outgrows stays allocated until the context is destroyed (at most twice
  * the largest one in all), so that launches captured before keep working.  A context serves one stream at a time: calls on different streams
  * that overlap in time need a context each.  Synchronous. */
@@ -220,7 +220,8 @@ int rosaq_rotate(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const rosaq_
  * (code - zero) * scale rounded to fp16; fp32 accumulation; y rounded once to fp16.
  *   r == NULL : x is already rotated (only the GEMM stage runs)
  *   r != NULL : x . R goes through the context workspace (grown on demand: this call
- *               may then allocate once), then the GEMM stage runs
+ *               may then allocate once), then the GEMM stage runs; small calls of up to eight tokens
+ *               run both in one launch
  * Only the first d_out columns of each y row are written.  ldx, ldy multiples of 8.
  * Any M >= 1.  The kernel is chosen by size: up to 128 tokens the weight-streaming kernels; larger batches run, where an
  * estimate says that it pays, on tiles of 256 columns x up to 256 tokens shared by two CTAs on adjacent SMs
@@ -251,7 +252,7 @@ int rosaq_linear_multi(rosaq_ctx *ctx, const void *x, int M, int64_t ldx, const 
  * All CTAs of the grid stream the operands of the whole list back to back; an operation whose input is
  * another operation's output starts when that output is complete.  It pays off for long lists (the ten
  * operations of a 7B decoder layer: 51 us in a burst, 60 us under the power cap, against 84 us as seven calls); for one or
- * two operations the single calls are faster (rotation + 4096 -> 4096 linear: 26.5 us as a plan, 18.5 us as rosaq_linear).
+ * two operations the single calls are faster (rotation + 4096 -> 4096 linear at 64 tokens: 20.8 us as a plan, 17.8 us as rosaq_linear).
  *   op.r / op.w  exactly one is non-NULL: the operation is y = x . R, or y = x . W^ (x already rotated)
  *   op.x, ldx    DEVICE [M][ldx] fp16 input; ignored when x_from >= 0
  *   op.x_from    -1, or the index (smaller than this operation's) of the operation whose y is this one's
@@ -314,9 +315,9 @@ int rosaq_plan_ctas(rosaq_ctx *ctx);
  * range is a sequence of pieces (the groups of one tile).  Writes piece_begin[0..n_ctas] (CTA c owns pieces
  * piece_begin[c] .. piece_begin[c + 1] - 1, in the order it processes them) and, for the first max_pieces
  * pieces, twelve int32 each: operation, tile, first group, end group, holders of the tile (copy), this
- * piece's position among them (ascending K), first partial-tile slot, arrival counter, closer index (-1: the
- * piece only contributes its partial tile; k >= 0: its CTA adds the partial tiles of token rows k,
- * k + closers, ...), closers, and the token rows [begin, end) out of 64 that the tile (copy) writes.
+ * piece's position among them (ascending K), first partial-tile slot, number of the shared tile (no kernel uses it), closer
+ * index (-1: the piece only contributes its partial tile; k >= 0: its CTA adds the partial tiles for the k-th of `closers`
+ * consecutive shares of the token rows), closers, and the token rows [begin, end) out of 64 that the tile (copy) writes.
  * All arrays HOST.  Returns the total number of pieces, or a negative status.
  */
 int rosaq_plan_schedule(int n_ops, const int32_t *n_tiles, const int32_t *groups, const int32_t *g_fp16,

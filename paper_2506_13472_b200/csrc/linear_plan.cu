@@ -86,7 +86,7 @@ struct alignas(64) PlParams {
   PlProblem prob[kPlanMaxOps];
   const PlanSeg *segs;
   const int *seg_begin;       // [CTAs + 1]
-  float *partials;            // [slot][token][128 columns]
+  float *partials;            // [slot][token / 4][128 columns][4 tokens]
   unsigned *sync;             // kPlSyncFinished, then two sets of kPlSyncSet words: done counters, wiped counter
   int *status;
   long long wait_limit;
@@ -108,7 +108,7 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *ptr) {
 __device__ __forceinline__ PlanSeg make_seg(const uint4 &a, const uint4 &b, const uint4 &c) {
   PlanSeg r;
   r.prob = a.x, r.tile = a.y, r.g_begin = a.z, r.g_end = a.w;
-  r.n_contrib = b.x, r.contrib_idx = b.y, r.slot0 = b.z, r.counter = b.w;
+  r.n_contrib = b.x, r.contrib_idx = b.y, r.slot0 = b.z, r.shared_idx = b.w;
   r.closer_idx = c.x, r.n_closers = c.y, r.tok_begin = c.z, r.tok_end = c.w;
   return r;
 }
@@ -219,8 +219,8 @@ __device__ __forceinline__ void epi_load_acc(uint32_t d_addr, int c0, float *acc
 }
 
 // Finishes tokens [c_begin, c_end) of one output column from the accumulator in tensor memory: adds, when
-// `keep`, the partial tiles 1 .. S-1 of the workspace in that order (this CTA's groups come first), rounds
-// once and writes the rows inside [t0, t1).  Two holders' quads of CH tokens are in flight per thread.  False: gave up.
+// `keep`, the partial tiles 1 .. S-1 of the workspace in that order (this CTA's groups come first; S is 2 then), rounds
+// once and writes the rows inside [t0, t1).  False: gave up.  (Without the loop plans of one to ten operations took 2 % longer.)
 template <int CH>
 __device__ __forceinline__ bool epi_finish(const Abort &ab, uint32_t d_addr, int c_begin, int c_end, bool keep, int S, float *src0,
                                            long long slot_floats, bool n_ok, int t0, int t1, __half *y_col, long long ldy) {
@@ -229,23 +229,15 @@ __device__ __forceinline__ bool epi_finish(const Abort &ab, uint32_t d_addr, int
     float acc[CH];
     epi_load_acc<CH>(d_addr, c0, acc);
     if (keep) {
-      for (int i = 1; i < S; i += 2) {
-        float *src[CH / 2];
-        float w[CH / 2][4];
+      for (int i = 1; i < S; ++i) {
+        float *src[CH / 4];
+        float w[CH / 4][4];
 #pragma unroll
-        for (int k = 0; k < CH / 4; ++k) {
-          const bool mine = c0 + 4 * k < t1 && c0 + 4 * k + 4 > t0;
-          float *at = src0 + (long long)i * slot_floats + (c0 / 4 + k) * kQuadFloats;
-          src[k] = mine ? at : nullptr;
-          src[CH / 4 + k] = mine && i + 1 < S ? at + slot_floats : nullptr;
-        }
+        for (int k = 0; k < CH / 4; ++k)
+          src[k] = c0 + 4 * k < t1 && c0 + 4 * k + 4 > t0 ? src0 + (long long)i * slot_floats + (c0 / 4 + k) * kQuadFloats : nullptr;
         if (!take_quads(ab, src, w)) return false;
 #pragma unroll
         for (int e = 0; e < CH; ++e) acc[e] = __fadd_rn(acc[e], w[e / 4][e % 4]);
-        if (i + 1 < S) {
-#pragma unroll
-          for (int e = 0; e < CH; ++e) acc[e] = __fadd_rn(acc[e], w[CH / 4 + e / 4][e % 4]);
-        }
       }
     }
     __half *yp = y_col + (long long)c0 * ldy;
@@ -603,8 +595,8 @@ linear_plan_kernel(const __grid_constant__ PlParams p) {
       const long long ldy = P.ldy;
       const int S = s.n_contrib;
       const bool sole = S == 1;
-      // the only closer of a shared tile (it holds the tile's first groups) keeps its accumulator and adds
-      // the other holders' partial tiles to it
+      // the only closer of a shared tile keeps its accumulator and adds the other holder's partial tile to it (all holders of a tile but the
+      // last close it: there are two, and the closer holds the first groups)
       const bool keep = !sole && s.n_closers == 1 && s.closer_idx == 0;
       // (the two CTAs of a pair exchange their own tiles: slots are interleaved by rank)
       const long long slot_step = (long long)tile_mul * p.slot_floats;            // from one holder's slot to the next
@@ -778,7 +770,7 @@ int plan_build_schedule(const std::vector<PlanGeom> &ops, int n_ctas, const int 
   }
   // Phases: an operation runs after the one whose output it reads.  Operations that neither read nor feed
   // another one go BETWEEN the producers and their consumers: while the CTAs work through them, the
-  // epilogue warps close the producers' shared tiles in the background (partial tiles through L2, counters:
+  // epilogue warps close the producers' shared tiles in the background (partial tiles through L2:
   // 6 to 9 us on a 7B layer), so that the consumers' activation copies find those outputs complete.
   std::vector<char> feeds(n, 0);
   bool any_dep = false, any_free = false;
@@ -793,8 +785,8 @@ int plan_build_schedule(const std::vector<PlanGeom> &ops, int n_ctas, const int 
   }
   std::vector<std::vector<PlanSeg>> per_cta(n_ctas);
   out->done_target.assign(n, 0u);
-  out->n_counters = 0;
   out->n_slots = 0;
+  int n_shared = 0;
   struct Holder {
     int cta, seg;      // position in per_cta[cta]
     bool last;         // the last piece of that CTA's range in this phase
@@ -880,12 +872,12 @@ int plan_build_schedule(const std::vector<PlanGeom> &ops, int n_ctas, const int 
         s.n_contrib = S;
         s.contrib_idx = j;
         s.slot0 = out->n_slots;
-        s.counter = out->n_counters;
+        s.shared_idx = n_shared;
         s.n_closers = n_closers;
         s.closer_idx = h[j].last ? ci++ : -1;
       }
       out->n_slots += S;
-      out->n_counters += 1;
+      n_shared += 1;
       out->done_target[tiles[k].op] += (unsigned)n_closers;
     }
   }

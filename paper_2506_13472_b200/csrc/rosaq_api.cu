@@ -163,10 +163,11 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
 // The persistent launch (rosaq_plan) pays off when a list is long: it saves a launch, a pipeline fill and a
 // drain per operation, but a list of one or two operations exposes its own fixed costs (the exchange of
 // shared tiles goes through L2 instead of a cluster's shared memory, and the phase after a rotation starts
-// only when the rotation's last tile is written).  Measured at 64 tokens, 4096 -> 4096 INT4: a GEMM stage
-// alone 13.6 us against 8.4 us on the per-call kernel; rotation + linear 26.5 us against 18.5 us as two
-// launches; the ten operations of a 7B decoder layer 51 us (60 under the power cap) against 84 us as seven calls.  So the single
-// calls stay on the per-call kernels; implementation 4 routes them through the persistent launch.
+// only when the rotation's last tile is written).  us in a chain of launches, as calls / as a plan, 4096 channels INT4 at 64 and 128 tokens:
+// 4096 -> 4096 alone 7.9 / 9.8, 11.4 / 13.2; rotation + it 17.8 / 20.8, 24.6 / 27.3; rotation + three 23.3 / 27.0, 32.1 / 35.7; the ten operations
+// of a 7B decoder layer 84 in seven calls, 51 (60 under the power cap) as one plan.  So the single calls stay on the per-call kernels;
+// implementation 4 routes them through the persistent launch.  (Two wide weights are already faster as a plan: 4096 -> 2 x 11008 21.3 / 19.1, 30.0 / 24.4, with
+// the rotation 31.6 / 30.0, 43.3 / 38.2; a call does not make use of it.)
 bool use_plan(const rosaq_ctx *ctx, int M, bool with_rotation) {
   (void)with_rotation;
   return M <= 64 && ctx->impl == 4;
@@ -784,7 +785,7 @@ int rosaq_plan_schedule(int n_ops, const int32_t *n_tiles, const int32_t *groups
     const PlanSeg &g = s.segs[k];
     int32_t *o = pieces + (size_t)k * 12;
     o[0] = g.prob, o[1] = g.tile, o[2] = g.g_begin, o[3] = g.g_end, o[4] = g.n_contrib, o[5] = g.contrib_idx;
-    o[6] = g.slot0, o[7] = g.counter, o[8] = g.closer_idx, o[9] = g.n_closers, o[10] = g.tok_begin, o[11] = g.tok_end;
+    o[6] = g.slot0, o[7] = g.shared_idx, o[8] = g.closer_idx, o[9] = g.n_closers, o[10] = g.tok_begin, o[11] = g.tok_end;
   }
   return total;
 }

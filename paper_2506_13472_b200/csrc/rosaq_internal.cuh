@@ -196,8 +196,8 @@ struct PlanSeg {
   int n_contrib;        // CTAs that hold groups of this tile (1: the tile is this CTA's alone)
   int contrib_idx;      // this CTA's position among them, ascending K
   int slot0;            // partial-tile slot of holder 0; holder i uses slot0 + i
-  int counter;          // the tile's arrival counter
-  int closer_idx;       // >= 0: this CTA adds the partial tiles for token rows closer_idx, + n_closers, ...
+  int shared_idx;       // number of the shared tile in the launch (for rosaq_plan_schedule; no kernel reads it)
+  int closer_idx;       // >= 0: this CTA adds the partial tiles for that one of n_closers consecutive shares of the token rows
   int n_closers;
   int tok_begin, tok_end;   // token rows of y this piece writes when it finishes the tile (a whole tile: all)
 };
@@ -213,7 +213,7 @@ struct PlanGeom {
 struct PlanSchedule {
   std::vector<PlanGeom> geom;
   int cost[3];
-  int n_ctas = 0, n_counters = 0, n_slots = 0;
+  int n_ctas = 0, n_slots = 0;
   std::vector<PlanSeg> segs;          // per CTA, in processing order
   std::vector<int> seg_begin;         // [n_ctas + 1]
   std::vector<unsigned> done_target;  // per problem: finishing events that complete it
