@@ -25,7 +25,8 @@ pytestmark = pytest.mark.gpu
     (np.float16, 300, 704, 8),        # head blocks that start inside a block of 64 channels: 88 channels,
     (np.float16, 90, 576, 4),         # 144 (two row tiles),
     (np.float16, 200, 4160, 8),       # 520 (pairs)
-    (np.float32, 70, 136, 1)])        # one split
+    (np.float32, 70, 136, 1),         # one split
+    (np.float32, 515, 2048, 1)])      # 136 tiles in two: steps of eight, mirrored shares
 def test_calib_cov_splits(dtype, n_tokens, d, n_blocks):
     X = synth.ActivationLaw(d, 1.0, seed=47, key=f"covs{d}").sample(n_tokens, "X", dtype)
     dh, half = d // n_blocks, n_tokens // 2 // 8 * 8
@@ -115,10 +116,11 @@ def test_a_long_calib_cov_does_not_use_up_the_waits_of_the_launch_behind_it():
         ctx.close()
 
 
-@pytest.mark.parametrize("n_tokens,n_blocks", [(509, 14), (509, 15), (7, 1), (17, 2)])
+@pytest.mark.parametrize("n_tokens,n_blocks", [(509, 14), (509, 15), (7, 1), (17, 2), (515, 14), (519, 15)])
 def test_calib_cov_either_step_of_the_fp32_kernel(n_tokens, n_blocks):
     """The fp32 kernel steps through sixteen tokens at a time where an SM has one CTA (up to 118 of them on 148 SMs), else through eight:
-    both sides of the line, tokens that fill no whole step, one step, less than one."""
+    both sides of the line (515 and 519 tokens in eight parts: 112 and 120 CTAs; 509 only in four), tokens that fill no whole step, one
+    step, less than one."""
     d = 128 * n_blocks
     X = synth.ActivationLaw(d, 1.0, seed=49, key=f"covk{d}").sample(n_tokens, "X", np.float32)
     ctx = rb.Context(0)
@@ -188,3 +190,26 @@ def test_calib_cov_behind_one_that_gave_up(d):
             assert ctx.last_status() == rb.ROSAQ_OK
     finally:
         ctx.close()
+
+
+def test_calib_cov_of_values_that_are_no_numbers():
+    """A NaN and an infinity in one channel each, on the pairs that take tiles in turn (91 tiles): their rows and columns of C hold nothing
+    finite, everything else has the bits that it has without them."""
+    n_tokens, d = 200, 3328
+    X = torch.randn((n_tokens, d), generator=torch.Generator().manual_seed(54)).half().cuda()
+    X[5, 100], X[150, 3000] = 0, 0
+    ctx = rb.Context(0)
+    try:
+        want = torch.zeros((d, d), device="cuda")
+        ctx.calib_cov(X, want)
+        X[5, 100], X[150, 3000] = float("nan"), float("inf")
+        C = torch.zeros((d, d), device="cuda")
+        ctx.calib_cov(X, C)
+        assert ctx.last_status() == rb.ROSAQ_OK
+    finally:
+        ctx.close()
+    keep = torch.ones(d, dtype=torch.bool, device="cuda")
+    keep[100] = keep[3000] = False
+    assert torch.equal(C[keep][:, keep], want[keep][:, keep])
+    assert torch.all(torch.isnan(C[100])) and torch.all(torch.isnan(C[:, 100]))
+    assert not torch.any(torch.isfinite(C[3000])) and not torch.any(torch.isfinite(C[:, 3000]))

@@ -274,10 +274,36 @@ def test_plan_behind_one_that_gave_up(ctx, M, d, d_out):
         finally:
             ctx.set_wait_limit(old)
         if read:
-            assert ctx.last_status() in (rb.ROSAQ_OK, rb.ROSAQ_ERR_TIMEOUT)
+            assert ctx.last_status() == rb.ROSAQ_ERR_TIMEOUT
         for _ in range(3):
             y.fill_(float("nan"))
             plan.run()
             assert torch.equal(y.view(torch.int16), want.view(torch.int16))
-        assert ctx.last_status() in (rb.ROSAQ_OK, rb.ROSAQ_ERR_TIMEOUT)
+        assert ctx.last_status() == (rb.ROSAQ_OK if read else rb.ROSAQ_ERR_TIMEOUT)
+    plan.free()
+
+
+@pytest.mark.parametrize("M,d,d_out", [(16, 1024, 640), (64, 4096, 4096), (100, 1024, 3000)])
+def test_plan_with_values_that_are_no_numbers(ctx, M, d, d_out):
+    """A NaN and an infinity in the input of a plan whose tiles are shared: their partial sums, which no reader may take for a slot that is still
+    empty, reach the output rows of their tokens, all other rows keep their bits, and so does the plan's next run."""
+    rng = synth.rng_for(33, "nan", M, d)
+    w = ctx.quantize(dev(synth.weights(d, d_out, 33, "nan", outlier_frac=0.01)), None, bits=4, k_salient=128)
+    clean = dev(rng.standard_normal((M, d)).astype(np.float16))
+    x, y = clean.clone(), empty(M, d_out)
+    plan = ctx.plan_create(M, [(x, None, w, y)])
+    plan.run()
+    want = y.clone()
+    for i in range(3):
+        x.copy_(clean)
+        x[3, 5 + i * d // 3], x[M - 1, 9 + i * d // 3] = float("nan"), float("inf")     # (in the first, a middle and the last holder's groups)
+        plan.run()
+        assert ctx.last_status() == rb.ROSAQ_OK
+        assert torch.all(torch.isnan(y[3])) and not torch.any(torch.isfinite(y[M - 1]))
+        rest = [r for r in range(M) if r not in (3, M - 1)]
+        assert torch.equal(y[rest].view(torch.int16), want[rest].view(torch.int16))
+        x.copy_(clean)
+        plan.run()
+        assert torch.equal(y.view(torch.int16), want.view(torch.int16))
+    assert ctx.last_status() == rb.ROSAQ_OK
     plan.free()

@@ -127,7 +127,8 @@ def test_rotation_and_linears_in_one_launch(ctx, kind, d, widths, bits):
             old = ctx.set_wait_limit(1)
             ctx.linear_multi(x, ws, r)
             ctx.set_wait_limit(old)
-            assert ctx.last_status() in (rb.ROSAQ_OK, rb.ROSAQ_ERR_TIMEOUT)
+            status = ctx.last_status()                     # (the smallest may be done before the second poll)
+            assert status == rb.ROSAQ_ERR_TIMEOUT or (status == rb.ROSAQ_OK and widths != [2688])
         for _ in range(3):
             assert all(same(y, v) for y, v in zip(ctx.linear_multi(x, ws, r), want))
             assert same(ctx.linear(x, ws[0], r), want[0])
@@ -143,8 +144,9 @@ def test_rotation_and_linears_in_one_launch(ctx, kind, d, widths, bits):
 
 @pytest.mark.parametrize("M,d_in,widths,bits", [
     (1, 4736, [4736], 4),               # 40 units: eight warps, the most slices with an SM each ...
-    (1, 4864, [4600, 136], 4),          # ... 41: sixteen, the last round nearly empty; a ragged tile, two weights
-    (1, 4864, [4744], 4),               # one tile more
+    (1, 4864, [4472, 136], 4),          # ... 41: sixteen, the last round nearly empty; the most slices, a ragged tile, two weights
+    (1, 4864, [4600, 136], 4),          # one tile more: eight
+    (1, 4864, [4744], 4),
     (2, 4096, [328], 3),                # 35 and
     (7, 4224, [328], 3),                # 36 units of INT3
     (5, 13824, [2048], 4),              # x' of the most tokens next to the rings of sixteen warps,
