@@ -148,9 +148,9 @@ int run_gemm(rosaq_ctx *ctx, const __half *x, int M, long long ldx, int n, const
   // More than 128 tokens may run on 256-column tiles shared by pairs of CTAs, one dequantisation per 256 tokens; the
   // estimates of the two kernels decide.  Over 2000 launches the pick is 0.6 % slower than the fastest of the two and their
   // cuts on average, by more than 10 % on 34 (the constants were fitted to these kernels before their last changes); the margin keeps
-  // small launches, where the estimates err most, on the per-call kernel.  Per-call kernel / pairs, measured (us): 13824 -> 128 at 160 tokens 11.7 / 17.1, 4096 -> 4096 at 200 13.0 / 16.3, at 768
-  // 28.7 / 28.7, 4096 -> 11008 at 1900 160 / 138, 4096 -> 3 x 4096 at 200 27.0 / 25.9, 5120 x 5120 rotation at 200 18.8 / 17.1, at
-  // 1900 130 / 84.
+  // small launches, where the estimates err most, on the per-call kernel.  Per-call kernel / pairs, measured (us): 13824 -> 128 at
+  // 160 tokens 11.7 / 17.1, 4096 -> 4096 at 200 13.8 / 17.9, at 1900 62.4 / 60.2, 4096 -> 11008 at 1900 149 / 127, 4096 -> 3 x 4096 at 200 30.4 / 29.1,
+  // 5120 x 5120 rotation at 200 21.3 / 19.6, at 1900 126 / 77.5.
   constexpr double kMarginUs = 0.4;
   if (prefill_supported(*ts[0], col_map) && (ctx->impl == 5 || (ctx->impl == 0 && M > 128))) {
     const PrefillCut cut = prefill_choose(ctx, M, n, ts);
